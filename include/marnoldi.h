@@ -300,7 +300,10 @@ int marnoldi_member_energy(marnoldi_ctx *ctx, int member, double *band_energy, d
 int marnoldi_set_member_temperatures(marnoldi_ctx *ctx, int n_members, const double *kT);
 
 /*
- * Launch-shape autotuner of the Gram-Schmidt kernel (process-wide).
+ * Launch-shape autotuner of the Gram-Schmidt kernel (process-wide).  A shape is
+ * reported as values per thread and threads per CTA of the partial sums: a CTA
+ * thread of the kernel may carry several of these "threads" (four at present),
+ * which changes no sum.
  *   marnoldi_set_autotune: mode 0 (default, also when MARNOLDI_AUTOTUNE is
  *     unset or not "1") uses a fixed rule: 256 threads per CTA up to m = 4096,
  *     512 for FP32 vectors up to 8192, the streamed kernel for longer FP32

@@ -1,5 +1,5 @@
 // Device helpers shared by the Gram-Schmidt kernels (krylov.cu, gs_stream.cu):
-// error-free FP32 dot accumulators, fixed-order CTA reductions, and the FP64
+// error-free FP32 dot accumulators, fixed-order warp reductions, and the FP64
 // scalar step of one Krylov step (norm, breakdown test, the Gram matrix's new
 // column, the new row of L^-1 and the projection coefficients).
 #pragma once
@@ -86,60 +86,10 @@ template <> struct DotAcc<float> {
 };
 
 
-// Two FP32 lanes per instruction (add/sub/mul/fma .rn.f32x2, sm_100 and
-// later): each lane is rounded exactly as the scalar instruction would be, so
-// a pair of independent sums runs at half the instruction count.  The pairs
-// are formed and split inside the PTX (mov.b64 of two 32-bit registers), so
-// that the register allocator can keep them as register pairs.
-__device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c)
-{
-    float2 d;
-    asm("{\n\t.reg .b64 a, b, c, d;\n\t"
-        "mov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
-        "fma.rn.f32x2 d, a, b, c;\n\t"
-        "mov.b64 {%0, %1}, d;\n\t}"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return d;
-}
-
-// Two DotAcc<float> side by side (lane x and lane y), updated with packed
-// instructions: per lane the operations of DotAcc<float>::add (p = a b,
-// e = fma(a, b, -p), the two-sum of hi and p, lo += e + err).
-struct DotAcc2 {
-    float2 hi = make_float2(0.f, 0.f), lo = make_float2(0.f, 0.f);
-    __device__ __forceinline__ void add(float2 a, float2 b)
-    {
-        asm("{\n\t.reg .b64 a, b, p, np, e, h, l, s, bb, t, u, err;\n\t"
-            "mov.b64 a, {%4, %5};\n\tmov.b64 b, {%6, %7};\n\t"
-            "mov.b64 h, {%0, %1};\n\tmov.b64 l, {%2, %3};\n\t"
-            "mul.rn.f32x2 p, a, b;\n\t"
-            "xor.b64 np, p, 0x8000000080000000;\n\t"
-            "fma.rn.f32x2 e, a, b, np;\n\t"
-            "add.rn.f32x2 s, h, p;\n\t"
-            "sub.rn.f32x2 bb, s, h;\n\t"
-            "sub.rn.f32x2 t, s, bb;\n\t"
-            "sub.rn.f32x2 t, h, t;\n\t"
-            "sub.rn.f32x2 u, p, bb;\n\t"
-            "add.rn.f32x2 err, t, u;\n\t"
-            "add.rn.f32x2 e, e, err;\n\t"
-            "add.rn.f32x2 l, l, e;\n\t"
-            "mov.b64 {%0, %1}, s;\n\tmov.b64 {%2, %3}, l;\n\t}"
-            : "+f"(hi.x), "+f"(hi.y), "+f"(lo.x), "+f"(lo.y)
-            : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    }
-    __device__ __forceinline__ DotAcc<float> lane(int q) const
-    {
-        DotAcc<float> r;
-        r.hi = q ? hi.y : hi.x;
-        r.lo = q ? lo.y : lo.x;
-        return r;
-    }
-};
-
 // Two adjacent FP32 values as one 64-bit register (lane x = the lower
-// address), and the packed (f32x2) operations on such pairs; each lane is
-// rounded exactly as the scalar instruction would be.
+// address), and the packed operations on such pairs (add/sub/mul/fma .rn.f32x2,
+// sm_100 and later): each lane is rounded exactly as the scalar instruction
+// would be, at half the instruction count.
 __device__ __forceinline__ uint64_t lds2(const float *p)
 {
     uint64_t r;
@@ -158,6 +108,7 @@ __device__ __forceinline__ uint64_t fma_x2(uint64_t a, uint64_t b, uint64_t c)
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
 }
+__device__ __forceinline__ uint64_t neg_x2(uint64_t a) { return a ^ 0x8000000080000000ull; }
 __device__ __forceinline__ float lane_x(uint64_t a) { return __uint_as_float((unsigned)a); }
 __device__ __forceinline__ float lane_y(uint64_t a) { return __uint_as_float((unsigned)(a >> 32)); }
 
@@ -184,6 +135,26 @@ struct PairAcc {
             : "+l"(hi), "+l"(lo)
             : "l"(a), "l"(b));
     }
+    // The same with nb = -b given: fma(a, -b, p) is the exact negative of e, and
+    // lo -= (-e - err) rounds as lo += (e + err), so the bits are add()'s without
+    // the two integer instructions that negate p.
+    __device__ __forceinline__ void add(uint64_t a, uint64_t b, uint64_t nb)
+    {
+        asm("{\n\t.reg .b64 p, e, s, bb, t, u, err;\n\t"
+            "mul.rn.f32x2 p, %2, %3;\n\t"
+            "fma.rn.f32x2 e, %2, %4, p;\n\t"
+            "add.rn.f32x2 s, %0, p;\n\t"
+            "sub.rn.f32x2 bb, s, %0;\n\t"
+            "sub.rn.f32x2 t, s, bb;\n\t"
+            "sub.rn.f32x2 t, %0, t;\n\t"
+            "sub.rn.f32x2 u, p, bb;\n\t"
+            "add.rn.f32x2 err, t, u;\n\t"
+            "sub.rn.f32x2 e, e, err;\n\t"
+            "sub.rn.f32x2 %1, %1, e;\n\t"
+            "mov.b64 %0, s;\n\t}"
+            : "+l"(hi), "+l"(lo)
+            : "l"(a), "l"(b), "l"(nb));
+    }
     // the two lanes' sums, joined by a two-sum
     __device__ __forceinline__ DotAcc<float> joined() const
     {
@@ -201,51 +172,7 @@ struct PairAcc {
 // Vectors per block of the Gram-Schmidt sweeps (one CTA reduction each).
 constexpr int kGsBlock = 4;
 
-template <int T>
-__device__ __forceinline__ int live_values(int cnt, int warp)
-{
-    constexpr int NW = T / 32;
-    return cnt > warp ? (cnt - warp + NW - 1) / NW : 0;
-}
-
-// f(v, live) over the thread's first nv values, chunk by chunk; a compiler
-// barrier between chunks keeps one chunk's loads live at a time, and only the
-// last live chunk tests its values.
-template <int VPT, int kChunk, typename F>
-__device__ __forceinline__ void for_live(int nv, F &&f)
-{
-#pragma unroll
-    for (int v0 = 0; v0 < VPT; v0 += kChunk) {
-        if (v0 >= nv) break;
-        if (v0 + kChunk <= nv) {
-#pragma unroll
-            for (int q = 0; q < kChunk && v0 + q < VPT; ++q) f(v0 + q, true);
-        } else {
-#pragma unroll
-            for (int q = 0; q < kChunk && v0 + q < VPT; ++q) f(v0 + q, v0 + q < nv);
-        }
-        if (v0 + kChunk < VPT) asm volatile("" ::: "memory");
-    }
-}
-
-// Barrier of a group of the CTA's threads: 0 = the whole CTA, else the named
-// barrier `bar` over `nthreads` threads (whole warps).
-__device__ __forceinline__ void group_sync(int bar, int nthreads)
-{
-    if (bar == 0) __syncthreads();
-    else asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nthreads) : "memory");
-}
-
-// Sum of N <= 16 per-thread accumulators over a group of warps (the CTA, or
-// one of its halves) in a fixed order.  In each warp a reduce-scatter
-// butterfly over NP = 2^ceil(log2 N) slots leaves slot q on lanes
-// q (32 / NP) .. (q + 1) (32 / NP) - 1 (each lane sends half of its slots per
-// round, so N values cost about as many shuffles as two); then warp w of the
-// group sums values w, w + gnw, ... over its warps and its lane 0 runs
-// epi(q, total).  `buf` alternates the partial slots (part holds
-// 2 x 16 x stride doubles, stride >= gnw) so that two barriers per reduction
-// suffice; `bar` selects the group's barrier (0: the CTA's).
-// The warp step of block_sum: a reduce-scatter butterfly over NP =
+// Sums of N <= 16 accumulators over a warp: a reduce-scatter butterfly over NP =
 // 2^ceil(log2 N) slots; slot q (q < N) ends, summed over the warp, on lanes
 // q (32 / NP) .. (q + 1) (32 / NP) - 1 (each lane sends half of its slots per
 // round, so N values cost about as many shuffles as two).  Returns the lane's
@@ -277,33 +204,6 @@ __device__ __forceinline__ DotAcc<VT> warp_scatter(const DotAcc<VT> (&in)[N])
     return a[0];
 }
 
-// Sum of N <= 16 per-thread accumulators over a group of warps (the CTA, or
-// one of its halves) in a fixed order: warp_scatter in each warp, then warp w
-// of the group sums values w, w + gnw, ... over its warps and its lane 0 runs
-// epi(q, total).  `buf` alternates the partial slots (part holds
-// 2 x 16 x stride doubles, stride >= gnw) so that two barriers per reduction
-// suffice; `bar` selects the group's barrier (0: the CTA's).
-template <typename VT, int N, typename Epi>
-__device__ __forceinline__ void block_sum(const DotAcc<VT> (&in)[N], double *part, int &buf, Epi epi,
-                                          int gwarp, int gnw, int stride, int bar)
-{
-    constexpr int LOGN = N > 8 ? 4 : N > 4 ? 3 : N > 2 ? 2 : N > 1 ? 1 : 0;
-    const int lane = threadIdx.x & 31;
-    const DotAcc<VT> a0 = warp_scatter(in);
-    const int qm = lane >> (5 - LOGN);
-    if ((lane & ((32 >> LOGN) - 1)) == 0 && qm < N) part[(buf * 16 + qm) * stride + gwarp] = a0.pack();
-    group_sync(bar, gnw * 32);
-    for (int q = gwarp; q < N; q += gnw) {
-        DotAcc<VT> x;
-        if (lane < gnw) x.unpack(part[(buf * 16 + q) * stride + lane]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x.merge(x.shfl_xor(o));
-        if (lane == 0) epi(q, x.value());
-    }
-    group_sync(bar, gnw * 32);
-    buf ^= 1;
-}
-
 // sum over the warp of x (every lane holds the total)
 __device__ __forceinline__ double warp_total(double x)
 {
@@ -312,12 +212,31 @@ __device__ __forceinline__ double warp_total(double x)
     return x;
 }
 
+// Totals over the warp of eight values per lane: lane l gets that of x[l / 4].
+// A reduce-scatter over lanes 16, 8, 4 apart, then 2 and 1: nine additions for
+// eight totals, where eight calls of warp_total take forty (an FP64 addition
+// holds the SM's two-lane FP64 pipe for 16 cycles per warp).  Each total is the
+// sum of the same pairs in the same tree as warp_total's, so the bits are equal.
+__device__ __forceinline__ double warp_total8(const double (&x)[8])
+{
+    const int lane = threadIdx.x & 31;
+    double a[4], b[2];
+    const bool u16 = (lane & 16) != 0, u8 = (lane & 8) != 0, u4 = (lane & 4) != 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        a[j] = (u16 ? x[j + 4] : x[j]) + __shfl_xor_sync(kFull, u16 ? x[j] : x[j + 4], 16);
+#pragma unroll
+    for (int j = 0; j < 2; ++j) b[j] = (u8 ? a[j + 2] : a[j]) + __shfl_xor_sync(kFull, u8 ? a[j] : a[j + 2], 8);
+    double c = (u4 ? b[1] : b[0]) + __shfl_xor_sync(kFull, u4 ? b[0] : b[1], 4);
+    c += __shfl_xor_sync(kFull, c, 2);
+    return c + __shfl_xor_sync(kFull, c, 1);
+}
+
 // Shared-memory arrays of the scalar step (length >= nu each).
 template <typename VT>
 struct GsScalarSmem {
     double *ssc;    // s_i (i < n) in, s_n set here
-    double *ta;     // sweep totals a_i = w_i . u
-    double *tb;     // b_i = (S w_i) . u
+    double *tb;     // sweep totals b_i = (S w_i) . u
     double *tg;     // g_i = (S w_i) . w_n
     double *lrow;   // L^-1 G_{<n, n}
     double *nrow;   // the new row n of L^-1
@@ -329,21 +248,24 @@ struct GsScalarSmem {
 
 // The FP64 scalar step of Krylov step n for column c, run by the T threads
 // (thread index tid) that `sync` synchronises, after the sweep's totals are in
-// ta, tb, tg: beta_n and the breakdown test, s_n, G's column n and the entries
-// h_{m,n} of unit-norm vectors (into Hsub), the new row of L^-1 (into Lsub),
-// and, when need_w, the coefficients c = L^-T L^-1 p of s_n u into coef and
-// |L^-1 p|^2 into cn2[c].  Returns true when the subtraction w_{n+1} = s_n u -
-// sum coef_i w_i follows (false: the column stopped, or the last step).  Lsub
-// holds L^-1 (lower triangular), so every product is a matrix-vector product,
-// one warp per row or column, with no serial chain.
+// tb, tg: beta_n and the breakdown test, s_n, G's column n, the new row of
+// L^-1 (into Lsub), and, when need_w, the coefficients c = L^-T L^-1 p of
+// s_n u into coef and |L^-1 p|^2 into cn2[c].  Returns false when the column
+// stopped.  Lsub holds L^-1 (lower triangular), so every product is a
+// matrix-vector product with no serial chain; a warp takes eight rows (or
+// columns) at a time and reduces them together (warp_total8), and the two
+// products with the same rows (L^-1 G_{<n,n} and L^-1 p) share one pass.  The
+// step is bound by the FP64 pipe: one total per row and product spent 5 of
+// about 6.5 FP64 instructions per row on its reduction at nu = 100.
 template <typename VT, int T, typename Sync>
 __device__ __forceinline__ bool gs_scalars(int c, int n, int nu, int need_w, double tau2, int tid,
-                                           double *__restrict__ Hsub, double *__restrict__ Lsub,
+                                           double *__restrict__ Lsub,
                                            double *__restrict__ scale, double *__restrict__ cn2,
                                            int *__restrict__ status, int *__restrict__ nu_eff,
                                            GsScalarSmem<VT> sm, Sync sync)
 {
     const int warp = tid >> 5, lane = tid & 31;
+    constexpr int NW = T / 32;
     double *Lc = Lsub + (int64_t)c * nu * nu;   // L^-1, row-major, lower triangle
     if (tid == 0) {
         double sn = 1.0;   // slot 0 is stored normalised (G_00 = 1)
@@ -368,22 +290,35 @@ __device__ __forceinline__ bool gs_scalars(int c, int n, int nu, int need_w, dou
     sync();
     if (sm.stop) return false;
     const double sn = sm.ssc[n];
-    for (int m = tid; m <= n; m += T) {   // G_{mn}, p_m (of s_n u) and h_m of unit-norm vectors
+    for (int m = tid; m <= n; m += T) {   // G_{mn} and p_m (of s_n u) of unit-norm vectors
         const double f = sm.ssc[m] * sn;
         sm.tg[m] *= f;
         sm.tb[m] *= f;
-        const double h = sm.ta[m] * f;
-        Hsub[((int64_t)c * nu + m) * nu + n] = h;
-        Hsub[((int64_t)c * nu + n) * nu + m] = h;
     }
     sync();
-    constexpr int NW = T / 32;
-    // l = L^-1 G_{<n, n}
-    for (int r = warp; r < n; r += NW) {
-        double x = 0.0;
-        for (int m = lane; m <= r; m += 32) x = fma(Lc[(int64_t)r * nu + m], sm.tg[m], x);
-        x = warp_total(x);
-        if (lane == 0) sm.lrow[r] = x;
+    // l = L^-1 G_{<n, n} and z = L^-1 p (rows below n)
+    for (int r0 = 8 * warp; r0 < n; r0 += 8 * NW) {
+        double x[8], y[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[j] = y[j] = 0.0;
+        const int mend = min(r0 + 8, n);
+        for (int m = lane; m < mend; m += 32) {
+            const double g = sm.tg[m], pm = need_w ? sm.tb[m] : 0.0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (m <= r0 + j && r0 + j < n) {
+                    const double l = Lc[(int64_t)(r0 + j) * nu + m];
+                    x[j] = fma(l, g, x[j]);
+                    if (need_w) y[j] = fma(l, pm, y[j]);
+                }
+        }
+        const int r = r0 + (lane >> 2);
+        const double tx = warp_total8(x);
+        if ((lane & 3) == 0 && r < n) sm.lrow[r] = tx;
+        if (need_w) {
+            const double ty = warp_total8(y);
+            if ((lane & 3) == 0 && r < n) sm.zc[r] = ty;
+        }
     }
     sync();
     // d = sqrt(G_nn - |l|^2), G_nn = 1; the new row of L^-1 is (-l^T L^-1, 1) / d
@@ -406,13 +341,21 @@ __device__ __forceinline__ bool gs_scalars(int c, int n, int nu, int need_w, dou
     if (sm.stop) return false;
     const double dinv = sm.dinv;
     double *Ln = Lc + (int64_t)n * nu;
-    for (int m = warp; m < n; m += NW) {
-        double x = 0.0;
-        for (int r = m + lane; r < n; r += 32) x = fma(sm.lrow[r], Lc[(int64_t)r * nu + m], x);
-        x = warp_total(x);
-        if (lane == 0) {
-            sm.nrow[m] = -dinv * x;
-            Ln[m] = -dinv * x;
+    for (int m0 = 8 * warp; m0 < n; m0 += 8 * NW) {
+        double x[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[j] = 0.0;
+        for (int o = lane; m0 + o < n; o += 32)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int r = m0 + j + o;
+                if (r < n) x[j] = fma(sm.lrow[r], Lc[(int64_t)r * nu + m0 + j], x[j]);
+            }
+        const int m = m0 + (lane >> 2);
+        const double tx = warp_total8(x);
+        if ((lane & 3) == 0 && m < n) {
+            sm.nrow[m] = -dinv * tx;
+            Ln[m] = -dinv * tx;
         }
     }
     if (tid == 0) {
@@ -420,23 +363,30 @@ __device__ __forceinline__ bool gs_scalars(int c, int n, int nu, int need_w, dou
         Ln[n] = dinv;
     }
     sync();
-    if (!need_w) return false;
-    // z = L^-1 p, |z|^2 = |projection of s_n u|_S^2, c = L^-T z
-    for (int r = warp; r <= n; r += NW) {
-        const double *Lr = r == n ? sm.nrow : Lc + (int64_t)r * nu;
+    if (!need_w) return true;
+    // z's last entry; then c = L^-T z and |z|^2 = |projection of s_n u|_S^2
+    if (warp == 0) {
         double x = 0.0;
-        for (int m = lane; m <= r; m += 32) x = fma(Lr[m], sm.tb[m], x);
+        for (int m = lane; m <= n; m += 32) x = fma(sm.nrow[m], sm.tb[m], x);
         x = warp_total(x);
-        if (lane == 0) sm.zc[r] = x;
+        if (lane == 0) sm.zc[n] = x;
     }
     sync();
-    for (int m = warp; m <= n; m += NW) {
-        double x = 0.0;
-        for (int r = m + lane; r <= n; r += 32) x = fma(r == n ? sm.nrow[m] : Lc[(int64_t)r * nu + m], sm.zc[r], x);
-        x = warp_total(x);
-        if (lane == 0) sm.coef[m] = (VT)(x * sm.ssc[m]);
+    for (int m0 = 8 * warp; m0 <= n; m0 += 8 * NW) {
+        double x[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[j] = 0.0;
+        for (int o = lane; m0 + o <= n; o += 32)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int r = m0 + j + o;
+                if (r <= n) x[j] = fma(r == n ? sm.nrow[m0 + j] : Lc[(int64_t)r * nu + m0 + j], sm.zc[r], x[j]);
+            }
+        const int m = m0 + (lane >> 2);
+        const double tx = warp_total8(x);
+        if ((lane & 3) == 0 && m <= n) sm.coef[m] = (VT)(tx * sm.ssc[m]);
     }
-    if (warp == 0) {
+    if (warp == NW - 1) {
         double x = 0.0;
         for (int r = lane; r <= n; r += 32) x = fma(sm.zc[r], sm.zc[r], x);
         x = warp_total(x);

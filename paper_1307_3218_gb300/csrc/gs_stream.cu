@@ -13,9 +13,7 @@
 // grouped differently over the threads, so results agree with gs_kernel's
 // shapes to rounding.
 //
-// What differs is how the vectors reach the arithmetic.  gs_kernel loads them
-// with the CTA's own threads, so its loads and its reductions alternate in
-// step and HBM idles during every block reduction.  Here a producer warp
+// What differs is how the vectors reach the arithmetic.  Here a producer warp
 // feeds a ring of R slots; a slot holds one chunk (2 T entries, T / 16 tiles
 // of 32, for T consumer threads) of the four vectors w_i and the four S w_i
 // of a block and of u = H w_n, its lo word and w_n, copied by cp.async.bulk
@@ -413,9 +411,18 @@ __global__ void __launch_bounds__(T + 32, MINB) gs_stream_kernel(
     named_sync(1, T);   // every block's totals are stored
 
     // ---- the FP64 scalar step over the consumer threads, then meet the producer
-    const GsScalarSmem<float> sm{ssc, ta, tb, tg, lrow, nrow, zc, coef, bc_stop, bc_dinv};
-    const bool go = gs_scalars<float, T>(c, n, nu, need_w, tau2, tid, Hsub, Lsub, scale, cn2, status, nu_eff,
-                                         sm, [] { named_sync(1, T); });
+    const GsScalarSmem<float> sm{ssc, tb, tg, lrow, nrow, zc, coef, bc_stop, bc_dinv};
+    const bool live = gs_scalars<float, T>(c, n, nu, need_w, tau2, tid, Lsub, scale, cn2, status, nu_eff, sm,
+                                           [] { named_sync(1, T); });
+    if (live) {
+        const double sn = ssc[n];
+        for (int m = tid; m <= n; m += T) {   // h_m of unit-norm vectors
+            const double h = ta[m] * (ssc[m] * sn);
+            Hsub[((int64_t)c * nu + m) * nu + n] = h;
+            Hsub[((int64_t)c * nu + n) * nu + m] = h;
+        }
+    }
+    const bool go = live && need_w;
     if (tid == 0) s_go = go ? 1 : 0;
     named_sync(2, T + 32);
     if (!go) {

@@ -19,11 +19,12 @@
 //
 // Inner products are accumulated to FP64 accuracy where the result needs it;
 // in mixed precision the vectors, the SpMM and the Gram-Schmidt updates are
-// FP32.  Reductions use a fixed order (warp butterflies, then one warp over
-// the warps), so results do not depend on scheduling.
+// FP32.  Reductions use a fixed order (trees over the lanes, then over the
+// warps), so results do not depend on scheduling.
 #include "gs_common.cuh"
 
 #include <cstdio>
+#include <type_traits>
 
 namespace marnoldi {
 
@@ -35,13 +36,14 @@ const char *kernel_name(int kind)
     return (kind >= 0 && kind < KK_NKINDS) ? names[kind] : "?";
 }
 
-// Vectors up to 4096 entries run 256-thread CTAs (several columns share an SM
-// and overlap each other's reductions).  Longer FP32 vectors up to 8192
-// entries run 512-thread CTAs of 16 values per thread (two per SM); longer
-// FP32 vectors run the streamed kernel (gs_stream.cu) with 256 consumer
-// threads of 64 values and a producer warp, two CTAs per SM (shape {64, 288};
-// {32, 544}, one CTA of 512 consumer threads per SM, is the other streamed
-// shape); the rest run 1024-thread CTAs.  VPT is the power of two that covers m.
+// A shape {vpt, threads} of gs_kernel names its partial sums: `threads` chains
+// of vpt values each (m_pad = vpt threads), on a CTA of threads / 4 threads.
+// Vectors up to 4096 entries take 256 chains, FP32 vectors up to 8192 entries
+// 512; longer FP32 vectors run the streamed kernel (gs_stream.cu) with 256
+// consumer threads of 64 values and a producer warp, two CTAs per SM (shape
+// {64, 288}; {32, 544}, one CTA of 512 consumer threads per SM, is the other
+// streamed shape); the rest take 1024 chains.  vpt is the power of two that
+// covers m.
 ColumnShape column_shape(int64_t m, int prec)
 {
     if (prec == 1 && m > 4096 && m <= 8192) return ColumnShape{16, 512, 8192};
@@ -239,296 +241,611 @@ __global__ void __launch_bounds__(256) spmm_hs_kernel(
 }
 
 // ------------------------------------------------------------------ Gram-Schmidt
-// One CTA of T threads (NW = T / 32 warps) per column; thread t owns the
-// values at positions p = t + v T (v < VPT) of the column's vectors, which are
-// stored in the column's tile order (tiles of 32 entries by hop count from the
-// column's atom).  Position tile k = w + NW v belongs to warp w, and vector i
-// vanishes past the first tcnt[i + 1] tiles (S w_i reaches one hop further
-// than w_i), so a warp's live values for vector i are its first
-// nv = ceil((tcnt[i + 1] - w) / NW): the sweeps stop there and read each
-// vector's support as one contiguous prefix.  The entries past a support are
-// exact zeros, so no sum changes.  T and m_pad = VPT T are compile-time
-// constants, so the offsets of the values and of the vector slots are load
-// immediates.
+// One CTA of T = C / 4 threads per column, for vectors of m_pad = nchunk C
+// entries.  Vectors are stored in the column's tile order (tiles of 32 entries
+// by hop count from the column's atom), and vector i vanishes past its first
+// tcnt[i + 1] tiles (S w_i reaches one hop further than w_i), so each sweep
+// reads a prefix; the entries past a support are exact zeros, so no sum
+// changes.  Thread t owns four entries of every chunk of C (FP32: positions
+// 4 t .. 4 t + 3, one 16-byte load; FP64: 2 t, 2 t + 1 and C / 2 further, two).
 //
 // Orthogonalisation (one pass, with the exact S-Gram matrix).  The stored
 // vectors w_i, scaled to unit S-norm (k_i = s_i w_i), are S-orthonormal only
 // up to rounding; their Gram matrix G = K^T S K = L L^T is kept exactly
 // through L^-1 (its new row every step from G's new column), so that every
-// solve with G is a pair of matrix-vector products.  Step n
-// forms, in one sweep over the stored vectors i <= n (blocks of kGsBlock
-// vectors, one CTA reduction each),
-//   a_i = w_i . u          H_sub entries of the stored basis (u = H w_n)
-//   b_i = (S w_i) . u      right-hand side of the S-projection of u
-//   g_i = (S w_i) . w_n    G's column n (g_n = beta_n^2)
-// then, in FP64 over the CTA, the S-projection coefficients c = G^-1 p of
-// s_n u onto span(K) and subtracts them in a streaming sweep with no
-// reductions: w_{n+1} = s_n u - sum_i c_i k_i.  Whatever rounding leaves
+// solve with G is a pair of matrix-vector products.  Step n makes two sweeps
+// over the stored vectors i <= n, in blocks of kGsBlock:
+//   1. over S w_i:  b_i = (S w_i) . u    right-hand side of the S-projection of u
+//                   g_i = (S w_i) . w_n  G's column n (g_n = beta_n^2)
+//      then, in FP64 over the CTA, the norm, the breakdown test and the
+//      S-projection coefficients c = G^-1 p of s_n u onto span(K);
+//   2. over w_i:    w_{n+1} = s_n u - sum_i c_i k_i, and
+//                   a_i = w_i . u        H_sub entries of the stored basis (u = H w_n)
+// a_i feeds nothing before the eigensolve, so it needs no sweep of its own:
+// two vector reads per stored vector and step, where a first sweep with a, b
+// and g and a second for the subtraction read three.  Whatever rounding leaves
 // along span(K) is carried by G, so the subspace problem, solved on
 // L^-1 H_sub L^-T, is the exact Rayleigh-Ritz projection on the stored
 // vectors.  The subspace is span{e_j, H e_j, ...} whatever the coefficients,
-// so in exact arithmetic this is the method's Arnoldi basis; per stored vector
-// and step it reads w_i and S w_i once for the coefficients and w_i once for
-// the subtraction (three vector reads, against four for two Gram-Schmidt
-// passes), and runs one reduction per block instead of two.
+// so in exact arithmetic this is the method's Arnoldi basis.
 //
 // In mixed precision a_i and g_i are accumulated error-free (exact FP32
 // products, two-sums, (hi, lo) pairs; the lo word of u, which only corrects
-// a_i by about 2^-24, through plain FMAs).  b_i is summed per thread with
-// plain FMAs (the CTA reduction stays accurate): its rounding only leaves a
-// component of w_{n+1} along span(K) at the level the FP32 subtraction leaves
-// anyway, which G records.  The coefficients and G are FP64.
-// u (and its lo word) and w sit in shared memory (or registers for small
-// VPT); w holds w_n during the coefficient sweep and w_{n+1} afterwards.
-template <typename VT, int VPT, int T>
-struct GsCfg {
-    static constexpr bool kLo = sizeof(VT) == 4;                    // u as (hi, lo) pair
-    static constexpr bool kWs = VPT >= (sizeof(VT) == 4 ? 8 : 4);    // w in smem
-    static constexpr bool kUs = kLo || !kWs || 2 * VPT * T * sizeof(VT) <= 160 * 1024;
-    static constexpr int kChunkDot = sizeof(VT) == 8 ? 1 : 2;        // values per batch of loads
-    static constexpr int kChunkUpd = sizeof(VT) == 8 ? 1 : 4;
-    static constexpr int kSmemVectors = (kUs ? 1 : 0) + (kLo ? 1 : 0) + (kWs ? 1 : 0);
+// a_i by about 2^-24, through plain FMAs).  b_i is summed with plain FMAs in C
+// chains per CTA (one per position modulo C; the sums of the chains stay
+// accurate): its rounding only leaves a component of w_{n+1} along span(K) at
+// the level the FP32 subtraction leaves anyway, which G records.  The chains
+// of b and g, and the tree that adds them up, are those of a CTA of C threads
+// of one entry per chunk each, so a shape's results do not depend on how many
+// of its chains a thread carries.  The coefficients and G are FP64.
+//
+// What bounds it: FP32 vectors, the issue slots (54 % at 0.51 of the HBM
+// bandwidth; about 32 FP32 operations per entry and stored vector, in packed
+// pairs) and the reductions, a fixed cost per warp and block of four vectors:
+// four entries per thread and chunk divide them by four against one thread per
+// chain.  FP64 vectors: the two-lane FP64 pipe, 93 % busy (four FMAs per entry
+// and stored vector).  Every copy goes through a ring in shared memory that
+// each thread fills for itself (cp.async), so that no registers wait for HBM
+// and a warp needs no barrier before its block's sums.
+// Per solve, against one thread per chain and a, b and g in one sweep (three
+// vector reads): 8,192 columns of 8,192 FP32 entries, nu = 30: 46.5 ms (was
+// 121.1); 24,000 of 1,024, nu = 30: 27.7 (47.8); 4,000 of 1,024, nu = 100: 50.8
+// (86.3); 2,048 of 2,048, nu = 100: 45.2 (72.0).  FP64: 4,004 of 4,096, nu = 30:
+// 50.8 (65.0); 2,048 of 16,384, nu = 30: 82.6 (100.1); 348 of 4,096, nu = 300:
+// 531 (681).
+
+// Four entries of a vector: FP32 as two packed pairs, FP64 as four doubles.
+template <typename VT> struct Quad;
+template <> struct Quad<float> {
+    uint64_t p[2];
+    __device__ __forceinline__ void lds(uint32_t a, int)
+    {
+        asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(p[0]), "=l"(p[1]) : "r"(a));
+    }
+};
+template <> struct Quad<double> {
+    double d[4];
+    __device__ __forceinline__ void lds(uint32_t a, int h)
+    {
+        asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(d[2 * h]), "=d"(d[2 * h + 1]) : "r"(a));
+    }
 };
 
-template <typename VT, int VPT, int T>
-__global__ void __launch_bounds__(T, T == 256 ? 4 : T == 512 ? 2 : 1) gs_kernel(
-    VT *__restrict__ K, VT *__restrict__ SK, const VT *__restrict__ U, const VT *__restrict__ Ulo,
+// 16 bytes global -> shared without a register; groups of such copies per thread.
+__device__ __forceinline__ void copy16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Dynamic shared memory: the ring (R stages of six quads per thread: four
+// stored vectors, u, and w_n or u's lo word), six FP64 arrays of nu entries, the
+// partial sums (sweep 1: b and g for kSpan vectors and C / 32 groups of 32
+// chains, FP64 per warp; sweep 2: a per vector and warp), the coefficients and
+// the support counts.
+template <typename VT, int C, int R>
+struct GsCfg {
+    static constexpr int T = C / 4;
+    static constexpr int NW = T / 32;
+    static constexpr int NP = sizeof(VT) == 4 ? C / 32 : NW;      // partial sums per total
+    static constexpr int kSpan = 32;                              // stored vectors per round of totals
+    static constexpr int kHalves = sizeof(VT) == 4 ? 1 : 2;       // 16-byte pieces per quad
+    static constexpr int kStage = 6 * kHalves * T * 16;           // bytes
+    // registers: FP32 96 (FP32 at 80: 54.8 against 46.6 ms on 8,192-entry
+    // vectors), FP64 (bound by its pipe, which few warps fill) about 150, but two
+    // CTAs for C = 1024 (91 against 96 ms on 16,384-entry vectors)
+    static constexpr int kMinCtas = sizeof(VT) == 4 ? 640 / T : C == 1024 ? 2 : 416 / T;
+    static constexpr __host__ __device__ int parts(int nu)        // doubles
+    {
+        return 2 * kSpan * NP > nu * NW ? 2 * kSpan * NP : nu * NW;
+    }
+    static size_t smem(int nu)
+    {
+        return (size_t)R * kStage + ((size_t)nu * 6 + parts(nu)) * sizeof(double) + (size_t)nu * sizeof(VT) +
+               (size_t)(nu + 2) * sizeof(int);
+    }
+};
+
+// f(integral constant count) for a run-time count in 1 .. N: a block's loops
+// over its vectors unroll for each count, so a short last block costs no FP64
+// work on vectors that do not exist (and no branch between independent FMAs).
+template <int N, typename F>
+__device__ __forceinline__ void for_count(int count, F &&f)
+{
+    if constexpr (N > 1) {
+        if (count < N) {
+            for_count<N - 1>(count, f);
+            return;
+        }
+    }
+    f(std::integral_constant<int, N>());
+}
+
+// The sums over groups of 32 chains of b and g for a block's four vectors
+// (FP32): bq[l], gq[l] hold the thread's four chains e.  A group is the chains
+// of eight lanes; its 32 chains x_0 .. x_31 are added in the tree of a
+// 32-lane reduce-scatter over twelve slots (slot 4 + l for b_l, 8 + l for
+// g_l): halves 16, 8, 4, 2, 1 apart, the first operand of each two-sum being
+// the half that the slot's number selects.  Lane j of the group ends with
+// q = j / 4 (b, g), l = j % 4.
+__device__ __forceinline__ uint64_t sel_x2(bool c, uint64_t a, uint64_t b) { return c ? a : b; }
+__device__ __forceinline__ PairAcc sel_x2(bool c, const PairAcc &a, const PairAcc &b)
+{
+    PairAcc r;
+    r.hi = sel_x2(c, a.hi, b.hi);
+    r.lo = sel_x2(c, a.lo, b.lo);
+    return r;
+}
+__device__ __forceinline__ PairAcc shfl_x2(const PairAcc &a, int o)
+{
+    PairAcc r;
+    r.hi = __shfl_xor_sync(kFull, a.hi, o);
+    r.lo = __shfl_xor_sync(kFull, a.lo, o);
+    return r;
+}
+// Per lane of the pair, first.merge(second), own being the first when
+// own_first: hi and the two-sum's error are symmetric in the operands, only
+// lo = lo_first + (lo_second + error) is not.
+__device__ __forceinline__ PairAcc merge_x2(bool own_first, const PairAcc &own, const PairAcc &other)
+{
+    PairAcc r;
+    uint64_t err;
+    asm("{\n\t.reg .b64 bb, t, u;\n\t"
+        "add.rn.f32x2 %0, %2, %3;\n\t"
+        "sub.rn.f32x2 bb, %0, %2;\n\t"
+        "sub.rn.f32x2 t, %0, bb;\n\t"
+        "sub.rn.f32x2 t, %2, t;\n\t"
+        "sub.rn.f32x2 u, %3, bb;\n\t"
+        "add.rn.f32x2 %1, t, u;\n\t}"
+        : "=&l"(r.hi), "=l"(err)
+        : "l"(own.hi), "l"(other.hi));
+    asm("{\n\t.reg .b64 t;\n\t"
+        "add.rn.f32x2 t, %2, %3;\n\t"
+        "add.rn.f32x2 %0, %1, t;\n\t}"
+        : "=l"(r.lo)
+        : "l"(sel_x2(own_first, own.lo, other.lo)), "l"(sel_x2(own_first, other.lo, own.lo)), "l"(err));
+    return r;
+}
+__device__ __forceinline__ DotAcc<float> chain_tree(const uint64_t (&bq)[kGsBlock][2], const PairAcc (&gq)[kGsBlock][2])
+{
+    const int lane = threadIdx.x & 31;
+    const bool j2 = (lane & 4) != 0, j1 = (lane & 2) != 0, j0 = (lane & 1) != 0;
+    // 16 chains apart = 4 lanes apart: lanes 0-3 take b, lanes 4-7 g; both
+    // keep their own half first
+    PairAcc a[4][2];
+#pragma unroll
+    for (int l = 0; l < 4; ++l)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            PairAcc b;
+            b.hi = bq[l][h];
+            a[l][h] = merge_x2(true, sel_x2(j2, gq[l][h], b), shfl_x2(sel_x2(j2, b, gq[l][h]), 4));
+        }
+    // 8 chains = 2 lanes apart: lane bit 1 takes vectors l / 2; b's first
+    // operand is the upper half, g's the lower
+    PairAcc c2[2][2];
+#pragma unroll
+    for (int l = 0; l < 2; ++l)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            c2[l][h] = merge_x2(j1 != j2, sel_x2(j1, a[l + 2][h], a[l][h]), shfl_x2(sel_x2(j1, a[l][h], a[l + 2][h]), 2));
+    // 4 chains = 1 lane apart: lane bit 0 takes l % 2; the first operand is the
+    // half numbered l / 2
+    PairAcc c1[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        c1[h] = merge_x2(j0 == j1, sel_x2(j0, c2[1][h], c2[0][h]), shfl_x2(sel_x2(j0, c2[0][h], c2[1][h]), 1));
+    // 2 chains apart (first: the half numbered l % 2), then neighbours
+    return merge_x2(!j0, c1[0], c1[1]).joined();
+}
+
+template <typename VT, int C, int R>
+__global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R>::kMinCtas) gs_kernel(
+    VT *__restrict__ K, const VT *__restrict__ SK, const VT *__restrict__ U, const VT *__restrict__ Ulo,
     double *__restrict__ Hsub, double *__restrict__ Lsub, double *__restrict__ scale,
     double *__restrict__ cn2, int *__restrict__ status, int *__restrict__ nu_eff,
-    const int *__restrict__ tcnt, int n, int nu, int need_w, double tau2)
+    const int *__restrict__ tcnt, int64_t MP, int n, int nu, int need_w, double tau2)
 {
-    using Cfg = GsCfg<VT, VPT, T>;
-    constexpr bool kWs = Cfg::kWs, kUs = Cfg::kUs, kLo = Cfg::kLo;
-    constexpr int kB = kGsBlock;
-    constexpr int64_t MP = (int64_t)VPT * T;   // m_pad
+    using Cfg = GsCfg<VT, C, R>;
+    constexpr bool kF = sizeof(VT) == 4;
+    constexpr int T = Cfg::T, NW = Cfg::NW, NP = Cfg::NP, kB = kGsBlock, kH = Cfg::kHalves;
+    constexpr int TPC = C / 32;           // tiles per chunk
+    constexpr int SC = 4;                 // chunks per pass of sweep 2 (16 entries per thread)
     const int c = blockIdx.x;
     if (status[c] != 0) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    VT *us = reinterpret_cast<VT *>(smem_raw);             // u = H w_n, unscaled (if kUs)
-    VT *uls = us + (kUs ? MP : 0);                          // its lo word (mixed precision)
-    VT *ws = uls + (kLo ? MP : 0);                          // w_n, then w_{n+1} (if kWs)
-    __shared__ double red[2 * 16 * 32];   // reduction partials, two slots
-    __shared__ double ssc[kMaxNu];        // s_i, then s_n
-    __shared__ double ta[kMaxNu], tb[kMaxNu], tg[kMaxNu];   // the sweep's totals
-    __shared__ double lrow[kMaxNu];       // L^-1 G_{<n, n}
-    __shared__ double nrow[kMaxNu];       // the new row n of L^-1
-    __shared__ double zc[kMaxNu];         // L^-1 p
-    __shared__ int cnt_s[kMaxNu + 2];
-    __shared__ VT coef[kMaxNu];           // subtraction coefficients c_i s_i
+    double *ssc = reinterpret_cast<double *>(smem_raw + R * Cfg::kStage);   // s_i, then s_n
+    double *tb = ssc + nu, *tg = tb + nu;                   // the sweep's totals
+    double *lrow = tg + nu;                                 // L^-1 G_{<n, n}
+    double *nrow = lrow + nu;                               // the new row n of L^-1
+    double *zc = nrow + nu;                                 // L^-1 p
+    double *part = zc + nu;                                 // partial sums
+    VT *coef = reinterpret_cast<VT *>(part + Cfg::parts(nu));   // subtraction coefficients c_i s_i
+    int *cnt_s = reinterpret_cast<int *>(coef + nu);
     __shared__ int bc_stop;
     __shared__ double bc_dinv;
     const int64_t base = (int64_t)c * nu * MP;
-    int buf = 0;
-    auto live = [&](int cnt) { return live_values<T>(cnt, warp); };
-
     for (int i = tid; i < n; i += T) ssc[i] = scale[(int64_t)c * nu + i];
     for (int L = tid; L <= n + 1; L += T) {
         const int t = tcnt[(int64_t)c * (nu + 2) + L];
         cnt_s[L] = in_range(t, MP / 32 + 1, kChkSupportCount) ? t : (int)(MP / 32);
     }
     __syncthreads();
+    const int cnt_u = cnt_s[n + 1];                     // tiles of u's support (and of w_{n+1})
+    const int nb1 = (n + kB) / kB;                      // blocks of stored vectors
+    const int nch_u = (cnt_u + TPC - 1) / TPC, nch_all = (int)(MP / C);
+    // chunks of block b (its last vector has the largest support; u's is the last block's)
+    auto chunks = [&](int b) { return (cnt_s[min(b * kB + kB, n + 1)] + TPC - 1) / TPC; };
+    // this thread's entries of a chunk: 16-byte piece h at position off + h C / 2
+    const int off = kF ? 4 * tid : 2 * tid;
+    constexpr int kHT = TPC / 2;                        // tiles from a piece to the next
+    const char *Ut = reinterpret_cast<const char *>(U + (int64_t)c * MP + off);
+    const int64_t dW = reinterpret_cast<const char *>(K + base + (int64_t)n * MP) -
+                       reinterpret_cast<const char *>(U + (int64_t)c * MP);      // w_n, from u
+    const int64_t dL = kF ? reinterpret_cast<const char *>(Ulo) - reinterpret_cast<const char *>(U) : 0;   // u's lo word
+    const uint32_t vb = (uint32_t)(MP * sizeof(VT));    // bytes of a vector
+    constexpr uint32_t kCB = C * sizeof(VT);            // bytes of a chunk
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(smem_raw) + 16 * tid;
+    auto piece = [&](uint32_t slot, int j, int h) { return slot + (j * kH + h) * (T * 16); };
 
-    // u (hi, lo) and w_n on chip; zeros past their supports
-    const VT *u = U + (int64_t)c * MP + tid;
-    const VT *ul = kLo ? Ulo + (int64_t)c * MP + tid : nullptr;
-    const VT *wnp = K + base + (int64_t)n * MP + tid;
-    VT wr[kWs ? 1 : VPT];
-    auto wget = [&](int v) -> VT {
-        if constexpr (kWs) return ws[tid + v * T]; else return wr[v];
-    };
-    auto wset = [&](int v, VT x) {
-        if constexpr (kWs) ws[tid + v * T] = x; else wr[v] = x;
-    };
-    {
-        const int nvu = live(cnt_s[n + 1]), nvn = live(cnt_s[n]);
+    // One stage: a chunk of a block's vectors (nbk of them, at src and vb
+    // apart), of u and of a sixth vector (d6 bytes from u).  Every thread
+    // copies what it alone reads, so a stage needs no barrier, only the
+    // thread's own wait.  Tiles from cnt on, past the support of the block's
+    // last vector, are neither copied nor read; a shorter vector of the block
+    // holds exact zeros up to there, and so does w_n.
+    auto copy_stage = [&](uint32_t slot, const char *src, const char *u, int64_t d6, bool six, int nbk, int k, int cnt) {
 #pragma unroll
-        for (int v = 0; v < VPT; ++v) {
-            const int p = tid + v * T;
-            const bool a = v < nvu;
-            if constexpr (kUs) us[p] = a ? u[v * T] : VT(0);
-            if constexpr (kLo) uls[p] = a ? ul[v * T] : VT(0);
-            wset(v, v < nvn ? wnp[v * T] : VT(0));
-        }
-    }
-    auto block_live = [&](int i0, int nbk, int (&nvl)[kB]) {
-        int m = 0;
+        for (int h = 0; h < kH; ++h)
+            if (k + h * kHT < cnt) {
 #pragma unroll
-        for (int l = 0; l < kB; ++l) {
-            nvl[l] = l < nbk ? live(cnt_s[i0 + l + 1]) : 0;
-            m = max(m, nvl[l]);
-        }
-        return m;
-    };
-
-    // ---- coefficient sweep over the stored vectors i <= n.  With G = 2 the
-    // CTA's halves take alternate blocks of vectors, each over all entries
-    // (thread t of a half owns positions t + v T/2), and reduce on their own
-    // barriers, so that one half's loads overlap the other's reduction.  This
-    // pays for FP64 vectors (6 % on a 16,384-entry sweep); FP32 vectors, whose
-    // error-free sums need more registers, ran slower with it (spills, or
-    // fewer loads in flight) and keep one group.
-    constexpr int G = (sizeof(VT) == 8 && T == 1024 && kWs && VPT >= 8) ? 2 : 1;
-    constexpr int TG = T / G, VG = VPT * G;
-    const int grp = tid / TG, gtid = tid - grp * TG, gwarp = gtid >> 5;
-    double *gpart = red + grp * (2 * 16 * 32 / G);
-    const VT *ug = U + (int64_t)c * MP + gtid;
-    auto glive = [&](int cnt) { return live_values<TG>(cnt, gwarp); };
-    if constexpr (G > 1) __syncthreads();   // u and w_n were stored by other threads
-    for (int i0 = grp * kB; i0 <= n; i0 += G * kB) {
-        const int nbk = min(kB, n + 1 - i0);
-        int nvl[kB];
-        int nvmax = 0;
-#pragma unroll
-        for (int l = 0; l < kB; ++l) {
-            nvl[l] = l < nbk ? glive(cnt_s[i0 + l + 1]) : 0;
-            nvmax = max(nvmax, nvl[l]);
-        }
-        const VT *kb = K + base + (int64_t)i0 * MP + gtid;
-        const VT *skb = SK + base + (int64_t)i0 * MP + gtid;
-        DotAcc<VT> acc[3 * kB];   // [l] a, [kB + l] b, [2 kB + l] g
-        VT hl[kB], bp[kB];
-#pragma unroll
-        for (int l = 0; l < kB; ++l) hl[l] = bp[l] = VT(0);
-        for_live<VG, Cfg::kChunkDot>(nvmax, [&](int v, bool a) {
-            const int p = gtid + v * TG;
-            VT uu;
-            if constexpr (kUs) uu = us[p]; else uu = a ? ug[v * TG] : VT(0);
-            VT wn;
-            if constexpr (G > 1) wn = ws[p]; else wn = wget(v);
-#pragma unroll
-            for (int l = 0; l < kB; ++l) {
-                const bool al = a && v < nvl[l];
-                const VT kr = al ? kb[l * MP + v * TG] : VT(0);
-                const VT sr = al ? skb[l * MP + v * TG] : VT(0);
-                acc[l].add(kr, uu);
-                if constexpr (kLo) hl[l] = fma(kr, uls[p], hl[l]);
-                if (need_w) bp[l] = fma(sr, uu, bp[l]);
-                acc[2 * kB + l].add(sr, wn);
+                for (int l = 0; l < kB; ++l)
+                    if (l < nbk) copy16(piece(slot, l, h), src + l * vb + h * (kCB / 2));
+                copy16(piece(slot, 4, h), u + h * (kCB / 2));
+                if (six) copy16(piece(slot, 5, h), u + d6 + h * (kCB / 2));
             }
-        });
-#pragma unroll
-        for (int l = 0; l < kB; ++l) {
-            if constexpr (kLo) acc[l].add_lo(hl[l]);
-            acc[kB + l].set(bp[l]);
+    };
+    // the next stage to copy: block pb, chunk pv (of the pass at chunk p0 in sweep 2)
+    uint32_t pslot = ring;
+    int pb = 0, pv = 0, p0 = 0, pch = chunks(0), pcnt = cnt_s[min(kB, n + 1)];
+    const char *ps = reinterpret_cast<const char *>(SK + base + off), *pu = Ut;
+    int pk = off >> 5;   // tile of the thread's first piece
+    auto issue1 = [&] {   // sweep 1: the blocks in order, then nothing
+        if (pb < nb1) {
+            copy_stage(pslot, ps, pu, dW, true, n + 1 - pb * kB, pk, pcnt);
+            ps += kCB;
+            pu += kCB;
+            pk += TPC;
+            if (++pv == pch) {
+                ps += (int64_t)kB * vb - (int64_t)pch * kCB;
+                pu = Ut;
+                pk = off >> 5;
+                pv = 0;
+                if (++pb < nb1) {
+                    pch = chunks(pb);
+                    pcnt = cnt_s[min(pb * kB + kB, n + 1)];
+                }
+            }
         }
-        block_sum(acc, gpart, buf, [&](int q, double t) {
-            const int l = q % kB, i = i0 + l;
-            if (l >= nbk) return;
-            if (q < kB) ta[i] = t; else if (q < 2 * kB) tb[i] = t; else tg[i] = t;
-        }, gwarp, TG / 32, 32 / G, G > 1 ? 1 + grp : 0);
-    }
-    if constexpr (G > 1) __syncthreads();   // both halves' totals
+        copy_commit();
+        pslot = pslot == ring + (R - 1) * Cfg::kStage ? ring : pslot + Cfg::kStage;
+    };
+    auto seek2 = [&] {   // sweep 2: to block pb of the pass at chunk p0
+        pch = min(SC, chunks(pb) - p0);
+        pcnt = cnt_s[min(pb * kB + kB, n + 1)];
+        ps = reinterpret_cast<const char *>(K + base + off) + (int64_t)pb * kB * vb + p0 * kCB;
+        pu = Ut + p0 * kCB;
+        pk = (off >> 5) + p0 * TPC;
+        pv = 0;
+    };
+    auto issue2 = [&] {   // passes of SC chunks, in each the blocks that reach it, last first
+        if (p0 < nch_u) {
+            copy_stage(pslot, ps, pu, dL, kF, n + 1 - pb * kB, pk, pcnt);
+            ps += kCB;
+            pu += kCB;
+            pk += TPC;
+            if (++pv == pch) {
+                if (--pb < 0 || chunks(pb) <= p0) {
+                    pb = nb1 - 1;
+                    p0 += SC;
+                }
+                if (p0 < nch_u) seek2();
+            }
+        }
+        copy_commit();
+        pslot = pslot == ring + (R - 1) * Cfg::kStage ? ring : pslot + Cfg::kStage;
+    };
 
-    // ---- scalars, G's column, the new row of L^-1, the coefficients (FP64).
-    // Lc holds L^-1 (lower triangular), so every product below is a matrix-
-    // vector product, one warp per row or column, with no serial chain.
+    // ---- sweep 1: b_i and g_i
+    uint32_t slot = ring;
+    auto next = [&] { slot = slot == ring + (R - 1) * Cfg::kStage ? ring : slot + Cfg::kStage; };
+#pragma unroll 1
+    for (int s = 0; s + 1 < R; ++s) issue1();
+#pragma unroll 1
+    for (int b = 0; b < nb1; ++b) {
+        const int i0 = b * kB, nch = chunks(b), cnt = cnt_s[min(i0 + kB, n + 1)];
+        int k = off >> 5;
+        if constexpr (kF) {
+            uint64_t bq[kB][2];
+            PairAcc gq[kB][2];
+#pragma unroll
+            for (int l = 0; l < kB; ++l) bq[l][0] = bq[l][1] = 0;
+#pragma unroll 1
+            for (int v = 0; v < nch; ++v, k += TPC) {
+                issue1();
+                copy_wait<R - 1>();
+                if (k < cnt) {
+                    Quad<float> u, w;
+                    u.lds(piece(slot, 4, 0), 0);
+                    w.lds(piece(slot, 5, 0), 0);
+                    const uint64_t nw[2] = {neg_x2(w.p[0]), neg_x2(w.p[1])};
+#pragma unroll
+                    for (int l = 0; l < kB; ++l) {
+                        if (i0 + l > n) break;
+                        Quad<float> sr;
+                        sr.lds(piece(slot, l, 0), 0);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            bq[l][h] = fma_x2(sr.p[h], u.p[h], bq[l][h]);
+                            gq[l][h].add(sr.p[h], w.p[h], nw[h]);
+                        }
+                    }
+                }
+                next();
+            }
+            const DotAcc<float> r = chain_tree(bq, gq);
+            const int q = (lane >> 2) & 1, i = i0 + (lane & 3);
+            if (i <= n) part[((i % Cfg::kSpan) * 2 + q) * NP + 4 * warp + (lane >> 3)] = r.pack();
+        } else {
+            DotAcc<VT> acc[2 * kB];   // [l] b, [kB + l] g
+            for_count<kB>(min(kB, n + 1 - i0), [&](auto nbk) {
+#pragma unroll 1
+                for (int v = 0; v < nch; ++v, k += TPC) {
+                    issue1();
+                    copy_wait<R - 1>();
+#pragma unroll
+                    for (int h = 0; h < kH; ++h)
+                        if (k + h * kHT < cnt) {
+                            Quad<VT> sr[nbk], u, w;
+                            u.lds(piece(slot, 4, h), h);
+                            w.lds(piece(slot, 5, h), h);
+#pragma unroll
+                            for (int l = 0; l < nbk; ++l) sr[l].lds(piece(slot, l, h), h);
+#pragma unroll
+                            for (int e = 2 * h; e < 2 * h + 2; ++e)
+#pragma unroll
+                                for (int l = 0; l < nbk; ++l) {
+                                    if (need_w) acc[l].add(sr[l].d[e], u.d[e]);
+                                    acc[kB + l].add(sr[l].d[e], w.d[e]);
+                                }
+                        }
+                    next();
+                }
+            });
+            const DotAcc<VT> r = warp_scatter(acc);   // slot lane / 4
+            const int q = lane >> 4, i = i0 + ((lane >> 2) & 3);
+            if ((lane & 3) == 0 && i <= n) part[((i % Cfg::kSpan) * 2 + q) * NP + warp] = r.pack();
+        }
+        // totals every kSpan vectors: the groups of chains (warps) in the tree of a butterfly reduction
+        if ((i0 + kB) % Cfg::kSpan == 0 || b == nb1 - 1) {
+            const int j0 = i0 / Cfg::kSpan * Cfg::kSpan;
+            __syncthreads();
+            for (int x = tid; x < 2 * (min(i0 + kB, n + 1) - j0); x += T) {
+                DotAcc<VT> v[NP];
+#pragma unroll
+                for (int j = 0; j < NP; ++j) v[j].unpack(part[x * NP + j]);
+#pragma unroll
+                for (int o = NP / 2; o > 0; o >>= 1)
+#pragma unroll
+                    for (int j = 0; j < o; ++j) v[j].merge(v[j + o]);
+                ((x & 1) ? tg : tb)[j0 + (x >> 1)] = v[0].value();
+            }
+            __syncthreads();
+        }
+    }
+
+    // the first stages of sweep 2 are copied during the scalar step
+    pslot = slot = ring;
+    pb = nb1 - 1;
+    seek2();
+#pragma unroll 1
+    for (int s = 0; s + 1 < R; ++s) issue2();
+
+    // ---- scalars: the norm, G's column, the new row of L^-1, the coefficients
     {
-        const GsScalarSmem<VT> sm{ssc, ta, tb, tg, lrow, nrow, zc, coef, bc_stop, bc_dinv};
-        if (!gs_scalars<VT, T>(c, n, nu, need_w, tau2, tid, Hsub, Lsub, scale, cn2, status, nu_eff, sm,
-                               [] { __syncthreads(); }))
+        const GsScalarSmem<VT> sm{ssc, tb, tg, lrow, nrow, zc, coef, bc_stop, bc_dinv};
+        if (!gs_scalars<VT, T>(c, n, nu, need_w, tau2, tid, Lsub, scale, cn2, status, nu_eff, sm,
+                               [] { __syncthreads(); })) {
+            copy_wait<0>();
             return;
+        }
     }
 
-    // ---- w_{n+1} = s_n u - sum_i coef_i w_i: streaming subtraction, last block
-    // first (its vectors are the ones the sweep read last; its support is u's)
+    // ---- sweep 2: w_{n+1} = s_n u - sum_i coef_i w_i and a_i = w_i . u, last
+    // block first (its support is u's), SC chunks at a time with w_{n+1} in
+    // registers.  FP32 vectors: w_{n+1} is a (hi, lo) sum with exact products
+    // and two-sums, rounded to FP32 once (s_n u and the projection nearly
+    // cancel, so a plain FP32 chain would leave rounding errors of the size of
+    // s_n u, not of w_{n+1}, outside span(K)).
     const VT vsn = (VT)ssc[n];
-    const int nb1 = (n + kB) / kB;
-    for (int b = nb1 - 1; b >= 0; --b) {
-        const int i0 = b * kB, nbk = min(kB, n + 1 - i0);
-        int nvl[kB];
-        const int nvmax = block_live(i0, nbk, nvl);
-        const bool first = b == nb1 - 1;
-        const int nvs = first ? live(cnt_s[n + 1]) : nvmax;
-        const VT *kb = K + base + (int64_t)i0 * MP + tid;
-        VT co[kB];
+    VT *wo = K + base + (int64_t)(n + 1) * MP;   // the next slot, unnormalised, zeros included
+#pragma unroll 1
+    for (int v0 = 0; v0 < nch_u; v0 += SC) {
+        PairAcc x[kF ? SC : 1][2];
+        double xd[kF ? 1 : SC][4];
+#pragma unroll 1
+        for (int b = nb1 - 1; b >= 0; --b) {
+            const int i0 = b * kB, nch = chunks(b);
+            if (nch <= v0) break;   // the blocks before it have no larger support
+            const int cnt = cnt_s[min(i0 + kB, n + 1)];
+            VT cf[kB];
 #pragma unroll
-        for (int l = 0; l < kB; ++l) co[l] = l < nbk ? coef[i0 + l] : VT(0);
-        for_live<VPT, Cfg::kChunkUpd>(nvs, [&](int v, bool a) {
-            if constexpr (kLo) {
-                // FP32 vectors: the sum runs as a (hi, lo) pair (hi in w's
-                // place, lo in u's lo word, which is no longer needed), with
-                // exact products and two-sums, and is rounded to FP32 once
-                // at the end: s_n u and the projection nearly cancel, so a
-                // plain FP32 chain would leave rounding errors of the size of
-                // s_n u, not of w_{n+1}, outside span(K)
-                const int p = tid + v * T;
-                DotAcc<VT> x;
-                if (first) {
-                    x.add(vsn, us[p]);
-                    x.lo = __fmaf_rn(vsn, uls[p], x.lo);
-                } else {
-                    x.hi = wget(v);
-                    x.lo = uls[p];
+            for (int l = 0; l < kB; ++l) cf[l] = need_w && i0 + l <= n ? coef[i0 + l] : VT(0);
+            PairAcc pa[kF ? kB : 1];
+            DotAcc<VT> acc[kB];
+            if constexpr (kF) {
+#pragma unroll
+                for (int q = 0; q < SC; ++q) {
+                    if (v0 + q >= nch) break;
+                    issue2();
+                    copy_wait<R - 1>();
+                    if (((v0 + q) * C + off) >> 5 < cnt) {
+                        Quad<float> u, ul;
+                        u.lds(piece(slot, 4, 0), 0);
+                        ul.lds(piece(slot, 5, 0), 0);
+                        const uint64_t nu2[2] = {neg_x2(u.p[0]), neg_x2(u.p[1])};
+                        if (b == nb1 - 1) {
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                x[q][h] = PairAcc();
+                                x[q][h].add(pair_of(vsn), u.p[h], nu2[h]);
+                                x[q][h].lo = fma_x2(pair_of(vsn), ul.p[h], x[q][h].lo);
+                            }
+                        }
+#pragma unroll
+                        for (int l = 0; l < kB; ++l) {
+                            if (i0 + l > n) break;
+                            Quad<float> w;
+                            w.lds(piece(slot, l, 0), 0);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                pa[l].add(w.p[h], u.p[h], nu2[h]);
+                                pa[l].lo = fma_x2(w.p[h], ul.p[h], pa[l].lo);
+                                x[q][h].add(w.p[h], pair_of(-cf[l]), pair_of(cf[l]));
+                            }
+                        }
+                    }
+                    next();
                 }
-#pragma unroll
-                for (int l = 0; l < kB; ++l)
-                    x.add(-co[l], (a && v < nvl[l]) ? kb[l * MP + v * T] : VT(0));
-                wset(v, x.hi);
-                uls[p] = x.lo;
             } else {
-                VT x;
-                if (first) {
-                    VT uu;
-                    if constexpr (kUs) uu = us[tid + v * T]; else uu = a ? u[v * T] : VT(0);
-                    x = uu * vsn;
-                } else {
-                    x = wget(v);
-                }
+                for_count<kB>(min(kB, n + 1 - i0), [&](auto nbk) {
 #pragma unroll
-                for (int l = 0; l < kB; ++l)
-                    x = fma(-co[l], (a && v < nvl[l]) ? kb[l * MP + v * T] : VT(0), x);
-                wset(v, x);
+                    for (int q = 0; q < SC; ++q) {
+                        if (v0 + q >= nch) break;
+                        const int k = ((v0 + q) * C + off) >> 5;
+                        issue2();
+                        copy_wait<R - 1>();
+#pragma unroll
+                        for (int h = 0; h < kH; ++h)
+                            if (k + h * kHT < cnt) {
+                                Quad<VT> w[nbk], u;
+                                u.lds(piece(slot, 4, h), h);
+#pragma unroll
+                                for (int l = 0; l < nbk; ++l) w[l].lds(piece(slot, l, h), h);
+#pragma unroll
+                                for (int e = 2 * h; e < 2 * h + 2; ++e) {
+                                    if (b == nb1 - 1) xd[q][e] = u.d[e] * vsn;
+#pragma unroll
+                                    for (int l = 0; l < nbk; ++l) {
+                                        acc[l].add(w[l].d[e], u.d[e]);
+                                        if (need_w) xd[q][e] = fma(-cf[l], w[l].d[e], xd[q][e]);
+                                    }
+                                }
+                            }
+                        next();
+                    }
+                });
             }
-        });
-    }
-    VT *wo = K + base + (int64_t)(n + 1) * MP + tid;   // the next slot, unnormalised, zeros included
-    const int nvu = live(cnt_s[n + 1]);
+            if constexpr (kF) {
 #pragma unroll
-    for (int v = 0; v < VPT; ++v) {
-        VT x = VT(0);
-        if (v < nvu) {
-            if constexpr (kLo) x = __fadd_rn(wget(v), uls[tid + v * T]); else x = wget(v);
+                for (int l = 0; l < kB; ++l) acc[l] = pa[l].joined();
+            }
+            // the warp's sums (slot lane / 8), added up over the passes; every
+            // support holds tile 0, so the first pass sets them all
+            DotAcc<VT> r = warp_scatter(acc);
+            const int i = i0 + (lane >> 3);
+            if ((lane & 7) == 0 && i <= n) {
+                double *ps = part + i * NW + warp;
+                if (v0 > 0) {
+                    DotAcc<VT> y;
+                    y.unpack(*ps);
+                    r.merge(y);
+                }
+                *ps = r.pack();
+            }
         }
-        wo[v * T] = x;
+        if (need_w) {
+#pragma unroll
+            for (int q = 0; q < SC; ++q) {
+                const int v = v0 + q;
+                if (v >= nch_all) break;
+                if constexpr (kF) {
+                    float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if ((v * C + off) >> 5 < cnt_u)
+                        r = make_float4(__fadd_rn(lane_x(x[q][0].hi), lane_x(x[q][0].lo)),
+                                        __fadd_rn(lane_y(x[q][0].hi), lane_y(x[q][0].lo)),
+                                        __fadd_rn(lane_x(x[q][1].hi), lane_x(x[q][1].lo)),
+                                        __fadd_rn(lane_y(x[q][1].hi), lane_y(x[q][1].lo)));
+                    *reinterpret_cast<float4 *>(wo + v * C + off) = r;
+                } else {
+#pragma unroll
+                    for (int h = 0; h < kH; ++h)
+                        *reinterpret_cast<double2 *>(wo + v * C + off + h * (C / 2)) =
+                            (v * C + off + h * (C / 2)) >> 5 < cnt_u ? make_double2(xd[q][2 * h], xd[q][2 * h + 1])
+                                                          : make_double2(0.0, 0.0);
+                }
+            }
+        }
+    }
+    if (need_w) {   // zeros past the last pass
+        for (int v = (nch_u + SC - 1) / SC * SC; v < nch_all; ++v)
+#pragma unroll
+            for (int h = 0; h < kH; ++h)
+                *reinterpret_cast<float4 *>(wo + v * C + off + h * (C / 2)) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    copy_wait<0>();
+    __syncthreads();
+    const double sn = ssc[n];
+    for (int m = tid; m <= n; m += T) {   // h_m of unit-norm vectors
+        DotAcc<VT> s;
+        s.unpack(part[m * NW]);
+#pragma unroll
+        for (int j = 1; j < NW; ++j) {
+            DotAcc<VT> y;
+            y.unpack(part[m * NW + j]);
+            s.merge(y);
+        }
+        const double h = s.value() * (ssc[m] * sn);
+        Hsub[((int64_t)c * nu + m) * nu + n] = h;
+        Hsub[((int64_t)c * nu + n) * nu + m] = h;
     }
 }
 
-template <typename VT, int VPT, int T>
+template <typename VT, int C, int R>
 cudaError_t gs_dispatch(const KrylovBatch &b, int n, int need_w, double tau, cudaStream_t s)
 {
-    using Cfg = GsCfg<VT, VPT, T>;
-    if (b.shape.m_pad != (int64_t)VPT * T || (int64_t)b.ntile * 32 < b.shape.m_pad || !b.tcnt || !b.Lsub)
+    using Cfg = GsCfg<VT, C, R>;
+    if (b.shape.m_pad % C != 0 || (int64_t)b.ntile * 32 < b.shape.m_pad || !b.tcnt || !b.Lsub)
         return cudaErrorInvalidValue;
-    const size_t smem = (size_t)VPT * T * sizeof(VT) * Cfg::kSmemVectors;
-    cudaError_t e = allow_dynamic_smem((const void *)gs_kernel<VT, VPT, T>, smem);
+    const size_t smem = Cfg::smem(b.nu);
+    cudaError_t e = allow_dynamic_smem((const void *)gs_kernel<VT, C, R>, smem);
     if (e != cudaSuccess) return e;
-    gs_kernel<VT, VPT, T><<<b.nb, T, smem, s>>>(
-        (VT *)b.K, (VT *)b.SK, (const VT *)b.U, (const VT *)b.Ulo, b.Hsub, b.Lsub, b.scale, b.cn2,
-        b.status, b.nu_eff, b.tcnt, n, b.nu, need_w, tau * tau);
+    gs_kernel<VT, C, R><<<b.nb, Cfg::T, smem, s>>>(
+        (VT *)b.K, (const VT *)b.SK, (const VT *)b.U, (const VT *)b.Ulo, b.Hsub, b.Lsub, b.scale, b.cn2,
+        b.status, b.nu_eff, b.tcnt, b.shape.m_pad, n, b.nu, need_w, tau * tau);
     return cudaGetLastError();
 }
 
-template <typename VT, int T>
-cudaError_t gs_vpt(const KrylovBatch &b, int n, int need_w, double tau, cudaStream_t s)
-{
-    switch (b.shape.vpt) {
-    case 1: return gs_dispatch<VT, 1, T>(b, n, need_w, tau, s);
-    case 2: return gs_dispatch<VT, 2, T>(b, n, need_w, tau, s);
-    case 4: return gs_dispatch<VT, 4, T>(b, n, need_w, tau, s);
-    case 8: return gs_dispatch<VT, 8, T>(b, n, need_w, tau, s);
-    case 16: return gs_dispatch<VT, 16, T>(b, n, need_w, tau, s);
-    default: return cudaErrorInvalidValue;
-    }
-}
-
+// A shape of `threads` entries per chunk and vpt chunks: C = threads chains of
+// partial sums on a CTA of a quarter as many threads.  Ring stages: FP64 two
+// (its arithmetic covers the copies).  FP32 two up to 1,024 entries, where the
+// ring's shared memory would hold back the CTAs whose reductions cover each
+// other (24,000 columns, nu = 30: 28.9 ms against 32.6 with three), three above
+// (2,048 columns of 2,048 entries, nu = 100: 44.9 ms against 48.3 with two).
 template <typename VT>
 cudaError_t gs_shape(const KrylovBatch &b, int n, int need_w, double tau, cudaStream_t s)
 {
+    constexpr int R = sizeof(VT) == 4 ? 3 : 2;
+    if ((int64_t)b.shape.vpt * b.shape.threads != b.shape.m_pad) return cudaErrorInvalidValue;
     switch (b.shape.threads) {
-    case 256: return gs_vpt<VT, 256>(b, n, need_w, tau, s);
-    case 512: return gs_vpt<VT, 512>(b, n, need_w, tau, s);
-    case 1024: return gs_vpt<VT, 1024>(b, n, need_w, tau, s);
+    case 256:
+        if (R == 3 && b.shape.m_pad <= 1024) return gs_dispatch<VT, 256, 2>(b, n, need_w, tau, s);
+        return gs_dispatch<VT, 256, R>(b, n, need_w, tau, s);
+    case 512: return gs_dispatch<VT, 512, R>(b, n, need_w, tau, s);
+    case 1024: return gs_dispatch<VT, 1024, R>(b, n, need_w, tau, s);
     default: return cudaErrorInvalidValue;
     }
 }
