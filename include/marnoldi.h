@@ -306,15 +306,13 @@ int marnoldi_set_member_temperatures(marnoldi_ctx *ctx, int n_members, const dou
  * which changes no sum.
  *   marnoldi_set_autotune: mode 0 (default, also when MARNOLDI_AUTOTUNE is
  *     unset or not "1") uses a fixed rule: 256 threads per CTA up to m = 4096,
- *     512 for FP32 vectors up to 8192, the streamed kernel for longer FP32
- *     vectors (reported as 64 values per thread and 288 threads: 256
- *     threads and a producer warp that copies the vectors into shared memory
- *     with the bulk-copy engine), else 1024, values per thread covering m.
+ *     512 for FP32 vectors up to 8192, 256 pairs of sums for longer FP32
+ *     vectors (reported as 64 values and 288 threads), else 1024, values per
+ *     thread covering m.
  *     Mode 1: the first solve of each (precision, nu, global/regional, padded
  *     vector length) times every shape with the same padded length (threads
- *     256, 512 or 1024; for FP32 vectors of 16,384 entries also the two
- *     streamed shapes, 64 x 288 and 32 x 544: 512 consumer threads and the
- *     producer, one CTA per SM) on its first 1,216 columns, keeps the fastest for the
+ *     256, 512 or 1024; for FP32 vectors of 16,384 entries also 64 x 288 and
+ *     32 x 544, pairs of sums) on its first 1,216 columns, keeps the fastest for the
  *     rest of the process and, when MARNOLDI_TUNE_CACHE names a file, appends
  *     it there and reads earlier choices from it.  Shapes change the order of
  *     the kernel's partial sums, so results may differ by rounding between

@@ -1173,8 +1173,7 @@ int marnoldi_check_status(int *compiled, int *site, int64_t *index)
     *compiled = kCheckBuild ? 1 : 0;
     *site = 0;
     *index = 0;
-    cudaError_t (*take[])(unsigned long long *) = {check_take_krylov, check_take_region, check_take_outputs,
-                                                   check_take_gs_stream};
+    cudaError_t (*take[])(unsigned long long *) = {check_take_krylov, check_take_region, check_take_outputs};
     for (auto f : take) {
         unsigned long long w = 0;
         const cudaError_t e = f(&w);
@@ -1613,9 +1612,6 @@ int marnoldi_solve(marnoldi_ctx *c, const int64_t *columns, int64_t ncols, int n
     c->kT = kT;
     c->solved = true;
     for (int64_t q = 0; q < nc; ++q) {
-        if (est[q] & 4)
-            return fail(c, MARNOLDI_ETIMEOUT, "column %lld: a bounded wait of the Gram-Schmidt kernel gave up",
-                        (long long)c->cols[q]);
         if (est[q] & 2)
             return fail(c, MARNOLDI_ENOTSPD, "column %lld: a Krylov vector has non-positive S norm", (long long)c->cols[q]);
         if (est[q] & 1)

@@ -1,4 +1,4 @@
-// Device helpers shared by the Gram-Schmidt kernels (krylov.cu, gs_stream.cu):
+// Device helpers of the Gram-Schmidt kernel (krylov.cu):
 // error-free FP32 dot accumulators, fixed-order warp reductions, and the FP64
 // scalar step of one Krylov step (norm, breakdown test, the Gram matrix's new
 // column, the new row of L^-1 and the projection coefficients).
@@ -90,16 +90,16 @@ template <> struct DotAcc<float> {
 // address), and the packed operations on such pairs (add/sub/mul/fma .rn.f32x2,
 // sm_100 and later): each lane is rounded exactly as the scalar instruction
 // would be, at half the instruction count.
-__device__ __forceinline__ uint64_t lds2(const float *p)
-{
-    uint64_t r;
-    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)));
-    return r;
-}
 __device__ __forceinline__ uint64_t pair_of(float x)
 {
     uint64_t r;
     asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ uint64_t pack_x2(float x, float y)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
     return r;
 }
 __device__ __forceinline__ uint64_t fma_x2(uint64_t a, uint64_t b, uint64_t c)
@@ -113,31 +113,12 @@ __device__ __forceinline__ float lane_x(uint64_t a) { return __uint_as_float((un
 __device__ __forceinline__ float lane_y(uint64_t a) { return __uint_as_float((unsigned)(a >> 32)); }
 
 // Two DotAcc<float> (one per lane) in packed registers: per lane the
-// operations of DotAcc<float>::add (p = a b, e = fma(a, b, -p), the two-sum
-// of hi and p, lo += e + err).
+// operations of DotAcc<float>::add.
 struct PairAcc {
     uint64_t hi = 0, lo = 0;
-    __device__ __forceinline__ void add(uint64_t a, uint64_t b)
-    {
-        asm("{\n\t.reg .b64 p, np, e, s, bb, t, u, err;\n\t"
-            "mul.rn.f32x2 p, %2, %3;\n\t"
-            "xor.b64 np, p, 0x8000000080000000;\n\t"
-            "fma.rn.f32x2 e, %2, %3, np;\n\t"
-            "add.rn.f32x2 s, %0, p;\n\t"
-            "sub.rn.f32x2 bb, s, %0;\n\t"
-            "sub.rn.f32x2 t, s, bb;\n\t"
-            "sub.rn.f32x2 t, %0, t;\n\t"
-            "sub.rn.f32x2 u, p, bb;\n\t"
-            "add.rn.f32x2 err, t, u;\n\t"
-            "add.rn.f32x2 e, e, err;\n\t"
-            "add.rn.f32x2 %1, %1, e;\n\t"
-            "mov.b64 %0, s;\n\t}"
-            : "+l"(hi), "+l"(lo)
-            : "l"(a), "l"(b));
-    }
-    // The same with nb = -b given: fma(a, -b, p) is the exact negative of e, and
-    // lo -= (-e - err) rounds as lo += (e + err), so the bits are add()'s without
-    // the two integer instructions that negate p.
+    // += a b, with nb = -b given: fma(a, -b, p) is the exact negative of the
+    // product's error e, and lo -= (-e - err) rounds as lo += (e + err), so no
+    // integer instruction negates p
     __device__ __forceinline__ void add(uint64_t a, uint64_t b, uint64_t nb)
     {
         asm("{\n\t.reg .b64 p, e, s, bb, t, u, err;\n\t"

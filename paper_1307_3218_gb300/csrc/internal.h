@@ -67,8 +67,9 @@ constexpr int kMaxNu = 320;
 // Largest Krylov-vector length of global mode (one CTA holds a column's vector).
 constexpr int64_t kMaxGlobalM = 16384;
 
-// Threads per CTA and values per thread of the column-per-CTA kernels on
-// vectors of length m: m_pad = vpt * threads >= m, a multiple of 32.
+// Partial sums of the Gram-Schmidt kernel on vectors of length m: `threads`
+// chains of vpt values each (krylov.cu), m_pad = vpt * threads >= m, a multiple
+// of 32 (the two pair shapes below count 32 threads more).
 struct ColumnShape {
     int vpt;
     int threads;
@@ -80,10 +81,10 @@ ColumnShape column_shape(int64_t m, int prec);
 // were written.
 constexpr int kMaxShapes = 4;
 int column_shape_candidates(int64_t m_pad, int prec, ColumnShape *out);
-// The shapes of the streamed Gram-Schmidt kernel (gs_stream.cu), FP32
-// vectors of m_pad = 16,384 and a producer warp: 512 consumer threads of 32
-// values, {vpt 32, threads 544}, or 256 of 64 values, {vpt 64, threads 288}.
-bool gs_stream_shape(const ColumnShape &s, int prec);
+// The shapes of FP32 vectors of m_pad = 16,384 whose chains are joined in
+// neighbouring pairs first: {64, 288} is 256 pairs of chains of 32 values,
+// {32, 544} 512 pairs of 16 (values per pair, pairs + 32).
+bool gs_pair_shape(const ColumnShape &s, int prec);
 
 // ---------------------------------------------------------------- Krylov build
 // All pointers are device pointers.  Batch layout (c = batch column):
@@ -92,8 +93,7 @@ bool gs_stream_shape(const ColumnShape &s, int prec);
 //     k_i = scale[c][i] * w_i (scale = 1 / ||w_i||_S, set by the MGS of step i)
 //   U[c][r] at c * m_pad + r: H w_n of the current step
 //   Hsub[c][i][l] at (c * nu + i) * nu + l (double)
-// status[c]: 0 active, 1 stopped (breakdown), 2 non-positive S norm, 3 a bounded
-// wait of the streamed Gram-Schmidt kernel gave up.
+// status[c]: 0 active, 1 stopped (breakdown), 2 non-positive S norm.
 struct KrylovBatch {
     int prec;             // 0 FP64, 1 mixed (vectors float)
     int nb;               // columns in this batch
@@ -140,7 +140,7 @@ enum CheckSite : int {
     kChkRegionCol,        // region.cu: local column of a local block
     kChkRegionGather,     // region.cu: position of a gathered 4-vector
     kChkDensityOut,       // outputs.cu: density entry of a pattern row
-    kChkSupportCount,     // krylov.cu, gs_stream.cu: tiles of a support (at most m_pad / 32)
+    kChkSupportCount,     // krylov.cu: tiles of a support (at most m_pad / 32)
 };
 #ifdef MARNOLDI_CHECK
 constexpr bool kCheckBuild = true;
@@ -178,7 +178,6 @@ __device__ __forceinline__ constexpr bool in_range(int64_t, int64_t, int) { retu
 cudaError_t check_take_krylov(unsigned long long *w);
 cudaError_t check_take_region(unsigned long long *w);
 cudaError_t check_take_outputs(unsigned long long *w);
-cudaError_t check_take_gs_stream(unsigned long long *w);
 
 // Four consecutive values (16-byte aligned for float, 32 for double) in one or
 // two vector loads (read-only path) or stores.
@@ -284,7 +283,6 @@ cudaError_t launch_support(const DeviceMatrix &A, const RegionMaps *rm, const Kr
 cudaError_t launch_spmm_hs(const DeviceMatrix &A, const KrylovBatch &b, const void *X, int64_t ldx,
                            void *SY, int64_t ldsy, int lim, cudaStream_t s);
 cudaError_t launch_gs(const KrylovBatch &b, int n, int need_w, double tau, cudaStream_t s);
-cudaError_t launch_gs_stream(const KrylovBatch &b, int n, int need_w, double tau, cudaStream_t s);
 
 // ---------------------------------------------------------------- subspace eigensolve
 // Per solved column c (global index col0 + batch column):
@@ -296,7 +294,7 @@ struct ColumnState {
     int *nu_eff;
     double *eps, *w, *t, *P;
     const int64_t *p_off;
-    int *eig_status;     // bits: 1 QL did not converge, 2 non-positive S norm, 4 a wait gave up
+    int *eig_status;     // bits: 1 QL did not converge, 2 non-positive S norm
 };
 
 // Scratch of the three-kernel eigensolve, per chunk of subspaces:

@@ -39,15 +39,13 @@ const char *kernel_name(int kind)
 // A shape {vpt, threads} of gs_kernel names its partial sums: `threads` chains
 // of vpt values each (m_pad = vpt threads), on a CTA of threads / 4 threads.
 // Vectors up to 4096 entries take 256 chains, FP32 vectors up to 8192 entries
-// 512; longer FP32 vectors run the streamed kernel (gs_stream.cu) with 256
-// consumer threads of 64 values and a producer warp, two CTAs per SM (shape
-// {64, 288}; {32, 544}, one CTA of 512 consumer threads per SM, is the other
-// streamed shape); the rest take 1024 chains.  vpt is the power of two that
-// covers m.
+// 512, longer FP32 vectors 256 pairs of chains (shape {64, 288}; {32, 544}, 512
+// pairs, is the other pair shape), the rest 1024 chains.  vpt is the power of
+// two that covers m.
 ColumnShape column_shape(int64_t m, int prec)
 {
     if (prec == 1 && m > 4096 && m <= 8192) return ColumnShape{16, 512, 8192};
-    if (prec == 1 && m > 8192 && m <= 16384) return ColumnShape{64, 288, 16384};   // gs_stream.cu
+    if (prec == 1 && m > 8192 && m <= 16384) return ColumnShape{64, 288, 16384};
     const int T = m <= 4096 ? 256 : 1024;
     int v = 1;
     while (v < 16 && (int64_t)v * T < m) v *= 2;
@@ -61,8 +59,14 @@ int column_shape_candidates(int64_t m_pad, int prec, ColumnShape *out)
         for (int v = 1; v <= 16; v *= 2)
             if ((int64_t)v * T == m_pad) out[n++] = ColumnShape{v, T, m_pad};
     for (const ColumnShape st : {ColumnShape{32, 544, 16384}, ColumnShape{64, 288, 16384}})
-        if (m_pad == st.m_pad && gs_stream_shape(st, prec)) out[n++] = st;
+        if (m_pad == st.m_pad && gs_pair_shape(st, prec)) out[n++] = st;
     return n;
+}
+
+bool gs_pair_shape(const ColumnShape &s, int prec)
+{
+    return prec == 1 && s.m_pad == 16384 &&
+           ((s.vpt == 32 && s.threads == 544) || (s.vpt == 64 && s.threads == 288));
 }
 
 namespace {
@@ -277,7 +281,8 @@ __global__ void __launch_bounds__(256) spmm_hs_kernel(
 // the level the FP32 subtraction leaves anyway, which G records.  The chains
 // of b and g, and the tree that adds them up, are those of a CTA of C threads
 // of one entry per chunk each, so a shape's results do not depend on how many
-// of its chains a thread carries.  The coefficients and G are FP64.
+// of its chains a thread carries.  (Vectors of 16,384 FP32 entries join
+// neighbouring chains in pairs first.)  The coefficients and G are FP64.
 //
 // What bounds it: FP32 vectors, the issue slots (54 % at 0.51 of the HBM
 // bandwidth; about 32 FP32 operations per entry and stored vector, in packed
@@ -292,7 +297,11 @@ __global__ void __launch_bounds__(256) spmm_hs_kernel(
 // 121.1); 24,000 of 1,024, nu = 30: 27.7 (47.8); 4,000 of 1,024, nu = 100: 50.8
 // (86.3); 2,048 of 2,048, nu = 100: 45.2 (72.0).  FP64: 4,004 of 4,096, nu = 30:
 // 50.8 (65.0); 2,048 of 16,384, nu = 30: 82.6 (100.1); 348 of 4,096, nu = 300:
-// 531 (681).
+// 531 (681).  16,384 columns of 16,384 FP32 entries, nu = 30: 160.8 ms, where a
+// kernel with the stored vectors streamed by a producer warp's bulk copies, two
+// CTAs per SM, took 227.7: it read each vector three times and its 16 consumer
+// warps per SM waited for their own arithmetic's latency.  More ring stages hold
+// back CTAs: 161.4 ms with four, 165.4 with five.
 
 // Four entries of a vector: FP32 as two packed pairs, FP64 as four doubles.
 template <typename VT> struct Quad;
@@ -325,11 +334,11 @@ __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group 
 // partial sums (sweep 1: b and g for kSpan vectors and C / 32 groups of 32
 // chains, FP64 per warp; sweep 2: a per vector and warp), the coefficients and
 // the support counts.
-template <typename VT, int C, int R>
+template <typename VT, int C, int R, bool kPairs>
 struct GsCfg {
     static constexpr int T = C / 4;
     static constexpr int NW = T / 32;
-    static constexpr int NP = sizeof(VT) == 4 ? C / 32 : NW;      // partial sums per total
+    static constexpr int NP = kPairs ? C / 64 : sizeof(VT) == 4 ? C / 32 : NW;   // partial sums per total
     static constexpr int kSpan = 32;                              // stored vectors per round of totals
     static constexpr int kHalves = sizeof(VT) == 4 ? 1 : 2;       // 16-byte pieces per quad
     static constexpr int kStage = 6 * kHalves * T * 16;           // bytes
@@ -441,14 +450,40 @@ __device__ __forceinline__ DotAcc<float> chain_tree(const uint64_t (&bq)[kGsBloc
     return merge_x2(!j0, c1[0], c1[1]).joined();
 }
 
-template <typename VT, int C, int R>
-__global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R>::kMinCtas) gs_kernel(
+// The same for chains in pairs: two neighbouring chains are joined first (b by
+// a plain addition, g by a two-sum, lower lane first) and the 32 pairs of 16
+// lanes added in that tree.  Lanes j and j + 1 (j even) end with q = j / 8 % 2,
+// l = j / 2 % 4 of their 16 lanes.
+__device__ __forceinline__ DotAcc<float> pair_tree(const uint64_t (&bq)[kGsBlock][2], const PairAcc (&gq)[kGsBlock][2])
+{
+    const int lane = threadIdx.x & 31;
+    const bool j3 = (lane & 8) != 0, j2 = (lane & 4) != 0, j1 = (lane & 2) != 0, j0 = (lane & 1) != 0;
+    PairAcc a[4];
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+        PairAcc b, g;
+        b.hi = pack_x2(__fadd_rn(lane_x(bq[l][0]), lane_y(bq[l][0])), __fadd_rn(lane_x(bq[l][1]), lane_y(bq[l][1])));
+        const DotAcc<float> g0 = gq[l][0].joined(), g1 = gq[l][1].joined();
+        g.hi = pack_x2(g0.hi, g1.hi);
+        g.lo = pack_x2(g0.lo, g1.lo);
+        a[l] = merge_x2(true, sel_x2(j3, g, b), shfl_x2(sel_x2(j3, b, g), 8));
+    }
+    PairAcc c2[2];
+#pragma unroll
+    for (int l = 0; l < 2; ++l)
+        c2[l] = merge_x2(j2 != j3, sel_x2(j2, a[l + 2], a[l]), shfl_x2(sel_x2(j2, a[l], a[l + 2]), 4));
+    const PairAcc c1 = merge_x2(j1 == j2, sel_x2(j1, c2[1], c2[0]), shfl_x2(sel_x2(j1, c2[0], c2[1]), 2));
+    return merge_x2(j0 == j1, c1, shfl_x2(c1, 1)).joined();
+}
+
+template <typename VT, int C, int R, bool kPairs = false>
+__global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_kernel(
     VT *__restrict__ K, const VT *__restrict__ SK, const VT *__restrict__ U, const VT *__restrict__ Ulo,
     double *__restrict__ Hsub, double *__restrict__ Lsub, double *__restrict__ scale,
     double *__restrict__ cn2, int *__restrict__ status, int *__restrict__ nu_eff,
     const int *__restrict__ tcnt, int64_t MP, int n, int nu, int need_w, double tau2)
 {
-    using Cfg = GsCfg<VT, C, R>;
+    using Cfg = GsCfg<VT, C, R, kPairs>;
     constexpr bool kF = sizeof(VT) == 4;
     constexpr int T = Cfg::T, NW = Cfg::NW, NP = Cfg::NP, kB = kGsBlock, kH = Cfg::kHalves;
     constexpr int TPC = C / 32;           // tiles per chunk
@@ -596,9 +631,10 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R>::kMinCtas) gs_kernel(
                 }
                 next();
             }
-            const DotAcc<float> r = chain_tree(bq, gq);
-            const int q = (lane >> 2) & 1, i = i0 + (lane & 3);
-            if (i <= n) part[((i % Cfg::kSpan) * 2 + q) * NP + 4 * warp + (lane >> 3)] = r.pack();
+            const DotAcc<float> r = kPairs ? pair_tree(bq, gq) : chain_tree(bq, gq);
+            const int j = kPairs ? (lane & 15) >> 1 : lane & 7, i = i0 + (j & 3);
+            const int grp = kPairs ? 2 * warp + (lane >> 4) : 4 * warp + (lane >> 3);
+            if (i <= n) part[((i % Cfg::kSpan) * 2 + (j >> 2)) * NP + grp] = r.pack();
         } else {
             DotAcc<VT> acc[2 * kB];   // [l] b, [kB + l] g
             for_count<kB>(min(kB, n + 1 - i0), [&](auto nbk) {
@@ -637,10 +673,15 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R>::kMinCtas) gs_kernel(
                 DotAcc<VT> v[NP];
 #pragma unroll
                 for (int j = 0; j < NP; ++j) v[j].unpack(part[x * NP + j]);
+                if constexpr (kPairs) {   // in order
 #pragma unroll
-                for (int o = NP / 2; o > 0; o >>= 1)
+                    for (int j = 1; j < NP; ++j) v[0].merge(v[j]);
+                } else {
 #pragma unroll
-                    for (int j = 0; j < o; ++j) v[j].merge(v[j + o]);
+                    for (int o = NP / 2; o > 0; o >>= 1)
+#pragma unroll
+                        for (int j = 0; j < o; ++j) v[j].merge(v[j + o]);
+                }
                 ((x & 1) ? tg : tb)[j0 + (x >> 1)] = v[0].value();
             }
             __syncthreads();
@@ -814,16 +855,16 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R>::kMinCtas) gs_kernel(
     }
 }
 
-template <typename VT, int C, int R>
+template <typename VT, int C, int R, bool kPairs = false>
 cudaError_t gs_dispatch(const KrylovBatch &b, int n, int need_w, double tau, cudaStream_t s)
 {
-    using Cfg = GsCfg<VT, C, R>;
+    using Cfg = GsCfg<VT, C, R, kPairs>;
     if (b.shape.m_pad % C != 0 || (int64_t)b.ntile * 32 < b.shape.m_pad || !b.tcnt || !b.Lsub)
         return cudaErrorInvalidValue;
     const size_t smem = Cfg::smem(b.nu);
-    cudaError_t e = allow_dynamic_smem((const void *)gs_kernel<VT, C, R>, smem);
+    cudaError_t e = allow_dynamic_smem((const void *)gs_kernel<VT, C, R, kPairs>, smem);
     if (e != cudaSuccess) return e;
-    gs_kernel<VT, C, R><<<b.nb, Cfg::T, smem, s>>>(
+    gs_kernel<VT, C, R, kPairs><<<b.nb, Cfg::T, smem, s>>>(
         (VT *)b.K, (const VT *)b.SK, (const VT *)b.U, (const VT *)b.Ulo, b.Hsub, b.Lsub, b.scale, b.cn2,
         b.status, b.nu_eff, b.tcnt, b.shape.m_pad, n, b.nu, need_w, tau * tau);
     return cudaGetLastError();
@@ -898,7 +939,9 @@ cudaError_t launch_spmm_hs(const DeviceMatrix &A, const KrylovBatch &b, const vo
 
 cudaError_t launch_gs(const KrylovBatch &b, int n, int need_w, double tau, cudaStream_t s)
 {
-    if (gs_stream_shape(b.shape, b.prec)) return launch_gs_stream(b, n, need_w, tau, s);
+    if (gs_pair_shape(b.shape, b.prec))
+        return b.shape.threads == 288 ? gs_dispatch<float, 512, 3, true>(b, n, need_w, tau, s)
+                                      : gs_dispatch<float, 1024, 3, true>(b, n, need_w, tau, s);
     return b.prec == 0 ? gs_shape<double>(b, n, need_w, tau, s) : gs_shape<float>(b, n, need_w, tau, s);
 }
 
