@@ -662,7 +662,7 @@ struct SolvePlan {
     bool a_global;
     EigScratch es;   // sizes and chunk; the caller sets the pointers
     size_t oK, oSK, oU, oUl, oH, oL, oSc, oC, oS, oN, oRg, oRc, oRi, oRk, oRs, oTh, oTo, oTc;
-    size_t oED, oEE, oERQ, oERot, oESw, oENs, oEA, ws_bytes;
+    size_t oTr, oPn, oED, oEE, oERQ, oERot, oESw, oENs, oEA, ws_bytes;
 };
 
 // Workspace bytes per batch column, for the default batch size.
@@ -671,7 +671,7 @@ size_t per_column_bytes(const ColumnShape &shape, size_t vs, int nu, int region_
     const size_t reg = region_atoms > 0 ? (size_t)region_atoms * (12 + 8 * (size_t)maxrow) : 0;
     return al256((size_t)2 * nu * shape.m_pad * vs) + (size_t)2 * shape.m_pad * vs +
            (size_t)2 * nu * nu * 8 + (size_t)nu * 8 + 64 + reg + (size_t)(shape.m_pad / 32) * 3 +
-           (size_t)(nu + 2) * 4;
+           (size_t)(nu + 2) * 4 + (region_atoms > 0 ? 0 : (size_t)shape.m_pad * vs + (size_t)(shape.m_pad / 32) * 2);
 }
 
 // Batch size within [1, ncols] and the launch limits (one CTA per column, or
@@ -732,7 +732,9 @@ bool plan_solve(int64_t m_vec, int prec, int nu, int region_atoms, int maxrow, i
     p.oTh = p.oRs + (regional ? al256((size_t)B * 4) : 0);
     p.oTo = p.oTh + al256((size_t)B * nt);
     p.oTc = p.oTo + al256((size_t)B * nt * 2);
-    const size_t oEg = p.oTc + al256((size_t)B * (nu + 2) * 4);
+    p.oTr = p.oTc + al256((size_t)B * (nu + 2) * 4);
+    p.oPn = p.oTr + (regional ? 0 : al256((size_t)B * nt * 2));
+    const size_t oEg = p.oPn + (regional ? 0 : al256((size_t)panel_entries(B, nt) * vs));
 
     // eigensolve scratch, for chunks of at most es.chunk subspaces; H_sub in
     // shared memory when it fits, else in a global scratch per subspace
@@ -1396,6 +1398,8 @@ int marnoldi_solve(marnoldi_ctx *c, const int64_t *columns, int64_t ncols, int n
     kb.thop = (uint8_t *)(wb + plan.oTh);
     kb.tinv = (uint16_t *)(wb + plan.oTo);
     kb.tcnt = (int *)(wb + plan.oTc);
+    kb.tord = regional ? nullptr : (uint16_t *)(wb + plan.oTr);
+    kb.panel = regional ? nullptr : (void *)(wb + plan.oPn);
     EigScratch es = plan.es;
     es.D = (double *)(wb + plan.oED);
     es.E = (double *)(wb + plan.oEE);
@@ -1427,6 +1431,10 @@ int marnoldi_solve(marnoldi_ctx *c, const int64_t *columns, int64_t ncols, int n
         const int rows = regional ? region_atoms : (int)c->nbr;
         if ((rows & 7) && (r = launch(c, KK_INIT, [&] { return launch_zero_partial_tile(k, rows, c->stream); })))
             return r;
+        if (k.panel) {   // zero outside the supports, which only grow
+            const cudaError_t pe = cudaMemsetAsync(k.panel, 0, (size_t)panel_entries(k.nb, k.ntile) * vs, c->stream);
+            if (pe != cudaSuccess) return fail_cuda(c, pe, "panel clear");
+        }
         if ((r = launch(c, KK_INIT, [&] {
                  return regional ? launch_init_regional(c->A, c->rm, k, c->stream) : launch_init(c->A, k, c->stream);
              })))
@@ -1441,8 +1449,7 @@ int marnoldi_solve(marnoldi_ctx *c, const int64_t *columns, int64_t ncols, int n
                      })))
                     return r;
             } else if ((r = launch(c, KK_SPMM_HS, [&] {
-                            return launch_spmm_hs(c->A, k, Kn, (int64_t)nu * mp, SKn, (int64_t)nu * mp, n + 1,
-                                                  c->stream);
+                            return launch_spmm_hs(c->A, k, SKn, (int64_t)nu * mp, n + 1, c->stream);
                         }))) {
                 return r;
             }

@@ -125,7 +125,20 @@ struct KrylovBatch {
     uint8_t *thop = nullptr;
     uint16_t *tinv = nullptr;
     int *tcnt = nullptr;
+    // Global mode: the inverse of the tile order, tord[c * ntile + r] = the tile
+    // at position r, and w_n of the current step as the product's input panel,
+    //   panel[((g * 8 ntile + I) * kPanel + c % kPanel) * 4 + a],  g = c / kPanel
+    // (atom I, orbital a), zero outside the support; null in regional mode.
+    uint16_t *tord = nullptr;
+    void *panel = nullptr;
 };
+// Entries of the panel for nb columns of ntile tiles, and an atom's place in it.
+__host__ __device__ constexpr int64_t panel_entries(int64_t nb, int64_t ntile) { return (nb + 63) / 64 * 64 * ntile * 32; }
+constexpr int kPanel = 4;   // columns side by side in the panel (krylov.cu)
+__device__ __forceinline__ int64_t panel_pos(int ntile, int c, int64_t I)
+{
+    return (((int64_t)(c / kPanel) * (8 * (int64_t)ntile) + I) * kPanel + (c % kPanel)) * 4;
+}
 
 // ---------------------------------------------------------------- index checks
 // Built with -DMARNOLDI_CHECK, kernels test the indices they take from data
@@ -276,12 +289,11 @@ cudaError_t launch_init(const DeviceMatrix &A, const KrylovBatch &b, cudaStream_
 cudaError_t launch_zero_partial_tile(const KrylovBatch &b, int rows, cudaStream_t s);
 cudaError_t launch_support(const DeviceMatrix &A, const RegionMaps *rm, const KrylovBatch &b,
                            cudaStream_t s);
-// U (and Ulo) = H X and, when SY is not null, SY = S X for the batch (X and
-// SY with column strides ldx, ldsy; U with m_pad); rows of tiles with
-// thop > lim are written as zeros without being computed (X must vanish
-// outside thop <= lim - 1).
-cudaError_t launch_spmm_hs(const DeviceMatrix &A, const KrylovBatch &b, const void *X, int64_t ldx,
-                           void *SY, int64_t ldsy, int lim, cudaStream_t s);
+// U (and Ulo) = H x and, when SY is not null, SY = S x for the batch's panel x
+// (SY with column stride ldsy; U with m_pad); rows of tiles with thop > lim are
+// written as zeros without being computed (x vanishes outside thop <= lim - 1).
+cudaError_t launch_spmm_hs(const DeviceMatrix &A, const KrylovBatch &b, void *SY, int64_t ldsy, int lim,
+                           cudaStream_t s);
 cudaError_t launch_gs(const KrylovBatch &b, int n, int need_w, double tau, cudaStream_t s);
 
 // ---------------------------------------------------------------- subspace eigensolve

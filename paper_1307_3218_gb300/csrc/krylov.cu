@@ -81,7 +81,8 @@ __global__ void init_kernel(const int64_t *__restrict__ rp, const int32_t *__res
                             const int64_t *__restrict__ cols, VT *__restrict__ K,
                             VT *__restrict__ SK, double *__restrict__ scale,
                             int *__restrict__ status, int *__restrict__ nu_eff, int nu,
-                            int64_t m_pad, const uint16_t *__restrict__ tinv, int nb)
+                            int64_t m_pad, const uint16_t *__restrict__ tinv, int nb, VT *__restrict__ panel,
+                            int ntile)
 {
     const int c = blockIdx.x;
     const int64_t j = cols[c];
@@ -97,6 +98,7 @@ __global__ void init_kernel(const int64_t *__restrict__ rp, const int32_t *__res
     const double inv = 1.0 / sqrt(sdiag[j]);
     if (threadIdx.x == 0) {
         k0[vpos(tinv, nb, c, j)] = (VT)inv;
+        panel[panel_pos(ntile, c, J) + b] = (VT)inv;
         scale[(int64_t)c * nu] = 1.0;
         status[c] = 0;
         nu_eff[c] = nu;
@@ -112,41 +114,57 @@ __global__ void init_kernel(const int64_t *__restrict__ rp, const int32_t *__res
 }
 
 // ------------------------------------------------------------------ SpMM
-// Y[c] = A X[c] for the batch columns c < ncols.  Thread (tx, ty) of a 32x8 CTA
-// owns block row I = 8 blockIdx.x + ty of column c = 32 blockIdx.y + tx, so
-// the 32 lanes of a warp share block row I (the matrix block is a broadcast
-// load) and read 32 columns' 4-vectors, and the CTA's 8 rows are support tile
-// blockIdx.x.  Rows run fastest in the grid, so the CTAs in flight work on one
-// or two 32-column tiles whose input panels stay in L2 while their ~b gathers
-// per entry hit it.
-//
-// Column c's x and y are stored in its tile order: block row I at position
-// apos(I) = 8 tinv[I / 8] + I % 8 (4 entries each).  Support: row I of
-// column c vanishes when its tile lies more than `lim` hops from the column's
-// atom (thop > lim; the input vanishes beyond lim - 1).  A lane past the
-// support gathers nothing and a warp with no live lane only writes its zeros.
-struct RowLive {
-    bool live, act;
-};
-__device__ __forceinline__ RowLive row_live(const uint8_t *__restrict__ thop, int tile, int nb,
-                                            int c, int lim)
+__device__ __forceinline__ void lds_x4(uint32_t a, uint64_t (&v)[4])
 {
-    const bool live = c < nb;
-    return RowLive{live, live && (int)thop[(int64_t)tile * nb + c] <= lim};
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(a));
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(v[2]), "=l"(v[3]) : "r"(a + 16));
 }
-__device__ __forceinline__ int64_t apos(const uint16_t *__restrict__ tinv, int nb, int c, int64_t I)
+__device__ __forceinline__ void lds_d4(uint32_t a, double (&v)[4])
 {
-    return 8 * (int64_t)tinv[(I >> 3) * nb + c] + (I & 7);
+    asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "r"(a));
+    asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v[2]), "=d"(v[3]) : "r"(a + 16));
+}
+// (hi, lo) += (h + l) x per lane of the pairs, nx = -x: p = h x, its error and
+// l x (negated, so that no integer instruction negates p), and p added to hi
+// with a two-sum.
+__device__ __forceinline__ void spmm_add(uint64_t &hi, uint64_t &lo, uint64_t h, uint64_t l, uint64_t x, uint64_t nx)
+{
+    asm("{\n\t.reg .b64 p, e, s, bb, t, u, err;\n\t"
+        "mul.rn.f32x2 p, %2, %4;\n\t"
+        "fma.rn.f32x2 e, %2, %5, p;\n\t"
+        "fma.rn.f32x2 e, %3, %5, e;\n\t"
+        "add.rn.f32x2 s, %0, p;\n\t"
+        "sub.rn.f32x2 bb, s, %0;\n\t"
+        "sub.rn.f32x2 t, s, bb;\n\t"
+        "sub.rn.f32x2 t, %0, t;\n\t"
+        "sub.rn.f32x2 u, p, bb;\n\t"
+        "add.rn.f32x2 err, t, u;\n\t"
+        "sub.rn.f32x2 e, e, err;\n\t"
+        "sub.rn.f32x2 %1, %1, e;\n\t"
+        "mov.b64 %0, s;\n\t}"
+        : "+l"(hi), "+l"(lo)
+        : "l"(h), "l"(l), "l"(x), "l"(nx));
 }
 
 // H x and S x for the same panel in one pass (both feed the Gram-Schmidt step
 // of the same Krylov vector, and H and S share their block pattern): each x
-// entry is gathered once for both products.  Thread (tx, ty) of a 32x8 CTA
-// owns block row I = 8 blockIdx.x + ty (the CTA's 8 rows are support tile
-// blockIdx.x) for the two columns c = 64 blockIdx.y + tx and c + 32, so every
-// matrix block, a broadcast load across the warp, serves 64 columns.  Rows run
-// fastest in the grid, so the CTAs in flight work on one or two 64-column
-// tiles whose input panels stay in L2 while their ~b gathers per entry hit it.
+// entry is gathered once for both products.  A warp takes one block row for 64
+// columns, a lane the two columns 64 g + lane and 64 g + lane + 32; a CTA's W
+// warps take W consecutive rows, which share most of their neighbours.  Rows
+// run fastest in the grid, so the CTAs in flight work on a few column groups
+// whose input panels stay in L2.
+//
+// The input is the panel that the Gram-Schmidt step wrote beside the vector's
+// slot: atom-major, kPanel columns side by side, zero outside the supports.
+// Gathering a block's x from the columns' own slots, each in its own tile
+// order, touched 32 lines per load and held the L1 at 75 %: 16,384 columns of
+// 4,096 atoms, nu = 30, 190.1 ms, now 145.7 (the Gram-Schmidt step pays 9 ms for
+// the panel; 13 with 16 columns side by side, whose product is 0.8 ms faster).
+// Column c's y are stored in its tile order: block row I at position
+// 8 tinv[I / 8] + I % 8 (4 entries each).  Support: row I of column c vanishes
+// when its tile lies more than `lim` hops from the column's atom (thop > lim;
+// the input vanishes beyond lim - 1); a warp with no live lane only writes
+// zeros.
 //
 // FP64: plain FMAs.  Mixed precision (matrix blocks stored as 16 "hi" then 16
 // "lo" FP32 values, hi + lo = the FP64 value to about 2^-48): the subspace
@@ -156,91 +174,157 @@ __device__ __forceinline__ int64_t apos(const uint16_t *__restrict__ tinv, int n
 // errors collect in a second FP32 word, and u is written as a normalised
 // (hi, lo) FP32 pair; the Krylov vector itself continues from the hi word.
 // S x is plain FP32 with the hi values: its rounding only perturbs the
-// Gram-Schmidt coefficients and the norms, which the second pass and the
-// subspace Galerkin step absorb.
-template <typename VT, bool kS>
-__global__ void __launch_bounds__(256) spmm_hs_kernel(
-    int64_t nbr, const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
-    const VT *__restrict__ Hv, const VT *__restrict__ Sv, const VT *__restrict__ X, int64_t ldx,
+// Gram-Schmidt coefficients and the norms, which G and the subspace Galerkin
+// step absorb.  A lane's two columns share one packed instruction (f32x2).
+//
+// What bounds it: the FP32 pipe, 68 % busy (12 operations per matrix entry and
+// column); FP64: the FP64 pipe.  The warp's blocks go through its own two slots
+// of shared memory, each value twice (FP32), so that one 16-byte broadcast read
+// gives two packed operands; block q + 2 is on its way from L2 and block q + 1's
+// x entries are loaded while block q computes.
+template <typename VT> struct SpmmCfg {
+    static constexpr bool kF = sizeof(VT) == 4;
+    // shared memory per block: H hi, H lo and S, each value twice (FP32); H and S (FP64)
+    static constexpr int kSmem = kF ? 48 * 8 : 32 * 8;
+};
+
+template <typename VT, bool kS, int W>
+__global__ void __launch_bounds__(32 * W, (sizeof(VT) == 4 ? 20 : 16) / W) spmm_hs_kernel(
+    int nbr, const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
+    const VT *__restrict__ Hv, const VT *__restrict__ Sv, const VT *__restrict__ panel, int ntile,
     VT *__restrict__ U, VT *__restrict__ Ulo, int64_t ldu, VT *__restrict__ SY, int64_t ldsy,
     int ncols, const uint8_t *__restrict__ thop, const uint16_t *__restrict__ tinv, int lim)
 {
-    constexpr bool kF = sizeof(VT) == 4;
-    constexpr int BS = kF ? 32 : 16;   // stored values per block
-    const int64_t I = (int64_t)blockIdx.x * 8 + threadIdx.y;
+    using Cfg = SpmmCfg<VT>;
+    constexpr bool kF = Cfg::kF;
+    __shared__ __align__(16) unsigned char blk[W][2][Cfg::kSmem];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int I = (int)blockIdx.x * W + warp, tile = I >> 3;
     if (I >= nbr) return;   // uniform over the warp
     int cc[2];
-    RowLive L[2];
+    bool act = false;
     int64_t yo[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        cc[h] = blockIdx.y * 64 + 32 * h + threadIdx.x;
-        L[h] = row_live(thop, blockIdx.x, ncols, cc[h], lim);
-        yo[h] = L[h].live ? 4 * apos(tinv, ncols, cc[h], I) : 0;
+        cc[h] = (int)blockIdx.y * 64 + 32 * h + lane;
+        act |= cc[h] < ncols && (int)thop[(int64_t)tile * ncols + cc[h]] <= lim;
+        // no position: past the columns, or a row of another structure of a
+        // union, whose tiles may sit past this column's positions
+        yo[h] = cc[h] < ncols ? 32 * (int64_t)tinv[(int64_t)tile * ncols + cc[h]] + 4 * (I & 7) : ldu;
     }
-    VT hi[2][4], lo[2][4], sy[2][4];
+    uint64_t hi[4], lo[4], sy[4];   // FP32: per row entry, the two columns
+    double hd[2][4], sd[2][4];      // FP64
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int a = 0; a < 4; ++a) hi[h][a] = lo[h][a] = sy[h][a] = VT(0);
-    if (__any_sync(kFull, L[0].act || L[1].act)) {
-        const VT *x0 = X + (int64_t)(L[0].live ? cc[0] : 0) * ldx;
-        const VT *x1 = X + (int64_t)(L[1].live ? cc[1] : 0) * ldx;
-        const int64_t k1 = rp[I + 1];
-        for (int64_t k = rp[I]; k < k1; ++k) {
-            const int64_t J = ci[k];
-            VT xv[2][4] = {{VT(0), VT(0), VT(0), VT(0)}, {VT(0), VT(0), VT(0), VT(0)}};
-            if (L[0].act) {
-                const int64_t xp = 4 * apos(tinv, ncols, cc[0], J);
-                if (in_range(xp, ldu - 3, kChkSpmmGather)) load4(x0 + xp, xv[0]);
+    for (int a = 0; a < 4; ++a) {
+        hi[a] = lo[a] = sy[a] = 0;
+        hd[0][a] = hd[1][a] = sd[0][a] = sd[1][a] = 0.0;
+    }
+    if (__any_sync(kFull, act)) {
+        const int64_t k0 = rp[I];
+        const int nk = (int)(rp[I + 1] - k0);
+        const VT *xp0 = panel + panel_pos(ntile, cc[0], 0);
+        const int dx = 32 / kPanel * ntile * (32 * kPanel);   // to the column 32 further
+        int jv = 0;   // column atoms of blocks 32 (q / 32) + lane
+        auto column = [&](int q) {
+            if ((q & 31) == 0) jv = k0 + q + lane < k0 + nk ? ci[k0 + q + lane] : 0;
+            return __shfl_sync(kFull, jv, q & 31);
+        };
+        // this lane's 16 bytes of a block: H (lanes 0-7), then S (FP32: its hi
+        // values only, lanes 8-11; FP64: lanes 8-15)
+        const bool loads = lane < 8 || (kS && lane < (kF ? 12 : 16));
+        const float4 *src = reinterpret_cast<const float4 *>(lane < 8 ? Hv : Sv) + 8 * k0 + (lane & 7);
+        auto fetch = [&](int q) { return loads && q < nk ? __ldg(src + 8 * q) : make_float4(0.f, 0.f, 0.f, 0.f); };
+        auto stage = [&](int q, const float4 &v) {
+            if (!loads) return;
+            float4 *d = reinterpret_cast<float4 *>(blk[warp][q & 1]);
+            if constexpr (kF) {
+                d[2 * lane] = make_float4(v.x, v.x, v.y, v.y);
+                d[2 * lane + 1] = make_float4(v.z, v.z, v.w, v.w);
+            } else {
+                d[lane] = v;
             }
-            if (L[1].act) {
-                const int64_t xp = 4 * apos(tinv, ncols, cc[1], J);
-                if (in_range(xp, ldu - 3, kChkSpmmGather)) load4(x1 + xp, xv[1]);
+        };
+        auto gather = [&](int J, VT (&x)[2][4]) {
+            if (!in_range(J, 8 * ntile, kChkSpmmGather)) J = 0;
+            const VT *p = xp0 + J * (4 * kPanel);
+            load4(p, x[0]);
+            load4(p + dx, x[1]);
+        };
+        VT xn[2][4];
+        float4 v = fetch(0);
+        gather(column(0), xn);
+        stage(0, v);
+        v = fetch(1);
+#pragma unroll 1
+        for (int q = 0; q < nk; ++q) {
+            __syncwarp();   // block q is staged, block q - 1 read
+            VT x[2][4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                x[0][e] = xn[0][e];
+                x[1][e] = xn[1][e];
             }
-            const VT *Hb = Hv + BS * k;
-            const VT *Sb = Sv + BS * k;
+            if (q + 1 < nk) {
+                stage(q + 1, v);
+                gather(column(q + 1), xn);
+                v = fetch(q + 2);
+            }
+            const uint32_t sb = (uint32_t)__cvta_generic_to_shared(blk[warp][q & 1]);
+            if constexpr (kF) {
+                uint64_t xp[4], nx[4];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                VT hr[4], sr[4], lr[4];
-                load4(Hb + 4 * a, hr);
-                if constexpr (kS) load4(Sb + 4 * a, sr);
-                if constexpr (kF) load4(Hb + 16 + 4 * a, lr);
+                for (int e = 0; e < 4; ++e) {
+                    xp[e] = pack_x2(x[0][e], x[1][e]);
+                    nx[e] = neg_x2(xp[e]);
+                }
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
+                for (int a = 0; a < 4; ++a) {
+                    uint64_t h4[4], l4[4], s4[4];
+                    lds_x4(sb + 32 * a, h4);
+                    lds_x4(sb + 128 + 32 * a, l4);
+                    if constexpr (kS) lds_x4(sb + 256 + 32 * a, s4);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        if constexpr (kF) {
-                            const float p = __fmul_rn(hr[q], xv[h][q]);
-                            const float e = __fmaf_rn(hr[q], xv[h][q], -p);
-                            df_add(hi[h][a], lo[h][a], p, __fmaf_rn(lr[q], xv[h][q], e));
-                        } else {
-                            hi[h][a] = fma(hr[q], xv[h][q], hi[h][a]);
-                        }
-                        if constexpr (kS) sy[h][a] = fma(sr[q], xv[h][q], sy[h][a]);
+                    for (int e = 0; e < 4; ++e) {
+                        spmm_add(hi[a], lo[a], h4[e], l4[e], xp[e], nx[e]);
+                        if constexpr (kS) sy[a] = fma_x2(s4[e], xp[e], sy[a]);
                     }
+                }
+            } else {
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    double h4[4], s4[4];
+                    lds_d4(sb + 32 * a, h4);
+                    if constexpr (kS) lds_d4(sb + 128 + 32 * a, s4);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            hd[h][a] = fma(h4[e], x[h][e], hd[h][a]);
+                            if constexpr (kS) sd[h][a] = fma(s4[e], x[h][e], sd[h][a]);
+                        }
                 }
             }
         }
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        // rows outside the support get their zeros, except rows of another
-        // structure of a union, whose tiles may sit past this column's positions
-        if (!L[h].live || yo[h] >= ldu) continue;
+        if (yo[h] >= ldu) continue;
         if constexpr (kF) {
-            float yh[4], yl[4];
+            float yh[4], yl[4], ys[4];
 #pragma unroll
             for (int a = 0; a < 4; ++a) {   // renormalise: yh = fl(hi + lo), yl = the rest
-                yh[a] = __fadd_rn(hi[h][a], lo[h][a]);
-                yl[a] = __fsub_rn(lo[h][a], __fsub_rn(yh[a], hi[h][a]));
+                const float fh = h ? lane_y(hi[a]) : lane_x(hi[a]), fl = h ? lane_y(lo[a]) : lane_x(lo[a]);
+                yh[a] = __fadd_rn(fh, fl);
+                yl[a] = __fsub_rn(fl, __fsub_rn(yh[a], fh));
+                ys[a] = h ? lane_y(sy[a]) : lane_x(sy[a]);
             }
             store4(U + (int64_t)cc[h] * ldu + yo[h], yh);
             store4(Ulo + (int64_t)cc[h] * ldu + yo[h], yl);
+            if constexpr (kS) store4(SY + (int64_t)cc[h] * ldsy + yo[h], ys);
         } else {
-            store4(U + (int64_t)cc[h] * ldu + yo[h], hi[h]);
+            store4(U + (int64_t)cc[h] * ldu + yo[h], hd[h]);
+            if constexpr (kS) store4(SY + (int64_t)cc[h] * ldsy + yo[h], sd[h]);
         }
-        if constexpr (kS) store4(SY + (int64_t)cc[h] * ldsy + yo[h], sy[h]);
     }
 }
 
@@ -481,7 +565,8 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
     VT *__restrict__ K, const VT *__restrict__ SK, const VT *__restrict__ U, const VT *__restrict__ Ulo,
     double *__restrict__ Hsub, double *__restrict__ Lsub, double *__restrict__ scale,
     double *__restrict__ cn2, int *__restrict__ status, int *__restrict__ nu_eff,
-    const int *__restrict__ tcnt, int64_t MP, int n, int nu, int need_w, double tau2)
+    const int *__restrict__ tcnt, const uint16_t *__restrict__ tord, VT *__restrict__ panel, int ntile, int64_t MP,
+    int n, int nu, int need_w, double tau2)
 {
     using Cfg = GsCfg<VT, C, R, kPairs>;
     constexpr bool kF = sizeof(VT) == 4;
@@ -713,6 +798,11 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
     // s_n u, not of w_{n+1}, outside span(K)).
     const VT vsn = (VT)ssc[n];
     VT *wo = K + base + (int64_t)(n + 1) * MP;   // the next slot, unnormalised, zeros included
+    // and, in global mode, its entries as the next product's input
+    auto panel_at = [&](int p) {
+        const int I = 8 * tord[(int64_t)c * ntile + (p >> 5)] + ((p >> 2) & 7);
+        return panel + panel_pos(ntile, c, I) + (p & 3);
+    };
 #pragma unroll 1
     for (int v0 = 0; v0 < nch_u; v0 += SC) {
         PairAcc x[kF ? SC : 1][2];
@@ -821,12 +911,16 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
                                         __fadd_rn(lane_x(x[q][1].hi), lane_x(x[q][1].lo)),
                                         __fadd_rn(lane_y(x[q][1].hi), lane_y(x[q][1].lo)));
                     *reinterpret_cast<float4 *>(wo + v * C + off) = r;
+                    if (panel && (v * C + off) >> 5 < cnt_u) *reinterpret_cast<float4 *>(panel_at(v * C + off)) = r;
                 } else {
 #pragma unroll
-                    for (int h = 0; h < kH; ++h)
-                        *reinterpret_cast<double2 *>(wo + v * C + off + h * (C / 2)) =
-                            (v * C + off + h * (C / 2)) >> 5 < cnt_u ? make_double2(xd[q][2 * h], xd[q][2 * h + 1])
-                                                          : make_double2(0.0, 0.0);
+                    for (int h = 0; h < kH; ++h) {
+                        const int p = v * C + off + h * (C / 2);
+                        const bool a = p >> 5 < cnt_u;
+                        const double2 r = a ? make_double2(xd[q][2 * h], xd[q][2 * h + 1]) : make_double2(0.0, 0.0);
+                        *reinterpret_cast<double2 *>(wo + p) = r;
+                        if (panel && a) *reinterpret_cast<double2 *>(panel_at(p)) = r;
+                    }
                 }
             }
         }
@@ -866,7 +960,7 @@ cudaError_t gs_dispatch(const KrylovBatch &b, int n, int need_w, double tau, cud
     if (e != cudaSuccess) return e;
     gs_kernel<VT, C, R, kPairs><<<b.nb, Cfg::T, smem, s>>>(
         (VT *)b.K, (const VT *)b.SK, (const VT *)b.U, (const VT *)b.Ulo, b.Hsub, b.Lsub, b.scale, b.cn2,
-        b.status, b.nu_eff, b.tcnt, b.shape.m_pad, n, b.nu, need_w, tau * tau);
+        b.status, b.nu_eff, b.tcnt, b.tord, (VT *)b.panel, b.ntile, b.shape.m_pad, n, b.nu, need_w, tau * tau);
     return cudaGetLastError();
 }
 
@@ -900,41 +994,46 @@ cudaError_t launch_init(const DeviceMatrix &A, const KrylovBatch &b, cudaStream_
     if (b.prec == 0)
         init_kernel<double><<<b.nb, 256, 0, s>>>(A.rp, A.ci, A.Sd, A.sdiag, b.cols, (double *)b.K,
                                                  (double *)b.SK, b.scale, b.status, b.nu_eff, b.nu,
-                                                 b.shape.m_pad, b.tinv, b.nb);
+                                                 b.shape.m_pad, b.tinv, b.nb, (double *)b.panel, b.ntile);
     else
         init_kernel<float><<<b.nb, 256, 0, s>>>(A.rp, A.ci, A.Sd, A.sdiag, b.cols, (float *)b.K,
                                                 (float *)b.SK, b.scale, b.status, b.nu_eff, b.nu,
-                                                b.shape.m_pad, b.tinv, b.nb);
+                                                b.shape.m_pad, b.tinv, b.nb, (float *)b.panel, b.ntile);
     return cudaGetLastError();
 }
 
-cudaError_t launch_spmm_hs(const DeviceMatrix &A, const KrylovBatch &b, const void *X, int64_t ldx,
-                           void *SY, int64_t ldsy, int lim, cudaStream_t s)
+namespace {
+
+constexpr int64_t kSpmmWarps = 152 * 8;   // fewest warps of a launch with several per CTA
+
+template <typename VT, bool kS>
+cudaError_t spmm_hs(const DeviceMatrix &A, const VT *Hv, const VT *Sv, const KrylovBatch &b, void *SY,
+                    int64_t ldsy, int lim, cudaStream_t s)
 {
-    if (!b.thop || !b.tinv || b.ntile * 8 < A.nbr) return cudaErrorInvalidValue;
-    const dim3 block(32, 8);
-    const dim3 grid((unsigned)((A.nbr + 7) / 8), (unsigned)((b.nb + 63) / 64));
-    const int64_t ldu = b.shape.m_pad;
-    if (b.prec == 0) {
-        if (SY)
-            spmm_hs_kernel<double, true><<<grid, block, 0, s>>>(
-                A.nbr, A.rp, A.ci, A.Hd, A.Sd, (const double *)X, ldx, (double *)b.U, nullptr, ldu,
-                (double *)SY, ldsy, b.nb, b.thop, b.tinv, lim);
-        else
-            spmm_hs_kernel<double, false><<<grid, block, 0, s>>>(
-                A.nbr, A.rp, A.ci, A.Hd, A.Sd, (const double *)X, ldx, (double *)b.U, nullptr, ldu,
-                nullptr, 0, b.nb, b.thop, b.tinv, lim);
-    } else {
-        if (SY)
-            spmm_hs_kernel<float, true><<<grid, block, 0, s>>>(
-                A.nbr, A.rp, A.ci, A.Hf, A.Sf, (const float *)X, ldx, (float *)b.U, (float *)b.Ulo, ldu,
-                (float *)SY, ldsy, b.nb, b.thop, b.tinv, lim);
-        else
-            spmm_hs_kernel<float, false><<<grid, block, 0, s>>>(
-                A.nbr, A.rp, A.ci, A.Hf, A.Sf, (const float *)X, ldx, (float *)b.U, (float *)b.Ulo, ldu,
-                nullptr, 0, b.nb, b.thop, b.tinv, lim);
-    }
+    const int64_t ng = (b.nb + 63) / 64, ldu = b.shape.m_pad;
+    auto go = [&](auto w) {
+        constexpr int W = decltype(w)::value;
+        spmm_hs_kernel<VT, kS, W><<<dim3((unsigned)((A.nbr + W - 1) / W), (unsigned)ng), 32 * W, 0, s>>>(
+            (int)A.nbr, A.rp, A.ci, Hv, Sv, (const VT *)b.panel, b.ntile, (VT *)b.U, (VT *)b.Ulo, ldu, (VT *)SY, ldsy, b.nb,
+            b.thop, b.tinv, lim);
+    };
+    // four rows per CTA; one when that leaves SMs without work (64 atoms, 256
+    // columns: 1.30 ms against 2.18 per FP64 solve of nu = 30, 0.37 against 0.79 mixed)
+    if (A.nbr * ng >= kSpmmWarps) go(std::integral_constant<int, 4>());
+    else go(std::integral_constant<int, 1>());
     return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_spmm_hs(const DeviceMatrix &A, const KrylovBatch &b, void *SY, int64_t ldsy, int lim,
+                           cudaStream_t s)
+{
+    if (!b.thop || !b.tinv || !b.panel || b.ntile * 8 < A.nbr) return cudaErrorInvalidValue;
+    if (b.prec == 0)
+        return SY ? spmm_hs<double, true>(A, A.Hd, A.Sd, b, SY, ldsy, lim, s)
+                  : spmm_hs<double, false>(A, A.Hd, A.Sd, b, SY, ldsy, lim, s);
+    return SY ? spmm_hs<float, true>(A, A.Hf, A.Sf, b, SY, ldsy, lim, s)
+              : spmm_hs<float, false>(A, A.Hf, A.Sf, b, SY, ldsy, lim, s);
 }
 
 cudaError_t launch_gs(const KrylovBatch &b, int n, int need_w, double tau, cudaStream_t s)

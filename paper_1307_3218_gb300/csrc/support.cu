@@ -33,7 +33,8 @@ __global__ void __launch_bounds__(256) support_kernel(
     const int64_t *__restrict__ rp, const int32_t *__restrict__ ci, int nbr,
     const int *__restrict__ reg, int n_reg, int maxrow, const int *__restrict__ lcnt,
     const int *__restrict__ lci, const int64_t *__restrict__ cols, int nb, int ntile, int maxlev,
-    int nlev, uint8_t *__restrict__ thop, uint16_t *__restrict__ tinv, int *__restrict__ tcnt)
+    int nlev, uint8_t *__restrict__ thop, uint16_t *__restrict__ tinv, int *__restrict__ tcnt,
+    uint16_t *__restrict__ tord)
 {
     extern __shared__ uint8_t dist[];   // per atom (global or local index)
     __shared__ uint8_t th[kMaxTiles];
@@ -90,7 +91,9 @@ __global__ void __launch_bounds__(256) support_kernel(
         int tail = run;
         for (int t = 0; t < ntile; ++t) {
             const int h = th[t];
-            tinv[(int64_t)t * nb + c] = (uint16_t)(h <= maxlev ? start[h]++ : tail++);
+            const int r = h <= maxlev ? start[h]++ : tail++;
+            tinv[(int64_t)t * nb + c] = (uint16_t)r;
+            if (tord) tord[(int64_t)c * ntile + r] = (uint16_t)t;
         }
     }
 }
@@ -149,12 +152,12 @@ cudaError_t launch_support(const DeviceMatrix &A, const RegionMaps *rm, const Kr
         if (rm->n_reg > kMaxRegion) return cudaErrorInvalidValue;
         support_kernel<true><<<b.nb, 256, rm->n_reg, s>>>(
             A.rp, A.ci, (int)A.nbr, rm->reg, rm->n_reg, rm->maxrow, rm->lcnt, rm->lci, b.cols, b.nb,
-            b.ntile, maxlev, nlev, b.thop, b.tinv, b.tcnt);
+            b.ntile, maxlev, nlev, b.thop, b.tinv, b.tcnt, nullptr);
     } else {
         if (A.nbr > kMaxGlobalM / 4) return cudaErrorInvalidValue;
         support_kernel<false><<<b.nb, 256, (size_t)A.nbr, s>>>(
             A.rp, A.ci, (int)A.nbr, nullptr, 0, 0, nullptr, nullptr, b.cols, b.nb, b.ntile, maxlev,
-            nlev, b.thop, b.tinv, b.tcnt);
+            nlev, b.thop, b.tinv, b.tcnt, b.tord);
     }
     return cudaGetLastError();
 }
