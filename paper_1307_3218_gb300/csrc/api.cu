@@ -662,7 +662,7 @@ struct SolvePlan {
     bool a_global;
     EigScratch es;   // sizes and chunk; the caller sets the pointers
     size_t oK, oSK, oU, oUl, oH, oL, oSc, oC, oS, oN, oRg, oRc, oRi, oRk, oRs, oTh, oTo, oTc;
-    size_t oTr, oPn, oED, oEE, oERQ, oERot, oESw, oENs, oEA, ws_bytes;
+    size_t oTr, oPn, oED, oEE, oEV, oERot, oESw, oENs, oEA, ws_bytes;
 };
 
 // Workspace bytes per batch column, for the default batch size.
@@ -747,7 +747,7 @@ bool plan_solve(int64_t m_vec, int prec, int nu, int region_atoms, int maxrow, i
     p.a_global = eig_smem_bytes(nu, es.nr_max, false) > kSmemCap;
     if (eig_smem_bytes(nu, es.nr_max, p.a_global) > kSmemCap) return false;
     const size_t a_per_sub = p.a_global ? (size_t)nu * (nu | 1) * 8 : 0;
-    const size_t per_sub = al256((size_t)(2 + es.nr_max) * nu * 8) + al256((size_t)es.rcap * 16) +
+    const size_t per_sub = al256((size_t)(2 + nu) * nu * 8) + al256((size_t)es.rcap * 16) +
                            al256((size_t)es.scap * 8) + 8 + a_per_sub;
     // the QL kernel runs one subspace per lane and its time hardly grows with the chunk (it is
     // latency-bound), so chunks are as large as 12 GB of scratch allow: at nu = 100 a whole
@@ -756,8 +756,8 @@ bool plan_solve(int64_t m_vec, int prec, int nu, int region_atoms, int maxrow, i
     const size_t ceig = (size_t)es.chunk;
     p.oED = oEg;
     p.oEE = p.oED + al256(ceig * nu * 8);
-    p.oERQ = p.oEE + al256(ceig * nu * 8);
-    p.oERot = p.oERQ + al256(ceig * es.nr_max * nu * 8);
+    p.oEV = p.oEE + al256(ceig * nu * 8);
+    p.oERot = p.oEV + al256(ceig * nu * nu * 8);
     p.oESw = p.oERot + al256(ceig * es.rcap * 16);
     p.oENs = p.oESw + al256(ceig * es.scap * 8);
     p.oEA = p.oENs + al256(ceig * 4);
@@ -1403,7 +1403,7 @@ int marnoldi_solve(marnoldi_ctx *c, const int64_t *columns, int64_t ncols, int n
     EigScratch es = plan.es;
     es.D = (double *)(wb + plan.oED);
     es.E = (double *)(wb + plan.oEE);
-    es.RQ = (double *)(wb + plan.oERQ);
+    es.V = (double *)(wb + plan.oEV);
     es.rot = (double2 *)(wb + plan.oERot);
     es.sweep = (int2 *)(wb + plan.oESw);
     es.nsweep = (int *)(wb + plan.oENs);

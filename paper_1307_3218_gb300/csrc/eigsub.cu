@@ -10,19 +10,25 @@
 // reflections and T = Z Lambda Z^T by the implicit-shift QL algorithm
 // (Bowdler, Martin, Reinsch & Wilkinson 1968), so R V = (R Q) Z.  Three
 // kernels per chunk of subspaces:
-//   eig_tridiag_kernel  one CTA per subspace: the reflections, applied to H_sub
-//                       and to R (never forming Q); writes d, e and R Q
-//   eig_ql_kernel       one LANE per subspace (32 subspaces per warp): the
-//                       QL recurrence, which is a serial chain of FP64
-//                       divisions and square roots per subspace.  Running 32
-//                       chains side by side fills GB300's narrow FP64 pipe
-//                       instead of issuing one useful lane per instruction.
-//                       Every Givens rotation (c, s) and every sweep's
-//                       index range is logged.
-//   eig_apply_kernel    one CTA per subspace: each thread replays the log on
-//                       its rows of R Q, then the levels are ranked and
-//                       eps, w_a = sqrt(S_jj) (R V)[0][a] (R V)[1][a], t and
-//                       P_j are written in ascending order of eps.
+//   eig_tridiag_kernel  one CTA per subspace: the reflections, applied to H_sub;
+//                       writes d, e and the reflectors
+//   eig_ql_kernel       one LANE per subspace: the QL recurrence, a serial chain
+//                       of FP64 divisions and square roots per subspace.
+//                       Every rotation is logged, as the two coefficients of
+//                       a fast plane rotation, and every sweep's index range.
+//   eig_apply_kernel    one CTA per subspace, a thread per row of R: the
+//                       reflectors, then the rotations of the log; the levels
+//                       are ranked and eps, w_a = sqrt(S_jj) (R V)[0][a] (R V)[1][a],
+//                       t and P_j are written in ascending order of eps.
+// All three are bound by FP64 instructions (64 cycles each on a warp's
+// scheduler): their sum where many warps run, else the longest chain.  The reflections used
+// to reach R in the first kernel, whose other threads waited and whose shared
+// memory then held one CTA per SM (nu = 100), and a rotation took four FP64
+// instructions per row.  Per solve, before and after (tridiagonalisation, QL,
+// rows): 24,000 subspaces of nu = 30: 13.9 + 2.1 + 12.0 -> 6.0 + 2.3 + 10.2 ms;
+// 4,000 of nu = 100: 60.6 + 16.7 + 23.6 -> 27.5 + 11.3 + 22.8; 348 of nu = 300:
+// 91.5 + 159.9 + 54.7 -> 41.9 + 88.9 + 55.5; 256 of nu = 30: 0.30 + 1.66 + 0.27 ->
+// 0.27 + 1.13 + 0.25.
 #include "internal.h"
 
 #include <math_constants.h>
@@ -34,9 +40,10 @@ namespace marnoldi {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kTriThreads = 256;
-constexpr int kApplyThreads = 128;
+constexpr int kTriThreads = 256;    // most threads of the tridiagonalisation
+constexpr int kApplyThreads = 128;  // most threads of the rows' kernel
 constexpr int kQlMaxIter = 30;      // QL iterations per eigenvalue
+constexpr int kQlWarps = 152;       // one QL warp per SM
 
 __device__ __forceinline__ double warp_sum(double s)
 {
@@ -45,27 +52,21 @@ __device__ __forceinline__ double warp_sum(double s)
     return s;
 }
 
-
 // ------------------------------------------------------------------ tridiagonalisation
-// A = Q T Q^T with Q = P_0 P_1 ... P_{n-3}; R <- R P_0 P_1 ... (R Q).
-// A is symmetric: after the L^-1 transform only its lower triangle is formed
-// and updated (the product A v reads it by rows left of the diagonal and by
-// columns below), which halves the FP64 work of the rank-2 updates and saves
-// two thirds of the second transform's.
-// Shared memory: A [n][lda], R [nr_max][lda] (lda = nu | 1, odd, so that the
-// per-thread row walks of R spread over the banks), v, e, scalars.  When A
-// does not fit (nu above about 110), it lives in a global scratch of
-// nu x lda doubles per subspace (Ag), which the CTA's sweeps keep in L2
-// (720 KB at nu = 300), and shared memory holds R and the vectors only.
-template <typename VT>
+// A = Q T Q^T with Q = P_0 P_1 ... P_{n-3}, P_k = I - tau_k v_k v_k^T on the
+// entries k + 1 ...  A is symmetric: after the L^-1 transform only its lower
+// triangle is formed and updated (the product A v reads it by rows left of the
+// diagonal and by columns below).
+// Shared memory: A [n][lda] (lda = nu | 1, odd, so that the per-thread row
+// walks spread over the banks), v, e, q.  When A and R do not fit one CTA's
+// shared memory (nu above about 110), A lives in a global scratch of nu x lda
+// doubles per subspace (Ag), which the CTA's sweeps keep in L2 (720 KB at
+// nu = 300).  A thread per row of A: the CTA has as many threads as nu needs.
+// Reflector k goes to V[sc][k][0 .. n - k - 2], tau_k to V[sc][k][nu - 1].
 __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
-    const double *__restrict__ Hsub, const int *__restrict__ bnu_eff,
-    const double *__restrict__ bscale, const VT *__restrict__ K, int64_t m_pad,
-    const uint16_t *__restrict__ tinv, int nb, int nu,
-    const int64_t *__restrict__ bcols, const int64_t *__restrict__ rp,
-    const int32_t *__restrict__ ci, const int *__restrict__ reg, int n_reg, int cofs,
-    double *__restrict__ D, double *__restrict__ E, double *__restrict__ RQ, int nr_max,
-    double *__restrict__ Ag, const double *__restrict__ Lsub, const double *__restrict__ proj)
+    const double *__restrict__ Hsub, const int *__restrict__ bnu_eff, int nu, int cofs,
+    double *__restrict__ D, double *__restrict__ E, double *__restrict__ V, double *__restrict__ Ag,
+    const double *__restrict__ Lsub)
 {
     const int sc = blockIdx.x;
     const int c = cofs + sc;
@@ -74,52 +75,26 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
     const int lda = nu | 1;
     extern __shared__ __align__(16) double sm[];
     double *A = Ag ? Ag + (size_t)sc * nu * lda : sm;
-    double *R = Ag ? sm : A + (size_t)nu * lda;
-    double *v = R + (size_t)nr_max * lda;
+    double *v = Ag ? sm : A + (size_t)nu * lda;
     double *ev = v + nu;
+    double *qv = ev + nu;
+    double *Vc = V + (int64_t)sc * nu * nu;
     __shared__ double sc4[4];
+    __shared__ double wpart[kTriThreads / 32];
     __shared__ int skip;
 
-    // rows of R: e_1, q = K^T e_j, and K_pat (zero for atoms outside a region)
-    const int64_t j = bcols[c];
-    const int64_t J = j >> 2;
-    const int *Rg = reg ? reg + (int64_t)c * n_reg : nullptr;
-    const int pJ = Rg ? find_sorted(Rg, n_reg, (int)J) : 0;
-    const int64_t jl = Rg ? 4 * (int64_t)(pJ < 0 ? 0 : pJ) + (j & 3) : j;
-    const int64_t kb = rp[J];
-    const int npat = 4 * (int)(rp[J + 1] - kb);
-    const int nr = npat + 2 + (proj ? 1 : 0);   // the projection row last
-    const VT *Kc = K + (int64_t)c * nu * m_pad;
     for (int idx = tid; idx < n * n; idx += T) {
         const int i = idx / n, l = idx - (idx / n) * n;
         A[i * lda + l] = 0.5 * (Hsub[((int64_t)c * nu + i) * nu + l] +
                                 Hsub[((int64_t)c * nu + l) * nu + i]);
     }
-    for (int idx = tid; idx < nr * n; idx += T) {
-        const int r = idx / n, i = idx - (idx / n) * n;
-        const double si = bscale[(int64_t)c * nu + i];
-        double val;
-        if (r == 0) {
-            val = i == 0 ? 1.0 : 0.0;
-        } else if (r == 1) {
-            val = si * (double)Kc[(int64_t)i * m_pad + vpos(tinv, nb, c, jl)];
-        } else if (r == npat + 2) {
-            val = si * proj[(int64_t)c * nu + i];
-        } else {
-            const int atom = ci[kb + ((r - 2) >> 2)];
-            const int64_t lr = Rg ? find_sorted(Rg, n_reg, atom) : atom;
-            val = lr >= 0 ? si * (double)Kc[(int64_t)i * m_pad + vpos(tinv, nb, c, 4 * lr + ((r - 2) & 3))]
-                          : 0.0;
-        }
-        R[r * lda + i] = val;
-    }
     __syncthreads();
     // The stored basis K~ has unit S-norms and S-Gram matrix G = L L^T, so the
     // S-orthonormal basis K = K~ L^-T carries the subspace problem
-    // A = L^-1 H~ L^-T and the rows q^T = q~^T L^-T and K_pat = K~_pat L^-T
-    // (row 0, e_1^T, is unchanged: K^T S e_j = sqrt(S_jj) e_1).  Lsub holds
-    // L^-1 (lower triangular); the products run in place from the last row
-    // (column) down, which only reads rows (columns) not yet replaced.
+    // A = L^-1 H~ L^-T.  Lsub holds L^-1 (lower triangular); the products run
+    // in place from the last row (column) down, which only reads rows
+    // (columns) not yet replaced.  Four sums side by side keep the FP64 pipe
+    // supplied.
     const double *Lc = Lsub + (int64_t)c * nu * nu;
     constexpr int kPer = (kMaxNu + kTriThreads - 1) / kTriThreads;   // entries per thread
     for (int i = n - 1; i >= 0; --i) {   // A <- L^-1 A, row i at a time
@@ -128,10 +103,15 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
 #pragma unroll
         for (int q = 0; q < kPer; ++q) {
             const int col = tid + q * T;
-            double s = 0.0;
-            if (col < n)
-                for (int m = 0; m <= i; ++m) s = fma(Li[m], A[m * lda + col], s);
-            x[q] = s;
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            if (col < n) {
+                int m = 0;
+                for (; m + 3 <= i; m += 4)
+#pragma unroll
+                    for (int z = 0; z < 4; ++z) s[z] = fma(Li[m + z], A[(m + z) * lda + col], s[z]);
+                for (; m <= i; ++m) s[0] = fma(Li[m], A[m * lda + col], s[0]);
+            }
+            x[q] = (s[0] + s[1]) + (s[2] + s[3]);
         }
         __syncthreads();
 #pragma unroll
@@ -149,10 +129,15 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
 #pragma unroll
         for (int q = 0; q < kPer; ++q) {
             const int row = tid + q * T;
-            double s = 0.0;
-            if (row >= i && row < n)
-                for (int m = 0; m <= i; ++m) s = fma(A[row * lda + m], Li[m], s);
-            x[q] = s;
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            if (row >= i && row < n) {
+                int m = 0;
+                for (; m + 3 <= i; m += 4)
+#pragma unroll
+                    for (int z = 0; z < 4; ++z) s[z] = fma(A[row * lda + m + z], Li[m + z], s[z]);
+                for (; m <= i; ++m) s[0] = fma(A[row * lda + m], Li[m], s[0]);
+            }
+            x[q] = (s[0] + s[1]) + (s[2] + s[3]);
         }
         __syncthreads();
 #pragma unroll
@@ -160,16 +145,6 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
             if (tid + q * T >= i && tid + q * T < n) A[(tid + q * T) * lda + i] = x[q];
         __syncthreads();
     }
-    for (int r = 1 + tid; r < nr; r += T) {   // R's rows 1..: R <- R L^-T, one row per thread
-        double *x = R + r * lda;
-        for (int i = n - 1; i >= 0; --i) {
-            const double *Li = Lc + (int64_t)i * nu;
-            double s = 0.0;
-            for (int m = 0; m <= i; ++m) s = fma(x[m], Li[m], s);
-            x[i] = s;
-        }
-    }
-    __syncthreads();
 
     for (int k = 0; k + 2 < n; ++k) {
         const int L = n - k - 1;  // x = A[k+1 .. n-1][k]
@@ -185,6 +160,7 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
                 if (tail == 0.0) {
                     skip = 1;
                     ev[k] = x0;
+                    Vc[(int64_t)k * nu + nu - 1] = 0.0;
                 } else {
                     const double s = tail + x0 * x0;
                     const double alpha = -copysign(sqrt(s), x0);
@@ -193,6 +169,7 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
                     ev[k] = alpha;
                     sc4[0] = 2.0 / (v0 * v0 + tail);   // reflector I - tau v v^T
                     sc4[1] = v0;
+                    Vc[(int64_t)k * nu + nu - 1] = sc4[0];
                 }
             }
         }
@@ -202,46 +179,48 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
             continue;
         }
         const double tauh = sc4[0];
-        for (int l = tid; l < L; l += T) v[l] = (l == 0) ? sc4[1] : A[(k + 1 + l) * lda + k];
+        for (int l = tid; l < L; l += T) {
+            const double x = (l == 0) ? sc4[1] : A[(k + 1 + l) * lda + k];
+            v[l] = x;
+            Vc[(int64_t)k * nu + l] = x;
+        }
         __syncthreads();
         // p = tau A_sub v from A_sub's lower triangle, one entry per thread: row
         // col left of the diagonal (stride lda, odd, across the threads), then
         // column col from the diagonal down (consecutive addresses); p goes to
         // the scratch after e
-        double *qv = ev + nu;
         double vp = 0.0;
         for (int col = tid; col < L; col += T) {
-            const double *Ar = A + (k + 1 + col) * lda + (k + 1);
-            double pl = 0.0;
-            for (int m = 0; m < col; ++m) pl = fma(Ar[m], v[m], pl);
-            for (int m = col; m < L; ++m) pl = fma(A[(k + 1 + m) * lda + (k + 1 + col)], v[m], pl);
-            pl *= tauh;
+            const double *Ar = A + (k + 1 + col) * lda + (k + 1), *Ac = A + (k + 1) * lda + (k + 1 + col);
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            int m = 0;
+            for (; m + 3 < col; m += 4)
+#pragma unroll
+                for (int z = 0; z < 4; ++z) s[z] = fma(Ar[m + z], v[m + z], s[z]);
+            for (; m < col; ++m) s[0] = fma(Ar[m], v[m], s[0]);
+            for (; m + 3 < L; m += 4)
+#pragma unroll
+                for (int z = 0; z < 4; ++z) s[z] = fma(Ac[(m + z) * lda], v[m + z], s[z]);
+            for (; m < L; ++m) s[0] = fma(Ac[m * lda], v[m], s[0]);
+            const double pl = ((s[0] + s[1]) + (s[2] + s[3])) * tauh;
             qv[col] = pl;
             vp = fma(v[col], pl, vp);
         }
         // K = (tau/2) v . p
-        __shared__ double wpart[kTriThreads / 32];
         vp = warp_sum(vp);
         if ((tid & 31) == 0) wpart[tid >> 5] = vp;
         __syncthreads();
-        if (tid == 0) {
-            double s = 0.0;
-            for (int q = 0; q < T / 32; ++q) s += wpart[q];
-            sc4[2] = 0.5 * tauh * s;
-        }
+        double kk = 0.0;
+        for (int q = 0; q < T / 32; ++q) kk += wpart[q];
+        kk *= 0.5 * tauh;
         __syncthreads();
-        for (int col = tid; col < L; col += T) qv[col] = fma(-sc4[2], v[col], qv[col]);   // q = p - K v
+        for (int col = tid; col < L; col += T) qv[col] = fma(-kk, v[col], qv[col]);   // q = p - K v
         __syncthreads();
-        for (int idx = tid; idx < L * L; idx += T) {  // A_sub -= v q^T + q v^T, lower triangle
-            const int a = idx / L, b = idx - (idx / L) * L;
-            if (a >= b) A[(k + 1 + a) * lda + (k + 1 + b)] -= v[a] * qv[b] + qv[a] * v[b];
-        }
-        for (int r = tid; r < nr; r += T) {  // R <- R (I - tau v v^T) on columns k+1..
-            double *row = R + r * lda + (k + 1);
-            double s = 0.0;
-            for (int m = 0; m < L; ++m) s = fma(row[m], v[m], s);
-            s *= tauh;
-            for (int m = 0; m < L; ++m) row[m] = fma(-s, v[m], row[m]);
+        // A_sub -= v q^T + q v^T, lower triangle: a warp per row
+        for (int a = tid >> 5; a < L; a += T / 32) {
+            const double va = v[a], qa = qv[a];
+            double *Ar = A + (k + 1 + a) * lda + (k + 1);
+            for (int b = tid & 31; b <= a; b += 32) Ar[b] = fma(-va, qv[b], fma(-qa, v[b], Ar[b]));
         }
         __syncthreads();
     }
@@ -250,148 +229,355 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
         Dc[i] = A[i * lda + i];
         Ec[i] = i + 2 < n ? ev[i] : (i + 2 == n ? A[(n - 1) * lda + (n - 2)] : 0.0);
     }
-    double *RQc = RQ + (int64_t)sc * nr_max * nu;
-    for (int idx = tid; idx < nr * n; idx += T) {
-        const int r = idx / n, i = idx - (idx / n) * n;
-        RQc[(int64_t)r * nu + i] = R[r * lda + i];
-    }
+}
+
+// 1 / sqrt(a) and 1 / a of normal numbers from the hardware's 20-bit estimates
+// by one step of third order (the binomial series of (1 - e)^(-1/2) and
+// (1 - e)^(-1) in the estimate's defect e, cut after e^2): what is left is the
+// rounding, about 1 ulp.  Few FP64 instructions (five and three) and no branch
+// for special values.
+__device__ __forceinline__ double series_rsqrt(double a)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-(a * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ double series_rcp(double a)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-a, y, 1.0);
+    return fma(y, fma(e, e, e), y);
 }
 
 // ------------------------------------------------------------------ batched QL
-// Lane = subspace.  d and e live in shared memory as [i][lane].  Rotations go
-// to rot[sc][0 .. rcap), sweeps (m, lo) to sweep[sc][0 .. scap); nsweep[sc]
-// receives the sweep count, or -1 (no convergence in kQlMaxIter iterations for
-// some level, or a full log).  Eigenvalues overwrite D, unsorted.
-__global__ void __launch_bounds__(32) eig_ql_kernel(const int *__restrict__ bnu_eff, int cofs,
-                                                    int nb, int nu, double *__restrict__ D,
-                                                    const double *__restrict__ E,
+// Lane = subspace (lanes < nl of a warp; nl shrinks with the chunk so that few
+// subspaces still spread over the SMs).  d and e live in shared memory as
+// [i][lane].  The lanes run their sweeps side by side, each at its own level l:
+// a lane that finishes a level early goes on with the next one instead of
+// waiting for the others.
+//
+// What bounds it: one warp's FP64 instruction holds its scheduler's FP64 unit
+// for 64 cycles whatever the number of active lanes, and a subspace's rotations
+// are one chain; so the time is that chain's count of FP64 instructions (20 per
+// rotation).  Tests that need no FP64 arithmetic (is e(m) negligible, which of
+// |c|, |s| is larger) are made on the exponents, and what the chain does not
+// wait for runs in the CTA's second warp, on another scheduler: it follows one
+// sweep behind and turns each logged rotation into the form the rows use.
+//
+// Rotation (c, s) of the columns i, i + 1 of a row x takes
+//   x_{i+1}' = s x_i + c x_{i+1},  x_i' = c x_i - s x_{i+1};
+// the log holds it for x = diag(scale) y (the same for all rows) so that a row
+// takes two multiply-adds instead of four FP64 instructions (fast plane
+// rotations, W. M. Gentleman 1973).  With (p, q) = (y_{i+1}, y_i) when
+// |c| >= |s|, else (y_i, y_{i+1}),
+//   y_{i+1}' = p + alpha q,  y_i' = q + beta p,
+// where alpha beta <= 0 and a rotation shrinks the two scales by no more than
+// 0.7: over the rotations of nu <= 320 they stay far above underflow, and a
+// scale below 1e-280 counts as no convergence.  rot = (alpha, |beta|), the
+// second negative for the second form.
+// Rotations go to rot[sc][0 .. rcap), sweeps (m, lo) to sweep[sc][0 .. scap);
+// nsweep[sc] receives the sweep count, or -1 (no convergence in kQlMaxIter
+// iterations for some level, or a full log).  Eigenvalues overwrite D,
+// unsorted, the scales E.
+__device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+__global__ void __launch_bounds__(64) eig_ql_kernel(const int *__restrict__ bnu_eff, int cofs,
+                                                    int nb, int nu, int nl, double *__restrict__ D,
+                                                    double *__restrict__ E,
                                                     double2 *__restrict__ rot, int64_t rcap,
                                                     int2 *__restrict__ sweep, int64_t scap,
                                                     int *__restrict__ nsweep)
 {
     extern __shared__ __align__(16) double qsm[];
-    const int lane = threadIdx.x;
-    const int sc = blockIdx.x * 32 + lane;
-    if (sc >= nb) return;
-    double *d = qsm;                 // d[i] at d[i * 32 + lane]
-    double *e = qsm + (size_t)nu * 32;
-    const int n = bnu_eff[cofs + sc];
-    for (int i = 0; i < n; ++i) {
-        d[i * 32 + lane] = D[(int64_t)sc * nu + i];
-        e[i * 32 + lane] = E[(int64_t)sc * nu + i];
+    __shared__ int4 trip[2][32];   // a lane's sweep: m, lo, rotations, -; double-buffered
+    __shared__ int more[2];
+    __shared__ int fail[32];
+    const int lane = threadIdx.x & 31, sc = blockIdx.x * nl + lane;
+    const bool mine = lane < nl && sc < nb, first = threadIdx.x < 32;
+    double *d = qsm + (mine ? lane : 0);             // d[i] at d[i * nl]
+    double *e = d + (size_t)nu * nl;
+    double *w = e + (size_t)nu * nl;                 // the scales (second warp)
+    const int n = mine ? bnu_eff[cofs + sc] : 0;
+    double2 *rl = rot + (int64_t)(mine ? sc : 0) * rcap;
+#define DD(i) d[(i) * nl]
+#define EE(i) e[(i) * nl]
+#define WW(i) w[(i) * nl]
+    if (!first) {
+        for (int i = 0; i < n; ++i) WW(i) = 1.0;
+        bool bad = false;
+        for (int t = 0;; t ^= 1) {
+            __syncthreads();   // sweep t is logged
+            if (!more[t]) break;
+            const int4 tr = trip[t][lane];
+            double2 *r = rl;
+            rl += mine ? tr.z : 0;
+            double2 cs = tr.z > 0 ? r[0] : make_double2(1.0, 0.0);
+            double wj = tr.z > 0 ? WW(tr.x) : 1.0;
+            for (int q = 0; __any_sync(kFull, q < tr.z); ++q)
+                if (q < tr.z) {
+                    const int i = tr.x - 1 - q;
+                    const double cth = cs.x, s = cs.y, wi = WW(i);
+                    if (q + 1 < tr.z) cs = r[q + 1];
+                    const bool cf = (__double2hiint(cth) & 0x7fffffff) >= (__double2hiint(s) & 0x7fffffff);
+                    const double num = cf ? s : cth, den = cf ? cth : s;
+                    const double wp = cf ? wi : wj, wq = cf ? wj : wi;
+                    const double alpha = (num * wp) * series_rcp(den * wq);
+                    const double beta = fabs((num * wq) * series_rcp(den * wp));
+                    r[q] = make_double2(alpha, cf ? beta : -beta);
+                    WW(i + 1) = den * wq;
+                    wj = cf ? den * wp : -(den * wp);
+                    bad |= exponent_of(wj) < 1023 - 930;
+                }
+            if (tr.z > 0) WW(tr.x - tr.z) = wj;
+        }
+        if (mine) {
+            for (int i = 0; i < n; ++i) E[(int64_t)sc * nu + i] = WW(i);
+            fail[lane] = bad;
+        }
+        __syncthreads();
+        return;
     }
-#define DD(i) d[(i) * 32 + lane]
-#define EE(i) e[(i) * 32 + lane]
-    double2 *rl = rot + (int64_t)sc * rcap;
-    int2 *sl = sweep + (int64_t)sc * scap;
+    for (int i = 0; i < n; ++i) {
+        d[i * nl] = D[(int64_t)sc * nu + i];
+        e[i * nl] = E[(int64_t)sc * nu + i];
+    }
+    int2 *sl = sweep + (int64_t)(mine ? sc : 0) * scap;
     int64_t nrot = 0;
-    int nsw = 0;
-    bool failed = false;
-    for (int l = 0; l < n && !failed; ++l) {
-        int iter = 0;
-        while (true) {
-            int m = l;
-            for (; m < n - 1; ++m)
-                if (fabs(EE(m)) <= DBL_EPSILON * (fabs(DD(m)) + fabs(DD(m + 1)))) break;
-            if (m == l) break;
-            if (++iter > kQlMaxIter || nrot + (m - l) > rcap || nsw >= scap) {
-                failed = true;
-                break;
+    int nsw = 0, l = 0, iter = 0;
+    bool failed = false, done = n == 0;
+    // every trip: each unfinished lane's next sweep; at most kQlMaxIter per level
+    for (int t = 0;; t ^= 1) {
+        int m = l;
+        bool go = false;
+        while (!done && !go) {
+            for (m = l; m < n - 1; ++m) {
+                // |e| > eps (|d| + |d'|) for sure when e's exponent is above the
+                // larger of the others' less 50
+                const double em = EE(m), d0 = DD(m), d1 = DD(m + 1);
+                if (exponent_of(em) > max(exponent_of(d0), exponent_of(d1)) - 50) continue;
+                if (fabs(em) <= DBL_EPSILON * (fabs(d0) + fabs(d1))) break;
             }
-            double g = (DD(l + 1) - DD(l)) / (2.0 * EE(l));
-            double r = hypot(g, 1.0);
-            g = DD(m) - DD(l) + EE(l) / (g + copysign(r, g));
-            double s = 1.0, cth = 1.0, p = 0.0;
-            int i = m - 1;
-            bool under = false;
-            for (; i >= l; --i) {
-                const double f = s * EE(i), b = cth * EE(i);
-                // r = |(f, g)| as one square root and one reciprocal (the
-                // levels and couplings are bounded by the spectrum's width, so
-                // f^2 + g^2 neither overflows nor underflows to zero unless
-                // both are zero)
+            if (m == l) {
+                iter = 0;
+                done = ++l >= n;
+            } else if (++iter > kQlMaxIter || nrot + (m - l) > rcap || nsw >= scap) {
+                failed = done = true;
+            } else {
+                go = true;
+            }
+        }
+        const bool any = __any_sync(kFull, go);
+        double g = 0.0, s = 1.0, cth = 1.0, p = 0.0;
+        int i = -1, lo = 0;
+        if (go) {
+            g = (DD(l + 1) - DD(l)) / (2.0 * EE(l));
+            g = DD(m) - DD(l) + EE(l) / (g + copysign(sqrt(fma(g, g, 1.0)), g));
+            i = m - 1;
+            lo = l;
+        }
+        bool under = false;
+        double dj = go ? DD(m) : 0.0;   // d(i + 1)
+        while (__any_sync(kFull, i >= lo)) {
+            if (i >= lo) {
+                const double ei = EE(i), di = DD(i), f = s * ei, b = cth * ei;
+                // r = |(f, g)| (the levels and couplings are bounded by the
+                // spectrum's width, so f^2 + g^2 neither overflows nor
+                // underflows unless both are as good as zero)
                 const double ss = fma(f, f, g * g);
-                r = sqrt(ss);
-                EE(i + 1) = r;
-                if (r == 0.0) {
-                    DD(i + 1) -= p;
+                if (exponent_of(ss) == 0) {
+                    EE(i + 1) = 0.0;
+                    DD(i + 1) = dj - p;
                     EE(m) = 0.0;
                     under = true;
-                    break;
+                    lo = i + 1;
+                } else {
+                    const double rinv = series_rsqrt(ss);
+                    EE(i + 1) = ss * rinv;
+                    s = f * rinv;
+                    cth = g * rinv;
+                    rl[nrot++] = make_double2(cth, s);
+                    g = dj - p;
+                    const double r = fma(cth + cth, b, (di - g) * s);
+                    p = s * r;
+                    DD(i + 1) = g + p;
+                    dj = di;
+                    g = fma(cth, r, -b);
+                    --i;
                 }
-                const double rinv = 1.0 / r;
-                s = f * rinv;
-                cth = g * rinv;
-                g = DD(i + 1) - p;
-                r = (DD(i) - g) * s + 2.0 * cth * b;
-                p = s * r;
-                DD(i + 1) = g + p;
-                g = cth * r - b;
-                rl[nrot++] = make_double2(cth, s);
             }
-            sl[nsw++] = make_int2(m, under ? i + 1 : l);
+        }
+        if (go) {
+            sl[nsw++] = make_int2(m, lo);
             if (!under) {
-                DD(l) -= p;
+                DD(l) = dj - p;
                 EE(l) = g;
                 EE(m) = 0.0;
             }
         }
+        trip[t][lane] = make_int4(m, lo, go ? m - lo : 0, 0);
+        if (lane == 0) more[t] = any;
+        __syncthreads();
+        if (!any) break;
     }
+    __syncthreads();   // the second warp's last sweep
+    if (!mine) return;
     for (int i = 0; i < n; ++i) D[(int64_t)sc * nu + i] = DD(i);
-    nsweep[sc] = failed ? -1 : nsw;
+    nsweep[sc] = failed || fail[lane] ? -1 : nsw;
 #undef DD
 #undef EE
+#undef WW
 }
 
-// ------------------------------------------------------------------ replay and outputs
+// ------------------------------------------------------------------ rows and outputs
+// A thread per row of R = [e_1; q; K_pat; (v^T w_i)], in shared memory as
+// [nr_max][ldr] (ldr odd): R L^-T, the reflectors, the rotations, the scales.
+// A warp's lanes hold the next 32 rotations in registers and broadcast them
+// with shuffles while the following 32 are on their way.
+template <typename VT>
 __global__ void __launch_bounds__(kApplyThreads) eig_apply_kernel(
     const int *__restrict__ bnu_eff, const int *__restrict__ bstatus, int cofs, int nu,
-    const int64_t *__restrict__ bcols, const double *__restrict__ sdiag,
-    const int64_t *__restrict__ rp, int64_t col0, const double *__restrict__ D,
-    const double *__restrict__ RQ, int nr_max, const double2 *__restrict__ rot, int64_t rcap,
-    const int2 *__restrict__ sweep, int64_t scap, const int *__restrict__ nsweep,
-    int *__restrict__ nu_eff_out, double *__restrict__ eps_out, double *__restrict__ w_out,
-    double *__restrict__ t_out, double *__restrict__ P_out, const int64_t *__restrict__ p_off,
-    int *__restrict__ eig_status, double *__restrict__ proj_out)
+    const double *__restrict__ bscale, const VT *__restrict__ K, int64_t m_pad, const uint16_t *__restrict__ tinv,
+    int nb, const int64_t *__restrict__ bcols, const double *__restrict__ sdiag,
+    const int64_t *__restrict__ rp, const int32_t *__restrict__ ci, const int *__restrict__ reg, int n_reg,
+    int64_t col0, const double *__restrict__ D, const double *__restrict__ W, const double *__restrict__ V,
+    const double *__restrict__ Lsub, const double *__restrict__ proj, int nr_max,
+    const double2 *__restrict__ rot, int64_t rcap, const int2 *__restrict__ sweep, int64_t scap,
+    const int *__restrict__ nsweep, int *__restrict__ nu_eff_out, double *__restrict__ eps_out,
+    double *__restrict__ w_out, double *__restrict__ t_out, double *__restrict__ P_out,
+    const int64_t *__restrict__ p_off, int *__restrict__ eig_status, double *__restrict__ proj_out)
 {
     const int sc = blockIdx.x;
     const int c = cofs + sc;
     const int64_t g = col0 + c;
     const int n = bnu_eff[c];
-    const int tid = threadIdx.x, T = blockDim.x;
+    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
     const int ldr = nu | 1;
     extern __shared__ __align__(16) double asm_[];
     double *R = asm_;
     double *d = R + (size_t)nr_max * ldr;
-    int *perm = reinterpret_cast<int *>(d + nu);
+    double *wsc = d + nu;
+    int *perm = reinterpret_cast<int *>(wsc + nu);
+    // rows of R: e_1, q = K^T e_j, and K_pat (zero for atoms outside a region)
     const int64_t j = bcols[c];
     const int64_t J = j >> 2;
-    const int npat = 4 * (int)(rp[J + 1] - rp[J]);
-    const int nr = npat + 2 + (proj_out ? 1 : 0);
-    const double *RQc = RQ + (int64_t)sc * nr_max * nu;
-    for (int idx = tid; idx < nr * n; idx += T) {
-        const int r = idx / n, i = idx - (idx / n) * n;
-        R[r * ldr + i] = RQc[(int64_t)r * nu + i];
+    const int *Rg = reg ? reg + (int64_t)c * n_reg : nullptr;
+    const int pJ = Rg ? find_sorted(Rg, n_reg, (int)J) : 0;
+    const int64_t jl = Rg ? 4 * (int64_t)(pJ < 0 ? 0 : pJ) + (j & 3) : j;
+    const int64_t kb = rp[J];
+    const int npat = 4 * (int)(rp[J + 1] - kb);
+    const int nr = npat + 2 + (proj ? 1 : 0);   // the projection row last
+    const VT *Kc = K + (int64_t)c * nu * m_pad;
+    for (int r = tid; r < nr; r += T) {
+        int64_t pos = -1;   // the row's position in the column's vectors
+        if (r == 1) {
+            pos = vpos(tinv, nb, c, jl);
+        } else if (r >= 2 && r < npat + 2) {
+            const int atom = ci[kb + ((r - 2) >> 2)];
+            const int64_t lr = Rg ? find_sorted(Rg, n_reg, atom) : atom;
+            if (lr >= 0) pos = vpos(tinv, nb, c, 4 * lr + ((r - 2) & 3));
+        }
+        double *x = R + r * ldr;
+        const double *si = bscale + (int64_t)c * nu;
+        for (int i = 0; i < n; ++i)
+            x[i] = r == 0 ? (i == 0 ? 1.0 : 0.0)
+                   : r == npat + 2 ? si[i] * proj[(int64_t)c * nu + i]
+                   : pos >= 0 ? si[i] * (double)Kc[(int64_t)i * m_pad + pos] : 0.0;
     }
-    for (int i = tid; i < n; i += T) d[i] = D[(int64_t)sc * nu + i];
-    __syncthreads();
+    for (int i = tid; i < n; i += T) {
+        d[i] = D[(int64_t)sc * nu + i];
+        wsc[i] = W[(int64_t)sc * nu + i];
+    }
+    const double *Lc = Lsub + (int64_t)c * nu * nu, *Vc = V + (int64_t)sc * nu * nu;
     const int nsw = nsweep[sc];
-    // each thread replays the whole log on its rows
     const double2 *rl = rot + (int64_t)sc * rcap;
     const int2 *sl = sweep + (int64_t)sc * scap;
-    for (int r = tid; r < nr; r += T) {
-        double *row = R + r * ldr;
-        int64_t ptr = 0;
-        for (int s = 0; s < nsw; ++s) {
-            const int2 sw = sl[s];
-            for (int i = sw.x - 1; i >= sw.y; --i) {
-                const double2 cs = rl[ptr++];
-                const double f = row[i + 1];
-                row[i + 1] = fma(cs.y, row[i], cs.x * f);
-                row[i] = fma(cs.x, row[i], -cs.y * f);
+    // whole warps run a row pass (the shuffles); a lane without a row reads and
+    // stores nothing
+    for (int r0 = tid - lane; r0 < nr; r0 += T) {
+        const bool own = r0 + lane < nr;
+        double *x = R + (own ? r0 + lane : 0) * ldr;
+        if (own) {
+            // rows 1..: R <- R L^-T (row 0, e_1^T, is unchanged: K^T S e_j =
+            // sqrt(S_jj) e_1), four entries at a time from the last down
+            if (r0 + lane > 0) {
+                for (int i = n - 1; i >= 0; i -= 4) {
+                    double s[4] = {0.0, 0.0, 0.0, 0.0};
+                    const double *L0 = Lc + (int64_t)i * nu;
+                    const int lo = i - 3;
+                    for (int m = 0; m <= lo; ++m) {   // lo < 0: the general loop below
+                        const double xm = x[m];
+#pragma unroll
+                        for (int z = 0; z < 4; ++z) s[z] = fma(xm, L0[m - (int64_t)z * nu], s[z]);
+                    }
+                    for (int m = lo < 0 ? 0 : lo + 1; m <= i; ++m) {
+                        const double xm = x[m];
+#pragma unroll
+                        for (int z = 0; z < 4; ++z)
+                            if (i - z >= m) s[z] = fma(xm, L0[m - (int64_t)z * nu], s[z]);
+                    }
+#pragma unroll
+                    for (int z = 0; z < 4; ++z)
+                        if (i - z >= 0) x[i - z] = s[z];
+                }
+            }
+            for (int k = 0; k + 2 < n; ++k) {   // R <- R (I - tau v v^T) on columns k + 1 ..
+                const int L = n - k - 1;
+                const double *v = Vc + (int64_t)k * nu;
+                const double tau = v[nu - 1];
+                if (tau == 0.0) continue;
+                double *row = x + k + 1;
+                double s[4] = {0.0, 0.0, 0.0, 0.0};
+                int m = 0;
+                for (; m + 3 < L; m += 4)
+#pragma unroll
+                    for (int z = 0; z < 4; ++z) s[z] = fma(row[m + z], v[m + z], s[z]);
+                for (; m < L; ++m) s[0] = fma(row[m], v[m], s[0]);
+                const double f = -tau * ((s[0] + s[1]) + (s[2] + s[3]));
+#pragma unroll 4
+                for (m = 0; m < L; ++m) row[m] = fma(f, v[m], row[m]);
             }
         }
+        __syncwarp();
+        // the next rotation's coefficients and the next entry are fetched before
+        // the current rotation's multiply-adds: the chain through carry is then
+        // one multiply-add per rotation
+        int64_t ptr = 0;   // rotation held by lane 0
+        double2 cur = lane < rcap ? rl[lane] : make_double2(0.0, 0.0);
+        double2 nxt = 32 + lane < rcap ? rl[32 + lane] : make_double2(0.0, 0.0);
+        int at = 0;
+        double alpha = __shfl_sync(kFull, cur.x, 0), bs = __shfl_sync(kFull, cur.y, 0);
+        int2 sw = nsw > 0 ? sl[0] : make_int2(0, 0);
+        for (int q = 0; q < nsw; ++q) {
+            const int2 sn = q + 1 < nsw ? sl[q + 1] : make_int2(0, 0);
+            double carry = own ? x[sw.x] : 0.0;
+            double yi = own && sw.x > sw.y ? x[sw.x - 1] : 0.0;
+            for (int i = sw.x - 1; i >= sw.y; --i) {
+                const double al = alpha, y = yi;
+                const bool sf = __double2hiint(bs) < 0;
+                // beta = -sign(alpha) |bs|
+                const double beta = __hiloint2double((__double2hiint(bs) & 0x7fffffff) |
+                                                         (~__double2hiint(al) & 0x80000000),
+                                                     __double2loint(bs));
+                if (++at == 32) {
+                    at = 0;
+                    ptr += 32;
+                    cur = nxt;
+                    if (ptr + 32 + lane < rcap) nxt = rl[ptr + 32 + lane];
+                }
+                alpha = __shfl_sync(kFull, cur.x, at);
+                bs = __shfl_sync(kFull, cur.y, at);
+                if (own && i > sw.y) yi = x[i - 1];
+                const double p = sf ? y : carry, qq = sf ? carry : y;
+                carry = fma(beta, p, qq);
+                if (own) x[i + 1] = fma(al, qq, p);
+            }
+            if (own) x[sw.y] = carry;
+            sw = sn;
+        }
     }
+    __syncthreads();
     // rank of every level (ties by index): ascending order; a NaN level (from
     // non-finite input) ranks as +inf, so the ranks always form a permutation
     auto key = [&](int b) { const double x = d[b]; return x != x ? CUDART_INF : x; };
@@ -411,18 +597,18 @@ __global__ void __launch_bounds__(kApplyThreads) eig_apply_kernel(
         if (a < n) {
             const int src = perm[a];
             ea = d[src];
-            ta = R[1 * ldr + src];
-            wa = sq * R[src] * ta;
+            ta = R[1 * ldr + src] * wsc[src];
+            wa = sq * (R[src] * wsc[src]) * ta;
         }
         eps_out[g * nu + a] = ea;
         t_out[g * nu + a] = ta;
         w_out[g * nu + a] = wa;
-        if (proj_out) proj_out[g * nu + a] = a < n ? R[(npat + 2) * ldr + perm[a]] : 0.0;
+        if (proj_out) proj_out[g * nu + a] = a < n ? R[(npat + 2) * ldr + perm[a]] * wsc[perm[a]] : 0.0;
     }
     double *P = P_out + p_off[g];
     for (int idx = tid; idx < npat * nu; idx += T) {
         const int r = idx / nu, a = idx - (idx / nu) * nu;
-        P[idx] = a < n ? R[(r + 2) * ldr + perm[a]] : 0.0;
+        P[idx] = a < n ? R[(r + 2) * ldr + perm[a]] * wsc[perm[a]] : 0.0;
     }
     if (tid == 0) {
         nu_eff_out[g] = n;
@@ -430,62 +616,64 @@ __global__ void __launch_bounds__(kApplyThreads) eig_apply_kernel(
     }
 }
 
-template <typename VT>
-cudaError_t tridiag_dispatch(const DeviceMatrix &A, const KrylovBatch &b, const RegionMaps *rm,
-                             const EigScratch &es, int cofs, int nb2, cudaStream_t s)
+size_t eig_apply_smem(int nu, int nr_max)
 {
-    const int nu = b.nu;
-    const size_t smem = eig_tridiag_smem(nu, es.nr_max, es.Ag != nullptr);
-    cudaError_t e = allow_dynamic_smem((const void *)eig_tridiag_kernel<VT>, smem);
+    return (size_t)nr_max * (nu | 1) * sizeof(double) + (size_t)nu * (2 * sizeof(double) + sizeof(int));
+}
+
+template <typename VT>
+cudaError_t apply_dispatch(const DeviceMatrix &A, const KrylovBatch &b, const ColumnState &st, int64_t col0,
+                           const RegionMaps *rm, const EigScratch &es, int cofs, int nb2, cudaStream_t s)
+{
+    const size_t smem = eig_apply_smem(b.nu, es.nr_max);
+    cudaError_t e = allow_dynamic_smem((const void *)eig_apply_kernel<VT>, smem);
     if (e != cudaSuccess) return e;
-    eig_tridiag_kernel<VT><<<nb2, kTriThreads, smem, s>>>(
-        b.Hsub, b.nu_eff, b.scale, (const VT *)b.K, b.shape.m_pad, b.tinv, b.nb, nu, b.cols, A.rp, A.ci,
-        rm ? rm->reg : nullptr, rm ? rm->n_reg : 0, cofs, es.D, es.E, es.RQ, es.nr_max, es.Ag, b.Lsub,
-        es.proj);
+    const int threads = std::min(kApplyThreads, (es.nr_max + 31) / 32 * 32);
+    eig_apply_kernel<VT><<<nb2, threads, smem, s>>>(
+        b.nu_eff, b.status, cofs, b.nu, b.scale, (const VT *)b.K, b.shape.m_pad, b.tinv, b.nb, b.cols, A.sdiag, A.rp,
+        A.ci, rm ? rm->reg : nullptr, rm ? rm->n_reg : 0, col0, es.D, es.E, es.V, b.Lsub, es.proj, es.nr_max, es.rot,
+        es.rcap, es.sweep, es.scap, es.nsweep, st.nu_eff, st.eps, st.w, st.t, st.P, st.p_off, st.eig_status,
+        es.proj ? es.proj_out : nullptr);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-size_t eig_tridiag_smem(int nu, int nr_max, bool a_global)
-{
-    const size_t lda = (size_t)(nu | 1);
-    return ((size_t)((a_global ? 0 : nu) + nr_max) * lda + 3 * (size_t)nu) * sizeof(double);
-}
-
+// What a solve is refused by: the shared memory that H_sub (unless a_global)
+// and the rows of R take together with their vectors.
 size_t eig_smem_bytes(int nu, int nr_max, bool a_global)
 {
     const size_t lda = (size_t)(nu | 1);
-    const size_t tri = eig_tridiag_smem(nu, nr_max, a_global);
-    const size_t app = (size_t)nr_max * lda * sizeof(double) + (size_t)nu * (sizeof(double) + sizeof(int));
+    const size_t tri = ((size_t)((a_global ? 0 : nu) + nr_max) * lda + 3 * (size_t)nu) * sizeof(double);
     const size_t ql = (size_t)2 * nu * 32 * sizeof(double);
-    return std::max(tri, std::max(app, ql));
+    return std::max(tri, ql);
 }
 
 cudaError_t launch_eig(const DeviceMatrix &A, const KrylovBatch &b, const ColumnState &st,
                        int64_t col0, const RegionMaps *rm, const EigScratch &es, cudaStream_t s)
 {
     if ((es.proj == nullptr) != (es.proj_out == nullptr)) return cudaErrorInvalidValue;
-    const int nu = b.nu, ldr = nu | 1;
-    const size_t qsmem = (size_t)2 * nu * 32 * sizeof(double);
-    const size_t asmem = (size_t)es.nr_max * ldr * sizeof(double) + (size_t)nu * (sizeof(double) + sizeof(int));
-    cudaError_t e;
-    if ((e = allow_dynamic_smem((const void *)eig_ql_kernel, qsmem)) != cudaSuccess ||
-        (e = allow_dynamic_smem((const void *)eig_apply_kernel, asmem)) != cudaSuccess)
-        return e;
+    const int nu = b.nu;
+    const size_t tsmem = ((size_t)(es.Ag ? 0 : nu) * (nu | 1) + 3 * (size_t)nu) * sizeof(double);
+    const int tthreads = std::min(kTriThreads, (nu + 31) / 32 * 32);
+    cudaError_t e = allow_dynamic_smem((const void *)eig_tridiag_kernel, tsmem);
+    if (e != cudaSuccess) return e;
     for (int cofs = 0; cofs < b.nb; cofs += es.chunk) {
         const int nb2 = b.nb - cofs < es.chunk ? b.nb - cofs : es.chunk;
-        e = b.prec == 0 ? tridiag_dispatch<double>(A, b, rm, es, cofs, nb2, s)
-                        : tridiag_dispatch<float>(A, b, rm, es, cofs, nb2, s);
+        eig_tridiag_kernel<<<nb2, tthreads, tsmem, s>>>(b.Hsub, b.nu_eff, nu, cofs, es.D, es.E, es.V, es.Ag, b.Lsub);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        // subspaces per warp: as few as leave one warp per SM (a sweep of the
+        // warp is as long as its longest lane's), 16 when 32 would not fit
+        int nl = 3 * (size_t)nu * 32 * sizeof(double) > (size_t)227 * 1024 ? 16 : 32;
+        while (nl > 1 && (nb2 + nl / 2 - 1) / (nl / 2) <= kQlWarps) nl /= 2;
+        const size_t qsmem = (size_t)3 * nu * nl * sizeof(double);
+        if ((e = allow_dynamic_smem((const void *)eig_ql_kernel, qsmem)) != cudaSuccess) return e;
+        eig_ql_kernel<<<(nb2 + nl - 1) / nl, 64, qsmem, s>>>(b.nu_eff, cofs, nb2, nu, nl, es.D, es.E, es.rot,
+                                                            es.rcap, es.sweep, es.scap, es.nsweep);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = b.prec == 0 ? apply_dispatch<double>(A, b, st, col0, rm, es, cofs, nb2, s)
+                        : apply_dispatch<float>(A, b, st, col0, rm, es, cofs, nb2, s);
         if (e != cudaSuccess) return e;
-        eig_ql_kernel<<<(nb2 + 31) / 32, 32, qsmem, s>>>(b.nu_eff, cofs, nb2, nu, es.D, es.E, es.rot,
-                                                           es.rcap, es.sweep, es.scap, es.nsweep);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        eig_apply_kernel<<<nb2, kApplyThreads, asmem, s>>>(
-            b.nu_eff, b.status, cofs, nu, b.cols, A.sdiag, A.rp, col0, es.D, es.RQ, es.nr_max,
-            es.rot, es.rcap, es.sweep, es.scap, es.nsweep, st.nu_eff, st.eps, st.w, st.t, st.P,
-            st.p_off, st.eig_status, es.proj ? es.proj_out : nullptr);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }

@@ -310,13 +310,13 @@ struct ColumnState {
 };
 
 // Scratch of the three-kernel eigensolve, per chunk of subspaces:
-//   D, E [chunk][nu] (tridiagonal, then levels), RQ [chunk][nr_max][nu] (rows
-//   e_1, q, K_pat times Q, then times Z), rot [chunk][rcap] Givens (c, s),
-//   sweep [chunk][scap] (m, lo), nsweep [chunk] (-1: QL failed).
+//   D, E [chunk][nu] (tridiagonal, then levels and column scales), V [chunk][nu]
+//   [nu] (Householder reflectors), rot [chunk][rcap] rotations, sweep
+//   [chunk][scap] (m, lo), nsweep [chunk] (-1: QL failed).
 struct EigScratch {
     int chunk = 0, nr_max = 0;
     int64_t rcap = 0, scap = 0;
-    double *D = nullptr, *E = nullptr, *RQ = nullptr;
+    double *D = nullptr, *E = nullptr, *V = nullptr;
     double2 *rot = nullptr;
     int2 *sweep = nullptr;
     int *nsweep = nullptr;
@@ -327,9 +327,8 @@ struct EigScratch {
     const double *proj = nullptr;
     double *proj_out = nullptr;
 };
-// Dynamic shared memory of the tridiagonalisation and the largest one of the
-// eigensolve kernels, with H_sub in shared (a_global = false) or global memory.
-size_t eig_tridiag_smem(int nu, int nr_max, bool a_global);
+// Shared memory that bounds nu and the pattern rows, with H_sub in shared
+// (a_global = false) or global memory.
 size_t eig_smem_bytes(int nu, int nr_max, bool a_global);
 
 cudaError_t launch_eig(const DeviceMatrix &A, const KrylovBatch &b, const ColumnState &st,
