@@ -516,7 +516,7 @@ def main():
     step_s = float(tmax.item())
     value = world * ncols / step_s
     stats = res["stats"]
-    launches = sum(v[0] for v in stats.values())
+    launches = sum(v[0] for k, v in stats.items() if k != "bisect_step")   # steps, not kernels
     peaks = read_peaks()
 
     # roofline of the dominant kernel over the timed region (vector length: M, or 4 n_reg)

@@ -33,12 +33,11 @@ constexpr double kTauFp64 = 1e-10;
 constexpr double kTauMixed = 1e-5;
 
 // Reduction scratch of a context: partial sums, the reduction output, the
-// level range, the bisection state and the reductions' ticket.
+// reductions' ticket and the scratch of one bisection.
 constexpr size_t kOffOut = 2 * kReduceBlocks * sizeof(double);
-constexpr size_t kOffRange = kOffOut + 2 * sizeof(double);
-constexpr size_t kOffBisect = kOffRange + 2 * sizeof(double);
-constexpr size_t kOffTicket = kOffBisect + ((sizeof(BisectState) + 15) & ~(size_t)15);
-constexpr size_t kScratchBytes = kOffTicket + 16;
+constexpr size_t kOffTicket = kOffOut + 2 * sizeof(double);
+constexpr size_t kOffBisect = kOffTicket + 16;
+constexpr size_t kScratchBytes = kOffBisect + bisect_bytes(1);
 
 }  // namespace
 
@@ -186,8 +185,8 @@ struct marnoldi_ctx {
     // reduction scratch and pinned read-back
     double *d_partial = nullptr;
     unsigned *d_ticket = nullptr;
-    double *d_out = nullptr, *d_range = nullptr;
-    BisectState *d_bisect = nullptr;
+    double *d_out = nullptr;
+    void *d_bisect = nullptr;   // bisect_bytes(1)
     double *h_out = nullptr;   // 128-byte pinned read-back slot
 
     // solved state
@@ -798,6 +797,43 @@ ColumnState column_view(const ColumnState &st, int64_t c0, int64_t c1)
     return v;
 }
 
+BisectTask bisect_task(const ColumnState &st, double kT, double ne)
+{
+    BisectTask t{};
+    t.ncols = st.ncols;
+    t.nu = st.nu;
+    t.nu_eff = st.nu_eff;
+    t.eps = st.eps;
+    t.w = st.w;
+    t.kT = kT;
+    t.Ne = ne;
+    return t;
+}
+
+// n bisections on the device, one read-back of their states.
+int bisect(marnoldi_ctx *c, const BisectTask *tasks, int n, void *scratch, BisectState *bs)
+{
+    int rc = launch(c, KK_COUNT, [&] { return launch_bisection(tasks, n, scratch, c->stream); });
+    if (rc) return rc;
+    // one state through the pinned slot, several through pageable memory
+    void *to = n == 1 ? (void *)c->h_out : (void *)bs;
+    const cudaError_t e = cudaMemcpyAsync(to, (char *)scratch + bisect_states(n), n * sizeof(BisectState),
+                                          cudaMemcpyDeviceToHost, c->stream);
+    if (e != cudaSuccess) return fail_cuda(c, e, "bisection read-back");
+    if ((rc = sync(c, "bisection"))) return rc;
+    if (n == 1) memcpy(bs, c->h_out, sizeof *bs);
+    // one launch was counted; the range, the loop's counts, and the bisections'
+    // steps (which end the counts)
+    int counts = 0;
+    c->launches[KK_MINMAX] += 1;
+    for (int q = 0; q < n; ++q) {
+        counts = std::max(counts, bs[q].steps - 1);
+        c->launches[KK_BISECT] += bs[q].steps;
+    }
+    c->launches[KK_COUNT] += counts - 1;
+    return MARNOLDI_OK;
+}
+
 void free_state(marnoldi_ctx *c)
 {
     if (c->state) dfree(c, c->state, c->state_bytes);
@@ -1039,8 +1075,7 @@ int marnoldi::setup_with_allocator(marnoldi_ctx **out, int64_t n_block_rows, con
     c->owned.push_back({p, kScratchBytes});
     c->d_partial = (double *)p;
     c->d_out = (double *)((char *)p + kOffOut);
-    c->d_range = (double *)((char *)p + kOffRange);
-    c->d_bisect = (BisectState *)((char *)p + kOffBisect);
+    c->d_bisect = (char *)p + kOffBisect;
     c->d_ticket = (unsigned *)((char *)p + kOffTicket);
     cudaError_t e = cudaMemsetAsync(p, 0, kScratchBytes, c->stream);
     if (e == cudaSuccess && !(c->h_out = pinned_slot())) e = cudaErrorMemoryAllocation;
@@ -1567,35 +1602,32 @@ int marnoldi_solve(marnoldi_ctx *c, const int64_t *columns, int64_t ncols, int n
         }
         col0[nmem] = nc;
         std::vector<double> mmu(nmem), mN(nmem), mE(nmem);
+        std::vector<BisectTask> tasks(nmem);
+        std::vector<BisectState> bs(nmem);
         for (size_t m = 0; m < nmem; ++m) {
-            const double ne = members ? c->mem_ne[m] : electron_count;
-            const double mkT = members && !c->mem_kT.empty() ? c->mem_kT[m] : kT;
             const ColumnState sub = column_view(c->st, col0[m], col0[m + 1]);
             if (sub.ncols == 0)
                 return fail(c, MARNOLDI_EINVAL, "member %zu has no real orbitals", m);
-            if ((rc = launch(c, KK_COUNT, [&] {
-                     return launch_bisection(sub, mkT, ne, c->d_partial, c->d_ticket, c->d_range, c->d_out,
-                                             c->d_bisect, c->stream);
-                 })))
-                return rc;
-            e = cudaMemcpyAsync(c->h_out, c->d_bisect, sizeof(BisectState), cudaMemcpyDeviceToHost, c->stream);
-            if (e != cudaSuccess) return fail_cuda(c, e, "bisection read-back");
-            if ((rc = sync(c, "bisection"))) return rc;
-            BisectState bs;
-            memcpy(&bs, c->h_out, sizeof bs);
-            // one launch each of the range and of the graph was counted; add the
-            // loop's kernels (a step and a count per iteration)
-            c->launches[KK_MINMAX] += 1;
-            c->launches[KK_COUNT] += bs.steps - 1;
-            c->launches[KK_BISECT] += bs.steps;
-            if (bs.status == 1)
+            tasks[m] = bisect_task(sub, members && !c->mem_kT.empty() ? c->mem_kT[m] : kT,
+                                   members ? c->mem_ne[m] : electron_count);
+        }
+        // scratch: the context's for one bisection; the members' side by side
+        // in the batch workspace, which nothing needs any more
+        const size_t need = bisect_bytes(nmem);
+        DeviceBuffer own(c, nmem > 1 && need > c->ws_bytes ? need : 0);
+        void *scratch = nmem == 1 ? c->d_bisect : own.get() ? (void *)own.get() : c->ws;
+        if (nmem > 1 && need > c->ws_bytes && !own.get())
+            return fail(c, MARNOLDI_ENOMEM, "device allocation for the members' bisections failed");
+        if ((rc = bisect(c, tasks.data(), (int)nmem, scratch, bs.data()))) return rc;
+        for (size_t m = 0; m < nmem; ++m) {
+            if (bs[m].status == 1)
                 return fail(c, MARNOLDI_ENOCONV, "electron count %.6g outside [N(lo) = %.6g, N(hi) = %.6g]%s",
-                            ne, bs.Nlo, bs.Nhi, members ? " for a member" : "");
-            mmu[m] = bs.mu;
-            mN[m] = bs.N;
-            mE[m] = bs.E;
-            N += bs.N;
-            E += bs.E;
+                            tasks[m].Ne, bs[m].Nlo, bs[m].Nhi, members ? " for a member" : "");
+            mmu[m] = bs[m].mu;
+            mN[m] = bs[m].N;
+            mE[m] = bs[m].E;
+            N += bs[m].N;
+            E += bs[m].E;
         }
         mu = mmu[0];
         if (members) {
@@ -1791,19 +1823,10 @@ int marnoldi_eigenstate(marnoldi_ctx *c, int64_t k, double sigma, double *eps_k,
     auto eta = [&](double n, double *out) -> int {
         if (n <= 0.0) { *out = -INFINITY; return MARNOLDI_OK; }
         if (n >= (double)m_real) { *out = INFINITY; return MARNOLDI_OK; }
-        int rc = launch(c, KK_COUNT, [&] {
-            return launch_bisection(c->st, sigma, 2.0 * n, c->d_partial, c->d_ticket, c->d_range, c->d_out,
-                                    c->d_bisect, c->stream);
-        });
-        if (rc) return rc;
-        cudaError_t e = cudaMemcpyAsync(c->h_out, c->d_bisect, sizeof(BisectState), cudaMemcpyDeviceToHost, c->stream);
-        if (e != cudaSuccess) return fail_cuda(c, e, "bisection read-back");
-        if ((rc = sync(c, "eigenstate bisection"))) return rc;
+        const BisectTask task = bisect_task(c->st, sigma, 2.0 * n);
         BisectState bs;
-        memcpy(&bs, c->h_out, sizeof bs);
-        c->launches[KK_MINMAX] += 1;
-        c->launches[KK_COUNT] += bs.steps - 1;
-        c->launches[KK_BISECT] += bs.steps;
+        const int rc = bisect(c, &task, 1, c->d_bisect, &bs);
+        if (rc) return rc;
         if (bs.status == 1) return fail(c, MARNOLDI_ENOCONV, "n = %.6g outside the bracket of the levels", n);
         *out = bs.mu;
         return MARNOLDI_OK;
@@ -1876,8 +1899,7 @@ int marnoldi_eigenstate(marnoldi_ctx *c, int64_t k, double sigma, double *eps_k,
         v->owned.push_back({p, kScratchBytes});
         v->d_partial = (double *)p;
         v->d_out = (double *)((char *)p + kOffOut);
-        v->d_range = (double *)((char *)p + kOffRange);
-        v->d_bisect = (BisectState *)((char *)p + kOffBisect);
+        v->d_bisect = (char *)p + kOffBisect;
         v->d_ticket = (unsigned *)((char *)p + kOffTicket);
         e = cudaMemsetAsync(p, 0, kScratchBytes, v->stream);
         if (e != cudaSuccess) return done(fail_cuda(c, e, "eigenstate scratch"));

@@ -346,16 +346,32 @@ cudaError_t launch_minmax(const ColumnState &st, double *partial, unsigned *tick
 constexpr double kBisectBracketKT = 40.0;
 constexpr double kBisectRtol = 1e-12;
 constexpr int kBisectMaxit = 200;
-struct BisectState {
+struct alignas(16) BisectState {
     double lo, hi, mu, N, E, Nlo, Nhi;
     int it, phase, status, steps;   // status 1: N_e outside [N(lo), N(hi)]
 };
-// Level range into range[0..1], then a CUDA graph with a while node that
-// alternates bisect_step_kernel and count_kernel (mu read from bs->mu) until
-// the step ends the loop; bs holds the result once the stream reaches it.
-cudaError_t launch_bisection(const ColumnState &st, double kT, double electron_count, double *partial,
-                             unsigned *ticket, double *range, double *out, BisectState *bs,
-                             cudaStream_t s);
+// One bisection: its columns, kT and electron count; the rest is set by
+// launch_bisection (places in the scratch).
+struct alignas(16) BisectTask {
+    int64_t ncols;
+    int nu;
+    const int *nu_eff;
+    const double *eps, *w;
+    double kT, Ne;
+    double *partial;
+    unsigned *ticket;
+    BisectState *bs;
+};
+// Device scratch of n bisections: the tasks, n BisectState (at bisect_states),
+// tickets and a count of the unfinished ones, all uploaded, then the partial sums.
+constexpr size_t bisect_states(size_t n) { return n * ((sizeof(BisectTask) + 15) / 16 * 16); }
+constexpr size_t bisect_tickets(size_t n) { return bisect_states(n) + n * ((sizeof(BisectState) + 15) / 16 * 16); }
+constexpr size_t bisect_partials(size_t n) { return bisect_tickets(n) + (n + 1 + 3) / 4 * 4 * sizeof(unsigned); }
+constexpr size_t bisect_bytes(size_t n) { return bisect_partials(n) + n * 2 * kReduceBlocks * sizeof(double); }
+// n bisections side by side: the level ranges, then a CUDA graph with a while
+// node whose counts (mu read from each task's state) end in a bisection step,
+// until every one is done; the states hold the results once the stream gets there.
+cudaError_t launch_bisection(const BisectTask *tasks, int n, void *scratch, cudaStream_t s);
 // The k-th eigen level and vector (eigstate.cu).
 //   launch_window   colmax[c] = max_a |t_a W_a|, colarg[c] its level, argmax[0] the column
 //                   of the largest (W_a = f((eps_a - hi) / sigma) - f((eps_a - lo) / sigma))

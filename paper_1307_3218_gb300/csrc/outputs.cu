@@ -9,6 +9,10 @@
 // with t = V^T K^T e_j and f(x) = 1 / (1 + e^x) at x = (eps - mu) / kT.
 #include "internal.h"
 
+#include <algorithm>
+#include <cstring>
+#include <vector>
+
 namespace marnoldi {
 namespace {
 
@@ -47,9 +51,11 @@ __device__ __forceinline__ double2 block_reduce2(double a, double b)
 
 // Per-block partials, then the last block to finish (atomic ticket) combines
 // them: each thread folds the partials q = tid, tid + blockDim.x, ... and the
-// block reduces those in its fixed order.  No thread waits on another block.
+// block reduces those in its fixed order.  True, with the totals in t, for one
+// thread of the grid (of a row blockIdx.y of it).  No thread waits on another
+// block.
 template <int OP>
-__device__ void finish_reduce(double a, double b, double *partial, unsigned *ticket, double *out)
+__device__ bool finish_reduce(double a, double b, double *partial, unsigned *ticket, double2 &t)
 {
     __shared__ int last;
     const double2 r = block_reduce2<OP>(a, b);
@@ -60,27 +66,23 @@ __device__ void finish_reduce(double a, double b, double *partial, unsigned *tic
         last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
     }
     __syncthreads();
-    if (last) {   // uniform over the block
-        __threadfence();
-        const volatile double *vp = partial;
-        double x = OP == 0 ? 0.0 : INFINITY, y = OP == 0 ? 0.0 : -INFINITY;
-        for (unsigned q = threadIdx.x; q < gridDim.x; q += blockDim.x) {
-            if (OP == 0) { x += vp[2 * q]; y += vp[2 * q + 1]; }
-            else { x = fmin(x, vp[2 * q]); y = fmax(y, vp[2 * q + 1]); }
-        }
-        const double2 t = block_reduce2<OP>(x, y);
-        if (threadIdx.x == 0) {
-            out[0] = t.x;
-            out[1] = t.y;
-            *ticket = 0u;
-        }
+    if (!last) return false;   // uniform over the block
+    __threadfence();
+    const volatile double *vp = partial;
+    double x = OP == 0 ? 0.0 : INFINITY, y = OP == 0 ? 0.0 : -INFINITY;
+    for (unsigned q = threadIdx.x; q < gridDim.x; q += blockDim.x) {
+        if (OP == 0) { x += vp[2 * q]; y += vp[2 * q + 1]; }
+        else { x = fmin(x, vp[2 * q]); y = fmax(y, vp[2 * q + 1]); }
     }
+    t = block_reduce2<OP>(x, y);
+    if (threadIdx.x != 0) return false;
+    *ticket = 0u;
+    return true;
 }
 
-__global__ void __launch_bounds__(256) minmax_kernel(int64_t total, int nu,
-                                                     const int *__restrict__ nu_eff,
-                                                     const double *__restrict__ eps,
-                                                     double *partial, unsigned *ticket, double *out)
+// Smallest and largest level over this thread's share of the levels.
+__device__ __forceinline__ double2 range_partial(int64_t total, int nu, const int *__restrict__ nu_eff,
+                                                 const double *__restrict__ eps)
 {
     double lo = INFINITY, hi = -INFINITY;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -91,7 +93,20 @@ __global__ void __launch_bounds__(256) minmax_kernel(int64_t total, int nu,
             hi = fmax(hi, eps[idx]);
         }
     }
-    finish_reduce<1>(lo, hi, partial, ticket, out);
+    return make_double2(lo, hi);
+}
+
+__global__ void __launch_bounds__(256) minmax_kernel(int64_t total, int nu,
+                                                     const int *__restrict__ nu_eff,
+                                                     const double *__restrict__ eps,
+                                                     double *partial, unsigned *ticket, double *out)
+{
+    const double2 r = range_partial(total, nu, nu_eff, eps);
+    double2 t;
+    if (finish_reduce<1>(r.x, r.y, partial, ticket, t)) {
+        out[0] = t.x;
+        out[1] = t.y;
+    }
 }
 
 // Beyond |x| = 40 the Fermi function needs no exponential: for x < -40,
@@ -103,15 +118,11 @@ constexpr double kFermiCut = 40.0;
 // in consecutive lanes, so that the lanes of a warp hold levels at similar
 // energies and mostly agree on whether the exponential is needed; levels
 // a >= nu_eff[c] are skipped; the per-thread sums are reduced in a fixed
-// order.  mu from mu_dev when given (the bisection graph), else mu_val.
-__global__ void __launch_bounds__(256) count_kernel(int64_t ncols, int nu,
-                                                    const int *__restrict__ nu_eff,
-                                                    const double *__restrict__ eps,
-                                                    const double *__restrict__ w, double mu_val,
-                                                    const double *__restrict__ mu_dev, double kT,
-                                                    double *partial, unsigned *ticket, double *out)
+// order.
+__device__ __forceinline__ double2 count_partial(int64_t ncols, int nu, const int *__restrict__ nu_eff,
+                                                 const double *__restrict__ eps, const double *__restrict__ w,
+                                                 double mu, double kT)
 {
-    const double mu = mu_dev ? *mu_dev : mu_val;
     const double cut = kFermiCut * kT;
     const int64_t total = ncols * nu, stride = (int64_t)gridDim.x * blockDim.x;
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -133,38 +144,65 @@ __global__ void __launch_bounds__(256) count_kernel(int64_t ncols, int nu,
             ++a;
         }
     }
-    finish_reduce<0>(sn, se, partial, ticket, out);
+    return make_double2(sn, se);
 }
 
-// One step of the Fermi-level bisection, run by one thread between two level
-// counts inside the graph's while loop (same bracket, halving and stopping
-// rule as a host loop would apply): phase 0 sets the bracket from the level
-// range and asks for N(lo), phase 1 asks for N(hi), phase 2 checks that the
-// bracket holds N_e, phase 3 halves until |N - N_e| <= rtol N_e or maxit
-// halvings.  `steps` bounds the loop whatever the counts hold.
-__global__ void bisect_step_kernel(BisectState *bs, const double *__restrict__ range,
-                                   const double *__restrict__ out, double kT, double Ne,
-                                   cudaGraphConditionalHandle loop)
+__global__ void __launch_bounds__(256) count_kernel(int64_t ncols, int nu,
+                                                    const int *__restrict__ nu_eff,
+                                                    const double *__restrict__ eps,
+                                                    const double *__restrict__ w, double mu, double kT,
+                                                    double *partial, unsigned *ticket, double *out)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    BisectState s = *bs;
+    const double2 r = count_partial(ncols, nu, nu_eff, eps, w, mu, kT);
+    double2 t;
+    if (finish_reduce<0>(r.x, r.y, partial, ticket, t)) {
+        out[0] = t.x;
+        out[1] = t.y;
+    }
+}
+
+// Bisection blockIdx.y: the level range and the bracket.
+__global__ void __launch_bounds__(256) bisect_range_kernel(const BisectTask *__restrict__ tasks)
+{
+    const BisectTask q = tasks[blockIdx.y];
+    const double2 r = range_partial(q.ncols * q.nu, q.nu, q.nu_eff, q.eps);
+    double2 t;
+    if (finish_reduce<1>(r.x, r.y, q.partial, q.ticket, t)) {
+        // rounded like the host's (min - 40 kT): no contraction into an FMA
+        q.bs->lo = __dsub_rn(t.x, __dmul_rn(kBisectBracketKT, q.kT));
+        q.bs->hi = __dadd_rn(t.y, __dmul_rn(kBisectBracketKT, q.kT));
+        q.bs->mu = q.bs->lo;
+        q.bs->phase = 1;
+        q.bs->steps = 1;
+    }
+}
+
+// Bisection blockIdx.y: N and E at its mu; the last block to finish then takes
+// the bisection's step (same bracket, halving and stopping rule as a host loop
+// would apply): phase 1 was N(lo) and asks for N(hi), phase 2 checks that the
+// bracket holds N_e, phase 3 halves until |N - N_e| <= rtol N_e or maxit
+// halvings, phase 4 is done.  `steps` bounds the loop whatever the counts hold.
+// The last bisection to finish ends the graph's while loop.  A step in a
+// kernel of its own, one thread between two counts, took half of the loop's time.
+__global__ void __launch_bounds__(256) bisect_count_kernel(const BisectTask *__restrict__ tasks, int *active,
+                                                           cudaGraphConditionalHandle loop)
+{
+    const BisectTask q = tasks[blockIdx.y];
+    if (q.bs->phase == 4) return;   // uniform: set by an earlier launch
+    const double2 r = count_partial(q.ncols, q.nu, q.nu_eff, q.eps, q.w, q.bs->mu, q.kT);
+    double2 t;
+    if (!finish_reduce<0>(r.x, r.y, q.partial, q.ticket, t)) return;
+    BisectState s = *q.bs;
     bool more = true;
     switch (s.phase) {
-    case 0:
-        // rounded like the host's (min - 40 kT): no contraction into an FMA
-        s.lo = __dsub_rn(range[0], __dmul_rn(kBisectBracketKT, kT));
-        s.hi = __dadd_rn(range[1], __dmul_rn(kBisectBracketKT, kT));
-        s.mu = s.lo;
-        s.phase = 1;
-        break;
     case 1:
-        s.Nlo = out[0];
+        s.Nlo = t.x;
         s.mu = s.hi;
         s.phase = 2;
         break;
     case 2:
-        s.Nhi = out[0];
-        if (!(s.Nlo <= Ne && Ne <= s.Nhi)) {
+        s.Nhi = t.x;
+        if (!(s.Nlo <= q.Ne && q.Ne <= s.Nhi)) {
             s.status = 1;
             more = false;
         } else {
@@ -174,12 +212,12 @@ __global__ void bisect_step_kernel(BisectState *bs, const double *__restrict__ r
         }
         break;
     case 3:
-        s.N = out[0];
-        s.E = out[1];
-        if (fabs(s.N - Ne) <= kBisectRtol * Ne || s.it >= kBisectMaxit) {
+        s.N = t.x;
+        s.E = t.y;
+        if (fabs(s.N - q.Ne) <= kBisectRtol * q.Ne || s.it >= kBisectMaxit) {
             more = false;
         } else {
-            if (s.N < Ne) s.lo = s.mu; else s.hi = s.mu;
+            if (s.N < q.Ne) s.lo = s.mu; else s.hi = s.mu;
             s.mu = 0.5 * (s.lo + s.hi);
             ++s.it;
         }
@@ -189,8 +227,8 @@ __global__ void bisect_step_kernel(BisectState *bs, const double *__restrict__ r
     }
     if (++s.steps >= kBisectMaxit + 3) more = false;
     if (!more) s.phase = 4;
-    *bs = s;
-    cudaGraphSetConditional(loop, more ? 1u : 0u);
+    *q.bs = s;
+    if (!more && atomicSub(active, 1) == 1) cudaGraphSetConditional(loop, 0u);
 }
 
 // One CTA per solved column: y = 2 f t (and 2 f eps t), then the pattern rows
@@ -327,33 +365,57 @@ cudaError_t launch_forces(const DeviceMatrix &A, const double *rho, const double
     return cudaGetLastError();
 }
 
+// Blocks of a reduction over `total` levels: those that hold any, at most
+// kReduceBlocks (a block without levels would add exact zeros).
+static unsigned reduce_blocks(int64_t total)
+{
+    return (unsigned)std::min<int64_t>(kReduceBlocks, std::max<int64_t>(1, (total + 255) / 256));
+}
+
 cudaError_t launch_minmax(const ColumnState &st, double *partial, unsigned *ticket, double *out,
                           cudaStream_t s)
 {
-    minmax_kernel<<<kReduceBlocks, 256, 0, s>>>(st.ncols * st.nu, st.nu, st.nu_eff, st.eps,
-                                                 partial, ticket, out);
+    minmax_kernel<<<reduce_blocks(st.ncols * st.nu), 256, 0, s>>>(st.ncols * st.nu, st.nu, st.nu_eff, st.eps,
+                                                                  partial, ticket, out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_count(const ColumnState &st, double mu, double kT, double *partial,
                          unsigned *ticket, double *out, cudaStream_t s)
 {
-    count_kernel<<<kReduceBlocks, 256, 0, s>>>(st.ncols, st.nu, st.nu_eff, st.eps, st.w, mu, nullptr,
-                                                kT, partial, ticket, out);
+    count_kernel<<<reduce_blocks(st.ncols * st.nu), 256, 0, s>>>(st.ncols, st.nu, st.nu_eff, st.eps, st.w, mu, kT,
+                                                                 partial, ticket, out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_bisection(const ColumnState &st, double kT, double electron_count, double *partial,
-                             unsigned *ticket, double *range, double *out, BisectState *bs,
-                             cudaStream_t s)
+cudaError_t launch_bisection(const BisectTask *tasks, int n, void *scratch, cudaStream_t s)
 {
-    // the level range, then one graph whose while node alternates a bisection
-    // step and a level count until the step clears the loop condition
-    minmax_kernel<<<kReduceBlocks, 256, 0, s>>>(st.ncols * st.nu, st.nu, st.nu_eff, st.eps, partial,
-                                                 ticket, range);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemsetAsync(bs, 0, sizeof(BisectState), s);
+    // the tasks with their places in the scratch, the zeroed states and
+    // tickets and the number of bisections, in one upload
+    char *dev = (char *)scratch;
+    std::vector<char> up(bisect_partials(n), 0);
+    int64_t total = 1;
+    for (int q = 0; q < n; ++q) {
+        BisectTask t = tasks[q];
+        t.bs = (BisectState *)(dev + bisect_states(n) + q * (bisect_tickets(1) - bisect_states(1)));
+        t.ticket = (unsigned *)(dev + bisect_tickets(n)) + q;
+        t.partial = (double *)(dev + bisect_partials(n)) + q * 2 * kReduceBlocks;
+        memcpy(up.data() + q * bisect_states(1), &t, sizeof t);
+        total = std::max<int64_t>(total, t.ncols * t.nu);
+    }
+    static_assert(sizeof(BisectTask) % 16 == 0 && sizeof(BisectState) % 16 == 0, "arrays without gaps");
+    int *active = (int *)(dev + bisect_tickets(n)) + n;
+    memcpy(up.data() + ((char *)active - dev), &n, sizeof n);
+    cudaError_t e = cudaMemcpyAsync(dev, up.data(), up.size(), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
+    const BisectTask *td = (const BisectTask *)dev;
+    const dim3 grid(reduce_blocks(total), (unsigned)n);
+    bisect_range_kernel<<<grid, 256, 0, s>>>(td);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // one graph whose while node counts (and steps) until every bisection is
+    // done; a pass of the loop holds several counts, since a pass costs more
+    // than a count that finds its bisection finished
+    constexpr int kCounts = 4;
     cudaGraph_t g = nullptr;
     cudaGraphExec_t ex = nullptr;
     cudaStream_t cap = nullptr;
@@ -374,9 +436,7 @@ cudaError_t launch_bisection(const ColumnState &st, double kT, double electron_c
         cudaGraph_t body = np.conditional.phGraph_out[0];
         e = cudaStreamBeginCaptureToGraph(cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            bisect_step_kernel<<<1, 32, 0, cap>>>(bs, range, out, kT, electron_count, loop);
-            count_kernel<<<kReduceBlocks, 256, 0, cap>>>(st.ncols, st.nu, st.nu_eff, st.eps, st.w, 0.0,
-                                                          &bs->mu, kT, partial, ticket, out);
+            for (int q = 0; q < kCounts; ++q) bisect_count_kernel<<<grid, 256, 0, cap>>>(td, active, loop);
             const cudaError_t el = cudaGetLastError();
             e = cudaStreamEndCapture(cap, &body);
             if (e == cudaSuccess) e = el;
