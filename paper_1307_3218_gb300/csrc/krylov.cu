@@ -148,8 +148,8 @@ __device__ __forceinline__ void spmm_add(uint64_t &hi, uint64_t &lo, uint64_t h,
 
 // H x and S x for the same panel in one pass (both feed the Gram-Schmidt step
 // of the same Krylov vector, and H and S share their block pattern): each x
-// entry is gathered once for both products.  A warp takes one block row for 64
-// columns, a lane the two columns 64 g + lane and 64 g + lane + 32; a CTA's W
+// entry is gathered once for both products.  A warp takes one block row for 32 NC
+// columns, a lane the columns 32 NC g + lane (+ 32); a CTA's W
 // warps take W consecutive rows, which share most of their neighbours.  Rows
 // run fastest in the grid, so the CTAs in flight work on a few column groups
 // whose input panels stay in L2.
@@ -188,7 +188,7 @@ template <typename VT> struct SpmmCfg {
     static constexpr int kSmem = kF ? 48 * 8 : 32 * 8;
 };
 
-template <typename VT, bool kS, int W>
+template <typename VT, bool kS, int W, int NC>
 __global__ void __launch_bounds__(32 * W, (sizeof(VT) == 4 ? 20 : 16) / W) spmm_hs_kernel(
     int nbr, const int64_t *__restrict__ rp, const int32_t *__restrict__ ci,
     const VT *__restrict__ Hv, const VT *__restrict__ Sv, const VT *__restrict__ panel, int ntile,
@@ -197,27 +197,29 @@ __global__ void __launch_bounds__(32 * W, (sizeof(VT) == 4 ? 20 : 16) / W) spmm_
 {
     using Cfg = SpmmCfg<VT>;
     constexpr bool kF = Cfg::kF;
+    static_assert(!kF || NC == 2, "FP32 columns go in pairs");
     __shared__ __align__(16) unsigned char blk[W][2][Cfg::kSmem];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int I = (int)blockIdx.x * W + warp, tile = I >> 3;
     if (I >= nbr) return;   // uniform over the warp
-    int cc[2];
+    int cc[NC];
     bool act = false;
-    int64_t yo[2];
+    int64_t yo[NC];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        cc[h] = (int)blockIdx.y * 64 + 32 * h + lane;
+    for (int h = 0; h < NC; ++h) {
+        cc[h] = (int)blockIdx.y * (32 * NC) + 32 * h + lane;
         act |= cc[h] < ncols && (int)thop[(int64_t)tile * ncols + cc[h]] <= lim;
         // no position: past the columns, or a row of another structure of a
         // union, whose tiles may sit past this column's positions
         yo[h] = cc[h] < ncols ? 32 * (int64_t)tinv[(int64_t)tile * ncols + cc[h]] + 4 * (I & 7) : ldu;
     }
     uint64_t hi[4], lo[4], sy[4];   // FP32: per row entry, the two columns
-    double hd[2][4], sd[2][4];      // FP64
+    double hd[NC][4], sd[NC][4];    // FP64
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
         hi[a] = lo[a] = sy[a] = 0;
-        hd[0][a] = hd[1][a] = sd[0][a] = sd[1][a] = 0.0;
+#pragma unroll
+        for (int h = 0; h < NC; ++h) hd[h][a] = sd[h][a] = 0.0;
     }
     if (__any_sync(kFull, act)) {
         const int64_t k0 = rp[I];
@@ -244,13 +246,13 @@ __global__ void __launch_bounds__(32 * W, (sizeof(VT) == 4 ? 20 : 16) / W) spmm_
                 d[lane] = v;
             }
         };
-        auto gather = [&](int J, VT (&x)[2][4]) {
+        auto gather = [&](int J, VT (&x)[NC][4]) {
             if (!in_range(J, 8 * ntile, kChkSpmmGather)) J = 0;
             const VT *p = xp0 + J * (4 * kPanel);
-            load4(p, x[0]);
-            load4(p + dx, x[1]);
+#pragma unroll
+            for (int h = 0; h < NC; ++h) load4(p + h * dx, x[h]);
         };
-        VT xn[2][4];
+        VT xn[NC][4];
         float4 v = fetch(0);
         gather(column(0), xn);
         stage(0, v);
@@ -258,12 +260,11 @@ __global__ void __launch_bounds__(32 * W, (sizeof(VT) == 4 ? 20 : 16) / W) spmm_
 #pragma unroll 1
         for (int q = 0; q < nk; ++q) {
             __syncwarp();   // block q is staged, block q - 1 read
-            VT x[2][4];
+            VT x[NC][4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                x[0][e] = xn[0][e];
-                x[1][e] = xn[1][e];
-            }
+            for (int h = 0; h < NC; ++h)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) x[h][e] = xn[h][e];
             if (q + 1 < nk) {
                 stage(q + 1, v);
                 gather(column(q + 1), xn);
@@ -298,7 +299,7 @@ __global__ void __launch_bounds__(32 * W, (sizeof(VT) == 4 ? 20 : 16) / W) spmm_
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
+                        for (int h = 0; h < NC; ++h) {
                             hd[h][a] = fma(h4[e], x[h][e], hd[h][a]);
                             if constexpr (kS) sd[h][a] = fma(s4[e], x[h][e], sd[h][a]);
                         }
@@ -307,7 +308,7 @@ __global__ void __launch_bounds__(32 * W, (sizeof(VT) == 4 ? 20 : 16) / W) spmm_
         }
     }
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < NC; ++h) {
         if (yo[h] >= ldu) continue;
         if constexpr (kF) {
             float yh[4], yl[4], ys[4];
@@ -1011,16 +1012,19 @@ cudaError_t spmm_hs(const DeviceMatrix &A, const VT *Hv, const VT *Sv, const Kry
                     int64_t ldsy, int lim, cudaStream_t s)
 {
     const int64_t ng = (b.nb + 63) / 64, ldu = b.shape.m_pad;
-    auto go = [&](auto w) {
-        constexpr int W = decltype(w)::value;
-        spmm_hs_kernel<VT, kS, W><<<dim3((unsigned)((A.nbr + W - 1) / W), (unsigned)ng), 32 * W, 0, s>>>(
+    auto go = [&](auto w, auto nc) {
+        constexpr int W = decltype(w)::value, NC = decltype(nc)::value;
+        const dim3 grid((unsigned)((A.nbr + W - 1) / W), (unsigned)((b.nb + 32 * NC - 1) / (32 * NC)));
+        spmm_hs_kernel<VT, kS, W, NC><<<grid, 32 * W, 0, s>>>(
             (int)A.nbr, A.rp, A.ci, Hv, Sv, (const VT *)b.panel, b.ntile, (VT *)b.U, (VT *)b.Ulo, ldu, (VT *)SY, ldsy, b.nb,
             b.thop, b.tinv, lim);
     };
-    // four rows per CTA; one when that leaves SMs without work (64 atoms, 256
-    // columns: 1.30 ms against 2.18 per FP64 solve of nu = 30, 0.37 against 0.79 mixed)
-    if (A.nbr * ng >= kSpmmWarps) go(std::integral_constant<int, 4>());
-    else go(std::integral_constant<int, 1>());
+    // four rows per CTA; one when that leaves SMs without work, and then one FP64
+    // column per lane (an FP64 instruction holds the warp's scheduler for 64
+    // cycles): 64 atoms, 256 columns, nu = 30: FP64 0.79 ms against 1.30 with two
+    // columns and 2.18 with eight rows per CTA, mixed 0.37 against 0.79
+    if (A.nbr * ng >= kSpmmWarps) go(std::integral_constant<int, 4>(), std::integral_constant<int, 2>());
+    else go(std::integral_constant<int, 1>(), std::integral_constant<int, sizeof(VT) == 4 ? 2 : 1>());
     return cudaGetLastError();
 }
 }  // namespace
