@@ -25,10 +25,10 @@
 // to reach R in the first kernel, whose other threads waited and whose shared
 // memory then held one CTA per SM (nu = 100), and a rotation took four FP64
 // instructions per row.  Per solve, before and after (tridiagonalisation, QL,
-// rows): 24,000 subspaces of nu = 30: 13.9 + 2.1 + 12.0 -> 6.0 + 2.3 + 10.2 ms;
-// 4,000 of nu = 100: 60.6 + 16.7 + 23.6 -> 27.5 + 11.3 + 22.8; 348 of nu = 300:
-// 91.5 + 159.9 + 54.7 -> 41.9 + 88.9 + 55.5; 256 of nu = 30: 0.30 + 1.66 + 0.27 ->
-// 0.27 + 1.13 + 0.25.
+// rows): 24,000 subspaces of nu = 30: 13.9 + 2.1 + 12.0 -> 5.2 + 2.3 + 10.2 ms;
+// 4,000 of nu = 100: 60.6 + 16.7 + 23.6 -> 16.5 + 11.3 + 22.8; 348 of nu = 300:
+// 91.5 + 159.9 + 54.7 -> 36.8 + 88.9 + 55.5; 256 of nu = 30: 0.30 + 1.66 + 0.27 ->
+// 0.24 + 1.13 + 0.25.
 #include "internal.h"
 
 #include <math_constants.h>
@@ -54,15 +54,18 @@ __device__ __forceinline__ double warp_sum(double s)
 
 // ------------------------------------------------------------------ tridiagonalisation
 // A = Q T Q^T with Q = P_0 P_1 ... P_{n-3}, P_k = I - tau_k v_k v_k^T on the
-// entries k + 1 ...  A is symmetric: after the L^-1 transform only its lower
-// triangle is formed and updated (the product A v reads it by rows left of the
-// diagonal and by columns below).
-// Shared memory: A [n][lda] (lda = nu | 1, odd, so that the per-thread row
-// walks spread over the banks), v, e, q.  When A and R do not fit one CTA's
-// shared memory (nu above about 110), A lives in a global scratch of nu x lda
-// doubles per subspace (Ag), which the CTA's sweeps keep in L2 (720 KB at
-// nu = 300).  A thread per row of A: the CTA has as many threads as nu needs.
+// entries k + 1 ...  A is symmetric and only its lower triangle is kept, row by
+// row without gaps: entry (i, j <= i) at i (i + 1) / 2 + j.  Half the shared
+// memory lets five CTAs share an SM at nu = 100 (two with the square), whose
+// phases between barriers then overlap: 16.5 ms for 4,000 subspaces, 27.5 with
+// the square.
+// Shared memory: A, v, e, q.  When A and R do not fit one CTA's shared memory
+// (nu above about 110), A lives in a global scratch per subspace (Ag), which
+// the CTA's sweeps keep in L2 (360 KB at nu = 300).  A thread per row of A: the
+// CTA has as many threads as nu needs.
 // Reflector k goes to V[sc][k][0 .. n - k - 2], tau_k to V[sc][k][nu - 1].
+__device__ __forceinline__ int tri(int i) { return i * (i + 1) / 2; }
+
 __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
     const double *__restrict__ Hsub, const int *__restrict__ bnu_eff, int nu, int cofs,
     double *__restrict__ D, double *__restrict__ E, double *__restrict__ V, double *__restrict__ Ag,
@@ -72,10 +75,9 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
     const int c = cofs + sc;
     const int n = bnu_eff[c];
     const int tid = threadIdx.x, T = blockDim.x;
-    const int lda = nu | 1;
     extern __shared__ __align__(16) double sm[];
-    double *A = Ag ? Ag + (size_t)sc * nu * lda : sm;
-    double *v = Ag ? sm : A + (size_t)nu * lda;
+    double *A = Ag ? Ag + (size_t)sc * nu * (nu | 1) : sm;
+    double *v = Ag ? sm : A + tri(nu);
     double *ev = v + nu;
     double *qv = ev + nu;
     double *Vc = V + (int64_t)sc * nu * nu;
@@ -83,46 +85,51 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
     __shared__ double wpart[kTriThreads / 32];
     __shared__ int skip;
 
-    for (int idx = tid; idx < n * n; idx += T) {
-        const int i = idx / n, l = idx - (idx / n) * n;
-        A[i * lda + l] = 0.5 * (Hsub[((int64_t)c * nu + i) * nu + l] +
-                                Hsub[((int64_t)c * nu + l) * nu + i]);
-    }
+    for (int i = tid >> 5; i < n; i += T / 32)
+        for (int l = tid & 31; l <= i; l += 32)
+            A[tri(i) + l] = 0.5 * (Hsub[((int64_t)c * nu + i) * nu + l] + Hsub[((int64_t)c * nu + l) * nu + i]);
     __syncthreads();
     // The stored basis K~ has unit S-norms and S-Gram matrix G = L L^T, so the
     // S-orthonormal basis K = K~ L^-T carries the subspace problem
-    // A = L^-1 H~ L^-T.  Lsub holds L^-1 (lower triangular); the products run
-    // in place from the last row (column) down, which only reads rows
-    // (columns) not yet replaced.  Four sums side by side keep the FP64 pipe
-    // supplied.
+    // A = L^-1 H~ L^-T.  Lsub holds L^-1 (lower triangular).  First the lower
+    // triangle of W = L^-1 A, row i from the last up: it reads rows m <= i of A
+    // (and, by symmetry, their columns), which are not yet replaced.  Four
+    // sums side by side keep the FP64 pipe supplied.
     const double *Lc = Lsub + (int64_t)c * nu * nu;
     constexpr int kPer = (kMaxNu + kTriThreads - 1) / kTriThreads;   // entries per thread
-    for (int i = n - 1; i >= 0; --i) {   // A <- L^-1 A, row i at a time
+    for (int i = n - 1; i >= 0; --i) {
         const double *Li = Lc + (int64_t)i * nu;
         double x[kPer];
 #pragma unroll
         for (int q = 0; q < kPer; ++q) {
             const int col = tid + q * T;
             double s[4] = {0.0, 0.0, 0.0, 0.0};
-            if (col < n) {
-                int m = 0;
+            if (col <= i) {
+                // row col left of the diagonal, then down column col, chosen per
+                // lane: two loops would run every lane through both bounds
+                const int r0 = tri(col);
+                int m = 0, d = col;   // d = tri(m) + col
                 for (; m + 3 <= i; m += 4)
 #pragma unroll
-                    for (int z = 0; z < 4; ++z) s[z] = fma(Li[m + z], A[(m + z) * lda + col], s[z]);
-                for (; m <= i; ++m) s[0] = fma(Li[m], A[m * lda + col], s[0]);
+                    for (int z = 0; z < 4; ++z) {
+                        s[z] = fma(Li[m + z], A[m + z < col ? r0 + m + z : d], s[z]);
+                        d += m + z + 1;
+                    }
+                for (; m <= i; ++m) {
+                    s[0] = fma(Li[m], A[m < col ? r0 + m : d], s[0]);
+                    d += m + 1;
+                }
             }
             x[q] = (s[0] + s[1]) + (s[2] + s[3]);
         }
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < kPer; ++q)
-            if (tid + q * T < n) A[i * lda + tid + q * T] = x[q];
+            if (tid + q * T <= i) A[tri(i) + tid + q * T] = x[q];
         __syncthreads();
     }
-    // A <- A L^-T, column i at a time, rows i.. only: the result is symmetric
-    // and from here on only its lower triangle (diagonal included) is read or
-    // written.  Column i reads columns m <= i, which are not yet replaced, at
-    // rows >= i.
+    // then W L^-T, column i from the last on, rows i ..: it reads columns m <= i
+    // of W, not yet replaced
     for (int i = n - 1; i >= 0; --i) {
         const double *Li = Lc + (int64_t)i * nu;
         double x[kPer];
@@ -131,18 +138,19 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
             const int row = tid + q * T;
             double s[4] = {0.0, 0.0, 0.0, 0.0};
             if (row >= i && row < n) {
+                const double *Ar = A + tri(row);
                 int m = 0;
                 for (; m + 3 <= i; m += 4)
 #pragma unroll
-                    for (int z = 0; z < 4; ++z) s[z] = fma(A[row * lda + m + z], Li[m + z], s[z]);
-                for (; m <= i; ++m) s[0] = fma(A[row * lda + m], Li[m], s[0]);
+                    for (int z = 0; z < 4; ++z) s[z] = fma(Ar[m + z], Li[m + z], s[z]);
+                for (; m <= i; ++m) s[0] = fma(Ar[m], Li[m], s[0]);
             }
             x[q] = (s[0] + s[1]) + (s[2] + s[3]);
         }
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < kPer; ++q)
-            if (tid + q * T >= i && tid + q * T < n) A[(tid + q * T) * lda + i] = x[q];
+            if (tid + q * T >= i && tid + q * T < n) A[tri(tid + q * T) + i] = x[q];
         __syncthreads();
     }
 
@@ -151,12 +159,12 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
         if (tid < 32) {
             double tail = 0.0;
             for (int l = 1 + tid; l < L; l += 32) {
-                const double x = A[(k + 1 + l) * lda + k];
+                const double x = A[tri(k + 1 + l) + k];
                 tail += x * x;
             }
             tail = warp_sum(tail);
             if (tid == 0) {
-                const double x0 = A[(k + 1) * lda + k];
+                const double x0 = A[tri(k + 1) + k];
                 if (tail == 0.0) {
                     skip = 1;
                     ev[k] = x0;
@@ -180,28 +188,27 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
         }
         const double tauh = sc4[0];
         for (int l = tid; l < L; l += T) {
-            const double x = (l == 0) ? sc4[1] : A[(k + 1 + l) * lda + k];
+            const double x = (l == 0) ? sc4[1] : A[tri(k + 1 + l) + k];
             v[l] = x;
             Vc[(int64_t)k * nu + l] = x;
         }
         __syncthreads();
-        // p = tau A_sub v from A_sub's lower triangle, one entry per thread: row
-        // col left of the diagonal (stride lda, odd, across the threads), then
-        // column col from the diagonal down (consecutive addresses); p goes to
-        // the scratch after e
+        // p = tau A_sub v, one entry per thread; p goes to q
         double vp = 0.0;
         for (int col = tid; col < L; col += T) {
-            const double *Ar = A + (k + 1 + col) * lda + (k + 1), *Ac = A + (k + 1) * lda + (k + 1 + col);
+            const int r0 = tri(k + 1 + col) + (k + 1);
             double s[4] = {0.0, 0.0, 0.0, 0.0};
-            int m = 0;
-            for (; m + 3 < col; m += 4)
-#pragma unroll
-                for (int z = 0; z < 4; ++z) s[z] = fma(Ar[m + z], v[m + z], s[z]);
-            for (; m < col; ++m) s[0] = fma(Ar[m], v[m], s[0]);
+            int m = 0, d = tri(k + 1) + (k + 1 + col);
             for (; m + 3 < L; m += 4)
 #pragma unroll
-                for (int z = 0; z < 4; ++z) s[z] = fma(Ac[(m + z) * lda], v[m + z], s[z]);
-            for (; m < L; ++m) s[0] = fma(Ac[m * lda], v[m], s[0]);
+                for (int z = 0; z < 4; ++z) {
+                    s[z] = fma(A[m + z < col ? r0 + m + z : d], v[m + z], s[z]);
+                    d += k + m + z + 2;
+                }
+            for (; m < L; ++m) {
+                s[0] = fma(A[m < col ? r0 + m : d], v[m], s[0]);
+                d += k + m + 2;
+            }
             const double pl = ((s[0] + s[1]) + (s[2] + s[3])) * tauh;
             qv[col] = pl;
             vp = fma(v[col], pl, vp);
@@ -216,18 +223,18 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
         __syncthreads();
         for (int col = tid; col < L; col += T) qv[col] = fma(-kk, v[col], qv[col]);   // q = p - K v
         __syncthreads();
-        // A_sub -= v q^T + q v^T, lower triangle: a warp per row
+        // A_sub -= v q^T + q v^T: a warp per row
         for (int a = tid >> 5; a < L; a += T / 32) {
             const double va = v[a], qa = qv[a];
-            double *Ar = A + (k + 1 + a) * lda + (k + 1);
+            double *Ar = A + tri(k + 1 + a) + (k + 1);
             for (int b = tid & 31; b <= a; b += 32) Ar[b] = fma(-va, qv[b], fma(-qa, v[b], Ar[b]));
         }
         __syncthreads();
     }
     double *Dc = D + (int64_t)sc * nu, *Ec = E + (int64_t)sc * nu;
     for (int i = tid; i < n; i += T) {
-        Dc[i] = A[i * lda + i];
-        Ec[i] = i + 2 < n ? ev[i] : (i + 2 == n ? A[(n - 1) * lda + (n - 2)] : 0.0);
+        Dc[i] = A[tri(i) + i];
+        Ec[i] = i + 2 < n ? ev[i] : (i + 2 == n ? A[tri(n - 1) + (n - 2)] : 0.0);
     }
 }
 
@@ -654,7 +661,7 @@ cudaError_t launch_eig(const DeviceMatrix &A, const KrylovBatch &b, const Column
 {
     if ((es.proj == nullptr) != (es.proj_out == nullptr)) return cudaErrorInvalidValue;
     const int nu = b.nu;
-    const size_t tsmem = ((size_t)(es.Ag ? 0 : nu) * (nu | 1) + 3 * (size_t)nu) * sizeof(double);
+    const size_t tsmem = ((es.Ag ? 0 : (size_t)nu * (nu + 1) / 2) + 3 * (size_t)nu) * sizeof(double);
     const int tthreads = std::min(kTriThreads, (nu + 31) / 32 * 32);
     cudaError_t e = allow_dynamic_smem((const void *)eig_tridiag_kernel, tsmem);
     if (e != cudaSuccess) return e;
