@@ -1,4 +1,4 @@
-// Device helpers of the Gram-Schmidt kernel (krylov.cu):
+// Device helpers of the Krylov build (krylov.cu, region.cu): packed and
 // error-free FP32 dot accumulators, fixed-order warp reductions, and the FP64
 // scalar step of one Krylov step (norm, breakdown test, the Gram matrix's new
 // column, the new row of L^-1 and the projection coefficients).
@@ -149,6 +149,28 @@ struct PairAcc {
         return r;
     }
 };
+
+// (hi, lo) += (h + l) x per lane of the pairs, nx = -x: p = h x, its error and
+// l x (negated, so that no integer instruction negates p), and p added to hi
+// with a two-sum.
+__device__ __forceinline__ void spmm_add(uint64_t &hi, uint64_t &lo, uint64_t h, uint64_t l, uint64_t x, uint64_t nx)
+{
+    asm("{\n\t.reg .b64 p, e, s, bb, t, u, err;\n\t"
+        "mul.rn.f32x2 p, %2, %4;\n\t"
+        "fma.rn.f32x2 e, %2, %5, p;\n\t"
+        "fma.rn.f32x2 e, %3, %5, e;\n\t"
+        "add.rn.f32x2 s, %0, p;\n\t"
+        "sub.rn.f32x2 bb, s, %0;\n\t"
+        "sub.rn.f32x2 t, s, bb;\n\t"
+        "sub.rn.f32x2 t, %0, t;\n\t"
+        "sub.rn.f32x2 u, p, bb;\n\t"
+        "add.rn.f32x2 err, t, u;\n\t"
+        "sub.rn.f32x2 e, e, err;\n\t"
+        "sub.rn.f32x2 %1, %1, e;\n\t"
+        "mov.b64 %0, s;\n\t}"
+        : "+l"(hi), "+l"(lo)
+        : "l"(h), "l"(l), "l"(x), "l"(nx));
+}
 
 // Vectors per block of the Gram-Schmidt sweeps (one CTA reduction each).
 constexpr int kGsBlock = 4;

@@ -124,28 +124,6 @@ __device__ __forceinline__ void lds_d4(uint32_t a, double (&v)[4])
     asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "r"(a));
     asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v[2]), "=d"(v[3]) : "r"(a + 16));
 }
-// (hi, lo) += (h + l) x per lane of the pairs, nx = -x: p = h x, its error and
-// l x (negated, so that no integer instruction negates p), and p added to hi
-// with a two-sum.
-__device__ __forceinline__ void spmm_add(uint64_t &hi, uint64_t &lo, uint64_t h, uint64_t l, uint64_t x, uint64_t nx)
-{
-    asm("{\n\t.reg .b64 p, e, s, bb, t, u, err;\n\t"
-        "mul.rn.f32x2 p, %2, %4;\n\t"
-        "fma.rn.f32x2 e, %2, %5, p;\n\t"
-        "fma.rn.f32x2 e, %3, %5, e;\n\t"
-        "add.rn.f32x2 s, %0, p;\n\t"
-        "sub.rn.f32x2 bb, s, %0;\n\t"
-        "sub.rn.f32x2 t, s, bb;\n\t"
-        "sub.rn.f32x2 t, %0, t;\n\t"
-        "sub.rn.f32x2 u, p, bb;\n\t"
-        "add.rn.f32x2 err, t, u;\n\t"
-        "sub.rn.f32x2 e, e, err;\n\t"
-        "sub.rn.f32x2 %1, %1, e;\n\t"
-        "mov.b64 %0, s;\n\t}"
-        : "+l"(hi), "+l"(lo)
-        : "l"(h), "l"(l), "l"(x), "l"(nx));
-}
-
 // H x and S x for the same panel in one pass (both feed the Gram-Schmidt step
 // of the same Krylov vector, and H and S share their block pattern): each x
 // entry is gathered once for both products.  A warp takes one block row for 32 NC

@@ -22,15 +22,13 @@
 //                      atom's columns (each block read once for the group),
 //                      x and y of length m_pad >= 4 n_reg, matrix values
 //                      gathered from the global BSR through lgk
-#include "internal.h"
+#include "gs_common.cuh"
 
 #include <cfloat>
 #include <climits>
 
 namespace marnoldi {
 namespace {
-
-constexpr unsigned kFull = 0xffffffffu;
 
 // Squared minimum-image distance, summed as (dx^2 + dy^2) + dz^2 with every
 // operation rounded separately (no contraction), so the host-side checker can
@@ -235,15 +233,6 @@ __global__ void init_regional_kernel(const double *__restrict__ Sv, const double
     }
 }
 
-__device__ __forceinline__ void df_add(float &hi, float &lo, float h2, float l2)
-{
-    const float s = __fadd_rn(hi, h2);
-    const float bb = __fsub_rn(s, hi);
-    const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(h2, bb));
-    hi = s;
-    lo = __fadd_rn(lo, __fadd_rn(l2, err));
-}
-
 // y = H_local x and, with kS, S_local x in one pass (both feed the same
 // Gram-Schmidt step and share the local block list, so the x gathers and the
 // index reads serve both).  Lanes run over local block rows, so the
@@ -330,28 +319,29 @@ __device__ __forceinline__ void regional_rows(
     }
 }
 
-// Thread (x, y) of a 32x8 CTA: local row p = 32 blockIdx.x + x of group
-// g = 8 blockIdx.y + y, the batch columns gstart[g] .. gstart[g + 1] - 1 of one
-// atom (the host splits the batch into runs of one atom's columns of at most
-// G = reg_group<VT>()).  A full group takes one shared pass; a shorter one (an
-// atom with fewer real orbitals, or a run cut by the batch) runs its columns
-// one by one.  G is what the registers allow: FP64 accumulators for four
-// columns would leave one CTA per SM.
+// Columns of one atom that share a pass over the blocks: what the registers
+// allow (FP64 accumulators for four columns would leave one CTA per SM).
 template <typename VT>
 constexpr int reg_group()
 {
     return sizeof(VT) == 4 ? 4 : 2;
 }
 
-template <typename VT, bool kS>
+// FP64: thread (x, y) of a 32x8 CTA takes local row p = 32 blockIdx.x + x of
+// group g = 8 blockIdx.y + y, the batch columns gstart[g] .. gstart[g + 1] - 1 of
+// one atom (the host splits the batch into runs of one atom's columns of at
+// most G = reg_group<VT>()).  A full group takes one shared pass; a shorter one
+// (an atom with fewer real orbitals, or a run cut by the batch) runs its
+// columns one by one.  Bound by the FP64 pipe.
+template <bool kS>
 __global__ void __launch_bounds__(256) spmm_regional_hs_kernel(
     int n_reg, int maxrow, const int *__restrict__ lcnt, const int *__restrict__ lci,
-    const int *__restrict__ lgk, const VT *__restrict__ Hv, const VT *__restrict__ Sv,
-    const VT *__restrict__ X, int64_t ldx, VT *__restrict__ U, VT *__restrict__ Ulo, int64_t ldu,
-    VT *__restrict__ SY, int64_t ldsy, int ncols, const int *__restrict__ gstart, int ngroups,
+    const int *__restrict__ lgk, const double *__restrict__ Hv, const double *__restrict__ Sv,
+    const double *__restrict__ X, int64_t ldx, double *__restrict__ U, int64_t ldu,
+    double *__restrict__ SY, int64_t ldsy, int ncols, const int *__restrict__ gstart, int ngroups,
     const uint8_t *__restrict__ thop, const uint16_t *__restrict__ tinv, int lim)
 {
-    constexpr int G = reg_group<VT>();
+    constexpr int G = reg_group<double>();
     const int p = blockIdx.x * 32 + threadIdx.x;
     const int g = blockIdx.y * 8 + threadIdx.y;
     if (p >= n_reg || g >= ngroups) return;
@@ -359,13 +349,168 @@ __global__ void __launch_bounds__(256) spmm_regional_hs_kernel(
     const int c0 = gstart[g], c1 = min(gstart[g + 1], ncols);
     if (c0 >= c1) return;
     if (c1 - c0 == G) {
-        regional_rows<VT, kS, G>(p, c0, n_reg, maxrow, lcnt, lci, lgk, Hv, Sv, X, ldx, U, Ulo, ldu, SY, ldsy,
-                                 ncols, thop, tinv, lim);
+        regional_rows<double, kS, G>(p, c0, n_reg, maxrow, lcnt, lci, lgk, Hv, Sv, X, ldx, U, nullptr, ldu, SY, ldsy,
+                                     ncols, thop, tinv, lim);
     } else {
 #pragma unroll 1
         for (int c = c0; c < c1; ++c)
-            regional_rows<VT, kS, 1>(p, c, n_reg, maxrow, lcnt, lci, lgk, Hv, Sv, X, ldx, U, Ulo, ldu, SY, ldsy,
-                                     ncols, thop, tinv, lim);
+            regional_rows<double, kS, 1>(p, c, n_reg, maxrow, lcnt, lci, lgk, Hv, Sv, X, ldx, U, nullptr, ldu, SY,
+                                         ldsy, ncols, thop, tinv, lim);
+    }
+}
+
+// Mixed precision, groups of four columns: one CTA per group, the four columns'
+// x in shared memory, a lane per local row.  A lane's block is its own (the
+// lanes' blocks are 32 different ones), and reading it 16 bytes at a time looked
+// up 32 lines per load, which kept the L1 at 87 %; here twelve lanes copy one
+// block together (its lines are looked up once) into the warp's shared memory,
+// from where each lane reads its own.  The columns go through packed
+// instructions in pairs; every column's sums run in the same order as alone.
+// 24,000 columns, 256-atom regions, nu = 30: 21.5 ms, 27.2 with a lane reading
+// its own block; 4,000 columns, nu = 100: 14.6 (19.0).
+constexpr int kRegPitch = 52;   // floats per staged block: H hi and lo, S hi, and 4 that spread the banks
+
+template <bool kS>
+__global__ void __launch_bounds__(128, 3) spmm_regional_group_kernel(
+    int n_reg, int maxrow, const int *__restrict__ lcnt, const int *__restrict__ lci,
+    const int *__restrict__ lgk, const float *__restrict__ Hv, const float *__restrict__ Sv,
+    const float *__restrict__ X, int64_t ldx, float *__restrict__ U, float *__restrict__ Ulo, int64_t ldu,
+    float *__restrict__ SY, int64_t ldsy, int ncols, const int *__restrict__ gstart,
+    const uint8_t *__restrict__ thop, const uint16_t *__restrict__ tinv, int lim)
+{
+    constexpr int G = reg_group<float>(), NW = 4, kPieces = kS ? 12 : 8;
+    static_assert(G == 4, "two pairs of columns");
+    extern __shared__ __align__(16) float rsm[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    float *blk = rsm + warp * (2 * 32 * kRegPitch);    // two stages of 32 blocks
+    const int g = blockIdx.x;
+    // clipped to ncols: a run of the autotuner covers the batch's first columns only
+    const int c0 = gstart[g], c1 = min(gstart[g + 1], ncols);
+    if (c0 >= c1) return;
+    if (c1 - c0 < G) {   // an atom with fewer real orbitals, or a run cut by the batch: column by column
+        for (int c = c0; c < c1; ++c)
+            for (int p = tid; p < n_reg; p += 32 * NW)
+                regional_rows<float, kS, 1>(p, c, n_reg, maxrow, lcnt, lci, lgk, Hv, Sv, X, ldx, U, Ulo, ldu, SY,
+                                            ldsy, ncols, thop, tinv, lim);
+        return;
+    }
+    const float *xc = X + (int64_t)c0 * ldx;
+    const int64_t base = (int64_t)c0 * maxrow * n_reg;
+    const uint32_t sb = (uint32_t)__cvta_generic_to_shared(blk);
+    for (int p0 = 32 * warp; p0 < n_reg; p0 += 32 * NW) {
+        const int p = p0 + lane;
+        const bool row = p < n_reg;
+        const bool act = row && (int)thop[(int64_t)(p >> 3) * ncols + c0] <= lim;
+        const int cnt = act ? lcnt[(int64_t)c0 * n_reg + p] : 0;
+        const int most = __reduce_max_sync(kFull, cnt);
+        uint64_t hi[2][4], lo[2][4], sy[2][4];   // column pairs (0, 1) and (2, 3)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int a = 0; a < 4; ++a) hi[h][a] = lo[h][a] = sy[h][a] = 0;
+        auto block_of = [&](int s) { return s < cnt ? lgk[base + (int64_t)s * n_reg + p] : -1; };
+        auto column_of = [&](int s) { return s < cnt ? lci[base + (int64_t)s * n_reg + p] : -1; };
+        // position of local column q's entries, -1 for none
+        auto position = [&](int q) {
+            if (q < 0 || !in_range(q, n_reg, kChkRegionCol)) return -1;
+            const int xp = 32 * (int)tinv[(int64_t)(q >> 3) * ncols + c0] + 4 * (q & 7);
+            return in_range(xp, ldu - 3, kChkRegionGather) ? xp : -1;
+        };
+        auto copy = [&](int s, int k) {   // the lanes' blocks of slot s, k this lane's
+            const uint32_t st = sb + (s & 1) * (32 * kRegPitch * 4);
+#pragma unroll
+            for (int r = 0; r < kPieces; ++r) {
+                const int item = 32 * r + lane, b = item / kPieces, piece = item - b * kPieces;
+                const int kb = __shfl_sync(kFull, k, b);
+                const float *src = (piece < 8 ? Hv : Sv) + 32 * (int64_t)kb + 4 * (piece < 8 ? piece : piece - 8);
+                if (kb >= 0)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(st + 4 * (b * kRegPitch + 4 * piece)),
+                                 "l"(src)
+                                 : "memory");
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        auto gather = [&](int xp, float4 (&x)[G]) {
+#pragma unroll
+            for (int m = 0; m < G; ++m)
+                if (xp >= 0) x[m] = __ldg(reinterpret_cast<const float4 *>(xc + m * ldx + xp));
+        };
+        // blocks are copied one slot ahead, x one, the positions two, the indices three
+        __syncwarp();   // the last slots of the rows before have been read
+        copy(0, block_of(0));
+        int kn = block_of(1), x0p = position(column_of(0)), x1p = position(column_of(1)), q2 = column_of(2);
+        float4 xv[G], xw[G];
+        gather(x0p, xv);
+        for (int s = 0; s < most; ++s) {
+            __syncwarp();   // slot s - 1 has been read
+            if (s + 1 < most) copy(s + 1, kn);
+            else asm volatile("cp.async.commit_group;" ::: "memory");
+            gather(x1p, xw);
+            const int x2p = position(q2);
+            q2 = column_of(s + 3);
+            kn = block_of(s + 2);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncwarp();
+            if (x0p >= 0) {
+                uint64_t x[2][4], nx[2][4];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float4 u = xv[2 * h], v = xv[2 * h + 1];
+                    x[h][0] = pack_x2(u.x, v.x);
+                    x[h][1] = pack_x2(u.y, v.y);
+                    x[h][2] = pack_x2(u.z, v.z);
+                    x[h][3] = pack_x2(u.w, v.w);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) nx[h][e] = neg_x2(x[h][e]);
+                }
+                const float *B = blk + (s & 1) * (32 * kRegPitch) + lane * kRegPitch;
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    const float4 h4 = *reinterpret_cast<const float4 *>(B + 4 * a);
+                    const float4 l4 = *reinterpret_cast<const float4 *>(B + 16 + 4 * a);
+                    const float hv[4] = {h4.x, h4.y, h4.z, h4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
+                    float sv[4] = {0.f, 0.f, 0.f, 0.f};
+                    if constexpr (kS) {
+                        const float4 s4 = *reinterpret_cast<const float4 *>(B + 32 + 4 * a);
+                        sv[0] = s4.x; sv[1] = s4.y; sv[2] = s4.z; sv[3] = s4.w;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const uint64_t hp = pack_x2(hv[e], hv[e]), lp = pack_x2(lv[e], lv[e]);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) spmm_add(hi[h][a], lo[h][a], hp, lp, x[h][e], nx[h][e]);
+                        if constexpr (kS) {
+                            const uint64_t sp = pack_x2(sv[e], sv[e]);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) sy[h][a] = fma_x2(sp, x[h][e], sy[h][a]);
+                        }
+                    }
+                }
+            }
+            x0p = x1p;
+            x1p = x2p;
+#pragma unroll
+            for (int m = 0; m < G; ++m) xv[m] = xw[m];
+        }
+        if (!row) continue;
+        const int64_t yp = 32 * (int64_t)tinv[(int64_t)(p >> 3) * ncols + c0] + 4 * (p & 7);
+#pragma unroll
+        for (int m = 0; m < G; ++m) {
+            const int64_t c = c0 + m;
+            float yh[4], yl[4], ys[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const int sh = 32 * (m & 1);
+                const float fh = __uint_as_float((unsigned)(hi[m >> 1][a] >> sh));
+                const float fl = __uint_as_float((unsigned)(lo[m >> 1][a] >> sh));
+                yh[a] = __fadd_rn(fh, fl);
+                yl[a] = __fsub_rn(fl, __fsub_rn(yh[a], fh));
+                ys[a] = __uint_as_float((unsigned)(sy[m >> 1][a] >> sh));
+            }
+            store4(U + c * ldu + yp, yh);
+            store4(Ulo + c * ldu + yp, yl);
+            if constexpr (kS) store4(SY + c * ldsy + yp, ys);
+        }
     }
 }
 
@@ -384,22 +529,22 @@ cudaError_t launch_spmm_regional_hs(const DeviceMatrix &A, const RegionMaps &rm,
     const int64_t ldu = b.shape.m_pad;
     if (b.prec == 0) {
         if (SY)
-            spmm_regional_hs_kernel<double, true><<<grid, block, 0, s>>>(
-                rm.n_reg, rm.maxrow, rm.lcnt, rm.lci, rm.lgk, A.Hd, A.Sd, (const double *)X, ldx, (double *)b.U,
-                nullptr, ldu, (double *)SY, ldsy, b.nb, rm.gstart, rm.ngroups, b.thop, b.tinv, lim);
+            spmm_regional_hs_kernel<true><<<grid, block, 0, s>>>(
+                rm.n_reg, rm.maxrow, rm.lcnt, rm.lci, rm.lgk, A.Hd, A.Sd, (const double *)X, ldx, (double *)b.U, ldu, (double *)SY, ldsy, b.nb, rm.gstart, rm.ngroups, b.thop, b.tinv, lim);
         else
-            spmm_regional_hs_kernel<double, false><<<grid, block, 0, s>>>(
-                rm.n_reg, rm.maxrow, rm.lcnt, rm.lci, rm.lgk, A.Hd, A.Sd, (const double *)X, ldx, (double *)b.U,
-                nullptr, ldu, nullptr, 0, b.nb, rm.gstart, rm.ngroups, b.thop, b.tinv, lim);
+            spmm_regional_hs_kernel<false><<<grid, block, 0, s>>>(
+                rm.n_reg, rm.maxrow, rm.lcnt, rm.lci, rm.lgk, A.Hd, A.Sd, (const double *)X, ldx, (double *)b.U, ldu, nullptr, 0, b.nb, rm.gstart, rm.ngroups, b.thop, b.tinv, lim);
     } else {
-        if (SY)
-            spmm_regional_hs_kernel<float, true><<<grid, block, 0, s>>>(
+        const size_t smem = (size_t)4 * 2 * 32 * kRegPitch * sizeof(float);
+        auto go = [&](auto kernel) {
+            const cudaError_t e = allow_dynamic_smem((const void *)kernel, smem);
+            if (e != cudaSuccess) return e;
+            kernel<<<rm.ngroups, 128, smem, s>>>(
                 rm.n_reg, rm.maxrow, rm.lcnt, rm.lci, rm.lgk, A.Hf, A.Sf, (const float *)X, ldx, (float *)b.U,
-                (float *)b.Ulo, ldu, (float *)SY, ldsy, b.nb, rm.gstart, rm.ngroups, b.thop, b.tinv, lim);
-        else
-            spmm_regional_hs_kernel<float, false><<<grid, block, 0, s>>>(
-                rm.n_reg, rm.maxrow, rm.lcnt, rm.lci, rm.lgk, A.Hf, A.Sf, (const float *)X, ldx, (float *)b.U,
-                (float *)b.Ulo, ldu, nullptr, 0, b.nb, rm.gstart, rm.ngroups, b.thop, b.tinv, lim);
+                (float *)b.Ulo, ldu, (float *)SY, ldsy, b.nb, rm.gstart, b.thop, b.tinv, lim);
+            return cudaGetLastError();
+        };
+        return SY ? go(spmm_regional_group_kernel<true>) : go(spmm_regional_group_kernel<false>);
     }
     return cudaGetLastError();
 }
