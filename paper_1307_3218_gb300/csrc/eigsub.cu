@@ -41,7 +41,6 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kTriThreads = 256;    // most threads of the tridiagonalisation
-constexpr int kApplyThreads = 128;  // most threads of the rows' kernel
 constexpr int kQlMaxIter = 30;      // QL iterations per eigenvalue
 constexpr int kQlWarps = 152;       // one QL warp per SM
 
@@ -437,210 +436,248 @@ __global__ void __launch_bounds__(64) eig_ql_kernel(const int *__restrict__ bnu_
 #undef WW
 }
 
-// ------------------------------------------------------------------ rows and outputs
-// A thread per row of R = [e_1; q; K_pat; (v^T w_i)], in shared memory as
-// [nr_max][ldr] (ldr odd): R L^-T, the reflectors, the rotations, the scales.
-// A warp's lanes hold the next 32 rotations in registers and broadcast them
-// with shuffles while the following 32 are on their way.
-template <typename VT>
-__global__ void __launch_bounds__(kApplyThreads) eig_apply_kernel(
-    const int *__restrict__ bnu_eff, const int *__restrict__ bstatus, int cofs, int nu,
-    const double *__restrict__ bscale, const VT *__restrict__ K, int64_t m_pad, const uint16_t *__restrict__ tinv,
-    int nb, const int64_t *__restrict__ bcols, const double *__restrict__ sdiag,
-    const int64_t *__restrict__ rp, const int32_t *__restrict__ ci, const int *__restrict__ reg, int n_reg,
-    int64_t col0, const double *__restrict__ D, const double *__restrict__ W, const double *__restrict__ V,
-    const double *__restrict__ Lsub, const double *__restrict__ proj, int nr_max,
-    const double2 *__restrict__ rot, int64_t rcap, const int2 *__restrict__ sweep, int64_t scap,
-    const int *__restrict__ nsweep, int *__restrict__ nu_eff_out, double *__restrict__ eps_out,
-    double *__restrict__ w_out, double *__restrict__ t_out, double *__restrict__ P_out,
-    const int64_t *__restrict__ p_off, int *__restrict__ eig_status, double *__restrict__ proj_out)
+// ------------------------------------------------------------------ levels
+// A CTA per subspace: eps in ascending order (ties by index; a NaN level, from
+// non-finite input, ranks as +inf, so that the ranks always form a
+// permutation) and the order, which takes the place of the levels in D.  The
+// comparisons are of integers that order as the doubles do.
+__global__ void __launch_bounds__(128) eig_rank_kernel(
+    const int *__restrict__ bnu_eff, const int *__restrict__ bstatus, int cofs, int nu, int64_t col0,
+    double *__restrict__ D, const int *__restrict__ nsweep, int *__restrict__ nu_eff_out,
+    double *__restrict__ eps_out, int *__restrict__ eig_status)
 {
-    const int sc = blockIdx.x;
-    const int c = cofs + sc;
-    const int64_t g = col0 + c;
-    const int n = bnu_eff[c];
-    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
-    const int ldr = nu | 1;
     extern __shared__ __align__(16) double asm_[];
-    double *R = asm_;
-    double *d = R + (size_t)nr_max * ldr;
-    double *wsc = d + nu;
-    int *perm = reinterpret_cast<int *>(wsc + nu);
-    // rows of R: e_1, q = K^T e_j, and K_pat (zero for atoms outside a region)
-    const int64_t j = bcols[c];
-    const int64_t J = j >> 2;
-    const int *Rg = reg ? reg + (int64_t)c * n_reg : nullptr;
-    const int pJ = Rg ? find_sorted(Rg, n_reg, (int)J) : 0;
-    const int64_t jl = Rg ? 4 * (int64_t)(pJ < 0 ? 0 : pJ) + (j & 3) : j;
-    const int64_t kb = rp[J];
+    double *d = asm_;
+    uint64_t *key = reinterpret_cast<uint64_t *>(d + nu);
+    const int sc = blockIdx.x, c = cofs + sc, n = bnu_eff[c];
+    const int64_t g = col0 + c;
+    double *Dc = D + (int64_t)sc * nu;
+    int *order = reinterpret_cast<int *>(Dc);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const double x = Dc[i];
+        d[i] = x;
+        const uint64_t u = (uint64_t)__double_as_longlong(x != x ? CUDART_INF : x + 0.0);   // -0 as 0
+        key[i] = u >> 63 ? ~u : u | 0x8000000000000000ull;
+    }
+    __syncthreads();
+    for (int a = threadIdx.x; a < nu; a += blockDim.x) {
+        if (a >= n) {
+            eps_out[g * nu + a] = 0.0;
+            continue;
+        }
+        const uint64_t ka = key[a];
+        int rank = 0;
+        for (int b = 0; b < n; ++b) rank += key[b] < ka || (key[b] == ka && b < a);
+        order[rank] = a;
+        eps_out[g * nu + rank] = d[a];
+    }
+    if (threadIdx.x == 0) {
+        nu_eff_out[g] = n;
+        eig_status[g] = (nsweep[sc] < 0 ? 1 : 0) | (bstatus[c] == 2 ? 2 : 0);
+    }
+}
+
+// ------------------------------------------------------------------ rows and outputs
+// Rows of R = [e_1; q; K_pat; (v^T w_i)], one per lane: R L^-T, the
+// reflectors, the rotations, the scales.  Bound by FP64 instructions, which
+// cost as much for one lane as for 32, so the rows of all subspaces are packed
+// without gaps: a CTA is one warp and takes the next `rows` of them, of one
+// subspace or of several (a lane then follows its own subspace's log), in
+// shared memory as [rows][ldr] (ldr odd).  Every subspace has an even number
+// of rows, so its first two share a warp.  With a CTA per subspace, 75 rows
+// took three warps and their CTAs filled an SM's four schedulers unevenly.
+// 24,000 subspaces of nu = 30: 10.2 -> @A@ ms; 4,000 of nu = 100: 22.8 -> @B@;
+// 348 of nu = 300: 55.5 -> @C@.
+constexpr int kLogAhead = 4;   // rotations held in registers ahead of their use
+
+template <typename VT>
+__global__ void __launch_bounds__(32) eig_apply_kernel(
+    const int *__restrict__ bnu_eff, int cofs, int nb2, int nu, int rows, const double *__restrict__ bscale,
+    const VT *__restrict__ K, int64_t m_pad, const uint16_t *__restrict__ tinv, int nb,
+    const int64_t *__restrict__ bcols, const double *__restrict__ sdiag, const int64_t *__restrict__ rp,
+    const int32_t *__restrict__ ci, const int *__restrict__ reg, int n_reg, int64_t col0,
+    const double *__restrict__ D, const double *__restrict__ W, const double *__restrict__ V,
+    const double *__restrict__ Lsub, const double *__restrict__ proj, const double2 *__restrict__ rot, int64_t rcap,
+    const int2 *__restrict__ sweep, int64_t scap, const int *__restrict__ nsweep, double *__restrict__ w_out,
+    double *__restrict__ t_out, double *__restrict__ P_out, const int64_t *__restrict__ p_off,
+    double *__restrict__ proj_out)
+{
+    extern __shared__ __align__(16) double asm_[];
+    const int lane = threadIdx.x;
+    const int ldr = nu | 1;
+    // first row of subspace s among all rows: its pattern rows start at
+    // p_off / nu, and the others add two rows per subspace (four with a projection
+    // row, the last of them unused)
+    const int extra = proj ? 4 : 2;
+    const int64_t g0 = col0 + cofs, p0 = p_off[g0];
+    auto first = [&](int s) { return p_off[g0 + s] - p0 + (int64_t)extra * nu * s; };   // times nu
+    const int64_t at = (int64_t)blockIdx.x * rows + lane;
+    int lo = 0, hi = nb2;   // the last subspace whose first row is at or before `at`
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (first(mid) <= at * nu) lo = mid; else hi = mid;
+    }
+    const int sc = lo, c = cofs + sc;
+    const int64_t j = bcols[c], J = j >> 2, kb = rp[J];
     const int npat = 4 * (int)(rp[J + 1] - kb);
-    const int nr = npat + 2 + (proj ? 1 : 0);   // the projection row last
-    const VT *Kc = K + (int64_t)c * nu * m_pad;
-    for (int r = tid; r < nr; r += T) {
+    const int64_t r64 = at - first(sc) / nu;
+    const int r = r64 < npat + 2 + (proj ? 1 : 0) ? (int)r64 : -1;   // -1: past the rows
+    const bool own = lane < rows && r >= 0;
+    const int n = bnu_eff[c];
+    double *R = asm_ + 1;   // x[-1] is read ahead and not used
+    double *x = R + (lane < rows ? lane : 0) * ldr;
+    if (own) {
+        // q = K^T e_j and K_pat (zero for atoms outside a region)
+        const int *Rg = reg ? reg + (int64_t)c * n_reg : nullptr;
         int64_t pos = -1;   // the row's position in the column's vectors
         if (r == 1) {
-            pos = vpos(tinv, nb, c, jl);
+            const int pJ = Rg ? find_sorted(Rg, n_reg, (int)J) : 0;
+            pos = vpos(tinv, nb, c, Rg ? 4 * (int64_t)(pJ < 0 ? 0 : pJ) + (j & 3) : j);
         } else if (r >= 2 && r < npat + 2) {
             const int atom = ci[kb + ((r - 2) >> 2)];
             const int64_t lr = Rg ? find_sorted(Rg, n_reg, atom) : atom;
             if (lr >= 0) pos = vpos(tinv, nb, c, 4 * lr + ((r - 2) & 3));
         }
-        double *x = R + r * ldr;
+        const VT *Kc = K + (int64_t)c * nu * m_pad;
         const double *si = bscale + (int64_t)c * nu;
+#pragma unroll 4
         for (int i = 0; i < n; ++i)
             x[i] = r == 0 ? (i == 0 ? 1.0 : 0.0)
                    : r == npat + 2 ? si[i] * proj[(int64_t)c * nu + i]
                    : pos >= 0 ? si[i] * (double)Kc[(int64_t)i * m_pad + pos] : 0.0;
-    }
-    for (int i = tid; i < n; i += T) {
-        d[i] = D[(int64_t)sc * nu + i];
-        wsc[i] = W[(int64_t)sc * nu + i];
-    }
-    const double *Lc = Lsub + (int64_t)c * nu * nu, *Vc = V + (int64_t)sc * nu * nu;
-    const int nsw = nsweep[sc];
-    const double2 *rl = rot + (int64_t)sc * rcap;
-    const int2 *sl = sweep + (int64_t)sc * scap;
-    // whole warps run a row pass (the shuffles); a lane without a row reads and
-    // stores nothing
-    for (int r0 = tid - lane; r0 < nr; r0 += T) {
-        const bool own = r0 + lane < nr;
-        double *x = R + (own ? r0 + lane : 0) * ldr;
-        if (own) {
-            // rows 1..: R <- R L^-T (row 0, e_1^T, is unchanged: K^T S e_j =
-            // sqrt(S_jj) e_1), four entries at a time from the last down
-            if (r0 + lane > 0) {
-                for (int i = n - 1; i >= 0; i -= 4) {
-                    double s[4] = {0.0, 0.0, 0.0, 0.0};
-                    const double *L0 = Lc + (int64_t)i * nu;
-                    const int lo = i - 3;
-                    for (int m = 0; m <= lo; ++m) {   // lo < 0: the general loop below
-                        const double xm = x[m];
+        // rows 1..: R <- R L^-T (row 0, e_1^T, is unchanged: K^T S e_j =
+        // sqrt(S_jj) e_1), four entries at a time from the last down
+        const double *Lc = Lsub + (int64_t)c * nu * nu, *Vc = V + (int64_t)sc * nu * nu;
+        if (r > 0) {
+            for (int i = n - 1; i >= 0; i -= 4) {
+                double s[4] = {0.0, 0.0, 0.0, 0.0};
+                const double *L0 = Lc + (int64_t)i * nu;
+                const int lo4 = i - 3;
+                for (int m = 0; m <= lo4; ++m) {   // lo4 < 0: the general loop below
+                    const double xm = x[m];
 #pragma unroll
-                        for (int z = 0; z < 4; ++z) s[z] = fma(xm, L0[m - (int64_t)z * nu], s[z]);
-                    }
-                    for (int m = lo < 0 ? 0 : lo + 1; m <= i; ++m) {
-                        const double xm = x[m];
-#pragma unroll
-                        for (int z = 0; z < 4; ++z)
-                            if (i - z >= m) s[z] = fma(xm, L0[m - (int64_t)z * nu], s[z]);
-                    }
+                    for (int z = 0; z < 4; ++z) s[z] = fma(xm, L0[m - (int64_t)z * nu], s[z]);
+                }
+                for (int m = lo4 < 0 ? 0 : lo4 + 1; m <= i; ++m) {
+                    const double xm = x[m];
 #pragma unroll
                     for (int z = 0; z < 4; ++z)
-                        if (i - z >= 0) x[i - z] = s[z];
+                        if (i - z >= m) s[z] = fma(xm, L0[m - (int64_t)z * nu], s[z]);
                 }
-            }
-            for (int k = 0; k + 2 < n; ++k) {   // R <- R (I - tau v v^T) on columns k + 1 ..
-                const int L = n - k - 1;
-                const double *v = Vc + (int64_t)k * nu;
-                const double tau = v[nu - 1];
-                if (tau == 0.0) continue;
-                double *row = x + k + 1;
-                double s[4] = {0.0, 0.0, 0.0, 0.0};
-                int m = 0;
-                for (; m + 3 < L; m += 4)
 #pragma unroll
-                    for (int z = 0; z < 4; ++z) s[z] = fma(row[m + z], v[m + z], s[z]);
-                for (; m < L; ++m) s[0] = fma(row[m], v[m], s[0]);
-                const double f = -tau * ((s[0] + s[1]) + (s[2] + s[3]));
-#pragma unroll 4
-                for (m = 0; m < L; ++m) row[m] = fma(f, v[m], row[m]);
+                for (int z = 0; z < 4; ++z)
+                    if (i - z >= 0) x[i - z] = s[z];
             }
         }
-        __syncwarp();
-        // the next rotation's coefficients and the next entry are fetched before
-        // the current rotation's multiply-adds: the chain through carry is then
-        // one multiply-add per rotation
-        int64_t ptr = 0;   // rotation held by lane 0
-        double2 cur = lane < rcap ? rl[lane] : make_double2(0.0, 0.0);
-        double2 nxt = 32 + lane < rcap ? rl[32 + lane] : make_double2(0.0, 0.0);
-        int at = 0;
-        double alpha = __shfl_sync(kFull, cur.x, 0), bs = __shfl_sync(kFull, cur.y, 0);
+        for (int k = 0; k + 2 < n; ++k) {   // R <- R (I - tau v v^T) on columns k + 1 ..
+            const int L = n - k - 1;
+            const double *v = Vc + (int64_t)k * nu;
+            const double tau = v[nu - 1];
+            if (tau == 0.0) continue;
+            double *row = x + k + 1;
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            int m = 0;
+            for (; m + 3 < L; m += 4)
+#pragma unroll
+                for (int z = 0; z < 4; ++z) s[z] = fma(row[m + z], v[m + z], s[z]);
+            for (; m < L; ++m) s[0] = fma(row[m], v[m], s[0]);
+            const double f = -tau * ((s[0] + s[1]) + (s[2] + s[3]));
+#pragma unroll 4
+            for (m = 0; m < L; ++m) row[m] = fma(f, v[m], row[m]);
+        }
+        // the next rotations and the next entry are fetched before the current
+        // rotation's multiply-adds: the chain through carry is then one
+        const int nsw = nsweep[sc];
+        // multiply-add per rotation.  The log comes from DRAM, whose lines are
+        // asked for 64 rotations early; no branches, which would add to the chain
+        const double2 *rl = rot + (int64_t)sc * rcap;
+        const int2 *sl = sweep + (int64_t)sc * scap;
+        const int last = (int)rcap - 1;
+        double2 ring[kLogAhead];
+#pragma unroll
+        for (int z = 0; z < kLogAhead; ++z) ring[z] = rl[min(z, last)];
+        int ahead = kLogAhead;
         int2 sw = nsw > 0 ? sl[0] : make_int2(0, 0);
         for (int q = 0; q < nsw; ++q) {
             const int2 sn = q + 1 < nsw ? sl[q + 1] : make_int2(0, 0);
-            double carry = own ? x[sw.x] : 0.0;
-            double yi = own && sw.x > sw.y ? x[sw.x - 1] : 0.0;
+            double carry = x[sw.x];
+            double yi = x[sw.x - 1];
             for (int i = sw.x - 1; i >= sw.y; --i) {
-                const double al = alpha, y = yi;
+                const double al = ring[0].x, bs = ring[0].y, y = yi;
+#pragma unroll
+                for (int z = 0; z + 1 < kLogAhead; ++z) ring[z] = ring[z + 1];
+                ring[kLogAhead - 1] = rl[min(ahead, last)];
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(rl + min(ahead + 64, last)));
+                ++ahead;
+                yi = x[i - 1];
                 const bool sf = __double2hiint(bs) < 0;
                 // beta = -sign(alpha) |bs|
                 const double beta = __hiloint2double((__double2hiint(bs) & 0x7fffffff) |
                                                          (~__double2hiint(al) & 0x80000000),
                                                      __double2loint(bs));
-                if (++at == 32) {
-                    at = 0;
-                    ptr += 32;
-                    cur = nxt;
-                    if (ptr + 32 + lane < rcap) nxt = rl[ptr + 32 + lane];
-                }
-                alpha = __shfl_sync(kFull, cur.x, at);
-                bs = __shfl_sync(kFull, cur.y, at);
-                if (own && i > sw.y) yi = x[i - 1];
                 const double p = sf ? y : carry, qq = sf ? carry : y;
                 carry = fma(beta, p, qq);
-                if (own) x[i + 1] = fma(al, qq, p);
+                x[i + 1] = fma(al, qq, p);
             }
-            if (own) x[sw.y] = carry;
+            x[sw.y] = carry;
             sw = sn;
         }
     }
-    __syncthreads();
-    // rank of every level (ties by index): ascending order; a NaN level (from
-    // non-finite input) ranks as +inf, so the ranks always form a permutation
-    auto key = [&](int b) { const double x = d[b]; return x != x ? CUDART_INF : x; };
-    for (int a = tid; a < n; a += T) {
-        const double da = key(a);
-        int rank = 0;
-        for (int b = 0; b < n; ++b) {
-            const double db = key(b);
-            rank += (db < da) || (db == da && b < a);
+    __syncwarp();
+    // a row's outputs, in ascending order of eps: the lanes run over the levels
+    for (int l = 0; l < rows; ++l) {
+        const int rr = __shfl_sync(kFull, own ? r : -1, l);
+        const int s = __shfl_sync(kFull, sc, l);
+        if (rr < 1) continue;   // row 0 goes with row 1
+        const int np = __shfl_sync(kFull, npat, l), nn = __shfl_sync(kFull, n, l);
+        const int64_t go = g0 + s;
+        const int *order = reinterpret_cast<const int *>(D + (int64_t)s * nu);
+        const double *wsc = W + (int64_t)s * nu, *xl = R + l * ldr;
+        double *out = rr == 1 ? t_out + go * nu : rr == np + 2 ? proj_out + go * nu
+                                                               : P_out + p_off[go] + (int64_t)(rr - 2) * nu;
+        const double sq = rr == 1 ? sqrt(sdiag[bcols[cofs + s]]) : 0.0;
+        for (int a = lane; a < nu; a += 32) {
+            const int src = a < nn ? order[a] : 0;
+            const double y = a < nn ? xl[src] * wsc[src] : 0.0;
+            out[a] = y;
+            if (rr == 1) w_out[go * nu + a] = a < nn ? sq * (xl[src - ldr] * wsc[src]) * y : 0.0;
         }
-        perm[rank] = a;
-    }
-    __syncthreads();
-    const double sq = sqrt(sdiag[j]);
-    for (int a = tid; a < nu; a += T) {
-        double ea = 0.0, wa = 0.0, ta = 0.0;
-        if (a < n) {
-            const int src = perm[a];
-            ea = d[src];
-            ta = R[1 * ldr + src] * wsc[src];
-            wa = sq * (R[src] * wsc[src]) * ta;
-        }
-        eps_out[g * nu + a] = ea;
-        t_out[g * nu + a] = ta;
-        w_out[g * nu + a] = wa;
-        if (proj_out) proj_out[g * nu + a] = a < n ? R[(npat + 2) * ldr + perm[a]] * wsc[perm[a]] : 0.0;
-    }
-    double *P = P_out + p_off[g];
-    for (int idx = tid; idx < npat * nu; idx += T) {
-        const int r = idx / nu, a = idx - (idx / nu) * nu;
-        P[idx] = a < n ? R[(r + 2) * ldr + perm[a]] * wsc[perm[a]] : 0.0;
-    }
-    if (tid == 0) {
-        nu_eff_out[g] = n;
-        eig_status[g] = (nsw < 0 ? 1 : 0) | (bstatus[c] == 2 ? 2 : 0);
     }
 }
 
-size_t eig_apply_smem(int nu, int nr_max)
+// Rows per warp: 32, or fewer where that lets another warp share the SM and
+// fewer than two per scheduler fit (nu above about 100): the most rows per
+// turn of the fullest scheduler.
+int apply_rows(int nu)
 {
-    return (size_t)nr_max * (nu | 1) * sizeof(double) + (size_t)nu * (2 * sizeof(double) + sizeof(int));
+    int best = 32;
+    double rate = 0.0;
+    for (int rows = 32; rows >= 16; rows -= 2) {
+        const int ctas = (int)((size_t)228 * 1024 / (((size_t)rows * (nu | 1) + 1) * sizeof(double) + 1024));
+        const double x = (double)rows * ctas / ((ctas + 3) / 4);
+        if (ctas > 0 && x > rate) {
+            rate = x;
+            best = rows;
+        }
+        if (ctas >= 8) break;
+    }
+    return best;
 }
 
 template <typename VT>
 cudaError_t apply_dispatch(const DeviceMatrix &A, const KrylovBatch &b, const ColumnState &st, int64_t col0,
                            const RegionMaps *rm, const EigScratch &es, int cofs, int nb2, cudaStream_t s)
 {
-    const size_t smem = eig_apply_smem(b.nu, es.nr_max);
+    const int rows = apply_rows(b.nu);
+    const size_t smem = ((size_t)rows * (b.nu | 1) + 1) * sizeof(double);
     cudaError_t e = allow_dynamic_smem((const void *)eig_apply_kernel<VT>, smem);
     if (e != cudaSuccess) return e;
-    const int threads = std::min(kApplyThreads, (es.nr_max + 31) / 32 * 32);
-    eig_apply_kernel<VT><<<nb2, threads, smem, s>>>(
-        b.nu_eff, b.status, cofs, b.nu, b.scale, (const VT *)b.K, b.shape.m_pad, b.tinv, b.nb, b.cols, A.sdiag, A.rp,
-        A.ci, rm ? rm->reg : nullptr, rm ? rm->n_reg : 0, col0, es.D, es.E, es.V, b.Lsub, es.proj, es.nr_max, es.rot,
-        es.rcap, es.sweep, es.scap, es.nsweep, st.nu_eff, st.eps, st.w, st.t, st.P, st.p_off, st.eig_status,
-        es.proj ? es.proj_out : nullptr);
+    // nr_max bounds a subspace's rows (odd; an even number is laid out)
+    const unsigned grid = (unsigned)(((int64_t)nb2 * (es.nr_max + 1) + rows - 1) / rows);
+    eig_apply_kernel<VT><<<grid, 32, smem, s>>>(
+        b.nu_eff, cofs, nb2, b.nu, rows, b.scale, (const VT *)b.K, b.shape.m_pad, b.tinv, b.nb, b.cols, A.sdiag, A.rp,
+        A.ci, rm ? rm->reg : nullptr, rm ? rm->n_reg : 0, col0, es.D, es.E, es.V, b.Lsub, es.proj, es.rot, es.rcap,
+        es.sweep, es.scap, es.nsweep, st.w, st.t, st.P, st.p_off, es.proj ? es.proj_out : nullptr);
     return cudaGetLastError();
 }
 
@@ -677,6 +714,10 @@ cudaError_t launch_eig(const DeviceMatrix &A, const KrylovBatch &b, const Column
         if ((e = allow_dynamic_smem((const void *)eig_ql_kernel, qsmem)) != cudaSuccess) return e;
         eig_ql_kernel<<<(nb2 + nl - 1) / nl, 64, qsmem, s>>>(b.nu_eff, cofs, nb2, nu, nl, es.D, es.E, es.rot,
                                                             es.rcap, es.sweep, es.scap, es.nsweep);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        const size_t rsmem = (size_t)2 * nu * sizeof(double);
+        eig_rank_kernel<<<nb2, std::min(128, (nu + 31) / 32 * 32), rsmem, s>>>(
+            b.nu_eff, b.status, cofs, nu, col0, es.D, es.nsweep, st.nu_eff, st.eps, st.eig_status);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         e = b.prec == 0 ? apply_dispatch<double>(A, b, st, col0, rm, es, cofs, nb2, s)
                         : apply_dispatch<float>(A, b, st, col0, rm, es, cofs, nb2, s);
