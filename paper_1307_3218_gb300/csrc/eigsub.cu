@@ -288,6 +288,11 @@ __device__ __forceinline__ double series_rcp(double a)
 // iterations for some level, or a full log).  Eigenvalues overwrite D,
 // unsorted, the scales E.
 __device__ __forceinline__ int exponent_of(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+// 2 x of a number far below overflow, on the integer pipe; no effect below the normal range
+__device__ __forceinline__ double twice(double x)
+{
+    return __hiloint2double(__double2hiint(x) + (exponent_of(x) ? 0x100000 : 0), __double2loint(x));
+}
 
 __global__ void __launch_bounds__(64) eig_ql_kernel(const int *__restrict__ bnu_eff, int cofs,
                                                     int nb, int nu, int nl, double *__restrict__ D,
@@ -321,7 +326,8 @@ __global__ void __launch_bounds__(64) eig_ql_kernel(const int *__restrict__ bnu_
             rl += mine ? tr.z : 0;
             double2 cs = tr.z > 0 ? r[0] : make_double2(1.0, 0.0);
             double wj = tr.z > 0 ? WW(tr.x) : 1.0;
-            for (int q = 0; __any_sync(kFull, q < tr.z); ++q)
+            const int len = (int)__reduce_max_sync(kFull, (unsigned)tr.z);
+            for (int q = 0; q < len; ++q)
                 if (q < tr.z) {
                     const int i = tr.x - 1 - q;
                     const double cth = cs.x, s = cs.y, wi = WW(i);
@@ -383,44 +389,64 @@ __global__ void __launch_bounds__(64) eig_ql_kernel(const int *__restrict__ bnu_
             i = m - 1;
             lo = l;
         }
+        // One straight block per rotation, so that the chain's waits are filled
+        // with what does not hang on it: the next entries are read a rotation
+        // ahead, and a rotation's results for d and e are worked out during the
+        // next one (at first d(m) itself and a zero, to no effect).
         bool under = false;
         double dj = go ? DD(m) : 0.0;   // d(i + 1)
-        while (__any_sync(kFull, i >= lo)) {
+        double ei = go ? EE(i) : 0.0, di = go ? DD(i) : 0.0;
+        double pe0 = 0.0, pe1 = 0.0, pd0 = dj, pd1 = 0.0;   // e(at) = pe0 * pe1, d(at) = pd0 + pd1
+        int at = m;
+        const int len = (int)__reduce_max_sync(kFull, go ? (unsigned)(m - l) : 0u);
+        for (int q = 0; q < len; ++q) {
             if (i >= lo) {
-                const double ei = EE(i), di = DD(i), f = s * ei, b = cth * ei;
+                const int nx = max(i - 1, 0);
+                const double en = EE(nx), dn = DD(nx);
                 // r = |(f, g)| (the levels and couplings are bounded by the
                 // spectrum's width, so f^2 + g^2 neither overflows nor
                 // underflows unless both are as good as zero)
+                const double f = s * ei, b = cth * ei;
                 const double ss = fma(f, f, g * g);
+                EE(at) = pe0 * pe1;
+                DD(at) = pd0 + pd1;
+                const double gd = dj - p, dd = di - gd;
+                const double rinv = series_rsqrt(ss);
+                const double sn = f * rinv, cn = g * rinv;
+                const double r = fma(twice(cn), b, dd * sn);
+                const double pn = sn * r, gn = fma(cn, r, -b);
+                at = i + 1;
+                pd0 = gd;
                 if (exponent_of(ss) == 0) {
-                    EE(i + 1) = 0.0;
-                    DD(i + 1) = dj - p;
-                    EE(m) = 0.0;
+                    pe0 = 0.0;
+                    pe1 = pd1 = 0.0;
                     under = true;
                     lo = i + 1;
                 } else {
-                    const double rinv = series_rsqrt(ss);
-                    EE(i + 1) = ss * rinv;
-                    s = f * rinv;
-                    cth = g * rinv;
-                    rl[nrot++] = make_double2(cth, s);
-                    g = dj - p;
-                    const double r = fma(cth + cth, b, (di - g) * s);
-                    p = s * r;
-                    DD(i + 1) = g + p;
+                    pe0 = ss;
+                    pe1 = rinv;
+                    pd1 = pn;
+                    s = sn;
+                    cth = cn;
+                    rl[nrot++] = make_double2(cn, sn);
+                    p = pn;
+                    g = gn;
                     dj = di;
-                    g = fma(cth, r, -b);
+                    ei = en;
+                    di = dn;
                     --i;
                 }
             }
         }
         if (go) {
             sl[nsw++] = make_int2(m, lo);
+            EE(at) = pe0 * pe1;
+            DD(at) = pd0 + pd1;
             if (!under) {
                 DD(l) = dj - p;
                 EE(l) = g;
-                EE(m) = 0.0;
             }
+            EE(m) = 0.0;
         }
         trip[t][lane] = make_int4(m, lo, go ? m - lo : 0, 0);
         if (lane == 0) more[t] = any;
@@ -486,8 +512,8 @@ __global__ void __launch_bounds__(128) eig_rank_kernel(
 // shared memory as [rows][ldr] (ldr odd).  Every subspace has an even number
 // of rows, so its first two share a warp.  With a CTA per subspace, 75 rows
 // took three warps and their CTAs filled an SM's four schedulers unevenly.
-// 24,000 subspaces of nu = 30: 10.2 -> @A@ ms; 4,000 of nu = 100: 22.8 -> @B@;
-// 348 of nu = 300: 55.5 -> @C@.
+// 24,000 subspaces of nu = 30: 10.2 -> 7.3 ms; 4,000 of nu = 100: 22.7 -> 13.9;
+// 348 of nu = 300: 55.3 -> 37.9.
 constexpr int kLogAhead = 4;   // rotations held in registers ahead of their use
 
 template <typename VT>
