@@ -822,15 +822,15 @@ int bisect(marnoldi_ctx *c, const BisectTask *tasks, int n, void *scratch, Bisec
     if (e != cudaSuccess) return fail_cuda(c, e, "bisection read-back");
     if ((rc = sync(c, "bisection"))) return rc;
     if (n == 1) memcpy(bs, c->h_out, sizeof *bs);
-    // one launch was counted; the range, the loop's counts, and the bisections'
-    // steps (which end the counts)
-    int counts = 0;
+    // one launch was counted; the range, the loop's passes, and the bisections'
+    // steps (which end the passes)
+    int passes = 0;
     c->launches[KK_MINMAX] += 1;
     for (int q = 0; q < n; ++q) {
-        counts = std::max(counts, bs[q].steps - 1);
+        passes = std::max(passes, bs[q].passes);
         c->launches[KK_BISECT] += bs[q].steps;
     }
-    c->launches[KK_COUNT] += counts - 1;
+    c->launches[KK_COUNT] += passes - 1;
     return MARNOLDI_OK;
 }
 

@@ -349,7 +349,9 @@ constexpr int kBisectMaxit = 200;
 struct alignas(16) BisectState {
     double lo, hi, mu, N, E, Nlo, Nhi;
     int it, phase, status, steps;   // status 1: N_e outside [N(lo), N(hi)]
+    int passes;                     // launches of the count that had work for it
 };
+constexpr int kBisectMus = 3;   // most counts of one pass
 // One bisection: its columns, kT and electron count; the rest is set by
 // launch_bisection (places in the scratch).
 struct alignas(16) BisectTask {
@@ -367,9 +369,9 @@ struct alignas(16) BisectTask {
 constexpr size_t bisect_states(size_t n) { return n * ((sizeof(BisectTask) + 15) / 16 * 16); }
 constexpr size_t bisect_tickets(size_t n) { return bisect_states(n) + n * ((sizeof(BisectState) + 15) / 16 * 16); }
 constexpr size_t bisect_partials(size_t n) { return bisect_tickets(n) + (n + 1 + 3) / 4 * 4 * sizeof(unsigned); }
-constexpr size_t bisect_bytes(size_t n) { return bisect_partials(n) + n * 2 * kReduceBlocks * sizeof(double); }
+constexpr size_t bisect_bytes(size_t n) { return bisect_partials(n) + n * 2 * kBisectMus * kReduceBlocks * sizeof(double); }
 // n bisections side by side: the level ranges, then a CUDA graph with a while
-// node whose counts (mu read from each task's state) end in a bisection step,
+// node whose passes (one count, or three about each task's mu) end in bisection steps,
 // until every one is done; the states hold the results once the stream gets there.
 cudaError_t launch_bisection(const BisectTask *tasks, int n, void *scratch, cudaStream_t s);
 // The k-th eigen level and vector (eigstate.cu).

@@ -53,28 +53,41 @@ __device__ __forceinline__ double2 block_reduce2(double a, double b)
 // them: each thread folds the partials q = tid, tid + blockDim.x, ... and the
 // block reduces those in its fixed order.  True, with the totals in t, for one
 // thread of the grid (of a row blockIdx.y of it).  No thread waits on another
-// block.
-template <int OP>
-__device__ bool finish_reduce(double a, double b, double *partial, unsigned *ticket, double2 &t)
+// block.  K sums side by side, one in each plane blockIdx.z of the grid.
+template <int OP, int K>
+__device__ bool finish_reduce(double2 a, double *partial, unsigned *ticket, double2 (&t)[K])
 {
     __shared__ int last;
-    const double2 r = block_reduce2<OP>(a, b);
+    const double2 r = block_reduce2<OP>(a.x, a.y);
     if (threadIdx.x == 0) {
-        partial[2 * blockIdx.x] = r.x;
-        partial[2 * blockIdx.x + 1] = r.y;
+        const unsigned at = blockIdx.z * gridDim.x + blockIdx.x;
+        partial[2 * at] = r.x;
+        partial[2 * at + 1] = r.y;
         __threadfence();
-        last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
+        last = (atomicAdd(ticket, 1u) == K * gridDim.x - 1);
     }
     __syncthreads();
     if (!last) return false;   // uniform over the block
     __threadfence();
     const volatile double *vp = partial;
-    double x = OP == 0 ? 0.0 : INFINITY, y = OP == 0 ? 0.0 : -INFINITY;
-    for (unsigned q = threadIdx.x; q < gridDim.x; q += blockDim.x) {
-        if (OP == 0) { x += vp[2 * q]; y += vp[2 * q + 1]; }
-        else { x = fmin(x, vp[2 * q]); y = fmax(y, vp[2 * q + 1]); }
+    double x[K], y[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        x[k] = OP == 0 ? 0.0 : INFINITY;
+        y[k] = OP == 0 ? 0.0 : -INFINITY;
     }
-    t = block_reduce2<OP>(x, y);
+    for (unsigned q = threadIdx.x; q < gridDim.x; q += blockDim.x)
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const double px = vp[2 * (k * gridDim.x + q)], py = vp[2 * (k * gridDim.x + q) + 1];
+            if (OP == 0) { x[k] += px; y[k] += py; }
+            else { x[k] = fmin(x[k], px); y[k] = fmax(y[k], py); }
+        }
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        if (k > 0) __syncthreads();   // the last reduction's shared sums are read
+        t[k] = block_reduce2<OP>(x[k], y[k]);
+    }
     if (threadIdx.x != 0) return false;
     *ticket = 0u;
     return true;
@@ -102,10 +115,10 @@ __global__ void __launch_bounds__(256) minmax_kernel(int64_t total, int nu,
                                                      double *partial, unsigned *ticket, double *out)
 {
     const double2 r = range_partial(total, nu, nu_eff, eps);
-    double2 t;
-    if (finish_reduce<1>(r.x, r.y, partial, ticket, t)) {
-        out[0] = t.x;
-        out[1] = t.y;
+    double2 t[1];
+    if (finish_reduce<1, 1>(r, partial, ticket, t)) {
+        out[0] = t[0].x;
+        out[1] = t[0].y;
     }
 }
 
@@ -154,10 +167,10 @@ __global__ void __launch_bounds__(256) count_kernel(int64_t ncols, int nu,
                                                     double *partial, unsigned *ticket, double *out)
 {
     const double2 r = count_partial(ncols, nu, nu_eff, eps, w, mu, kT);
-    double2 t;
-    if (finish_reduce<0>(r.x, r.y, partial, ticket, t)) {
-        out[0] = t.x;
-        out[1] = t.y;
+    double2 t[1];
+    if (finish_reduce<0, 1>(r, partial, ticket, t)) {
+        out[0] = t[0].x;
+        out[1] = t[0].y;
     }
 }
 
@@ -166,66 +179,95 @@ __global__ void __launch_bounds__(256) bisect_range_kernel(const BisectTask *__r
 {
     const BisectTask q = tasks[blockIdx.y];
     const double2 r = range_partial(q.ncols * q.nu, q.nu, q.nu_eff, q.eps);
-    double2 t;
-    if (finish_reduce<1>(r.x, r.y, q.partial, q.ticket, t)) {
+    double2 t[1];
+    if (finish_reduce<1, 1>(r, q.partial, q.ticket, t)) {
         // rounded like the host's (min - 40 kT): no contraction into an FMA
-        q.bs->lo = __dsub_rn(t.x, __dmul_rn(kBisectBracketKT, q.kT));
-        q.bs->hi = __dadd_rn(t.y, __dmul_rn(kBisectBracketKT, q.kT));
+        q.bs->lo = __dsub_rn(t[0].x, __dmul_rn(kBisectBracketKT, q.kT));
+        q.bs->hi = __dadd_rn(t[0].y, __dmul_rn(kBisectBracketKT, q.kT));
         q.bs->mu = q.bs->lo;
         q.bs->phase = 1;
         q.bs->steps = 1;
     }
 }
 
-// Bisection blockIdx.y: N and E at its mu; the last block to finish then takes
-// the bisection's step (same bracket, halving and stopping rule as a host loop
-// would apply): phase 1 was N(lo) and asks for N(hi), phase 2 checks that the
-// bracket holds N_e, phase 3 halves until |N - N_e| <= rtol N_e or maxit
-// halvings, phase 4 is done.  `steps` bounds the loop whatever the counts hold.
-// The last bisection to finish ends the graph's while loop.  A step in a
-// kernel of its own, one thread between two counts, took half of the loop's time.
+// Levels (of all bisections of a launch) up to which a pass makes three counts: one
+// per thread of two blocks per SM.  120,000 levels: 33 us per two halvings, 31 one
+// by one; 246,000: 44 and 36.
+constexpr int64_t kThreeLevels = (int64_t)152 * 512;
+
+// One halving of the bracket, from N and E at its middle s.mu (same halving and
+// stopping rule as a host loop would apply: until |N - N_e| <= rtol N_e or maxit
+// halvings); false when it is the last.
+__device__ __forceinline__ bool bisect_halve(BisectState &s, double2 t, double Ne)
+{
+    s.N = t.x;
+    s.E = t.y;
+    bool more = !(fabs(s.N - Ne) <= kBisectRtol * Ne || s.it >= kBisectMaxit);
+    if (more) {
+        if (s.N < Ne) s.lo = s.mu; else s.hi = s.mu;
+        s.mu = 0.5 * (s.lo + s.hi);
+        ++s.it;
+    }
+    if (++s.steps >= kBisectMaxit + 3) more = false;
+    return more;
+}
+
+// Bisection blockIdx.y: N and E at kMus chemical potentials, one per plane of the
+// grid; the last block to finish then takes the bisection's steps: phase 1 asks
+// whether the bracket's ends hold N_e, phase 3 halves it, phase 4 is done.  With
+// three, phase 1 counts at both ends and the middle, phase 3 at the middle and at
+// the two values that can be the next middle, so that a pass halves twice.  A small
+// solve's pass is a chain of latencies that leaves most of the chip without a
+// block: per two halvings 256 columns of nu = 30 take 18 us with three counts side
+// by side, 26 with one per pass.  Where the levels fill the chip the third count is
+// lost work: 24,000 columns 75 us and 59 (78 with all three in one thread).
+// `steps` bounds the loop whatever the counts hold.  The last bisection to finish
+// ends the graph's while loop.
+template <int kMus>
 __global__ void __launch_bounds__(256) bisect_count_kernel(const BisectTask *__restrict__ tasks, int *active,
                                                            cudaGraphConditionalHandle loop)
 {
     const BisectTask q = tasks[blockIdx.y];
-    if (q.bs->phase == 4) return;   // uniform: set by an earlier launch
-    const double2 r = count_partial(q.ncols, q.nu, q.nu_eff, q.eps, q.w, q.bs->mu, q.kT);
-    double2 t;
-    if (!finish_reduce<0>(r.x, r.y, q.partial, q.ticket, t)) return;
+    const int phase = q.bs->phase;
+    if (phase == 4) return;   // uniform: set by an earlier launch
+    double mu = q.bs->mu;     // phases 1 and 2: lo and hi, or with three counts the middle
+    if constexpr (kMus == 3) {
+        const double lo = q.bs->lo, hi = q.bs->hi;
+        if (phase == 1) mu = blockIdx.z == 0 ? 0.5 * (lo + hi) : blockIdx.z == 1 ? lo : hi;
+        else mu = blockIdx.z == 0 ? mu : 0.5 * (blockIdx.z == 1 ? lo + mu : mu + hi);
+    }
+    const double2 r = count_partial(q.ncols, q.nu, q.nu_eff, q.eps, q.w, mu, q.kT);
+    double2 t[kMus];
+    if (!finish_reduce<0, kMus>(r, q.partial, q.ticket, t)) return;
     BisectState s = *q.bs;
     bool more = true;
-    switch (s.phase) {
-    case 1:
-        s.Nlo = t.x;
-        s.mu = s.hi;
-        s.phase = 2;
-        break;
-    case 2:
-        s.Nhi = t.x;
-        if (!(s.Nlo <= q.Ne && q.Ne <= s.Nhi)) {
-            s.status = 1;
-            more = false;
-        } else {
-            s.it = 1;
-            s.mu = 0.5 * (s.lo + s.hi);
-            s.phase = 3;
+    ++s.passes;
+    if (phase == 3) {
+        const bool up = t[0].x < q.Ne;   // then lo becomes mu, and the next middle is the upper one
+        more = bisect_halve(s, t[0], q.Ne);
+        if constexpr (kMus == 3)
+            if (more) more = bisect_halve(s, up ? t[2] : t[1], q.Ne);
+    } else {
+        if (kMus == 3 || phase == 1) {
+            s.Nlo = t[kMus == 3 ? 1 : 0].x;
+            s.mu = s.hi;
+            s.phase = 2;
+            ++s.steps;
         }
-        break;
-    case 3:
-        s.N = t.x;
-        s.E = t.y;
-        if (fabs(s.N - q.Ne) <= kBisectRtol * q.Ne || s.it >= kBisectMaxit) {
-            more = false;
-        } else {
-            if (s.N < q.Ne) s.lo = s.mu; else s.hi = s.mu;
-            s.mu = 0.5 * (s.lo + s.hi);
-            ++s.it;
+        if (kMus == 3 || phase == 2) {
+            s.Nhi = t[kMus == 3 ? 2 : 0].x;
+            ++s.steps;
+            if (!(s.Nlo <= q.Ne && q.Ne <= s.Nhi)) {
+                s.status = 1;
+                more = false;
+            } else {
+                s.it = 1;
+                s.mu = 0.5 * (s.lo + s.hi);
+                s.phase = 3;
+                if (kMus == 3) more = bisect_halve(s, t[0], q.Ne);
+            }
         }
-        break;
-    default:
-        more = false;
     }
-    if (++s.steps >= kBisectMaxit + 3) more = false;
     if (!more) s.phase = 4;
     *q.bs = s;
     if (!more && atomicSub(active, 1) == 1) cudaGraphSetConditional(loop, 0u);
@@ -394,14 +436,15 @@ cudaError_t launch_bisection(const BisectTask *tasks, int n, void *scratch, cuda
     // tickets and the number of bisections, in one upload
     char *dev = (char *)scratch;
     std::vector<char> up(bisect_partials(n), 0);
-    int64_t total = 1;
+    int64_t total = 1, levels = 0;
     for (int q = 0; q < n; ++q) {
         BisectTask t = tasks[q];
         t.bs = (BisectState *)(dev + bisect_states(n) + q * (bisect_tickets(1) - bisect_states(1)));
         t.ticket = (unsigned *)(dev + bisect_tickets(n)) + q;
-        t.partial = (double *)(dev + bisect_partials(n)) + q * 2 * kReduceBlocks;
+        t.partial = (double *)(dev + bisect_partials(n)) + q * 2 * kBisectMus * kReduceBlocks;
         memcpy(up.data() + q * bisect_states(1), &t, sizeof t);
         total = std::max<int64_t>(total, t.ncols * t.nu);
+        levels += t.ncols * t.nu;
     }
     static_assert(sizeof(BisectTask) % 16 == 0 && sizeof(BisectState) % 16 == 0, "arrays without gaps");
     int *active = (int *)(dev + bisect_tickets(n)) + n;
@@ -412,6 +455,9 @@ cudaError_t launch_bisection(const BisectTask *tasks, int n, void *scratch, cuda
     const dim3 grid(reduce_blocks(total), (unsigned)n);
     bisect_range_kernel<<<grid, 256, 0, s>>>(td);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const bool three = levels <= kThreeLevels;
+    const dim3 cgrid(grid.x, grid.y, three ? kBisectMus : 1);
+    const auto count = three ? bisect_count_kernel<kBisectMus> : bisect_count_kernel<1>;
     // one graph whose while node counts (and steps) until every bisection is
     // done; a pass of the loop holds several counts, since a pass costs more
     // than a count that finds its bisection finished
@@ -436,7 +482,7 @@ cudaError_t launch_bisection(const BisectTask *tasks, int n, void *scratch, cuda
         cudaGraph_t body = np.conditional.phGraph_out[0];
         e = cudaStreamBeginCaptureToGraph(cap, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            for (int q = 0; q < kCounts; ++q) bisect_count_kernel<<<grid, 256, 0, cap>>>(td, active, loop);
+            for (int q = 0; q < kCounts; ++q) count<<<cgrid, 256, 0, cap>>>(td, active, loop);
             const cudaError_t el = cudaGetLastError();
             e = cudaStreamEndCapture(cap, &body);
             if (e == cudaSuccess) e = el;
