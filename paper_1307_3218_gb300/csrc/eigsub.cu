@@ -8,27 +8,27 @@
 //
 // H_sub is reduced to tridiagonal form T = Q^T H_sub Q by Householder
 // reflections and T = Z Lambda Z^T by the implicit-shift QL algorithm
-// (Bowdler, Martin, Reinsch & Wilkinson 1968), so R V = (R Q) Z.  Three
+// (Bowdler, Martin, Reinsch & Wilkinson 1968), so R V = (R Q) Z.  Four
 // kernels per chunk of subspaces:
 //   eig_tridiag_kernel  one CTA per subspace: the reflections, applied to H_sub;
 //                       writes d, e and the reflectors
 //   eig_ql_kernel       one LANE per subspace: the QL recurrence, a serial chain
-//                       of FP64 divisions and square roots per subspace.
-//                       Every rotation is logged, as the two coefficients of
-//                       a fast plane rotation, and every sweep's index range.
-//   eig_apply_kernel    one CTA per subspace, a thread per row of R: the
-//                       reflectors, then the rotations of the log; the levels
-//                       are ranked and eps, w_a = sqrt(S_jj) (R V)[0][a] (R V)[1][a],
-//                       t and P_j are written in ascending order of eps.
-// All three are bound by FP64 instructions (64 cycles each on a warp's
-// scheduler): their sum where many warps run, else the longest chain.  The reflections used
-// to reach R in the first kernel, whose other threads waited and whose shared
-// memory then held one CTA per SM (nu = 100), and a rotation took four FP64
-// instructions per row.  Per solve, before and after (tridiagonalisation, QL,
-// rows): 24,000 subspaces of nu = 30: 13.9 + 2.1 + 12.0 -> 5.2 + 2.3 + 10.2 ms;
-// 4,000 of nu = 100: 60.6 + 16.7 + 23.6 -> 16.5 + 11.3 + 22.8; 348 of nu = 300:
-// 91.5 + 159.9 + 54.7 -> 36.8 + 88.9 + 55.5; 256 of nu = 30: 0.30 + 1.66 + 0.27 ->
-// 0.24 + 1.13 + 0.25.
+//                       of FP64 operations per subspace.  Every rotation is
+//                       logged, as the two coefficients of a fast plane
+//                       rotation, and every sweep's index range.
+//   eig_rank_kernel     one CTA per subspace: the levels in ascending order
+//   eig_apply_kernel    one warp per 32 rows of R, packed over the subspaces:
+//                       L^-T, the reflectors, then the rotations of the log;
+//                       w_a = sqrt(S_jj) (R V)[0][a] (R V)[1][a], t and P_j are
+//                       written in ascending order of eps.
+// All but the ranking are bound by FP64 instructions (64 cycles each on a warp's
+// scheduler): their sum where many warps run, else the longest chain.  The
+// reflections used to reach R in the first kernel, whose other threads waited and
+// whose shared memory then held one CTA per SM (nu = 100), and a rotation took four
+// FP64 instructions per row.  Per solve, then and now (tridiagonalisation, QL, rows):
+// 24,000 subspaces of nu = 30: 13.9 + 2.1 + 12.0 -> 5.2 + 2.0 + 7.3 ms; 4,000 of
+// nu = 100: 60.6 + 16.7 + 23.6 -> 16.5 + 9.8 + 13.9; 348 of nu = 300: 91.5 + 159.9 +
+// 54.7 -> 36.8 + 77.0 + 37.7; 256 of nu = 30: 0.30 + 1.66 + 0.27 -> 0.24 + 1.02 + 0.25.
 #include "internal.h"
 
 #include <math_constants.h>
@@ -266,8 +266,9 @@ __device__ __forceinline__ double series_rcp(double a)
 //
 // What bounds it: one warp's FP64 instruction holds its scheduler's FP64 unit
 // for 64 cycles whatever the number of active lanes, and a subspace's rotations
-// are one chain; so the time is that chain's count of FP64 instructions (20 per
-// rotation).  Tests that need no FP64 arithmetic (is e(m) negligible, which of
+// are one chain; so the time is that chain's count of FP64 instructions (19 per
+// rotation, 1,216 cycles; about 1,500 are measured, the rest is the latency of the
+// chain through f, g and the square root).  Tests that need no FP64 arithmetic (is e(m) negligible, which of
 // |c|, |s| is larger) are made on the exponents, and what the chain does not
 // wait for runs in the CTA's second warp, on another scheduler: it follows one
 // sweep behind and turns each logged rotation into the form the rows use.

@@ -364,7 +364,9 @@ __global__ void __launch_bounds__(32 * W, (sizeof(VT) == 4 ? 20 : 16) / W) spmm_
 // kernel with the stored vectors streamed by a producer warp's bulk copies, two
 // CTAs per SM, took 227.7: it read each vector three times and its 16 consumer
 // warps per SM waited for their own arithmetic's latency.  More ring stages hold
-// back CTAs: 161.4 ms with four, 165.4 with five.
+// back CTAs: 161.4 ms with four, 165.4 with five.  The input panel of the next
+// product, written too since (see the SpMM), added 2.3 ms to the first figure, 0.7 to
+// the 2,048 columns and 10 to the last.
 
 // Four entries of a vector: FP32 as two packed pairs, FP64 as four doubles.
 template <typename VT> struct Quad;
