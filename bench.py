@@ -269,6 +269,15 @@ def gs_algorithmic_support(nu: int, tcnt, vbytes: int):
     return vals * vbytes, 2.0 * fmas
 
 
+def gs_two_reads(nu: int, by: float, tcnt, m: int, vbytes: int, ncols: int):
+    """The bytes `by` of gs_algorithmic_support (of gs_algorithmic when tcnt is None), which count a
+    third read of every stored vector, for the kernel's two: w_i feeds a_i and the subtraction at once."""
+    if tcnt is None:
+        return by - (nu * (nu - 1) // 2) * m * vbytes * ncols
+    E = 32.0 * np.asarray(tcnt).sum(axis=0)
+    return by - sum((nu - 1 - i) * E[i + 1] for i in range(nu - 1)) * vbytes
+
+
 def spmm_algorithmic(nu: int, m: int, nnzb: int, nbr: int, vbytes: int, ncols: int):
     """Per column and application: read x, write y (m values each); flops 2 * 16 nnzb."""
     apps = 2 * nu - 1
@@ -529,6 +538,7 @@ def main():
     if dom == "gs":
         by, fl = (gs_algorithmic_support(args.nu, tcnt, vb) if tcnt is not None
                   else gs_algorithmic(args.nu, m_vec, vb, ncols))
+        by = gs_two_reads(args.nu, by, tcnt, m_vec, vb, ncols)
     elif dom in ("spmm_H", "spmm_S", "spmm_HS"):
         by, fl = spmm_algorithmic(args.nu, m_vec, t.nnzb, t.n_block_rows, vb, ncols)
         if dom != "spmm_HS":
@@ -654,6 +664,7 @@ def main():
                 # the Gram-Schmidt kernel's HBM fraction at nu = 100 (support bytes)
                 tc100 = support_counts(t, cl, nu_x, column_m_pad(t.M))
                 by100, _ = gs_algorithmic_support(nu_x, tc100, 4)
+                by100 = gs_two_reads(nu_x, by100, tc100, t.M, 4, len(cl))
                 gs_n, gs_ms = rx["stats"]["gs"]
                 ach100 = by100 * 3 / (gs_ms / 1e3) / 1e9
                 pk = peaks.get("hbm_gbs", 6800.0)
