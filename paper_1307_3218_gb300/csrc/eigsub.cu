@@ -367,9 +367,10 @@ __global__ void __launch_bounds__(64) eig_ql_kernel(const int *__restrict__ bnu_
         while (!done && !go) {
             for (m = l; m < n - 1; ++m) {
                 // |e| > eps (|d| + |d'|) for sure when e's exponent is above the
-                // larger of the others' less 50
+                // larger of the others' less 50 and e is no zero or subnormal
+                // number (whose exponent field, 0, says nothing)
                 const double em = EE(m), d0 = DD(m), d1 = DD(m + 1);
-                if (exponent_of(em) > max(exponent_of(d0), exponent_of(d1)) - 50) continue;
+                if (exponent_of(em) > max(max(exponent_of(d0), exponent_of(d1)) - 50, 0)) continue;
                 if (fabs(em) <= DBL_EPSILON * (fabs(d0) + fabs(d1))) break;
             }
             if (m == l) {

@@ -1,0 +1,47 @@
+// Host entries for the tests of the eigensolver's device code, one translation unit with it:
+// eig_probe_ql runs the batched QL kernel on tridiagonal matrices given from the host.
+#include "eigsub.cu"
+
+#include <vector>
+
+namespace marnoldi {
+cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+}  // namespace marnoldi
+
+using namespace marnoldi;
+
+// nb matrices of order n: d [nb][n] (the levels on return), e [nb][n] (the column scales on
+// return), nsweep [nb]; nl matrices per warp.  Returns a CUDA error code.
+extern "C" int eig_probe_ql(int nb, int n, int nl, double *d, double *e, int *nsweep)
+{
+    const int64_t rcap = (int64_t)8 * n * n, scap = (int64_t)40 * n;
+    const size_t vals = (size_t)nb * n * sizeof(double);
+    int *nu_eff = nullptr, *ns = nullptr;
+    double *D = nullptr, *E = nullptr;
+    double2 *rot = nullptr;
+    int2 *sweep = nullptr;
+    const std::vector<int> order(nb, n);
+    cudaError_t err = cudaMalloc(&nu_eff, nb * sizeof(int));
+    if (!err) err = cudaMalloc(&ns, nb * sizeof(int));
+    if (!err) err = cudaMalloc(&D, vals);
+    if (!err) err = cudaMalloc(&E, vals);
+    if (!err) err = cudaMalloc(&rot, nb * rcap * sizeof(double2));
+    if (!err) err = cudaMalloc(&sweep, nb * scap * sizeof(int2));
+    if (!err) err = cudaMemcpy(nu_eff, order.data(), nb * sizeof(int), cudaMemcpyHostToDevice);
+    if (!err) err = cudaMemcpy(D, d, vals, cudaMemcpyHostToDevice);
+    if (!err) err = cudaMemcpy(E, e, vals, cudaMemcpyHostToDevice);
+    const size_t smem = (size_t)3 * n * nl * sizeof(double);
+    if (!err) err = allow_dynamic_smem((const void *)eig_ql_kernel, smem);
+    if (!err) {
+        eig_ql_kernel<<<(nb + nl - 1) / nl, 64, smem>>>(nu_eff, 0, nb, n, nl, D, E, rot, rcap, sweep, scap, ns);
+        err = cudaGetLastError();
+    }
+    if (!err) err = cudaMemcpy(d, D, vals, cudaMemcpyDeviceToHost);
+    if (!err) err = cudaMemcpy(e, E, vals, cudaMemcpyDeviceToHost);
+    if (!err) err = cudaMemcpy(nsweep, ns, nb * sizeof(int), cudaMemcpyDeviceToHost);
+    for (void *p : {(void *)nu_eff, (void *)ns, (void *)D, (void *)E, (void *)rot, (void *)sweep}) cudaFree(p);
+    return (int)err;
+}
