@@ -43,6 +43,7 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kTriThreads = 256;    // most threads of the tridiagonalisation
 constexpr int kQlMaxIter = 30;      // QL iterations per eigenvalue
 constexpr int kQlWarps = 152;       // one QL warp per SM
+constexpr int kScaleBits = 930;     // a column scale below 2^-930 counts as no convergence
 
 __device__ __forceinline__ double warp_sum(double s)
 {
@@ -295,6 +296,7 @@ __device__ __forceinline__ double twice(double x)
     return __hiloint2double(__double2hiint(x) + (exponent_of(x) ? 0x100000 : 0), __double2loint(x));
 }
 
+template <int kLostBits>
 __global__ void __launch_bounds__(64) eig_ql_kernel(const int *__restrict__ bnu_eff, int cofs,
                                                     int nb, int nu, int nl, double *__restrict__ D,
                                                     double *__restrict__ E,
@@ -318,7 +320,6 @@ __global__ void __launch_bounds__(64) eig_ql_kernel(const int *__restrict__ bnu_
 #define WW(i) w[(i) * nl]
     if (!first) {
         for (int i = 0; i < n; ++i) WW(i) = 1.0;
-        bool bad = false;
         for (int t = 0;; t ^= 1) {
             __syncthreads();   // sweep t is logged
             if (!more[t]) break;
@@ -341,13 +342,17 @@ __global__ void __launch_bounds__(64) eig_ql_kernel(const int *__restrict__ bnu_
                     r[q] = make_double2(alpha, cf ? beta : -beta);
                     WW(i + 1) = den * wq;
                     wj = cf ? den * wp : -(den * wp);
-                    bad |= exponent_of(wj) < 1023 - 930;
                 }
             if (tr.z > 0) WW(tr.x - tr.z) = wj;
         }
         if (mine) {
-            for (int i = 0; i < n; ++i) E[(int64_t)sc * nu + i] = WW(i);
-            fail[lane] = bad;
+            bool lost = false;   // rotations only shrink the scales: the last ones tell
+            for (int i = 0; i < n; ++i) {
+                const double wi = WW(i);
+                E[(int64_t)sc * nu + i] = wi;
+                lost |= exponent_of(wi) < 1023 - kLostBits;
+            }
+            fail[lane] = lost;
         }
         __syncthreads();
         return;
@@ -739,8 +744,8 @@ cudaError_t launch_eig(const DeviceMatrix &A, const KrylovBatch &b, const Column
         int nl = 3 * (size_t)nu * 32 * sizeof(double) > (size_t)227 * 1024 ? 16 : 32;
         while (nl > 1 && (nb2 + nl / 2 - 1) / (nl / 2) <= kQlWarps) nl /= 2;
         const size_t qsmem = (size_t)3 * nu * nl * sizeof(double);
-        if ((e = allow_dynamic_smem((const void *)eig_ql_kernel, qsmem)) != cudaSuccess) return e;
-        eig_ql_kernel<<<(nb2 + nl - 1) / nl, 64, qsmem, s>>>(b.nu_eff, cofs, nb2, nu, nl, es.D, es.E, es.rot,
+        if ((e = allow_dynamic_smem((const void *)eig_ql_kernel<kScaleBits>, qsmem)) != cudaSuccess) return e;
+        eig_ql_kernel<kScaleBits><<<(nb2 + nl - 1) / nl, 64, qsmem, s>>>(b.nu_eff, cofs, nb2, nu, nl, es.D, es.E, es.rot,
                                                             es.rcap, es.sweep, es.scap, es.nsweep);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         const size_t rsmem = (size_t)2 * nu * sizeof(double);

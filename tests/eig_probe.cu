@@ -13,9 +13,8 @@ cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes)
 
 using namespace marnoldi;
 
-// nb matrices of order n: d [nb][n] (the levels on return), e [nb][n] (the column scales on
-// return), nsweep [nb]; nl matrices per warp.  Returns a CUDA error code.
-extern "C" int eig_probe_ql(int nb, int n, int nl, double *d, double *e, int *nsweep)
+template <int kLostBits>
+static int ql(int nb, int n, int nl, double *d, double *e, int *nsweep)
 {
     const int64_t rcap = (int64_t)8 * n * n, scap = (int64_t)40 * n;
     const size_t vals = (size_t)nb * n * sizeof(double);
@@ -34,9 +33,10 @@ extern "C" int eig_probe_ql(int nb, int n, int nl, double *d, double *e, int *ns
     if (!err) err = cudaMemcpy(D, d, vals, cudaMemcpyHostToDevice);
     if (!err) err = cudaMemcpy(E, e, vals, cudaMemcpyHostToDevice);
     const size_t smem = (size_t)3 * n * nl * sizeof(double);
-    if (!err) err = allow_dynamic_smem((const void *)eig_ql_kernel, smem);
+    if (!err) err = allow_dynamic_smem((const void *)eig_ql_kernel<kLostBits>, smem);
     if (!err) {
-        eig_ql_kernel<<<(nb + nl - 1) / nl, 64, smem>>>(nu_eff, 0, nb, n, nl, D, E, rot, rcap, sweep, scap, ns);
+        eig_ql_kernel<kLostBits><<<(nb + nl - 1) / nl, 64, smem>>>(nu_eff, 0, nb, n, nl, D, E, rot, rcap, sweep, scap,
+                                                                   ns);
         err = cudaGetLastError();
     }
     if (!err) err = cudaMemcpy(d, D, vals, cudaMemcpyDeviceToHost);
@@ -44,4 +44,18 @@ extern "C" int eig_probe_ql(int nb, int n, int nl, double *d, double *e, int *ns
     if (!err) err = cudaMemcpy(nsweep, ns, nb * sizeof(int), cudaMemcpyDeviceToHost);
     for (void *p : {(void *)nu_eff, (void *)ns, (void *)D, (void *)E, (void *)rot, (void *)sweep}) cudaFree(p);
     return (int)err;
+}
+
+// nb matrices of order n: d [nb][n] (the levels on return), e [nb][n] (the column scales on
+// return), nsweep [nb]; nl matrices per warp; a scale counts as lost below 2^-bits (0: the
+// library's bound).  Returns a CUDA error code.
+extern "C" int eig_probe_ql(int nb, int n, int nl, int bits, double *d, double *e, int *nsweep)
+{
+    switch (bits) {
+    case 0: return ql<kScaleBits>(nb, n, nl, d, e, nsweep);
+    case 2: return ql<2>(nb, n, nl, d, e, nsweep);
+    case 4: return ql<4>(nb, n, nl, d, e, nsweep);
+    case 8: return ql<8>(nb, n, nl, d, e, nsweep);
+    default: return -1;
+    }
 }

@@ -30,11 +30,12 @@ def _ptr(a):
     return a.ctypes.data_as(C.c_void_p)
 
 
-def _ql(probe, d, e, nl=4):
-    """Levels, column scales and sweep counts of the tridiagonal matrices (d, e), e of d's length."""
+def _ql(probe, d, e, nl=4, bits=0):
+    """Levels, column scales and sweep counts of the tridiagonal matrices (d, e), e of d's length; a
+    scale below 2^-bits counts as lost (0: the library's bound)."""
     d, e = np.array(d, float), np.array(e, float)
     ns = np.zeros(d.shape[0], np.int32)
-    assert probe.eig_probe_ql(d.shape[0], d.shape[1], nl, _ptr(d), _ptr(e), _ptr(ns)) == 0
+    assert probe.eig_probe_ql(d.shape[0], d.shape[1], nl, bits, _ptr(d), _ptr(e), _ptr(ns)) == 0
     return d, e, ns
 
 
@@ -51,3 +52,17 @@ def test_negligible_couplings_of_zero_levels(probe, d, e):
     assert np.all(ns >= 0)
     for row in lv:
         np.testing.assert_allclose(np.sort(row), want, rtol=0, atol=8 * np.finfo(float).eps * np.abs(want).max())
+
+
+@pytest.mark.parametrize("bits", [2, 4, 8])
+@pytest.mark.parametrize("n", [2, 5, 20, 60])
+def test_every_lost_scale_is_reported(probe, n, bits):
+    """The scales only shrink, so a subspace has lost one exactly when one of those it ends with lies
+    below the bound, in whichever column: with a bound that ordinary matrices reach."""
+    rng = np.random.default_rng(n)
+    d, e = rng.standard_normal((256, n)), rng.standard_normal((256, n))
+    _, w, ns = _ql(probe, d, e, nl=32, bits=bits)
+    w0, ns0 = _ql(probe, d, e, nl=32)[1:]
+    np.testing.assert_array_equal(w, w0)
+    assert np.all(ns0 >= 0)
+    np.testing.assert_array_equal(ns < 0, np.abs(w).min(axis=1) < 2.0 ** -bits)
