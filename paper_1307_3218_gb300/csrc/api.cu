@@ -1618,13 +1618,14 @@ int marnoldi_solve(marnoldi_ctx *c, const int64_t *columns, int64_t ncols, int n
                                    members ? c->mem_ne[m] : electron_count);
         }
         // scratch: the context's for one bisection; the members' side by side
-        // in the batch workspace, which nothing needs any more
-        const size_t need = bisect_bytes(nmem);
-        DeviceBuffer own(c, nmem > 1 && need > c->ws_bytes ? need : 0);
-        void *scratch = nmem == 1 ? c->d_bisect : own.get() ? (void *)own.get() : c->ws;
-        if (nmem > 1 && need > c->ws_bytes && !own.get())
-            return fail(c, MARNOLDI_ENOMEM, "device allocation for the members' bisections failed");
-        if ((rc = bisect(c, tasks.data(), (int)nmem, scratch, bs.data()))) return rc;
+        // in the batch workspace, which nothing needs any more, as many at a
+        // time as it holds (all, unless the batches were very small)
+        size_t fit = nmem;
+        while (fit > 1 && bisect_bytes(fit) > c->ws_bytes) fit = (fit + 1) / 2;
+        for (size_t m = 0; m < nmem; m += fit) {
+            const int k = (int)std::min(fit, nmem - m);
+            if ((rc = bisect(c, tasks.data() + m, k, k == 1 ? c->d_bisect : c->ws, bs.data() + m))) return rc;
+        }
         for (size_t m = 0; m < nmem; ++m) {
             if (bs[m].status == 1)
                 return fail(c, MARNOLDI_ENOCONV, "electron count %.6g outside [N(lo) = %.6g, N(hi) = %.6g]%s",
