@@ -664,13 +664,16 @@ struct SolvePlan {
     size_t oTr, oPn, oED, oEE, oEV, oERot, oESw, oENs, oEA, ws_bytes;
 };
 
-// Workspace bytes per batch column, for the default batch size.
-size_t per_column_bytes(const ColumnShape &shape, size_t vs, int nu, int region_atoms, int maxrow)
+// Workspace bytes per batch column, for the default batch size.  The tile
+// arrays and the product's input panel (global mode) span all tiles of the
+// structure: a union's, where the vectors have one member's length.
+size_t per_column_bytes(const ColumnShape &shape, size_t vs, int nu, int region_atoms, int maxrow, int64_t ntile_min)
 {
     const size_t reg = region_atoms > 0 ? (size_t)region_atoms * (12 + 8 * (size_t)maxrow) : 0;
+    const size_t nt = std::max<size_t>((size_t)shape.m_pad / 32, (size_t)ntile_min);
     return al256((size_t)2 * nu * shape.m_pad * vs) + (size_t)2 * shape.m_pad * vs +
-           (size_t)2 * nu * nu * 8 + (size_t)nu * 8 + 64 + reg + (size_t)(shape.m_pad / 32) * 3 +
-           (size_t)(nu + 2) * 4 + (region_atoms > 0 ? 0 : (size_t)shape.m_pad * vs + (size_t)(shape.m_pad / 32) * 2);
+           (size_t)2 * nu * nu * 8 + (size_t)nu * 8 + 64 + reg + nt * 3 +
+           (size_t)(nu + 2) * 4 + (region_atoms > 0 ? 0 : nt * (32 * vs + 2));
 }
 
 // Batch size within [1, ncols] and the launch limits (one CTA per column, or
@@ -1345,7 +1348,7 @@ int marnoldi_solve(marnoldi_ctx *c, const int64_t *columns, int64_t ncols, int n
     int64_t B = c->batch_override;
     if (B <= 0) {
         const ColumnShape shape = column_shape(m_vec, c->prec);
-        const size_t per_col = per_column_bytes(shape, c->prec == 0 ? 8 : 4, nu, region_atoms, c->maxrow);
+        const size_t per_col = per_column_bytes(shape, c->prec == 0 ? 8 : 4, nu, region_atoms, c->maxrow, ntile_min);
         size_t freeb = 0, totb = 0;
         if (cudaMemGetInfo(&freeb, &totb) != cudaSuccess) { cudaGetLastError(); freeb = (size_t)8 << 30; }
         const size_t budget = std::min<size_t>(freeb / 2, (size_t)48 << 30);
