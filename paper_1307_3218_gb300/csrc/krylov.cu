@@ -308,8 +308,12 @@ __global__ void __launch_bounds__(32 * W, (sizeof(VT) == 4 ? 20 : 16) / W) spmm_
 }
 
 // ------------------------------------------------------------------ Gram-Schmidt
-// One CTA of T = C / 4 threads per column, for vectors of m_pad = nchunk C
-// entries.  Vectors are stored in the column's tile order (tiles of 32 entries
+// One CTA per column, of G groups of T = C / 4 threads, for vectors of m_pad =
+// nchunk C entries; G = 1, or 4 where columns are few (gs_shape).  The groups
+// share a step's work without touching a sum: in sweep 1 they take the blocks of
+// stored vectors in turn, in sweep 2 the passes of four chunks (whose sums a_i
+// are then added in the order of the passes at the end), and the scalar step
+// runs on all warps.  Vectors are stored in the column's tile order (tiles of 32 entries
 // by hop count from the column's atom), and vector i vanishes past its first
 // tcnt[i + 1] tiles (S w_i reaches one hop further than w_i), so each sweep
 // reads a prefix; the entries past a support are exact zeros, so no sum
@@ -397,27 +401,30 @@ __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group 
 // Dynamic shared memory: the ring (R stages of six quads per thread: four
 // stored vectors, u, and w_n or u's lo word), six FP64 arrays of nu entries, the
 // partial sums (sweep 1: b and g for kSpan vectors and C / 32 groups of 32
-// chains, FP64 per warp; sweep 2: a per vector and warp), the coefficients and
-// the support counts.
-template <typename VT, int C, int R, bool kPairs>
+// chains, FP64 per warp; sweep 2: a per vector and warp, with several groups
+// also per pass), the coefficients and the support counts.
+template <typename VT, int C, int R, int G, bool kPairs>
 struct GsCfg {
-    static constexpr int T = C / 4;
+    static constexpr int T = C / 4;                               // threads of a group
     static constexpr int NW = T / 32;
+    static constexpr int TA = G * T;                              // threads of the CTA
     static constexpr int NP = kPairs ? C / 64 : sizeof(VT) == 4 ? C / 32 : NW;   // partial sums per total
     static constexpr int kSpan = 32;                              // stored vectors per round of totals
     static constexpr int kHalves = sizeof(VT) == 4 ? 1 : 2;       // 16-byte pieces per quad
-    static constexpr int kStage = 6 * kHalves * T * 16;           // bytes
+    static constexpr int kStage = 6 * kHalves * TA * 16;          // bytes
+    static constexpr int kPass = 4;                               // chunks per pass of sweep 2 (16 entries per thread)
     // registers: FP32 96 (FP32 at 80: 54.8 against 46.6 ms on 8,192-entry
     // vectors), FP64 (bound by its pipe, which few warps fill) about 150, but two
     // CTAs for C = 1024 (91 against 96 ms on 16,384-entry vectors)
-    static constexpr int kMinCtas = sizeof(VT) == 4 ? 640 / T : C == 1024 ? 2 : 416 / T;
-    static constexpr __host__ __device__ int parts(int nu)        // doubles
+    static constexpr int kMinCtas = G > 1 ? 1 : sizeof(VT) == 4 ? 640 / T : C == 1024 ? 2 : 416 / T;
+    static constexpr __host__ __device__ int parts(int nu, int nchunk)   // doubles
     {
-        return 2 * kSpan * NP > nu * NW ? 2 * kSpan * NP : nu * NW;
+        const int a = nu * NW * (G > 1 ? (nchunk + kPass - 1) / kPass : 1);
+        return 2 * kSpan * NP > a ? 2 * kSpan * NP : a;
     }
-    static size_t smem(int nu)
+    static size_t smem(int nu, int nchunk)
     {
-        return (size_t)R * kStage + ((size_t)nu * 6 + parts(nu)) * sizeof(double) + (size_t)nu * sizeof(VT) +
+        return (size_t)R * kStage + ((size_t)nu * 6 + parts(nu, nchunk)) * sizeof(double) + (size_t)nu * sizeof(VT) +
                (size_t)(nu + 2) * sizeof(int);
     }
 };
@@ -541,22 +548,24 @@ __device__ __forceinline__ DotAcc<float> pair_tree(const uint64_t (&bq)[kGsBlock
     return merge_x2(j0 == j1, c1, shfl_x2(c1, 1)).joined();
 }
 
-template <typename VT, int C, int R, bool kPairs = false>
-__global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_kernel(
+template <typename VT, int C, int R, int G = 1, bool kPairs = false>
+__global__ void __launch_bounds__(G * C / 4, GsCfg<VT, C, R, G, kPairs>::kMinCtas) gs_kernel(
     VT *__restrict__ K, const VT *__restrict__ SK, const VT *__restrict__ U, const VT *__restrict__ Ulo,
     double *__restrict__ Hsub, double *__restrict__ Lsub, double *__restrict__ scale,
     double *__restrict__ cn2, int *__restrict__ status, int *__restrict__ nu_eff,
     const int *__restrict__ tcnt, const uint16_t *__restrict__ tord, VT *__restrict__ panel, int ntile, int64_t MP,
     int n, int nu, int need_w, double tau2)
 {
-    using Cfg = GsCfg<VT, C, R, kPairs>;
+    using Cfg = GsCfg<VT, C, R, G, kPairs>;
     constexpr bool kF = sizeof(VT) == 4;
-    constexpr int T = Cfg::T, NW = Cfg::NW, NP = Cfg::NP, kB = kGsBlock, kH = Cfg::kHalves;
+    constexpr int T = Cfg::T, TA = Cfg::TA, NW = Cfg::NW, NP = Cfg::NP, kB = kGsBlock, kH = Cfg::kHalves;
     constexpr int TPC = C / 32;           // tiles per chunk
-    constexpr int SC = 4;                 // chunks per pass of sweep 2 (16 entries per thread)
+    constexpr int SC = Cfg::kPass;
     const int c = blockIdx.x;
     if (status[c] != 0) return;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int ta = threadIdx.x;                              // thread of the CTA
+    const int group = G > 1 ? ta / T : 0, tid = G > 1 ? ta % T : ta;   // its group, thread and warp of the group
+    const int warp = tid >> 5, lane = tid & 31;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double *ssc = reinterpret_cast<double *>(smem_raw + R * Cfg::kStage);   // s_i, then s_n
     double *tb = ssc + nu, *tg = tb + nu;                   // the sweep's totals
@@ -564,13 +573,13 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
     double *nrow = lrow + nu;                               // the new row n of L^-1
     double *zc = nrow + nu;                                 // L^-1 p
     double *part = zc + nu;                                 // partial sums
-    VT *coef = reinterpret_cast<VT *>(part + Cfg::parts(nu));   // subtraction coefficients c_i s_i
+    VT *coef = reinterpret_cast<VT *>(part + Cfg::parts(nu, (int)(MP / C)));   // subtraction coefficients c_i s_i
     int *cnt_s = reinterpret_cast<int *>(coef + nu);
     __shared__ int bc_stop;
     __shared__ double bc_dinv;
     const int64_t base = (int64_t)c * nu * MP;
-    for (int i = tid; i < n; i += T) ssc[i] = scale[(int64_t)c * nu + i];
-    for (int L = tid; L <= n + 1; L += T) {
+    for (int i = ta; i < n; i += TA) ssc[i] = scale[(int64_t)c * nu + i];
+    for (int L = ta; L <= n + 1; L += TA) {
         const int t = tcnt[(int64_t)c * (nu + 2) + L];
         cnt_s[L] = in_range(t, MP / 32 + 1, kChkSupportCount) ? t : (int)(MP / 32);
     }
@@ -589,8 +598,8 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
     const int64_t dL = kF ? reinterpret_cast<const char *>(Ulo) - reinterpret_cast<const char *>(U) : 0;   // u's lo word
     const uint32_t vb = (uint32_t)(MP * sizeof(VT));    // bytes of a vector
     constexpr uint32_t kCB = C * sizeof(VT);            // bytes of a chunk
-    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(smem_raw) + 16 * tid;
-    auto piece = [&](uint32_t slot, int j, int h) { return slot + (j * kH + h) * (T * 16); };
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(smem_raw) + 16 * ta;
+    auto piece = [&](uint32_t slot, int j, int h) { return slot + (j * kH + h) * (TA * 16); };
 
     // One stage: a chunk of a block's vectors (nbk of them, at src and vb
     // apart), of u and of a sixth vector (d6 bytes from u).  Every thread
@@ -611,21 +620,21 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
     };
     // the next stage to copy: block pb, chunk pv (of the pass at chunk p0 in sweep 2)
     uint32_t pslot = ring;
-    int pb = 0, pv = 0, p0 = 0, pch = chunks(0), pcnt = cnt_s[min(kB, n + 1)];
-    const char *ps = reinterpret_cast<const char *>(SK + base + off), *pu = Ut;
+    int pb = group, pv = 0, p0 = 0, pch = chunks(pb), pcnt = cnt_s[min(pb * kB + kB, n + 1)];
+    const char *ps = reinterpret_cast<const char *>(SK + base + off) + (int64_t)pb * kB * vb, *pu = Ut;
     int pk = off >> 5;   // tile of the thread's first piece
-    auto issue1 = [&] {   // sweep 1: the blocks in order, then nothing
+    auto issue1 = [&] {   // sweep 1: the group's blocks in order, then nothing
         if (pb < nb1) {
             copy_stage(pslot, ps, pu, dW, true, n + 1 - pb * kB, pk, pcnt);
             ps += kCB;
             pu += kCB;
             pk += TPC;
             if (++pv == pch) {
-                ps += (int64_t)kB * vb - (int64_t)pch * kCB;
+                ps += (int64_t)(G * kB) * vb - (int64_t)pch * kCB;
                 pu = Ut;
                 pk = off >> 5;
                 pv = 0;
-                if (++pb < nb1) {
+                if ((pb += G) < nb1) {
                     pch = chunks(pb);
                     pcnt = cnt_s[min(pb * kB + kB, n + 1)];
                 }
@@ -642,7 +651,7 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
         pk = (off >> 5) + p0 * TPC;
         pv = 0;
     };
-    auto issue2 = [&] {   // passes of SC chunks, in each the blocks that reach it, last first
+    auto issue2 = [&] {   // the group's passes of SC chunks, in each the blocks that reach it, last first
         if (p0 < nch_u) {
             copy_stage(pslot, ps, pu, dL, kF, n + 1 - pb * kB, pk, pcnt);
             ps += kCB;
@@ -651,7 +660,7 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
             if (++pv == pch) {
                 if (--pb < 0 || chunks(pb) <= p0) {
                     pb = nb1 - 1;
-                    p0 += SC;
+                    p0 += G * SC;
                 }
                 if (p0 < nch_u) seek2();
             }
@@ -660,103 +669,108 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
         pslot = pslot == ring + (R - 1) * Cfg::kStage ? ring : pslot + Cfg::kStage;
     };
 
-    // ---- sweep 1: b_i and g_i
+    // ---- sweep 1: b_i and g_i, in rounds of kSpan vectors, the groups taking blocks in turn
+    constexpr int kRound = Cfg::kSpan / kB;
+    static_assert(kRound % G == 0, "every group keeps its place from round to round");
     uint32_t slot = ring;
     auto next = [&] { slot = slot == ring + (R - 1) * Cfg::kStage ? ring : slot + Cfg::kStage; };
 #pragma unroll 1
     for (int s = 0; s + 1 < R; ++s) issue1();
 #pragma unroll 1
-    for (int b = 0; b < nb1; ++b) {
-        const int i0 = b * kB, nch = chunks(b), cnt = cnt_s[min(i0 + kB, n + 1)];
-        int k = off >> 5;
-        if constexpr (kF) {
-            uint64_t bq[kB][2];
-            PairAcc gq[kB][2];
-#pragma unroll
-            for (int l = 0; l < kB; ++l) bq[l][0] = bq[l][1] = 0;
+    for (int b0 = 0; b0 < nb1; b0 += kRound) {
+        const int b1 = min(b0 + kRound, nb1);
 #pragma unroll 1
-            for (int v = 0; v < nch; ++v, k += TPC) {
-                issue1();
-                copy_wait<R - 1>();
-                if (k < cnt) {
-                    Quad<float> u, w;
-                    u.lds(piece(slot, 4, 0), 0);
-                    w.lds(piece(slot, 5, 0), 0);
-                    const uint64_t nw[2] = {neg_x2(w.p[0]), neg_x2(w.p[1])};
+        for (int b = b0 + group; b < b1; b += G) {
+            const int i0 = b * kB, nch = chunks(b), cnt = cnt_s[min(i0 + kB, n + 1)];
+            int k = off >> 5;
+            if constexpr (kF) {
+                uint64_t bq[kB][2];
+                PairAcc gq[kB][2];
 #pragma unroll
-                    for (int l = 0; l < kB; ++l) {
-                        if (i0 + l > n) break;
-                        Quad<float> sr;
-                        sr.lds(piece(slot, l, 0), 0);
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            bq[l][h] = fma_x2(sr.p[h], u.p[h], bq[l][h]);
-                            gq[l][h].add(sr.p[h], w.p[h], nw[h]);
-                        }
-                    }
-                }
-                next();
-            }
-            const DotAcc<float> r = kPairs ? pair_tree(bq, gq) : chain_tree(bq, gq);
-            const int j = kPairs ? (lane & 15) >> 1 : lane & 7, i = i0 + (j & 3);
-            const int grp = kPairs ? 2 * warp + (lane >> 4) : 4 * warp + (lane >> 3);
-            if (i <= n) part[((i % Cfg::kSpan) * 2 + (j >> 2)) * NP + grp] = r.pack();
-        } else {
-            DotAcc<VT> acc[2 * kB];   // [l] b, [kB + l] g
-            for_count<kB>(min(kB, n + 1 - i0), [&](auto nbk) {
+                for (int l = 0; l < kB; ++l) bq[l][0] = bq[l][1] = 0;
 #pragma unroll 1
                 for (int v = 0; v < nch; ++v, k += TPC) {
                     issue1();
                     copy_wait<R - 1>();
+                    if (k < cnt) {
+                        Quad<float> u, w;
+                        u.lds(piece(slot, 4, 0), 0);
+                        w.lds(piece(slot, 5, 0), 0);
+                        const uint64_t nw[2] = {neg_x2(w.p[0]), neg_x2(w.p[1])};
 #pragma unroll
-                    for (int h = 0; h < kH; ++h)
-                        if (k + h * kHT < cnt) {
-                            Quad<VT> sr[nbk], u, w;
-                            u.lds(piece(slot, 4, h), h);
-                            w.lds(piece(slot, 5, h), h);
+                        for (int l = 0; l < kB; ++l) {
+                            if (i0 + l > n) break;
+                            Quad<float> sr;
+                            sr.lds(piece(slot, l, 0), 0);
 #pragma unroll
-                            for (int l = 0; l < nbk; ++l) sr[l].lds(piece(slot, l, h), h);
-#pragma unroll
-                            for (int e = 2 * h; e < 2 * h + 2; ++e)
-#pragma unroll
-                                for (int l = 0; l < nbk; ++l) {
-                                    if (need_w) acc[l].add(sr[l].d[e], u.d[e]);
-                                    acc[kB + l].add(sr[l].d[e], w.d[e]);
-                                }
+                            for (int h = 0; h < 2; ++h) {
+                                bq[l][h] = fma_x2(sr.p[h], u.p[h], bq[l][h]);
+                                gq[l][h].add(sr.p[h], w.p[h], nw[h]);
+                            }
                         }
+                    }
                     next();
                 }
-            });
-            const DotAcc<VT> r = warp_scatter(acc);   // slot lane / 4
-            const int q = lane >> 4, i = i0 + ((lane >> 2) & 3);
-            if ((lane & 3) == 0 && i <= n) part[((i % Cfg::kSpan) * 2 + q) * NP + warp] = r.pack();
-        }
-        // totals every kSpan vectors: the groups of chains (warps) in the tree of a butterfly reduction
-        if ((i0 + kB) % Cfg::kSpan == 0 || b == nb1 - 1) {
-            const int j0 = i0 / Cfg::kSpan * Cfg::kSpan;
-            __syncthreads();
-            for (int x = tid; x < 2 * (min(i0 + kB, n + 1) - j0); x += T) {
-                DotAcc<VT> v[NP];
+                const DotAcc<float> r = kPairs ? pair_tree(bq, gq) : chain_tree(bq, gq);
+                const int j = kPairs ? (lane & 15) >> 1 : lane & 7, i = i0 + (j & 3);
+                const int grp = kPairs ? 2 * warp + (lane >> 4) : 4 * warp + (lane >> 3);
+                if (i <= n) part[((i % Cfg::kSpan) * 2 + (j >> 2)) * NP + grp] = r.pack();
+            } else {
+                DotAcc<VT> acc[2 * kB];   // [l] b, [kB + l] g
+                for_count<kB>(min(kB, n + 1 - i0), [&](auto nbk) {
+#pragma unroll 1
+                    for (int v = 0; v < nch; ++v, k += TPC) {
+                        issue1();
+                        copy_wait<R - 1>();
 #pragma unroll
-                for (int j = 0; j < NP; ++j) v[j].unpack(part[x * NP + j]);
-                if constexpr (kPairs) {   // in order
+                        for (int h = 0; h < kH; ++h)
+                            if (k + h * kHT < cnt) {
+                                Quad<VT> sr[nbk], u, w;
+                                u.lds(piece(slot, 4, h), h);
+                                w.lds(piece(slot, 5, h), h);
 #pragma unroll
-                    for (int j = 1; j < NP; ++j) v[0].merge(v[j]);
-                } else {
+                                for (int l = 0; l < nbk; ++l) sr[l].lds(piece(slot, l, h), h);
 #pragma unroll
-                    for (int o = NP / 2; o > 0; o >>= 1)
+                                for (int e = 2 * h; e < 2 * h + 2; ++e)
 #pragma unroll
-                        for (int j = 0; j < o; ++j) v[j].merge(v[j + o]);
-                }
-                ((x & 1) ? tg : tb)[j0 + (x >> 1)] = v[0].value();
+                                    for (int l = 0; l < nbk; ++l) {
+                                        if (need_w) acc[l].add(sr[l].d[e], u.d[e]);
+                                        acc[kB + l].add(sr[l].d[e], w.d[e]);
+                                    }
+                            }
+                        next();
+                    }
+                });
+                const DotAcc<VT> r = warp_scatter(acc);   // slot lane / 4
+                const int q = lane >> 4, i = i0 + ((lane >> 2) & 3);
+                if ((lane & 3) == 0 && i <= n) part[((i % Cfg::kSpan) * 2 + q) * NP + warp] = r.pack();
             }
-            __syncthreads();
         }
+        // totals of the round: the groups of chains (warps) in the tree of a butterfly reduction
+        const int j0 = b0 * kB;
+        __syncthreads();
+        for (int x = ta; x < 2 * (min(b1 * kB, n + 1) - j0); x += TA) {
+            DotAcc<VT> v[NP];
+#pragma unroll
+            for (int j = 0; j < NP; ++j) v[j].unpack(part[x * NP + j]);
+            if constexpr (kPairs) {   // in order
+#pragma unroll
+                for (int j = 1; j < NP; ++j) v[0].merge(v[j]);
+            } else {
+#pragma unroll
+                for (int o = NP / 2; o > 0; o >>= 1)
+#pragma unroll
+                    for (int j = 0; j < o; ++j) v[j].merge(v[j + o]);
+            }
+            ((x & 1) ? tg : tb)[j0 + (x >> 1)] = v[0].value();
+        }
+        __syncthreads();
     }
 
     // the first stages of sweep 2 are copied during the scalar step
     pslot = slot = ring;
     pb = nb1 - 1;
+    p0 = group * SC;
     seek2();
 #pragma unroll 1
     for (int s = 0; s + 1 < R; ++s) issue2();
@@ -764,7 +778,7 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
     // ---- scalars: the norm, G's column, the new row of L^-1, the coefficients
     {
         const GsScalarSmem<VT> sm{ssc, tb, tg, lrow, nrow, zc, coef, bc_stop, bc_dinv};
-        if (!gs_scalars<VT, T>(c, n, nu, need_w, tau2, tid, Lsub, scale, cn2, status, nu_eff, sm,
+        if (!gs_scalars<VT, TA>(c, n, nu, need_w, tau2, ta, Lsub, scale, cn2, status, nu_eff, sm,
                                [] { __syncthreads(); })) {
             copy_wait<0>();
             return;
@@ -785,7 +799,7 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
         return panel + panel_pos(ntile, c, I) + (p & 3);
     };
 #pragma unroll 1
-    for (int v0 = 0; v0 < nch_u; v0 += SC) {
+    for (int v0 = group * SC; v0 < nch_u; v0 += G * SC) {
         PairAcc x[kF ? SC : 1][2];
         double xd[kF ? 1 : SC][4];
 #pragma unroll 1
@@ -865,13 +879,14 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
 #pragma unroll
                 for (int l = 0; l < kB; ++l) acc[l] = pa[l].joined();
             }
-            // the warp's sums (slot lane / 8), added up over the passes; every
-            // support holds tile 0, so the first pass sets them all
+            // the warp's sums (slot lane / 8), added up over the passes (with
+            // several groups at the end); every support holds tile 0, so the
+            // first pass sets them all
             DotAcc<VT> r = warp_scatter(acc);
             const int i = i0 + (lane >> 3);
             if ((lane & 7) == 0 && i <= n) {
-                double *ps = part + i * NW + warp;
-                if (v0 > 0) {
+                double *ps = part + ((G > 1 ? v0 / SC * nu : 0) + i) * NW + warp;
+                if (G == 1 && v0 > 0) {
                     DotAcc<VT> y;
                     y.unpack(*ps);
                     r.merge(y);
@@ -907,7 +922,7 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
         }
     }
     if (need_w) {   // zeros past the last pass
-        for (int v = (nch_u + SC - 1) / SC * SC; v < nch_all; ++v)
+        for (int v = (nch_u + SC - 1) / SC * SC + group; v < nch_all; v += G)
 #pragma unroll
             for (int h = 0; h < kH; ++h)
                 *reinterpret_cast<float4 *>(wo + v * C + off + h * (C / 2)) = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -915,31 +930,38 @@ __global__ void __launch_bounds__(C / 4, GsCfg<VT, C, R, kPairs>::kMinCtas) gs_k
     copy_wait<0>();
     __syncthreads();
     const double sn = ssc[n];
-    for (int m = tid; m <= n; m += T) {   // h_m of unit-norm vectors
-        DotAcc<VT> s;
-        s.unpack(part[m * NW]);
-#pragma unroll
-        for (int j = 1; j < NW; ++j) {
+    for (int m = ta; m <= n; m += TA) {   // h_m of unit-norm vectors
+        const int np = G > 1 ? (chunks(m / kB) + SC - 1) / SC : 1;
+        auto sum_of = [&](int j) {   // warp j's, over the passes in order
             DotAcc<VT> y;
             y.unpack(part[m * NW + j]);
-            s.merge(y);
-        }
+            for (int p = 1; p < np; ++p) {
+                DotAcc<VT> z;
+                z.unpack(part[(p * nu + m) * NW + j]);
+                z.merge(y);
+                y = z;
+            }
+            return y;
+        };
+        DotAcc<VT> s = sum_of(0);
+#pragma unroll
+        for (int j = 1; j < NW; ++j) s.merge(sum_of(j));
         const double h = s.value() * (ssc[m] * sn);
         Hsub[((int64_t)c * nu + m) * nu + n] = h;
         Hsub[((int64_t)c * nu + n) * nu + m] = h;
     }
 }
 
-template <typename VT, int C, int R, bool kPairs = false>
+template <typename VT, int C, int R, int G = 1, bool kPairs = false>
 cudaError_t gs_dispatch(const KrylovBatch &b, int n, int need_w, double tau, cudaStream_t s)
 {
-    using Cfg = GsCfg<VT, C, R, kPairs>;
+    using Cfg = GsCfg<VT, C, R, G, kPairs>;
     if (b.shape.m_pad % C != 0 || (int64_t)b.ntile * 32 < b.shape.m_pad || !b.tcnt || !b.Lsub)
         return cudaErrorInvalidValue;
-    const size_t smem = Cfg::smem(b.nu);
-    cudaError_t e = allow_dynamic_smem((const void *)gs_kernel<VT, C, R, kPairs>, smem);
+    const size_t smem = Cfg::smem(b.nu, (int)(b.shape.m_pad / C));
+    cudaError_t e = allow_dynamic_smem((const void *)gs_kernel<VT, C, R, G, kPairs>, smem);
     if (e != cudaSuccess) return e;
-    gs_kernel<VT, C, R, kPairs><<<b.nb, Cfg::T, smem, s>>>(
+    gs_kernel<VT, C, R, G, kPairs><<<b.nb, Cfg::TA, smem, s>>>(
         (VT *)b.K, (const VT *)b.SK, (const VT *)b.U, (const VT *)b.Ulo, b.Hsub, b.Lsub, b.scale, b.cn2,
         b.status, b.nu_eff, b.tcnt, b.tord, (VT *)b.panel, b.ntile, b.shape.m_pad, n, b.nu, need_w, tau * tau);
     return cudaGetLastError();
@@ -951,16 +973,35 @@ cudaError_t gs_dispatch(const KrylovBatch &b, int n, int need_w, double tau, cud
 // ring's shared memory would hold back the CTAs whose reductions cover each
 // other (24,000 columns, nu = 30: 28.9 ms against 32.6 with three), three above
 // (2,048 columns of 2,048 entries, nu = 100: 44.9 ms against 48.3 with two).
+//
+// At most one column per SM: four groups of threads per CTA.  One group's two
+// warps reach two of the SM's four schedulers and hide little of each other's
+// latency, where nothing else runs on the SM.  Gram-Schmidt of a solve with one
+// group and with four (the Krylov vectors' bits are the same): FP64, 4,096
+// entries, nu = 200, 1 column 214 -> 90 ms, 150 columns 218 -> 92; nu = 30, 1
+// column 4.9 -> 2.4; 1,024 entries, nu = 30, 150 columns 1.78 -> 1.45; mixed,
+// 4,096 entries, nu = 100, 1 column 21.7 -> 7.6; 8,192 entries, nu = 100, 150
+// columns 21.7 -> 12.3 (13.7 with two groups).  With more columns the CTAs run in
+// two turns, or three: 300 columns, FP64, 4,096 entries, nu = 100 54.9 -> 46.8,
+// but 1,024 entries, nu = 60 6.8 -> 9.6; 340 columns 68.9 -> 69.7 and 7.8 -> 13.9.
+// FP64 shapes of 512 chains (only an autotuner's choice) would not fit the ring.
+constexpr int kGsFewColumns = 152;
+
 template <typename VT>
 cudaError_t gs_shape(const KrylovBatch &b, int n, int need_w, double tau, cudaStream_t s)
 {
     constexpr int R = sizeof(VT) == 4 ? 3 : 2;
     if ((int64_t)b.shape.vpt * b.shape.threads != b.shape.m_pad) return cudaErrorInvalidValue;
+    const bool few = b.nb <= kGsFewColumns;
     switch (b.shape.threads) {
     case 256:
+        if (few) return gs_dispatch<VT, 256, R, 4>(b, n, need_w, tau, s);
         if (R == 3 && b.shape.m_pad <= 1024) return gs_dispatch<VT, 256, 2>(b, n, need_w, tau, s);
         return gs_dispatch<VT, 256, R>(b, n, need_w, tau, s);
-    case 512: return gs_dispatch<VT, 512, R>(b, n, need_w, tau, s);
+    case 512:
+        if constexpr (sizeof(VT) == 4)
+            if (few) return gs_dispatch<VT, 512, R, 4>(b, n, need_w, tau, s);
+        return gs_dispatch<VT, 512, R>(b, n, need_w, tau, s);
     case 1024: return gs_dispatch<VT, 1024, R>(b, n, need_w, tau, s);
     default: return cudaErrorInvalidValue;
     }
@@ -1023,8 +1064,8 @@ cudaError_t launch_spmm_hs(const DeviceMatrix &A, const KrylovBatch &b, void *SY
 cudaError_t launch_gs(const KrylovBatch &b, int n, int need_w, double tau, cudaStream_t s)
 {
     if (gs_pair_shape(b.shape, b.prec))
-        return b.shape.threads == 288 ? gs_dispatch<float, 512, 3, true>(b, n, need_w, tau, s)
-                                      : gs_dispatch<float, 1024, 3, true>(b, n, need_w, tau, s);
+        return b.shape.threads == 288 ? gs_dispatch<float, 512, 3, 1, true>(b, n, need_w, tau, s)
+                                      : gs_dispatch<float, 1024, 3, 1, true>(b, n, need_w, tau, s);
     return b.prec == 0 ? gs_shape<double>(b, n, need_w, tau, s) : gs_shape<float>(b, n, need_w, tau, s);
 }
 
