@@ -383,37 +383,41 @@ __global__ void __launch_bounds__(256) spmm_regional_hs_kernel(
     }
 }
 
-// Mixed precision, groups of four columns: one CTA per group, the four columns'
-// x in shared memory, a lane per local row.  A lane's block is its own (the
-// lanes' blocks are 32 different ones), and reading it 16 bytes at a time looked
-// up 32 lines per load, which kept the L1 at 87 %; here twelve lanes copy one
-// block together (its lines are looked up once) into the warp's shared memory,
-// from where each lane reads its own.  The columns go through packed
-// instructions in pairs; every column's sums run in the same order as alone.
-// 24,000 columns, 256-atom regions, nu = 30: 21.5 ms, 27.2 with a lane reading
-// its own block; 4,000 columns, nu = 100: 14.6 (19.0).
+// Mixed precision, groups of four columns: one warp per 32 rows of a group, a
+// lane per local row.  A lane's block is its own (the lanes' blocks are 32
+// different ones), and reading it 16 bytes at a time looked up 32 lines per
+// load, which kept the L1 at 87 %; here twelve lanes copy one block together
+// (its lines are looked up once) into the warp's shared memory, from where each
+// lane reads its own.  The columns go through packed instructions in pairs;
+// every column's sums run in the same order as alone.  24,000 columns, 256-atom
+// regions, nu = 30: 20.2 ms, 27.2 with a lane reading its own block; 4,000
+// columns, nu = 100: 13.1 (19.0).  The warps need nothing of each other, so a CTA
+// is one: no CTA waits for its longest warp, and a few groups, or regions of few
+// rows, still spread over the SMs.  With a CTA of four warps per group that went
+// over all its rows: one atom of a 1,024-atom region, nu = 30, 3.4 ms, now 0.61;
+// 100 columns, one per atom, of 1,000-atom regions 3.6 -> 1.75; 8,000 columns of
+// 32-atom regions, nu = 20, 1.6 -> 0.86.  The rows of a group run fastest in the
+// grid, so that they share the group's x in L2.
 constexpr int kRegPitch = 52;   // floats per staged block: H hi and lo, S hi, and 4 that spread the banks
 
 template <bool kS>
-__global__ void __launch_bounds__(128, 3) spmm_regional_group_kernel(
+__global__ void __launch_bounds__(32, 12) spmm_regional_group_kernel(
     int n_reg, int maxrow, const int *__restrict__ lcnt, const int *__restrict__ lci,
     const int *__restrict__ lgk, const float *__restrict__ Hv, const float *__restrict__ Sv,
     const float *__restrict__ X, int64_t ldx, float *__restrict__ U, float *__restrict__ Ulo, int64_t ldu,
     float *__restrict__ SY, int64_t ldsy, int ncols, const int *__restrict__ gstart,
     const uint8_t *__restrict__ thop, const uint16_t *__restrict__ tinv, int lim)
 {
-    constexpr int G = reg_group<float>(), NW = 4, kPieces = kS ? 12 : 8;
+    constexpr int G = reg_group<float>(), kPieces = kS ? 12 : 8;
     static_assert(G == 4, "two pairs of columns");
-    extern __shared__ __align__(16) float rsm[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    float *blk = rsm + warp * (2 * 32 * kRegPitch);    // two stages of 32 blocks
-    const int g = blockIdx.x;
+    __shared__ __align__(16) float blk[2 * 32 * kRegPitch];   // two stages of 32 blocks
+    const int lane = threadIdx.x, g = blockIdx.y, p = 32 * (int)blockIdx.x + lane;
     // clipped to ncols: a run of the autotuner covers the batch's first columns only
     const int c0 = gstart[g], c1 = min(gstart[g + 1], ncols);
     if (c0 >= c1) return;
     if (c1 - c0 < G) {   // an atom with fewer real orbitals, or a run cut by the batch: column by column
-        for (int c = c0; c < c1; ++c)
-            for (int p = tid; p < n_reg; p += 32 * NW)
+        if (p < n_reg)
+            for (int c = c0; c < c1; ++c)
                 regional_rows<float, kS, 1>(p, c, n_reg, maxrow, lcnt, lci, lgk, Hv, Sv, X, ldx, U, Ulo, ldu, SY,
                                             ldsy, ncols, thop, tinv, lim);
         return;
@@ -421,120 +425,116 @@ __global__ void __launch_bounds__(128, 3) spmm_regional_group_kernel(
     const float *xc = X + (int64_t)c0 * ldx;
     const int64_t base = (int64_t)c0 * maxrow * n_reg;
     const uint32_t sb = (uint32_t)__cvta_generic_to_shared(blk);
-    for (int p0 = 32 * warp; p0 < n_reg; p0 += 32 * NW) {
-        const int p = p0 + lane;
-        const bool row = p < n_reg;
-        const bool act = row && (int)thop[(int64_t)(p >> 3) * ncols + c0] <= lim;
-        const int cnt = act ? lcnt[(int64_t)c0 * n_reg + p] : 0;
-        const int most = __reduce_max_sync(kFull, cnt);
-        uint64_t hi[2][4], lo[2][4], sy[2][4];   // column pairs (0, 1) and (2, 3)
+    const bool row = p < n_reg;
+    const bool act = row && (int)thop[(int64_t)(p >> 3) * ncols + c0] <= lim;
+    const int cnt = act ? lcnt[(int64_t)c0 * n_reg + p] : 0;
+    const int most = __reduce_max_sync(kFull, cnt);
+    uint64_t hi[2][4], lo[2][4], sy[2][4];   // column pairs (0, 1) and (2, 3)
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+    for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int a = 0; a < 4; ++a) hi[h][a] = lo[h][a] = sy[h][a] = 0;
-        auto block_of = [&](int s) { return s < cnt ? lgk[base + (int64_t)s * n_reg + p] : -1; };
-        auto column_of = [&](int s) { return s < cnt ? lci[base + (int64_t)s * n_reg + p] : -1; };
-        // position of local column q's entries, -1 for none
-        auto position = [&](int q) {
-            if (q < 0 || !in_range(q, n_reg, kChkRegionCol)) return -1;
-            const int xp = 32 * (int)tinv[(int64_t)(q >> 3) * ncols + c0] + 4 * (q & 7);
-            return in_range(xp, ldu - 3, kChkRegionGather) ? xp : -1;
-        };
-        auto copy = [&](int s, int k) {   // the lanes' blocks of slot s, k this lane's
-            const uint32_t st = sb + (s & 1) * (32 * kRegPitch * 4);
+        for (int a = 0; a < 4; ++a) hi[h][a] = lo[h][a] = sy[h][a] = 0;
+    auto block_of = [&](int s) { return s < cnt ? lgk[base + (int64_t)s * n_reg + p] : -1; };
+    auto column_of = [&](int s) { return s < cnt ? lci[base + (int64_t)s * n_reg + p] : -1; };
+    // position of local column q's entries, -1 for none
+    auto position = [&](int q) {
+        if (q < 0 || !in_range(q, n_reg, kChkRegionCol)) return -1;
+        const int xp = 32 * (int)tinv[(int64_t)(q >> 3) * ncols + c0] + 4 * (q & 7);
+        return in_range(xp, ldu - 3, kChkRegionGather) ? xp : -1;
+    };
+    auto copy = [&](int s, int k) {   // the lanes' blocks of slot s, k this lane's
+        const uint32_t st = sb + (s & 1) * (32 * kRegPitch * 4);
 #pragma unroll
-            for (int r = 0; r < kPieces; ++r) {
-                const int item = 32 * r + lane, b = item / kPieces, piece = item - b * kPieces;
-                const int kb = __shfl_sync(kFull, k, b);
-                const float *src = (piece < 8 ? Hv : Sv) + 32 * (int64_t)kb + 4 * (piece < 8 ? piece : piece - 8);
-                if (kb >= 0)
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(st + 4 * (b * kRegPitch + 4 * piece)),
-                                 "l"(src)
-                                 : "memory");
-            }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-        };
-        auto gather = [&](int xp, float4 (&x)[G]) {
-#pragma unroll
-            for (int m = 0; m < G; ++m)
-                if (xp >= 0) x[m] = __ldg(reinterpret_cast<const float4 *>(xc + m * ldx + xp));
-        };
-        // blocks are copied one slot ahead, x one, the positions two, the indices three
-        __syncwarp();   // the last slots of the rows before have been read
-        copy(0, block_of(0));
-        int kn = block_of(1), x0p = position(column_of(0)), x1p = position(column_of(1)), q2 = column_of(2);
-        float4 xv[G], xw[G];
-        gather(x0p, xv);
-        for (int s = 0; s < most; ++s) {
-            __syncwarp();   // slot s - 1 has been read
-            if (s + 1 < most) copy(s + 1, kn);
-            else asm volatile("cp.async.commit_group;" ::: "memory");
-            gather(x1p, xw);
-            const int x2p = position(q2);
-            q2 = column_of(s + 3);
-            kn = block_of(s + 2);
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-            __syncwarp();
-            if (x0p >= 0) {
-                uint64_t x[2][4], nx[2][4];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const float4 u = xv[2 * h], v = xv[2 * h + 1];
-                    x[h][0] = pack_x2(u.x, v.x);
-                    x[h][1] = pack_x2(u.y, v.y);
-                    x[h][2] = pack_x2(u.z, v.z);
-                    x[h][3] = pack_x2(u.w, v.w);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) nx[h][e] = neg_x2(x[h][e]);
-                }
-                const float *B = blk + (s & 1) * (32 * kRegPitch) + lane * kRegPitch;
-#pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    const float4 h4 = *reinterpret_cast<const float4 *>(B + 4 * a);
-                    const float4 l4 = *reinterpret_cast<const float4 *>(B + 16 + 4 * a);
-                    const float hv[4] = {h4.x, h4.y, h4.z, h4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
-                    float sv[4] = {0.f, 0.f, 0.f, 0.f};
-                    if constexpr (kS) {
-                        const float4 s4 = *reinterpret_cast<const float4 *>(B + 32 + 4 * a);
-                        sv[0] = s4.x; sv[1] = s4.y; sv[2] = s4.z; sv[3] = s4.w;
-                    }
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const uint64_t hp = pack_x2(hv[e], hv[e]), lp = pack_x2(lv[e], lv[e]);
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) spmm_add(hi[h][a], lo[h][a], hp, lp, x[h][e], nx[h][e]);
-                        if constexpr (kS) {
-                            const uint64_t sp = pack_x2(sv[e], sv[e]);
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) sy[h][a] = fma_x2(sp, x[h][e], sy[h][a]);
-                        }
-                    }
-                }
-            }
-            x0p = x1p;
-            x1p = x2p;
-#pragma unroll
-            for (int m = 0; m < G; ++m) xv[m] = xw[m];
+        for (int r = 0; r < kPieces; ++r) {
+            const int item = 32 * r + lane, b = item / kPieces, piece = item - b * kPieces;
+            const int kb = __shfl_sync(kFull, k, b);
+            const float *src = (piece < 8 ? Hv : Sv) + 32 * (int64_t)kb + 4 * (piece < 8 ? piece : piece - 8);
+            if (kb >= 0)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(st + 4 * (b * kRegPitch + 4 * piece)),
+                             "l"(src)
+                             : "memory");
         }
-        if (!row) continue;
-        const int64_t yp = 32 * (int64_t)tinv[(int64_t)(p >> 3) * ncols + c0] + 4 * (p & 7);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto gather = [&](int xp, float4 (&x)[G]) {
 #pragma unroll
-        for (int m = 0; m < G; ++m) {
-            const int64_t c = c0 + m;
-            float yh[4], yl[4], ys[4];
+        for (int m = 0; m < G; ++m)
+            if (xp >= 0) x[m] = __ldg(reinterpret_cast<const float4 *>(xc + m * ldx + xp));
+    };
+    // blocks are copied one slot ahead, x one, the positions two, the indices three
+    copy(0, block_of(0));
+    int kn = block_of(1), x0p = position(column_of(0)), x1p = position(column_of(1)), q2 = column_of(2);
+    float4 xv[G], xw[G];
+    gather(x0p, xv);
+    for (int s = 0; s < most; ++s) {
+        __syncwarp();   // slot s - 1 has been read
+        if (s + 1 < most) copy(s + 1, kn);
+        else asm volatile("cp.async.commit_group;" ::: "memory");
+        gather(x1p, xw);
+        const int x2p = position(q2);
+        q2 = column_of(s + 3);
+        kn = block_of(s + 2);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        if (x0p >= 0) {
+            uint64_t x[2][4], nx[2][4];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float4 u = xv[2 * h], v = xv[2 * h + 1];
+                x[h][0] = pack_x2(u.x, v.x);
+                x[h][1] = pack_x2(u.y, v.y);
+                x[h][2] = pack_x2(u.z, v.z);
+                x[h][3] = pack_x2(u.w, v.w);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) nx[h][e] = neg_x2(x[h][e]);
+            }
+            const float *B = blk + (s & 1) * (32 * kRegPitch) + lane * kRegPitch;
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
-                const int sh = 32 * (m & 1);
-                const float fh = __uint_as_float((unsigned)(hi[m >> 1][a] >> sh));
-                const float fl = __uint_as_float((unsigned)(lo[m >> 1][a] >> sh));
-                yh[a] = __fadd_rn(fh, fl);
-                yl[a] = __fsub_rn(fl, __fsub_rn(yh[a], fh));
-                ys[a] = __uint_as_float((unsigned)(sy[m >> 1][a] >> sh));
+                const float4 h4 = *reinterpret_cast<const float4 *>(B + 4 * a);
+                const float4 l4 = *reinterpret_cast<const float4 *>(B + 16 + 4 * a);
+                const float hv[4] = {h4.x, h4.y, h4.z, h4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
+                float sv[4] = {0.f, 0.f, 0.f, 0.f};
+                if constexpr (kS) {
+                    const float4 s4 = *reinterpret_cast<const float4 *>(B + 32 + 4 * a);
+                    sv[0] = s4.x; sv[1] = s4.y; sv[2] = s4.z; sv[3] = s4.w;
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const uint64_t hp = pack_x2(hv[e], hv[e]), lp = pack_x2(lv[e], lv[e]);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) spmm_add(hi[h][a], lo[h][a], hp, lp, x[h][e], nx[h][e]);
+                    if constexpr (kS) {
+                        const uint64_t sp = pack_x2(sv[e], sv[e]);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) sy[h][a] = fma_x2(sp, x[h][e], sy[h][a]);
+                    }
+                }
             }
-            store4(U + c * ldu + yp, yh);
-            store4(Ulo + c * ldu + yp, yl);
-            if constexpr (kS) store4(SY + c * ldsy + yp, ys);
         }
+        x0p = x1p;
+        x1p = x2p;
+#pragma unroll
+        for (int m = 0; m < G; ++m) xv[m] = xw[m];
+    }
+    if (!row) return;
+    const int64_t yp = 32 * (int64_t)tinv[(int64_t)(p >> 3) * ncols + c0] + 4 * (p & 7);
+#pragma unroll
+    for (int m = 0; m < G; ++m) {
+        const int64_t c = c0 + m;
+        float yh[4], yl[4], ys[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int sh = 32 * (m & 1);
+            const float fh = __uint_as_float((unsigned)(hi[m >> 1][a] >> sh));
+            const float fl = __uint_as_float((unsigned)(lo[m >> 1][a] >> sh));
+            yh[a] = __fadd_rn(fh, fl);
+            yl[a] = __fsub_rn(fl, __fsub_rn(yh[a], fh));
+            ys[a] = __uint_as_float((unsigned)(sy[m >> 1][a] >> sh));
+        }
+        store4(U + c * ldu + yp, yh);
+        store4(Ulo + c * ldu + yp, yl);
+        if constexpr (kS) store4(SY + c * ldsy + yp, ys);
     }
 }
 
@@ -559,16 +559,13 @@ cudaError_t launch_spmm_regional_hs(const DeviceMatrix &A, const RegionMaps &rm,
             spmm_regional_hs_kernel<false><<<grid, block, 0, s>>>(
                 rm.n_reg, rm.maxrow, rm.lcnt, rm.lci, rm.lgk, A.Hd, A.Sd, (const double *)X, ldx, (double *)b.U, ldu, nullptr, 0, b.nb, rm.gstart, rm.ngroups, b.thop, b.tinv, lim);
     } else {
-        const size_t smem = (size_t)4 * 2 * 32 * kRegPitch * sizeof(float);
+        const dim3 ggrid(grid.x, (unsigned)rm.ngroups);
         auto go = [&](auto kernel) {
-            const cudaError_t e = allow_dynamic_smem((const void *)kernel, smem);
-            if (e != cudaSuccess) return e;
-            kernel<<<rm.ngroups, 128, smem, s>>>(
+            kernel<<<ggrid, 32, 0, s>>>(
                 rm.n_reg, rm.maxrow, rm.lcnt, rm.lci, rm.lgk, A.Hf, A.Sf, (const float *)X, ldx, (float *)b.U,
                 (float *)b.Ulo, ldu, (float *)SY, ldsy, b.nb, rm.gstart, b.thop, b.tinv, lim);
-            return cudaGetLastError();
         };
-        return SY ? go(spmm_regional_group_kernel<true>) : go(spmm_regional_group_kernel<false>);
+        SY ? go(spmm_regional_group_kernel<true>) : go(spmm_regional_group_kernel<false>);
     }
     return cudaGetLastError();
 }
