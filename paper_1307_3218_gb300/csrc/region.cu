@@ -25,6 +25,7 @@
 #include "gs_common.cuh"
 
 #include <climits>
+#include <type_traits>
 
 namespace marnoldi {
 namespace {
@@ -261,63 +262,51 @@ __global__ void init_regional_kernel(const double *__restrict__ Sv, const double
 // Gram-Schmidt step and share the local block list, so the x gathers and the
 // index reads serve both).  Lanes run over local block rows, so the
 // local-structure reads coalesce and the x gathers stay inside the columns'
-// short local vectors.  FP32: H by exact products and two-sums over its hi + lo
-// values, output as a (hi, lo) pair (the subspace matrix entries use it), S by
-// FMAs over its hi values; FP64: FMAs.  Rows whose support tile lies more than
-// `lim` hops from the column's atom are exact zeros and are written without
-// being computed.
+// short local vectors.  FP64: FMAs; mixed precision: see group_rows.  Rows whose
+// support tile lies more than `lim` hops from the column's atom are exact zeros
+// and are written without being computed.
 //
 // The NC batch columns c0 .. c0 + NC - 1 belong to one atom here: a column's
 // region, local block lists and tile order depend only on its atom, so one
 // pass over the blocks, each block read once, serves all NC columns (the
 // lanes read different blocks, so the block reads are what the L1 spends its
 // time on).  Every column's sums run in the same order as alone.
-template <typename VT, bool kS, int NC>
+template <bool kS, int NC>
 __device__ __forceinline__ void regional_rows(
     int p, int c0, int n_reg, int maxrow, const int *__restrict__ lcnt, const int *__restrict__ lci,
-    const int *__restrict__ lgk, const VT *__restrict__ Hv, const VT *__restrict__ Sv,
-    const VT *__restrict__ X, int64_t ldx, VT *__restrict__ U, VT *__restrict__ Ulo, int64_t ldu,
-    VT *__restrict__ SY, int64_t ldsy, int ncols, const uint8_t *__restrict__ thop,
-    const uint16_t *__restrict__ tinv, int lim)
+    const int *__restrict__ lgk, const double *__restrict__ Hv, const double *__restrict__ Sv,
+    const double *__restrict__ X, int64_t ldx, double *__restrict__ U, int64_t ldu, double *__restrict__ SY,
+    int64_t ldsy, int ncols, const uint8_t *__restrict__ thop, const uint16_t *__restrict__ tinv, int lim)
 {
-    constexpr bool kF = sizeof(VT) == 4;
-    constexpr int stride = kF ? 32 : 16;
     const int64_t base = (int64_t)c0 * maxrow * n_reg;
     const bool act = (int)thop[(int64_t)(p >> 3) * ncols + c0] <= lim;
     const int cnt = act ? lcnt[(int64_t)c0 * n_reg + p] : 0;
-    VT acc[NC][4], acl[NC][4], sacc[NC][4];
+    double acc[NC][4], sacc[NC][4];
 #pragma unroll
     for (int m = 0; m < NC; ++m)
 #pragma unroll
-        for (int a = 0; a < 4; ++a) acc[m][a] = acl[m][a] = sacc[m][a] = VT(0);
+        for (int a = 0; a < 4; ++a) acc[m][a] = sacc[m][a] = 0.0;
     for (int s = 0; s < cnt; ++s) {
         const int q = lci[base + (int64_t)s * n_reg + p];
         const int64_t k = lgk[base + (int64_t)s * n_reg + p];
         if (!in_range(q, n_reg, kChkRegionCol)) continue;
         const int64_t xp = 32 * (int64_t)tinv[(int64_t)(q >> 3) * ncols + c0] + 4 * (q & 7);
         if (!in_range(xp, ldu - 3, kChkRegionGather)) continue;
-        VT xv[NC][4];
+        double xv[NC][4];
 #pragma unroll
         for (int m = 0; m < NC; ++m) load4(X + (int64_t)(c0 + m) * ldx + xp, xv[m]);
-        const VT *Hb = Hv + stride * k;
-        const VT *Sb = Sv + stride * k;
+        const double *Hb = Hv + 16 * k;
+        const double *Sb = Sv + 16 * k;
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
-            VT hr[4], lr[4], sr[4];
+            double hr[4], sr[4];
             load4(Hb + 4 * a, hr);
-            if constexpr (kF) load4(Hb + 16 + 4 * a, lr);
             if constexpr (kS) load4(Sb + 4 * a, sr);
 #pragma unroll
             for (int m = 0; m < NC; ++m) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    if constexpr (kF) {
-                        const float pr = __fmul_rn(hr[e], xv[m][e]);
-                        const float er = __fmaf_rn(hr[e], xv[m][e], -pr);
-                        df_add(acc[m][a], acl[m][a], pr, __fmaf_rn(lr[e], xv[m][e], er));
-                    } else {
-                        acc[m][a] = fma(hr[e], xv[m][e], acc[m][a]);
-                    }
+                    acc[m][a] = fma(hr[e], xv[m][e], acc[m][a]);
                     if constexpr (kS) sacc[m][a] = fma(sr[e], xv[m][e], sacc[m][a]);
                 }
             }
@@ -327,18 +316,7 @@ __device__ __forceinline__ void regional_rows(
 #pragma unroll
     for (int m = 0; m < NC; ++m) {
         const int64_t c = c0 + m;
-        if constexpr (kF) {
-            VT yh[4], yl[4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                yh[a] = __fadd_rn(acc[m][a], acl[m][a]);
-                yl[a] = __fsub_rn(acl[m][a], __fsub_rn(yh[a], acc[m][a]));
-            }
-            store4(U + c * ldu + yp, yh);
-            store4(Ulo + c * ldu + yp, yl);
-        } else {
-            store4(U + c * ldu + yp, acc[m]);
-        }
+        store4(U + c * ldu + yp, acc[m]);
         if constexpr (kS) store4(SY + c * ldsy + yp, sacc[m]);
     }
 }
@@ -373,25 +351,31 @@ __global__ void __launch_bounds__(256) spmm_regional_hs_kernel(
     const int c0 = gstart[g], c1 = min(gstart[g + 1], ncols);
     if (c0 >= c1) return;
     if (c1 - c0 == G) {
-        regional_rows<double, kS, G>(p, c0, n_reg, maxrow, lcnt, lci, lgk, Hv, Sv, X, ldx, U, nullptr, ldu, SY, ldsy,
-                                     ncols, thop, tinv, lim);
+        regional_rows<kS, G>(p, c0, n_reg, maxrow, lcnt, lci, lgk, Hv, Sv, X, ldx, U, ldu, SY, ldsy, ncols, thop, tinv,
+                             lim);
     } else {
 #pragma unroll 1
         for (int c = c0; c < c1; ++c)
-            regional_rows<double, kS, 1>(p, c, n_reg, maxrow, lcnt, lci, lgk, Hv, Sv, X, ldx, U, nullptr, ldu, SY,
-                                         ldsy, ncols, thop, tinv, lim);
+            regional_rows<kS, 1>(p, c, n_reg, maxrow, lcnt, lci, lgk, Hv, Sv, X, ldx, U, ldu, SY, ldsy, ncols, thop,
+                                 tinv, lim);
     }
 }
 
-// Mixed precision, groups of four columns: one warp per 32 rows of a group, a
-// lane per local row.  A lane's block is its own (the lanes' blocks are 32
+// Mixed precision, NC columns of one atom: one warp per 32 rows of the group, a
+// lane per local row.  H by exact products and two-sums over its hi + lo values,
+// output as a (hi, lo) pair (the subspace matrix entries use it), S by FMAs over
+// its hi values.  A lane's block is its own (the lanes' blocks are 32
 // different ones), and reading it 16 bytes at a time looked up 32 lines per
 // load, which kept the L1 at 87 %; here twelve lanes copy one block together
 // (its lines are looked up once) into the warp's shared memory, from where each
 // lane reads its own.  The columns go through packed instructions in pairs;
 // every column's sums run in the same order as alone.  24,000 columns, 256-atom
-// regions, nu = 30: 20.2 ms, 27.2 with a lane reading its own block; 4,000
-// columns, nu = 100: 13.1 (19.0).  The warps need nothing of each other, so a CTA
+// regions, nu = 30: 20.4 ms, 27.2 with a lane reading its own block; 4,000
+// columns, nu = 100: 13.2 (19.0).  An odd NC (an atom with fewer real orbitals, or
+// a run cut by the batch) takes its last column for both halves of a pair.  Groups
+// of one, two and three columns of 2,000 atoms: 4.6, 4.8 and 7.2 ms; one column
+// after another, a lane reading its own block, 7.5, 14.5 and 21.4.  (NC at run time
+// instead: 21.8 ms for the 24,000 columns.)  The warps need nothing of each other, so a CTA
 // is one: no CTA waits for its longest warp, and a few groups, or regions of few
 // rows, still spread over the SMs.  With a CTA of four warps per group that went
 // over all its rows: one atom of a 1,024-atom region, nu = 30, 3.4 ms, now 0.61;
@@ -400,28 +384,16 @@ __global__ void __launch_bounds__(256) spmm_regional_hs_kernel(
 // grid, so that they share the group's x in L2.
 constexpr int kRegPitch = 52;   // floats per staged block: H hi and lo, S hi, and 4 that spread the banks
 
-template <bool kS>
-__global__ void __launch_bounds__(32, 12) spmm_regional_group_kernel(
-    int n_reg, int maxrow, const int *__restrict__ lcnt, const int *__restrict__ lci,
-    const int *__restrict__ lgk, const float *__restrict__ Hv, const float *__restrict__ Sv,
-    const float *__restrict__ X, int64_t ldx, float *__restrict__ U, float *__restrict__ Ulo, int64_t ldu,
-    float *__restrict__ SY, int64_t ldsy, int ncols, const int *__restrict__ gstart,
+template <bool kS, int NC>
+__device__ __forceinline__ void group_rows(
+    float *blk, int p, int c0, int n_reg, int maxrow, const int *__restrict__ lcnt,
+    const int *__restrict__ lci, const int *__restrict__ lgk, const float *__restrict__ Hv,
+    const float *__restrict__ Sv, const float *__restrict__ X, int64_t ldx, float *__restrict__ U,
+    float *__restrict__ Ulo, int64_t ldu, float *__restrict__ SY, int64_t ldsy, int ncols,
     const uint8_t *__restrict__ thop, const uint16_t *__restrict__ tinv, int lim)
 {
-    constexpr int G = reg_group<float>(), kPieces = kS ? 12 : 8;
-    static_assert(G == 4, "two pairs of columns");
-    __shared__ __align__(16) float blk[2 * 32 * kRegPitch];   // two stages of 32 blocks
-    const int lane = threadIdx.x, g = blockIdx.y, p = 32 * (int)blockIdx.x + lane;
-    // clipped to ncols: a run of the autotuner covers the batch's first columns only
-    const int c0 = gstart[g], c1 = min(gstart[g + 1], ncols);
-    if (c0 >= c1) return;
-    if (c1 - c0 < G) {   // an atom with fewer real orbitals, or a run cut by the batch: column by column
-        if (p < n_reg)
-            for (int c = c0; c < c1; ++c)
-                regional_rows<float, kS, 1>(p, c, n_reg, maxrow, lcnt, lci, lgk, Hv, Sv, X, ldx, U, Ulo, ldu, SY,
-                                            ldsy, ncols, thop, tinv, lim);
-        return;
-    }
+    constexpr int kPieces = kS ? 12 : 8, NP = (NC + 1) / 2, G = 2 * NP;
+    const int lane = threadIdx.x;
     const float *xc = X + (int64_t)c0 * ldx;
     const int64_t base = (int64_t)c0 * maxrow * n_reg;
     const uint32_t sb = (uint32_t)__cvta_generic_to_shared(blk);
@@ -429,9 +401,9 @@ __global__ void __launch_bounds__(32, 12) spmm_regional_group_kernel(
     const bool act = row && (int)thop[(int64_t)(p >> 3) * ncols + c0] <= lim;
     const int cnt = act ? lcnt[(int64_t)c0 * n_reg + p] : 0;
     const int most = __reduce_max_sync(kFull, cnt);
-    uint64_t hi[2][4], lo[2][4], sy[2][4];   // column pairs (0, 1) and (2, 3)
+    uint64_t hi[NP][4], lo[NP][4], sy[NP][4];   // column pairs (0, 1) and (2, 3)
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+    for (int h = 0; h < NP; ++h)
 #pragma unroll
         for (int a = 0; a < 4; ++a) hi[h][a] = lo[h][a] = sy[h][a] = 0;
     auto block_of = [&](int s) { return s < cnt ? lgk[base + (int64_t)s * n_reg + p] : -1; };
@@ -459,7 +431,7 @@ __global__ void __launch_bounds__(32, 12) spmm_regional_group_kernel(
     auto gather = [&](int xp, float4 (&x)[G]) {
 #pragma unroll
         for (int m = 0; m < G; ++m)
-            if (xp >= 0) x[m] = __ldg(reinterpret_cast<const float4 *>(xc + m * ldx + xp));
+            if (xp >= 0) x[m] = __ldg(reinterpret_cast<const float4 *>(xc + (m < NC ? m : NC - 1) * ldx + xp));
     };
     // blocks are copied one slot ahead, x one, the positions two, the indices three
     copy(0, block_of(0));
@@ -477,9 +449,9 @@ __global__ void __launch_bounds__(32, 12) spmm_regional_group_kernel(
         asm volatile("cp.async.wait_group 1;" ::: "memory");
         __syncwarp();
         if (x0p >= 0) {
-            uint64_t x[2][4], nx[2][4];
+            uint64_t x[NP][4], nx[NP][4];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            for (int h = 0; h < NP; ++h) {
                 const float4 u = xv[2 * h], v = xv[2 * h + 1];
                 x[h][0] = pack_x2(u.x, v.x);
                 x[h][1] = pack_x2(u.y, v.y);
@@ -503,11 +475,11 @@ __global__ void __launch_bounds__(32, 12) spmm_regional_group_kernel(
                 for (int e = 0; e < 4; ++e) {
                     const uint64_t hp = pack_x2(hv[e], hv[e]), lp = pack_x2(lv[e], lv[e]);
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) spmm_add(hi[h][a], lo[h][a], hp, lp, x[h][e], nx[h][e]);
+                    for (int h = 0; h < NP; ++h) spmm_add(hi[h][a], lo[h][a], hp, lp, x[h][e], nx[h][e]);
                     if constexpr (kS) {
                         const uint64_t sp = pack_x2(sv[e], sv[e]);
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) sy[h][a] = fma_x2(sp, x[h][e], sy[h][a]);
+                        for (int h = 0; h < NP; ++h) sy[h][a] = fma_x2(sp, x[h][e], sy[h][a]);
                     }
                 }
             }
@@ -520,7 +492,7 @@ __global__ void __launch_bounds__(32, 12) spmm_regional_group_kernel(
     if (!row) return;
     const int64_t yp = 32 * (int64_t)tinv[(int64_t)(p >> 3) * ncols + c0] + 4 * (p & 7);
 #pragma unroll
-    for (int m = 0; m < G; ++m) {
+    for (int m = 0; m < NC; ++m) {
         const int64_t c = c0 + m;
         float yh[4], yl[4], ys[4];
 #pragma unroll
@@ -535,6 +507,32 @@ __global__ void __launch_bounds__(32, 12) spmm_regional_group_kernel(
         store4(U + c * ldu + yp, yh);
         store4(Ulo + c * ldu + yp, yl);
         if constexpr (kS) store4(SY + c * ldsy + yp, ys);
+    }
+}
+
+template <bool kS>
+__global__ void __launch_bounds__(32, 12) spmm_regional_group_kernel(
+    int n_reg, int maxrow, const int *__restrict__ lcnt, const int *__restrict__ lci,
+    const int *__restrict__ lgk, const float *__restrict__ Hv, const float *__restrict__ Sv,
+    const float *__restrict__ X, int64_t ldx, float *__restrict__ U, float *__restrict__ Ulo, int64_t ldu,
+    float *__restrict__ SY, int64_t ldsy, int ncols, const int *__restrict__ gstart,
+    const uint8_t *__restrict__ thop, const uint16_t *__restrict__ tinv, int lim)
+{
+    static_assert(reg_group<float>() == 4, "two pairs of columns");
+    __shared__ __align__(16) float blk[2 * 32 * kRegPitch];   // two stages of 32 blocks
+    const int g = blockIdx.y, p = 32 * (int)blockIdx.x + (int)threadIdx.x;
+    // clipped to ncols: a run of the autotuner covers the batch's first columns only
+    const int c0 = gstart[g], nc = min(gstart[g + 1], ncols) - c0;
+    auto rows = [&](auto n) {
+        group_rows<kS, decltype(n)::value>(blk, p, c0, n_reg, maxrow, lcnt, lci, lgk, Hv, Sv, X, ldx, U, Ulo, ldu, SY,
+                                           ldsy, ncols, thop, tinv, lim);
+    };
+    switch (nc) {
+    case 4: rows(std::integral_constant<int, 4>()); break;
+    case 3: rows(std::integral_constant<int, 3>()); break;
+    case 2: rows(std::integral_constant<int, 2>()); break;
+    case 1: rows(std::integral_constant<int, 1>()); break;
+    default: break;   // past ncols
     }
 }
 
