@@ -238,11 +238,11 @@ __global__ void __launch_bounds__(kTriThreads) eig_tridiag_kernel(
     }
 }
 
-// 1 / sqrt(a) and 1 / a of normal numbers from the hardware's 20-bit estimates
-// by one step of third order (the binomial series of (1 - e)^(-1/2) and
-// (1 - e)^(-1) in the estimate's defect e, cut after e^2): what is left is the
-// rounding, about 1 ulp.  Few FP64 instructions (five and three) and no branch
-// for special values.
+// 1 / sqrt(a) and 1 / a of normal numbers (with normal results) from the
+// hardware's 20-bit estimates by one step of third order (the binomial series of
+// (1 - e)^(-1/2) and (1 - e)^(-1) in the estimate's defect e, cut after e^2): what
+// is left is rounding, within 1.05 and 0.55 units of the last place.  Few FP64
+// instructions (five and three) and no branch for special values.
 __device__ __forceinline__ double series_rsqrt(double a)
 {
     double y;

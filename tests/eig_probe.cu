@@ -1,5 +1,6 @@
 // Host entries for the tests of the eigensolver's device code, one translation unit with it:
-// eig_probe_ql runs the batched QL kernel on tridiagonal matrices given from the host.
+// eig_probe_ql runs the batched QL kernel on tridiagonal matrices given from the host,
+// eig_probe_series the reciprocals of its rotations.
 #include "eigsub.cu"
 
 #include <vector>
@@ -58,4 +59,31 @@ extern "C" int eig_probe_ql(int nb, int n, int nl, int bits, double *d, double *
     case 8: return ql<8>(nb, n, nl, d, e, nsweep);
     default: return -1;
     }
+}
+
+static __global__ void series_kernel(int n, const double *x, double *out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    out[i] = x[i] > 0.0 ? series_rsqrt(x[i]) : 0.0;
+    out[n + i] = x[i] > 0.0 ? rsqrt(x[i]) : 0.0;
+    out[2 * n + i] = series_rcp(x[i]);
+    out[3 * n + i] = 1.0 / x[i];
+}
+
+// out [4][n]: series_rsqrt and CUDA's rsqrt (0 for x <= 0), series_rcp and 1 / x.
+extern "C" int eig_probe_series(int n, const double *x, double *out)
+{
+    double *X = nullptr, *Y = nullptr;
+    cudaError_t err = cudaMalloc(&X, n * sizeof(double));
+    if (!err) err = cudaMalloc(&Y, 4 * n * sizeof(double));
+    if (!err) err = cudaMemcpy(X, x, n * sizeof(double), cudaMemcpyHostToDevice);
+    if (!err) {
+        series_kernel<<<(n + 255) / 256, 256>>>(n, X, Y);
+        err = cudaGetLastError();
+    }
+    if (!err) err = cudaMemcpy(out, Y, 4 * n * sizeof(double), cudaMemcpyDeviceToHost);
+    cudaFree(X);
+    cudaFree(Y);
+    return (int)err;
 }

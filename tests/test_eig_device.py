@@ -2,8 +2,10 @@
 ever holds, but the code has to take."""
 
 import ctypes as C
+import math
 import os
 import subprocess
+from decimal import Decimal, getcontext
 
 import numpy as np
 import pytest
@@ -66,3 +68,34 @@ def test_every_lost_scale_is_reported(probe, n, bits):
     np.testing.assert_array_equal(w, w0)
     assert np.all(ns0 >= 0)
     np.testing.assert_array_equal(ns < 0, np.abs(w).min(axis=1) < 2.0 ** -bits)
+
+
+def _ulps(got, exact):
+    """|got - exact| in units of got's last place; exact in 50 digits."""
+    return np.array([float(abs(Decimal(float(g)) - e) / Decimal(math.ulp(float(g)))) for g, e in zip(got, exact)])
+
+
+def test_series_reciprocals(probe):
+    """series_rsqrt and series_rcp over mantissas, signs and the exponents whose results are normal.
+    With a 20-bit estimate, e = 1 - a y^2 is about 2^-19 and known to 2^-53: half of that on the result
+    is at most half a unit of its last place, the last rounding another half, what the series leaves out
+    (5/16 e^3) 0.02.  e = 1 - a y is exact to 2^-73: half a unit, and e^3 = 0.008.  CUDA's rsqrt is within
+    one unit, its quotient correctly rounded."""
+    rng = np.random.default_rng(0)
+    edge = np.array([1.0, 1.0 + 2.0 ** -52, 1.5, np.sqrt(2.0), 2.0 - 2.0 ** -52])
+    near = np.concatenate([rng.uniform(1.0, 2.0, 4000), np.linspace(1.0, 2.0, 2000, endpoint=False)])
+    x = np.concatenate([
+        np.ldexp(np.tile(edge, 2044), np.repeat(np.arange(-1021, 1023), edge.size) - 1),   # every exponent
+        near, 2.0 * near,
+        np.ldexp(rng.uniform(1.0, 2.0, 6000), rng.integers(-1021, 1020, 6000))])
+    x = np.concatenate([x, -x[::7]])
+    out = np.zeros((4, x.size))
+    assert probe.eig_probe_series(x.size, _ptr(x), _ptr(out)) == 0
+    getcontext().prec = 50
+    pos = x > 0
+    d = [Decimal(float(v)) for v in x]
+    root = [1 / v.sqrt() for v, p in zip(d, pos) if p]
+    assert _ulps(out[0][pos], root).max() <= 1.05
+    assert (np.abs(out[0] - out[1])[pos] / np.spacing(out[1][pos])).max() <= 2.05
+    assert _ulps(out[2], [1 / v for v in d]).max() <= 0.55
+    assert (np.abs(out[2] - out[3]) / np.spacing(np.abs(out[3]))).max() <= 1.05
