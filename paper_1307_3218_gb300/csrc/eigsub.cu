@@ -469,6 +469,18 @@ __global__ void __launch_bounds__(64) eig_ql_kernel(const int *__restrict__ bnu_
 #undef WW
 }
 
+size_t ql_smem(int nu, int nl) { return (size_t)3 * nu * nl * sizeof(double); }
+
+// Subspaces per warp: as few as leave one warp per SM (a sweep of the warp is
+// as long as its longest lane's), 16 when 32 would not fit a CTA's shared
+// memory beside the kernel's 1.2 KB of static arrays (nu above 300).
+int ql_lanes(int nu, int nb2)
+{
+    int nl = ql_smem(nu, 32) + 2048 > (size_t)227 * 1024 ? 16 : 32;
+    while (nl > 1 && (nb2 + nl / 2 - 1) / (nl / 2) <= kQlWarps) nl /= 2;
+    return nl;
+}
+
 // ------------------------------------------------------------------ levels
 // A CTA per subspace: eps in ascending order (ties by index; a NaN level, from
 // non-finite input, ranks as +inf, so that the ranks always form a
@@ -739,14 +751,11 @@ cudaError_t launch_eig(const DeviceMatrix &A, const KrylovBatch &b, const Column
         const int nb2 = b.nb - cofs < es.chunk ? b.nb - cofs : es.chunk;
         eig_tridiag_kernel<<<nb2, tthreads, tsmem, s>>>(b.Hsub, b.nu_eff, nu, cofs, es.D, es.E, es.V, es.Ag, b.Lsub);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        // subspaces per warp: as few as leave one warp per SM (a sweep of the
-        // warp is as long as its longest lane's), 16 when 32 would not fit
-        int nl = 3 * (size_t)nu * 32 * sizeof(double) > (size_t)227 * 1024 ? 16 : 32;
-        while (nl > 1 && (nb2 + nl / 2 - 1) / (nl / 2) <= kQlWarps) nl /= 2;
-        const size_t qsmem = (size_t)3 * nu * nl * sizeof(double);
+        const int nl = ql_lanes(nu, nb2);
+        const size_t qsmem = ql_smem(nu, nl);
         if ((e = allow_dynamic_smem((const void *)eig_ql_kernel<kScaleBits>, qsmem)) != cudaSuccess) return e;
-        eig_ql_kernel<kScaleBits><<<(nb2 + nl - 1) / nl, 64, qsmem, s>>>(b.nu_eff, cofs, nb2, nu, nl, es.D, es.E, es.rot,
-                                                            es.rcap, es.sweep, es.scap, es.nsweep);
+        eig_ql_kernel<kScaleBits><<<(nb2 + nl - 1) / nl, 64, qsmem, s>>>(
+            b.nu_eff, cofs, nb2, nu, nl, es.D, es.E, es.rot, es.rcap, es.sweep, es.scap, es.nsweep);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         const size_t rsmem = (size_t)2 * nu * sizeof(double);
         eig_rank_kernel<<<nb2, std::min(128, (nu + 31) / 32 * 32), rsmem, s>>>(

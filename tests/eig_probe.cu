@@ -87,3 +87,6 @@ extern "C" int eig_probe_series(int n, const double *x, double *out)
     cudaFree(Y);
     return (int)err;
 }
+
+// Dynamic shared memory of the QL kernel for a chunk of nb subspaces (no GPU needed).
+extern "C" int64_t eig_probe_ql_smem(int nu, int nb) { return (int64_t)ql_smem(nu, ql_lanes(nu, nb)); }
