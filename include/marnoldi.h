@@ -54,7 +54,7 @@ typedef enum {
     MARNOLDI_ENOTSPD = -2,   /* S shown not positive definite */
     MARNOLDI_ENOMEM = -3,    /* device or host allocation failed */
     MARNOLDI_ECUDA = -4,     /* a CUDA call failed */
-    MARNOLDI_ETIMEOUT = -5,  /* a bounded device loop ran out of iterations */
+    MARNOLDI_ETIMEOUT = -5,  /* reserved: no function returns it any more */
     MARNOLDI_ESTATE = -6,    /* call out of order (e.g. density before solve) */
     MARNOLDI_ENOCONV = -7,   /* the subspace eigensolver or the bisection did not converge */
     MARNOLDI_EPENDING = -8   /* a server request has not finished within the wait's timeout */

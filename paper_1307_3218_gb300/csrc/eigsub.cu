@@ -59,10 +59,10 @@ __device__ __forceinline__ double warp_sum(double s)
 // memory lets five CTAs share an SM at nu = 100 (two with the square), whose
 // phases between barriers then overlap: 16.5 ms for 4,000 subspaces, 27.5 with
 // the square.
-// Shared memory: A, v, e, q.  When A and R do not fit one CTA's shared memory
-// (nu above about 110), A lives in a global scratch per subspace (Ag), which
-// the CTA's sweeps keep in L2 (360 KB at nu = 300).  A thread per row of A: the
-// CTA has as many threads as nu needs.
+// Shared memory: A, v, e, q; where eig_smem_bytes says so (nu above 145 for
+// 12 blocks per row, 126 for 24) A lives in a global scratch per subspace (Ag)
+// instead, which the CTA's sweeps keep in L2 (360 KB at nu = 300).  A thread per
+// row of A: the CTA has as many threads as nu needs.
 // Reflector k goes to V[sc][k][0 .. n - k - 2], tau_k to V[sc][k][nu - 1].
 __device__ __forceinline__ int tri(int i) { return i * (i + 1) / 2; }
 
@@ -728,14 +728,14 @@ cudaError_t apply_dispatch(const DeviceMatrix &A, const KrylovBatch &b, const Co
 
 }  // namespace
 
-// What a solve is refused by: the shared memory that H_sub (unless a_global)
-// and the rows of R take together with their vectors.
+// The measure that a solve is refused by and that decides where A lives: the
+// full square of H_sub (unless a_global), all rows of R and three vectors in one
+// CTA's shared memory.  No kernel holds as much (A is a triangle, which would fit
+// up to nu = 237, and the rows go 32 at a time); which solves are accepted, and A's
+// place, have stayed as they were.
 size_t eig_smem_bytes(int nu, int nr_max, bool a_global)
 {
-    const size_t lda = (size_t)(nu | 1);
-    const size_t tri = ((size_t)((a_global ? 0 : nu) + nr_max) * lda + 3 * (size_t)nu) * sizeof(double);
-    const size_t ql = (size_t)2 * nu * 32 * sizeof(double);
-    return std::max(tri, ql);
+    return ((size_t)((a_global ? 0 : nu) + nr_max) * (size_t)(nu | 1) + 3 * (size_t)nu) * sizeof(double);
 }
 
 cudaError_t launch_eig(const DeviceMatrix &A, const KrylovBatch &b, const ColumnState &st,

@@ -44,7 +44,6 @@ template <> struct DotAcc<double> {
     }
     __device__ __forceinline__ double pack() const { return s; }
     __device__ __forceinline__ void unpack(double p) { s = p; }
-    __device__ __forceinline__ void set(double x) { s = x; }
 };
 template <> struct DotAcc<float> {
     float hi = 0.f, lo = 0.f;
@@ -55,8 +54,6 @@ template <> struct DotAcc<float> {
         df_add(hi, lo, p, e);
     }
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-    // fold in a correction of about 2^-24 relative to the sum
-    __device__ __forceinline__ void add_lo(float x) { lo = __fadd_rn(lo, x); }
     __device__ __forceinline__ void merge(const DotAcc &o) { df_add(hi, lo, o.hi, o.lo); }
     __device__ __forceinline__ DotAcc shfl_xor(int o) const
     {

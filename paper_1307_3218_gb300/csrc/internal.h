@@ -61,8 +61,8 @@ int footprint_of(const PatternStats &st, int precision, int nu, int region_atoms
 // only grows, and callers on several threads may race: one lock orders them.
 cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes);
 
-// Largest subspace dimension.  Up to about 110 the subspace matrix of the
-// eigensolve sits in shared memory, above that in a global scratch.
+// Largest subspace dimension.  The subspace matrix of the eigensolve sits in
+// shared memory or, for larger nu (eig_smem_bytes), in a global scratch.
 constexpr int kMaxNu = 320;
 // Largest Krylov-vector length of global mode (one CTA holds a column's vector).
 constexpr int64_t kMaxGlobalM = 16384;
@@ -309,7 +309,7 @@ struct ColumnState {
     int *eig_status;     // bits: 1 QL did not converge, 2 non-positive S norm
 };
 
-// Scratch of the three-kernel eigensolve, per chunk of subspaces:
+// Scratch of the eigensolve's kernels, per chunk of subspaces:
 //   D, E [chunk][nu] (tridiagonal, then levels and column scales), V [chunk][nu]
 //   [nu] (Householder reflectors), rot [chunk][rcap] rotations, sweep
 //   [chunk][scap] (m, lo), nsweep [chunk] (-1: QL failed).
@@ -327,8 +327,8 @@ struct EigScratch {
     const double *proj = nullptr;
     double *proj_out = nullptr;
 };
-// Shared memory that bounds nu and the pattern rows, with H_sub in shared
-// (a_global = false) or global memory.
+// The measure against a CTA's shared memory that bounds nu and the pattern rows,
+// with H_sub in shared (a_global = false) or global memory.
 size_t eig_smem_bytes(int nu, int nr_max, bool a_global);
 
 cudaError_t launch_eig(const DeviceMatrix &A, const KrylovBatch &b, const ColumnState &st,
