@@ -984,6 +984,9 @@ cudaError_t gs_dispatch(const KrylovBatch &b, int n, int need_w, double tau, cud
 // columns 21.7 -> 12.3 (13.7 with two groups).  With more columns the CTAs run in
 // two turns, or three: 300 columns, FP64, 4,096 entries, nu = 100 54.9 -> 46.8,
 // but 1,024 entries, nu = 60 6.8 -> 9.6; 340 columns 68.9 -> 69.7 and 7.8 -> 13.9.
+// 16,384 FP32 entries (256 pairs of chains), nu = 30, 1 column 3.2 -> 1.8, 150
+// columns 3.6 -> 2.25; nu = 100 36.8 -> 18.4 and 39.0 -> 21.8 (21.8 and 24.2 with
+// two groups and three ring stages; four groups leave room for two).
 // FP64 shapes of 512 chains (only an autotuner's choice) would not fit the ring.
 constexpr int kGsFewColumns = 152;
 
@@ -1063,9 +1066,12 @@ cudaError_t launch_spmm_hs(const DeviceMatrix &A, const KrylovBatch &b, void *SY
 
 cudaError_t launch_gs(const KrylovBatch &b, int n, int need_w, double tau, cudaStream_t s)
 {
-    if (gs_pair_shape(b.shape, b.prec))
+    if (gs_pair_shape(b.shape, b.prec)) {
+        if (b.shape.threads == 288 && b.nb <= kGsFewColumns)   // see gs_shape
+            return gs_dispatch<float, 512, 2, 4, true>(b, n, need_w, tau, s);
         return b.shape.threads == 288 ? gs_dispatch<float, 512, 3, 1, true>(b, n, need_w, tau, s)
                                       : gs_dispatch<float, 1024, 3, 1, true>(b, n, need_w, tau, s);
+    }
     return b.prec == 0 ? gs_shape<double>(b, n, need_w, tau, s) : gs_shape<float>(b, n, need_w, tau, s);
 }
 

@@ -15,6 +15,8 @@ pytestmark = pytest.mark.gpu
     (45, 3, 0, 0), (45, 3, 0, 1), (60, 34, 0, 0), (64, 33, 0, 1),       # vectors of 256 entries
     (250, 70, 0, 0), (250, 70, 0, 1), (500, 37, 0, 0), (505, 40, 0, 1), (1001, 30, 0, 0), (1001, 66, 0, 1),
     (1500, 30, 0, 1), (2048, 20, 0, 1),                                 # 8,192 FP32 entries
+    (2100, 34, 0, 1), (4001, 24, 0, 1),                                 # 16,384, chains in pairs
+    (1000, 320, 0, 0), (1500, 320, 0, 1), (2049, 320, 0, 1),            # the most shared memory
     (600, 20, 300, 0), (600, 20, 300, 1), (90, 257, 0, 0), (90, 260, 0, 1), (48, 12, 0, 0),
 ])
 def test_bits_do_not_depend_on_the_column_count(atoms, nu, region, prec):
