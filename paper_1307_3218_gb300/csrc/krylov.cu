@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(32 * W, (sizeof(VT) == 4 ? 20 : 16) / W) spmm_
 
 // ------------------------------------------------------------------ Gram-Schmidt
 // One CTA per column, of G groups of T = C / 4 threads, for vectors of m_pad =
-// nchunk C entries; G = 1, or 4 where columns are few (gs_shape).  The groups
+// nchunk C entries; G = 1, or 2 or 4 where columns are few (gs_shape).  The groups
 // share a step's work without touching a sum: in sweep 1 they take the blocks of
 // stored vectors in turn, in sweep 2 the passes of four chunks (whose sums a_i
 // are then added in the order of the passes at the end), and the scalar step
@@ -416,7 +416,7 @@ struct GsCfg {
     // registers: FP32 96 (FP32 at 80: 54.8 against 46.6 ms on 8,192-entry
     // vectors), FP64 (bound by its pipe, which few warps fill) about 150, but two
     // CTAs for C = 1024 (91 against 96 ms on 16,384-entry vectors)
-    static constexpr int kMinCtas = G > 1 ? 1 : sizeof(VT) == 4 ? 640 / T : C == 1024 ? 2 : 416 / T;
+    static constexpr int kMinCtas = G > 1 ? 2 : sizeof(VT) == 4 ? 640 / T : C == 1024 ? 2 : 416 / T;
     static constexpr __host__ __device__ int parts(int nu, int nchunk)   // doubles
     {
         const int a = nu * NW * (G > 1 ? (nchunk + kPass - 1) / kPass : 1);
@@ -974,20 +974,25 @@ cudaError_t gs_dispatch(const KrylovBatch &b, int n, int need_w, double tau, cud
 // other (24,000 columns, nu = 30: 28.9 ms against 32.6 with three), three above
 // (2,048 columns of 2,048 entries, nu = 100: 44.9 ms against 48.3 with two).
 //
-// At most one column per SM: four groups of threads per CTA.  One group's two
-// warps reach two of the SM's four schedulers and hide little of each other's
-// latency, where nothing else runs on the SM.  Gram-Schmidt of a solve with one
-// group and with four (the Krylov vectors' bits are the same): FP64, 4,096
-// entries, nu = 200, 1 column 214 -> 90 ms, 150 columns 218 -> 92; nu = 30, 1
-// column 4.9 -> 2.4; 1,024 entries, nu = 30, 150 columns 1.78 -> 1.45; mixed,
-// 4,096 entries, nu = 100, 1 column 21.7 -> 7.6; 8,192 entries, nu = 100, 150
-// columns 21.7 -> 12.3 (13.7 with two groups).  With more columns the CTAs run in
-// two turns, or three: 300 columns, FP64, 4,096 entries, nu = 100 54.9 -> 46.8,
-// but 1,024 entries, nu = 60 6.8 -> 9.6; 340 columns 68.9 -> 69.7 and 7.8 -> 13.9.
-// 16,384 FP32 entries (256 pairs of chains), nu = 30, 1 column 3.2 -> 1.8, 150
-// columns 3.6 -> 2.25; nu = 100 36.8 -> 18.4 and 39.0 -> 21.8 (21.8 and 24.2 with
-// two groups and three ring stages; four groups leave room for two).
-// FP64 shapes of 512 chains (only an autotuner's choice) would not fit the ring.
+// At most one column per SM: as many groups of threads as make eight warps, for
+// vectors of more than 1,024 entries.  One group's two (four) warps reach two of
+// the SM's four schedulers, or hide little of each other's latency, where nothing
+// else runs on the SM.  Gram-Schmidt of a solve with one group and with several
+// (the Krylov vectors' bits are the same): FP64, 4,096 entries, nu = 200, 1 column
+// 214 -> 90 ms, 150 columns 218 -> 92; nu = 30, 1 column 4.9 -> 2.4; mixed, 4,096
+// entries, nu = 100, 1 column 21.7 -> 7.8; 8,192 entries, nu = 100, 1 column 20.9 ->
+// 13.1, 150 columns 21.7 -> 14.0; 16,384 entries (256 pairs of chains), nu = 30, 1
+// column 3.2 -> 2.1, 150 columns 3.6 -> 2.5.
+// - Two CTAs per SM (at most 128 registers): solves of few columns also run side by
+//   side on several streams.  Mixed, 4,096 entries, nu = 60, 150 columns: one CTA
+//   per SM is 3 % faster alone, but eight streams take 46 ms per solve, with two
+//   CTAs 41 (one group 42).  8,192 entries: sixteen warps are 17 % faster alone, but
+//   four streams take 35 ms, with eight warps 31.5 (one group 31).
+// - Up to 1,024 entries alone 1.78 -> 1.45 ms (FP64, nu = 30, 150 columns), but four
+//   streams of such solves (nu = 60) 24.8 -> 26.7 ms per solve.
+// - With more columns the CTAs run in turns: 300 columns, FP64, nu = 100, 4,096
+//   entries 54.9 -> 46.8, but 340 columns 68.9 -> 69.7.
+// FP64 shapes of 512 chains (only an autotuner's choice) keep one group.
 constexpr int kGsFewColumns = 152;
 
 template <typename VT>
@@ -998,12 +1003,12 @@ cudaError_t gs_shape(const KrylovBatch &b, int n, int need_w, double tau, cudaSt
     const bool few = b.nb <= kGsFewColumns;
     switch (b.shape.threads) {
     case 256:
-        if (few) return gs_dispatch<VT, 256, R, 4>(b, n, need_w, tau, s);
+        if (few && b.shape.m_pad > 1024) return gs_dispatch<VT, 256, R, 4>(b, n, need_w, tau, s);
         if (R == 3 && b.shape.m_pad <= 1024) return gs_dispatch<VT, 256, 2>(b, n, need_w, tau, s);
         return gs_dispatch<VT, 256, R>(b, n, need_w, tau, s);
     case 512:
         if constexpr (sizeof(VT) == 4)
-            if (few) return gs_dispatch<VT, 512, R, 4>(b, n, need_w, tau, s);
+            if (few) return gs_dispatch<VT, 512, R, 2>(b, n, need_w, tau, s);
         return gs_dispatch<VT, 512, R>(b, n, need_w, tau, s);
     case 1024: return gs_dispatch<VT, 1024, R>(b, n, need_w, tau, s);
     default: return cudaErrorInvalidValue;
@@ -1068,7 +1073,7 @@ cudaError_t launch_gs(const KrylovBatch &b, int n, int need_w, double tau, cudaS
 {
     if (gs_pair_shape(b.shape, b.prec)) {
         if (b.shape.threads == 288 && b.nb <= kGsFewColumns)   // see gs_shape
-            return gs_dispatch<float, 512, 2, 4, true>(b, n, need_w, tau, s);
+            return gs_dispatch<float, 512, 3, 2, true>(b, n, need_w, tau, s);
         return b.shape.threads == 288 ? gs_dispatch<float, 512, 3, 1, true>(b, n, need_w, tau, s)
                                       : gs_dispatch<float, 1024, 3, 1, true>(b, n, need_w, tau, s);
     }
