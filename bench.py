@@ -40,16 +40,21 @@ UNIT = "columns/s"
 L2_FLUSH_BYTES = 256 << 20
 FP64_PEAK_NOTE = "152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz (nominal 1.25 TFLOP/s FP64)"
 # (dram__bytes_read + dram__bytes_write) / algorithmic bytes of one captured
-# Gram-Schmidt launch (ncu --set full, mixed precision, 608 columns, step n = 20,
-# algorithmic 1.929072e9 B read + 0.039846e9 B written over the supports), per
-# precision and launch shape (values per thread, threads) of the kernel that was
+# Gram-Schmidt launch (ncu, mixed precision, 608 columns, step n = 20, algorithmic
+# 1.365740e9 B over the supports, two reads per stored vector), per precision and launch shape (values per thread, threads) of the kernel that was
 # captured; a shape without an entry reports no traffic.  An entry must be
 # re-measured (or removed) whenever its kernel changes.
-GS_DRAM_PER_ALGORITHMIC = {}
-GS_DRAM_KERNEL = {}
+# gs_kernel<float, 512, 3, 1, true> (64 x 288): (1.769197e9 + 0.070595e9) / 1.365740e9;
+# gs_kernel<float, 1024, 3, 1, true> (32 x 544): (1.597046e9 + 0.070813e9) / 1.365740e9.  Above 1 by
+# what of u, its lo word and w_n, read again with every block of four vectors, misses L2.
+GS_DRAM_PER_ALGORITHMIC = {("mixed", (64, 288)): 1.3471, ("mixed", (32, 544)): 1.2212}
+GS_DRAM_KERNEL = {(64, 288): "gs_kernel<float, 512, 3, 1, true>", (32, 544): "gs_kernel<float, 1024, 3, 1, true>"}
 # SHA-256 of the sources of each captured kernel; when they differ from the files
 # on disk the capture no longer describes the kernel and no traffic is reported
-GS_DRAM_SOURCES = {}
+_GS_SOURCES = {
+    "paper_1307_3218_gb300/csrc/krylov.cu": "a428e04975558670775fa1444ff54048e4ded7bc7c4045431ed7236ec472f68c",
+    "paper_1307_3218_gb300/csrc/gs_common.cuh": "3abeb45f32e3a8d4457a515260691e045faeb073bf951111c941c0b73cac06bc"}
+GS_DRAM_SOURCES = {(64, 288): _GS_SOURCES, (32, 544): _GS_SOURCES}
 
 
 def capture_current(shape) -> bool:
